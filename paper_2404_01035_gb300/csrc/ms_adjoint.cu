@@ -955,7 +955,7 @@ ms_status ms_grad(ms_ctx* c, const void* dphi_T, const void* dmu_T, double* dpar
       char* src = slots + (size_t)(k - 1) * c->state_bytes;
       if (!encode_step_maps(*c->kern, &tm, &tmi, src, m)) return fail(c, MS_ERR_CUDA, "cuTensorMapEncodeTiled failed");
       const double t = m.t0 + (double)(s0 + k - 1) * m.dt;
-      e = c->kern->launch(&tm, &tmi, c->args.data(), m, t,
+      e = c->kern->launch(&tm, &tmi, src, c->args.data(), m, t,
                           slots + (size_t)k * c->state_bytes, c->codes[cs],
                           c->codes[1 - cs], lg, st);
       if (e != cudaSuccess) return cuda_fail(c, e, "segment recompute");

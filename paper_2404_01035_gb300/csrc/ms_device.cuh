@@ -81,6 +81,8 @@ struct StepArgs {
   Real delta[P];
   unsigned char aniso[P];   // delta_ab != 0
   unsigned char rotated[P]; // rotation differs from identity
+  unsigned char apair[P][4];   // the anisotropic pairs (a, b, pair index), sorted by b
+  int n_apairs;
   Real rot[P][9];
   Real cw[NP][NP];          // obstacle: 16 gamma/pi^2, well: 18 gamma
   Real g3[NP][NP][NP];      // third-order coefficients (only if has_g3)

@@ -86,11 +86,12 @@ struct StepKernel {
   // Fill the launch-argument blob from the model (all constants).
   void (*fill)(void* blob, const HostModel& m, int zchunk, int* status);
   // Launch one step: tm = tensor map of the input state (tile box), tmi =
-  // its interface-box map (split variants; may be NULL otherwise), t = time
+  // its interface-box map (split variants; may be NULL otherwise), in = the
+  // input state itself, t = time
   // of the input state, out = destination buffer, codes_in / codes_out =
   // segment codes of the input / output state.
-  cudaError_t (*launch)(const CUtensorMap* tm, const CUtensorMap* tmi, void* blob, const HostModel& m, double t, void* out,
-                        const uint8_t* codes_in, uint8_t* codes_out, const LaunchGeom& lg,
+  cudaError_t (*launch)(const CUtensorMap* tm, const CUtensorMap* tmi, const void* in, void* blob, const HostModel& m,
+                        double t, void* out, const uint8_t* codes_in, uint8_t* codes_out, const LaunchGeom& lg,
                         cudaStream_t st);
   // Recompute the segment codes of a state loaded from outside.
   cudaError_t (*codes)(const void* state, const HostModel& m, uint8_t* codes, cudaStream_t st);

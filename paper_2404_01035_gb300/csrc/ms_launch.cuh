@@ -9,6 +9,7 @@
 #include "ms_at.cuh"
 #include "ms_diag.cuh"
 #include "ms_internal.h"
+#include "ms_rows.cuh"
 #include "ms_split.cuh"
 #include "ms_step.cuh"
 
@@ -54,6 +55,16 @@ void fill_args(void* blob, const HostModel& m, int zchunk, int* status) {
       g.aniso[p] = m.delta[a][b] != 0.0;
       g.rotated[p] = m.rotated[a][b];
       for (int k = 0; k < 9; ++k) g.rot[p][k] = (Real)m.rot[a][b][k];
+    }
+  g.n_apairs = 0;
+  for (int b = 1; b < NP; ++b)
+    for (int a = 0; a < b; ++a) {
+      const int q = pair_index<NP>(a, b);
+      if (!g.aniso[q]) continue;
+      unsigned char* e = g.apair[g.n_apairs++];
+      e[0] = (unsigned char)a;
+      e[1] = (unsigned char)b;
+      e[2] = (unsigned char)q;
     }
   for (int a = 0; a < NP; ++a)
     for (int b = 0; b < NP; ++b)
@@ -153,9 +164,33 @@ inline bool plain_model(const HostModel& m) {
   return !m.has_g3 && m.noise_amp == 0.0 && !m.el && !m.gg;
 }
 
+// One boundary energy for every pair and no triple term: the sums over pairs
+// factorise (k_gp_rows).
+inline bool uniform_gamma(const HostModel& m) {
+  for (int a = 0; a < m.N; ++a)
+    for (int b = 0; b < m.N; ++b)
+      if (a != b && m.gamma[a][b] != m.gamma[0][1]) return false;
+  return !m.has_g3;
+}
+
+// The interface rows of the split step by k_gp_rows (many phases, one boundary energy).
+template <int NP, int NM, bool ANISO>
+cudaError_t launch_rows(const StepArgs<float, NP, NM>& g, const void* in, int sms, cudaStream_t st) {
+  using Sh = RowsShape<NP, NM>;
+  auto k = k_gp_rows<NP, NM, ANISO>;
+  static int per_sm = 0;   // resident CTAs per SM
+  if (per_sm == 0) {
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, Sh::THREADS, 0);
+    if (e != cudaSuccess) return e;
+    per_sm = per_sm < 1 ? 1 : per_sm;
+  }
+  k<<<sms * per_sm, Sh::THREADS, 0, st>>>(g, reinterpret_cast<const float*>(in));
+  return cudaGetLastError();
+}
+
 // Fused step: one kernel updates every cell.
 template <int DIM, int NP, int NM, class Real, int TX, int TY>
-cudaError_t launch_step(const CUtensorMap* tm, const CUtensorMap*, void* blob, const HostModel& m, double t,
+cudaError_t launch_step(const CUtensorMap* tm, const CUtensorMap*, const void*, void* blob, const HostModel& m, double t,
                         void* out, const uint8_t* codes_in, uint8_t* codes_out, const LaunchGeom& lg,
                         cudaStream_t st) {
   using Sh = StepShape<DIM, NP, NM, Real, TX, TY>;
@@ -175,8 +210,8 @@ cudaError_t launch_step(const CUtensorMap* tm, const CUtensorMap*, void* blob, c
 // Split 3-D FP32 step: the bulk streaming kernel (tm = mu-only tile map),
 // then the interface kernel over the rows it listed (tmi = interface boxes).
 template <int NP, int NM, int TY>
-cudaError_t launch_split(const CUtensorMap* tm, const CUtensorMap* tmi, void* blob, const HostModel& m, double t,
-                         void* out, const uint8_t* codes_in, uint8_t* codes_out, const LaunchGeom& lg,
+cudaError_t launch_split(const CUtensorMap* tm, const CUtensorMap* tmi, const void* in, void* blob,
+                         const HostModel& m, double t, void* out, const uint8_t* codes_in, uint8_t* codes_out, const LaunchGeom& lg,
                          cudaStream_t st) {
   using Ss = StreamShape<NP, NM, TY>;
   using Si = IfaceShape<NP, NM, float>;
@@ -220,6 +255,10 @@ cudaError_t launch_split(const CUtensorMap* tm, const CUtensorMap* tmi, void* bl
   }
   const int v = plain ? 1 : 0;
   ks<<<dim3(lg.tiles, lg.zchunks), Ss::NTHREADS, Ss::SMEM_BYTES, st>>>(*tm, g);
+  if constexpr (two)
+    if (uniform_gamma(m))
+      return g.n_apairs ? launch_rows<NP, NM, true>(g, in, lg.iface_blocks, st)
+                        : launch_rows<NP, NM, false>(g, in, lg.iface_blocks, st);
   ki<<<lg.iface_blocks * iface_per_sm[v], Si::THREADS, Si::SMEM_BYTES, st>>>(*tmi, g);
   if constexpr (two) kf<<<lg.iface_blocks * full_per_sm[v], Si::THREADS, Si::SMEM_BYTES, st>>>(*tmi, g);
   return cudaGetLastError();

@@ -535,8 +535,8 @@ ms_status launch_one_step(ms_ctx* c) {
     ms_status es = elastic_solve(c, c->buf[src]);
     if (es != MS_OK) return es;
   }
-  cudaError_t e = c->kern->launch(&c->tm[src], &c->tmi[src], c->args.data(), c->m, c->t, c->buf[dst], c->codes[src],
-                                  c->codes[dst], c->lg, c->stream);
+  cudaError_t e = c->kern->launch(&c->tm[src], &c->tmi[src], c->buf[src], c->args.data(), c->m, c->t, c->buf[dst],
+                                  c->codes[src], c->codes[dst], c->lg, c->stream);
   if (e == cudaSuccess && c->m.at)
     e = c->kern->at(c->buf[src], c->args.data(), c->m, c->t, c->buf[dst], c->codes[src], c->codes[dst], c->lg,
                     c->stream);

@@ -530,7 +530,8 @@ __device__ __forceinline__ void box_bulk_mu(const Real* c, const Real* cf, Real*
 // work is shared by two launches: MODE 0 takes the rows whose box holds at
 // most kSparseK phases (the compact update) and moves the others to a second
 // list, which MODE 1 updates with the full one (each kernel's registers then
-// fit its own path).  The last CTA to finish clears its list (ticket in
+// fit its own path); with one gamma for every pair k_gp_rows takes all rows
+// instead.  The last CTA to finish clears its list (ticket in
 // list[1]), so the launches can be replayed from a CUDA graph.
 template <int DIM, int NP, int NM, class Real, int MODE, int FEAT = kFeatAll>
 __global__ void __launch_bounds__(IfaceShape<NP, NM, Real>::THREADS, IfaceShape<NP, NM, Real>::MIN_BLOCKS)
