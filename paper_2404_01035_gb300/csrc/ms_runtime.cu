@@ -467,9 +467,12 @@ int default_zchunk(const HostModel& m, const StepKernel& k) {
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long long tiles = (long long)((m.nx + k.tx - 1) / k.tx) * ((m.ny + k.ty - 1) / k.ty);
-  // aim for >= 8 CTAs per SM worth of work units, chunks of 8..64 planes
+  // aim for >= 8 CTAs per SM worth of work units, chunks of 8..64 planes (split
+  // step: of 4..64, its streaming kernel is short on small grids: 64^3 eutectic
+  // 24.7 us with 4, 28.8 with 8, 39.1 with 16)
   int zc = 64;
-  while (zc > 8 && tiles * ((m.nz + zc - 1) / zc) < 8ll * sms) zc /= 2;
+  const int least = k.split ? 4 : 8;
+  while (zc > least && tiles * ((m.nz + zc - 1) / zc) < 8ll * sms) zc /= 2;
   return std::min(zc, m.nz);
 }
 
@@ -671,7 +674,19 @@ ms_status ms_create(const ms_grid* grid, int n_phases, int n_components, const m
     ms_destroy(c);
     return r;
   }
-  s = apply_launch(c, k, 0);
+  // the split step where one is compiled (3-D FP32): faster than the fused
+  // kernels at every size measured on a GB300 (us a step, fused / split:
+  // eutectic 24^3 87 / 17, 150x133x97 158 / 80, 256^3 769 / 196; 8-phase
+  // multigrain 24^3 329 / 19, 128^3 1733 / 231, 384^3 3646 / 389).  A grid too
+  // large for its work-list entries, or without memory for the lists, gets the
+  // fused kernel.
+  const StepKernel* split = nullptr;
+  if (c->m.dim == 3 && list_entry_fits(c->m))
+    for (auto* v : step_variants(c->m.dim, c->m.N, c->m.NM, c->m.dtype))
+      if (v->split) split = v;
+  s = MS_ERR_UNSUPPORTED;
+  if (split) s = apply_launch(c, split, 0);
+  if (s != MS_OK) s = apply_launch(c, k, 0);
   if (s == MS_OK) s = elastic_setup(c);
   if (s != MS_OK) {
     std::string m = c->err;
