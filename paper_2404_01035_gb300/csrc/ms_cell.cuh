@@ -475,6 +475,18 @@ __device__ __forceinline__ void gradient_terms(const Acc& A, const StepArgs<Real
   centre_term<DIM, NP, NM, Real, S, FEAT, ALL>(g, dp, ph, gcr, mask, Gc);
 }
 
+// Elasticity: -sigma : eps*^b joins each phase potential, from its el_rank
+// fields at the cell (grid cell index `cell` of `cells`).
+template <int NP, int NM, class Real, class S>
+__device__ __forceinline__ void add_elastic(const StepArgs<Real, NP, NM>& g, unsigned long long cell,
+                                            unsigned long long cells, S* psi) {
+  for (int s = 0; s < g.el_rank; ++s) {
+    const Real p = g.elw[s * cells + cell];
+#pragma unroll
+    for (int b = 0; b < NP; ++b) psi[b] = psi[b] + g.elc[b][s] * p;
+  }
+}
+
 // S4-S5 of the cell update from the gradient terms: the potential
 // derivative, the driving force, the rate of Eq. (phi_eqn) / (tau eps), the
 // explicit Euler step and the projection.  ph, mc: the cell's phi^n and mu^n;
@@ -509,11 +521,10 @@ __device__ __forceinline__ void phase_update(const StepArgs<Real, NP, NM>& g, co
   S psi[NP];
 #pragma unroll
   for (int b = 0; b < NP; ++b) psi[b] = gg ? S(Real(0)) : grand_potential<NP, NM, Real>(g, b, mc, s);
-  if ((FEAT & kFeatElastic) && g.elw) {   // elasticity: -sigma : eps*^b joins each phase potential
+  if ((FEAT & kFeatElastic) && g.elw) {
     const unsigned long long cell = gcell - (unsigned long long)g.zorg * (DIM == 3 ? (unsigned long long)g.nx * g.ny : g.nx);
     const unsigned long long cells = (unsigned long long)g.nx * g.ny * (DIM == 3 ? g.nz : 1);
-#pragma unroll
-    for (int b = 0; b < NP; ++b) psi[b] = psi[b] + g.elw[b * cells + cell];
+    add_elastic<NP, NM, Real, S>(g, cell, cells, psi);
   }
   S e1 = ph[0];
 #pragma unroll
@@ -921,11 +932,10 @@ __device__ __forceinline__ void gp_cell_sparse(const Acc& A, const StepArgs<Real
     Real psi[NP];
 #pragma unroll
     for (int b = 0; b < NP; ++b) psi[b] = gg ? Real(0) : grand_potential<NP, NM, Real>(g, b, mc, s);
-    if ((FEAT & kFeatElastic) && g.elw) {   // elasticity: -sigma : eps*^b joins each phase potential
+    if ((FEAT & kFeatElastic) && g.elw) {
       const unsigned long long cell = gcell - (unsigned long long)g.zorg * (DIM == 3 ? (unsigned long long)g.nx * g.ny : g.nx);
       const unsigned long long cells = (unsigned long long)g.nx * g.ny * (DIM == 3 ? g.nz : 1);
-#pragma unroll
-      for (int b = 0; b < NP; ++b) psi[b] += g.elw[b * cells + cell];
+      add_elastic<NP, NM, Real, Real>(g, cell, cells, psi);
     }
     Real e1 = ph[0];
 #pragma unroll

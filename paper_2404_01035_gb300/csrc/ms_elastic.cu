@@ -1,20 +1,32 @@
 // Elasticity with a homogeneous stiffness (MICROSIM paper, arXiv 2404.01035,
 // Sec. 2 "Elasticity implementation": the homogeneous case of its
-// Fourier-space equilibrium).  Before a step, from phi^n:
-//   1. k_el_eig:   eps*(x) = sum_a eps*^a h_a(phi)          (dense components)
-//   2. cuFFT R2C of every component
-//   3. k_el_spec:  t_i = C_ijmn k_j eps*_mn, G = (C_ijkl k_j k_l)^-1,
-//                  eps_kl = (k_k (G t)_l + k_l (G t)_k) / 2, zero at k = 0
-//                  (no homogeneous strain), Nyquist wavenumbers taken as 0
-//   4. cuFFT C2R back to the periodic strain
-//   5. k_el_force: sigma = C (eps - eps*), w_b = -sigma : eps*^b per phase,
-// and the step adds w_b to each phase potential psi_b, so that the phase rate
-// sees d f_el / d phi_a = sum_b w_b dh_b / dphi_a.  cuFFT is opened at run
-// time, so the library loads (and everything else runs) without it.
+// Fourier-space equilibrium).  The step needs w_b = -sigma : eps*^b of every
+// phase b, sigma = C (eps - eps*), where the strain eps is in equilibrium with
+// eps*(x) = sum_a eps*^a h_a(phi) (no homogeneous strain: zero at k = 0, and
+// Nyquist wavenumbers taken as 0).
+//
+// The eigenstrains of the phases span few directions (one, when all grains
+// share a dilatation): with a basis B^s of them, eps*^a = sum_s c_as B^s,
+//   eps*(x)  = sum_s e_s(x) B^s,             e_s = sum_a c_as h_a
+//   w_b      = -sum_s c_bs p_s(x),           p_s = B^s : sigma
+//   p_s(k)   = sum_s' [ (P^s k) . G(k) (P^s' k) - B^s : C : B^s' ] e_s'(k),
+// P^s = C : B^s, G = (C_ijkl k_j k_l)^-1, so the equilibrium takes rank
+// transforms each way instead of one per strain component (6 in 3-D), and no
+// pass over the cells after them.  Before a step:
+//   1. k_el_eig:  e_s(x), the constant of its phase where a segment code says
+//                 that the segment is pure
+//   2. cuFFT R2C of the rank fields
+//   3. k_el_spec: p_s(k) in place
+//   4. cuFFT C2R: p_s(x), which the step reads where it needs them.
+// What bounds it: memory passes.  7 grains with one dilatation, 128^3 FP32 on
+// a GB300, without the step: 230 us with one transform per component and
+// w_b stored per phase, see the figures at k_el_spec for this form.  cuFFT is
+// opened at run time, so the library loads (and everything else runs) without it.
 #include <cuda_runtime.h>
 #include <cufft.h>
 #include <dlfcn.h>
 
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 
@@ -58,43 +70,44 @@ const FftApi& fft_api() {
   return api;
 }
 
-// Symmetric components: 3-D (xx, yy, zz, yz, xz, xy), 2-D (xx, yy, xy).
-template <int DIM>
-struct Comp {
-  static constexpr int N = DIM == 3 ? 6 : 3;
-  __host__ __device__ static int index(int i, int j) {
-    if (i == j) return i;
-    if (DIM == 2) return 2;
-    const int s = i + j;   // (1,2) -> 3, (0,2) -> 4, (0,1) -> 5
-    return s == 3 ? 3 : (s == 2 ? 4 : 5);
-  }
-};
-
 template <class Real>
 struct ElConst {
+  Real c[kNMax][kElRank];          // e_s = sum_a c_as h_a
+  Real Pl[kElRank][3][3];          // B_ij C_ijkl
+  Real Pr[kElRank][3][3];          // C_ijkl B_kl
+  Real Q[kElRank][kElRank];        // B^s : C : B^s'
   Real C[3][3][3][3];
-  Real eig[kNMax][6];   // per phase, tensor components in Comp order
-  Real kstep[3];        // 2 pi / (n dx) per axis
-  int nx, ny, nz, nxh, pitch, nyp, xoff, zoff;
+  Real kstep[3];                   // 2 pi / (n dx) per axis
+  int rank, nx, ny, nz, nxh, pitch, nyp, xoff, zoff, segs;
   long long fstride, cells, ncplx;
 };
 
+// One warp per 32-cell row segment.
 template <int DIM, int NP, class Real>
-__global__ void k_el_eig(const ElConst<Real> q, const Real* __restrict__ st, Real* __restrict__ E) {
-  const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= q.cells) return;
-  const int x = (int)(idx % q.nx), y = (int)((idx / q.nx) % q.ny), z = (int)(idx / ((long long)q.nx * q.ny));
+__global__ void __launch_bounds__(256) k_el_eig(const __grid_constant__ ElConst<Real> q, const Real* __restrict__ st,
+                                                const uint8_t* __restrict__ codes, Real* __restrict__ E) {
+  const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (w >= (long long)q.segs * q.ny * q.nz) return;
+  const int sg = (int)(w % q.segs), y = (int)((w / q.segs) % q.ny), z = (int)(w / ((long long)q.segs * q.ny));
+  const int x = 32 * sg + lane;
+  if (x >= q.nx) return;
+  const long long idx = ((long long)z * q.ny + y) * q.nx + x;
+  const int code = codes[((long long)(z + q.zoff) * q.ny + y) * q.segs + sg] & kCodePhase;
+  if (code != 0) {   // the segment is pure: h is 1 for that phase, 0 for the others
+    for (int s = 0; s < q.rank; ++s) E[s * q.cells + idx] = q.c[code - 1][s];
+    return;
+  }
   const long long o = (long long)(DIM == 3 ? z + q.zoff : 0) * q.nyp * q.pitch + (long long)(y + 1) * q.pitch + x + q.xoff;
   Real ph[NP], h[NP];
 #pragma unroll
   for (int a = 0; a < NP; ++a) ph[a] = st[a * q.fstride + o];
   interp_h<NP>(ph, h);
-#pragma unroll
-  for (int c = 0; c < Comp<DIM>::N; ++c) {
+  for (int s = 0; s < q.rank; ++s) {
     Real e = Real(0);
 #pragma unroll
-    for (int a = 0; a < NP; ++a) e += h[a] * q.eig[a][c];
-    E[c * q.cells + idx] = e;
+    for (int a = 0; a < NP; ++a) e += h[a] * q.c[a][s];
+    E[s * q.cells + idx] = e;
   }
 }
 
@@ -110,9 +123,9 @@ __device__ __forceinline__ Real wavenumber(int i, int n, Real step) {
   return step * Real(2 * i < n ? i : i - n);
 }
 
-template <int DIM, class Real>
-__global__ void k_el_spec(const ElConst<Real> q, Cplx<Real>* __restrict__ S) {
-  using Cp = Comp<DIM>;
+// One thread per wavevector, all fields of it in place.
+template <int DIM, int RANK, class Real>
+__global__ void __launch_bounds__(256) k_el_spec(const __grid_constant__ ElConst<Real> q, Cplx<Real>* __restrict__ S) {
   const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (idx >= q.ncplx) return;
   const int mx = (int)(idx % q.nxh), my = (int)((idx / q.nxh) % q.ny), mz = (int)(idx / ((long long)q.nxh * q.ny));
@@ -121,127 +134,122 @@ __global__ void k_el_spec(const ElConst<Real> q, Cplx<Real>* __restrict__ S) {
   Real k2 = Real(0);
 #pragma unroll
   for (int d = 0; d < DIM; ++d) k2 += k[d] * k[d];
-  if (k2 == Real(0)) {
+  Cplx<Real> e[RANK];
 #pragma unroll
-    for (int c = 0; c < Cp::N; ++c) S[c * q.ncplx + idx] = Cplx<Real>{Real(0), Real(0)};
-    return;
-  }
-  Cplx<Real> e[Cp::N];
-#pragma unroll
-  for (int c = 0; c < Cp::N; ++c) e[c] = S[c * q.ncplx + idx];
-  // t_i = C_ijmn k_j e_mn; A_ik = C_ijkl k_j k_l
-  Cplx<Real> t[DIM];
-  Real A[DIM][DIM];
-#pragma unroll
-  for (int i = 0; i < DIM; ++i) {
-    t[i] = Cplx<Real>{Real(0), Real(0)};
-#pragma unroll
-    for (int j = 0; j < DIM; ++j)
-#pragma unroll
-      for (int m = 0; m < DIM; ++m)
-#pragma unroll
-        for (int n = 0; n < DIM; ++n) {
-          const Real ck = q.C[i][j][m][n] * k[j];
-          const Cplx<Real> v = e[Cp::index(m, n)];
-          t[i].re += ck * v.re;
-          t[i].im += ck * v.im;
-        }
-#pragma unroll
-    for (int kk = 0; kk < DIM; ++kk) {
-      Real a = Real(0);
-#pragma unroll
-      for (int j = 0; j < DIM; ++j)
-#pragma unroll
-        for (int l = 0; l < DIM; ++l) a += q.C[i][j][kk][l] * k[j] * k[l];
-      A[i][kk] = a;
-    }
-  }
-  // G = A^-1 (adjugate over the determinant)
-  Real G[DIM][DIM];
-  if constexpr (DIM == 2) {
-    const Real det = A[0][0] * A[1][1] - A[0][1] * A[1][0];
-    G[0][0] = A[1][1] / det;
-    G[0][1] = -A[0][1] / det;
-    G[1][0] = -A[1][0] / det;
-    G[1][1] = A[0][0] / det;
-  } else {
-    const Real c00 = A[1][1] * A[2][2] - A[1][2] * A[2][1], c01 = A[1][2] * A[2][0] - A[1][0] * A[2][2];
-    const Real c02 = A[1][0] * A[2][1] - A[1][1] * A[2][0];
-    const Real det = A[0][0] * c00 + A[0][1] * c01 + A[0][2] * c02;
-    G[0][0] = c00 / det;
-    G[1][0] = c01 / det;
-    G[2][0] = c02 / det;
-    G[0][1] = (A[0][2] * A[2][1] - A[0][1] * A[2][2]) / det;
-    G[1][1] = (A[0][0] * A[2][2] - A[0][2] * A[2][0]) / det;
-    G[2][1] = (A[0][1] * A[2][0] - A[0][0] * A[2][1]) / det;
-    G[0][2] = (A[0][1] * A[1][2] - A[0][2] * A[1][1]) / det;
-    G[1][2] = (A[0][2] * A[1][0] - A[0][0] * A[1][2]) / det;
-    G[2][2] = (A[0][0] * A[1][1] - A[0][1] * A[1][0]) / det;
-  }
-  Cplx<Real> gt[DIM];
-#pragma unroll
-  for (int kk = 0; kk < DIM; ++kk) {
-    gt[kk] = Cplx<Real>{Real(0), Real(0)};
-#pragma unroll
-    for (int i = 0; i < DIM; ++i) {
-      gt[kk].re += G[kk][i] * t[i].re;
-      gt[kk].im += G[kk][i] * t[i].im;
-    }
-  }
-  const Real scale = Real(1) / Real(q.cells);   // the inverse transform is unnormalised
-#pragma unroll
-  for (int i = 0; i < DIM; ++i)
-#pragma unroll
-    for (int j = i; j < DIM; ++j) {
-      const Real re = Real(0.5) * (k[i] * gt[j].re + k[j] * gt[i].re);
-      const Real im = Real(0.5) * (k[i] * gt[j].im + k[j] * gt[i].im);
-      S[Cp::index(i, j) * q.ncplx + idx] = Cplx<Real>{re * scale, im * scale};
-    }
-}
-
-template <int DIM, int NP, class Real>
-__global__ void k_el_force(const ElConst<Real> q, const Real* __restrict__ E, const Real* __restrict__ eps,
-                           Real* __restrict__ W) {
-  using Cp = Comp<DIM>;
-  const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= q.cells) return;
-  Real d[Cp::N];
-#pragma unroll
-  for (int c = 0; c < Cp::N; ++c) d[c] = eps[c * q.cells + idx] - E[c * q.cells + idx];
-  Real sig[Cp::N];
-#pragma unroll
-  for (int i = 0; i < DIM; ++i)
-#pragma unroll
-    for (int j = i; j < DIM; ++j) {
-      Real s = Real(0);
-#pragma unroll
-      for (int k = 0; k < DIM; ++k)
-#pragma unroll
-        for (int l = 0; l < DIM; ++l) s += q.C[i][j][k][l] * d[Cp::index(k, l)];
-      sig[Cp::index(i, j)] = s;
-    }
-#pragma unroll
-  for (int b = 0; b < NP; ++b) {
-    Real w = Real(0);
+  for (int s = 0; s < RANK; ++s) e[s] = S[s * q.ncplx + idx];
+  // v^s = Pr^s k and y^s = G v^s, G = A^-1 (adjugate over the determinant), A_ik = C_ijkl k_j k_l
+  Real yv[RANK][DIM];
+  if (k2 != Real(0)) {
+    Real A[DIM][DIM];
 #pragma unroll
     for (int i = 0; i < DIM; ++i)
 #pragma unroll
-      for (int j = 0; j < DIM; ++j) w += sig[Cp::index(i, j)] * q.eig[b][Cp::index(i, j)];
-    W[b * q.cells + idx] = -w;
+      for (int kk = 0; kk < DIM; ++kk) {
+        Real a = Real(0);
+#pragma unroll
+        for (int j = 0; j < DIM; ++j)
+#pragma unroll
+          for (int l = 0; l < DIM; ++l) a += q.C[i][j][kk][l] * k[j] * k[l];
+        A[i][kk] = a;
+      }
+    Real adj[DIM][DIM], det;
+    if constexpr (DIM == 2) {
+      det = A[0][0] * A[1][1] - A[0][1] * A[1][0];
+      adj[0][0] = A[1][1];
+      adj[0][1] = -A[0][1];
+      adj[1][0] = -A[1][0];
+      adj[1][1] = A[0][0];
+    } else {
+      adj[0][0] = A[1][1] * A[2][2] - A[1][2] * A[2][1];
+      adj[1][0] = A[1][2] * A[2][0] - A[1][0] * A[2][2];
+      adj[2][0] = A[1][0] * A[2][1] - A[1][1] * A[2][0];
+      det = A[0][0] * adj[0][0] + A[0][1] * adj[1][0] + A[0][2] * adj[2][0];
+      adj[0][1] = A[0][2] * A[2][1] - A[0][1] * A[2][2];
+      adj[1][1] = A[0][0] * A[2][2] - A[0][2] * A[2][0];
+      adj[2][1] = A[0][1] * A[2][0] - A[0][0] * A[2][1];
+      adj[0][2] = A[0][1] * A[1][2] - A[0][2] * A[1][1];
+      adj[1][2] = A[0][2] * A[1][0] - A[0][0] * A[1][2];
+      adj[2][2] = A[0][0] * A[1][1] - A[0][1] * A[1][0];
+    }
+#pragma unroll
+    for (int s = 0; s < RANK; ++s) {
+      Real v[DIM];
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) {
+        v[i] = Real(0);
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) v[i] += q.Pr[s][i][j] * k[j];
+      }
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) {
+        Real t = Real(0);
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) t += adj[i][j] * v[j];
+        yv[s][i] = t / det;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int s = 0; s < RANK; ++s)
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) yv[s][i] = Real(0);
+  }
+  const Real scale = Real(1) / Real(q.cells);   // the inverse transform is unnormalised
+#pragma unroll
+  for (int s = 0; s < RANK; ++s) {
+    Real v[DIM];
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) {
+      v[i] = Real(0);
+#pragma unroll
+      for (int j = 0; j < DIM; ++j) v[i] += q.Pl[s][i][j] * k[j];
+    }
+    Real re = Real(0), im = Real(0);
+#pragma unroll
+    for (int t = 0; t < RANK; ++t) {
+      Real K = -q.Q[s][t];
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) K += v[i] * yv[t][i];
+      re += K * e[t].re;
+      im += K * e[t].im;
+    }
+    S[s * q.ncplx + idx] = Cplx<Real>{re * scale, im * scale};
   }
 }
 
 template <class Real>
 ElConst<Real> make_const(const HostModel& m) {
   ElConst<Real> q{};
+  const ElasticBasis eb = elastic_basis(m);
+  q.rank = eb.rank;
+  for (int a = 0; a < m.N; ++a)
+    for (int s = 0; s < eb.rank; ++s) q.c[a][s] = (Real)eb.c[a][s];
+  const int dim = m.dim;
   for (int i = 0; i < 3; ++i)
     for (int j = 0; j < 3; ++j)
       for (int k = 0; k < 3; ++k)
         for (int l = 0; l < 3; ++l) q.C[i][j][k][l] = (Real)m.elC[i][j][k][l];
-  for (int a = 0; a < m.N; ++a)
-    for (int i = 0; i < m.dim; ++i)
-      for (int j = 0; j < m.dim; ++j)
-        q.eig[a][m.dim == 3 ? Comp<3>::index(i, j) : Comp<2>::index(i, j)] = (Real)m.eig[a][i][j];
+  for (int s = 0; s < eb.rank; ++s) {
+    for (int k = 0; k < dim; ++k)
+      for (int l = 0; l < dim; ++l) {
+        double pl = 0.0, pr = 0.0;
+        for (int i = 0; i < dim; ++i)
+          for (int j = 0; j < dim; ++j) {
+            pl += eb.B[s][i][j] * m.elC[i][j][k][l];
+            pr += m.elC[k][l][i][j] * eb.B[s][i][j];
+          }
+        q.Pl[s][k][l] = (Real)pl;
+        q.Pr[s][k][l] = (Real)pr;
+      }
+    for (int t = 0; t < eb.rank; ++t) {
+      double v = 0.0;
+      for (int i = 0; i < dim; ++i)
+        for (int j = 0; j < dim; ++j)
+          for (int k = 0; k < dim; ++k)
+            for (int l = 0; l < dim; ++l) v += eb.B[s][i][j] * m.elC[i][j][k][l] * eb.B[t][k][l];
+      q.Q[s][t] = (Real)v;
+    }
+  }
   const double two_pi = 6.28318530717958647692;
   q.kstep[0] = (Real)(two_pi / (m.nx * m.dx));
   q.kstep[1] = (Real)(two_pi / (m.ny * m.dx));
@@ -254,59 +262,103 @@ ElConst<Real> make_const(const HostModel& m) {
   q.nyp = m.nyp;
   q.xoff = m.xoff;
   q.zoff = m.zoff;
+  q.segs = segments(m);
   q.fstride = m.fstride;
   q.cells = (long long)m.nx * m.ny * q.nz;
   q.ncplx = (long long)q.nxh * m.ny * q.nz;
   return q;
 }
 
-template <int DIM, int NP, class Real>
-cudaError_t launch_el_cells(const ElConst<Real>& q, const void* st, ElasticState& s, int stage, cudaStream_t str) {
-  const int blocks = (int)((q.cells + 255) / 256);
-  if (stage == 0)
-    k_el_eig<DIM, NP, Real><<<blocks, 256, 0, str>>>(q, static_cast<const Real*>(st), static_cast<Real*>(s.E));
-  else
-    k_el_force<DIM, NP, Real><<<blocks, 256, 0, str>>>(q, static_cast<const Real*>(s.E),
-                                                        static_cast<const Real*>(s.eps), static_cast<Real*>(s.W));
+template <int DIM, class Real>
+cudaError_t launch_eig(int np, const ElConst<Real>& q, const void* st, const uint8_t* codes, ElasticState& s,
+                       cudaStream_t str) {
+  const unsigned blocks = (unsigned)(((long long)q.segs * q.ny * q.nz * 32 + 255) / 256);
+  const Real* p = static_cast<const Real*>(st);
+  Real* E = static_cast<Real*>(s.E);
+  switch (np) {
+    case 2: k_el_eig<DIM, 2, Real><<<blocks, 256, 0, str>>>(q, p, codes, E); break;
+    case 3: k_el_eig<DIM, 3, Real><<<blocks, 256, 0, str>>>(q, p, codes, E); break;
+    case 8: k_el_eig<DIM, 8, Real><<<blocks, 256, 0, str>>>(q, p, codes, E); break;
+    default: return cudaErrorInvalidValue;
+  }
   return cudaGetLastError();
 }
 
 template <int DIM, class Real>
-cudaError_t launch_el_np(int np, const ElConst<Real>& q, const void* st, ElasticState& s, int stage,
-                         cudaStream_t str) {
-  switch (np) {
-    case 2: return launch_el_cells<DIM, 2, Real>(q, st, s, stage, str);
-    case 3: return launch_el_cells<DIM, 3, Real>(q, st, s, stage, str);
-    case 8: return launch_el_cells<DIM, 8, Real>(q, st, s, stage, str);
+cudaError_t launch_spec(const ElConst<Real>& q, ElasticState& s, cudaStream_t str) {
+  const unsigned blocks = (unsigned)((q.ncplx + 255) / 256);
+  Cplx<Real>* S = static_cast<Cplx<Real>*>(s.spec);
+  switch (q.rank) {
+    case 1: k_el_spec<DIM, 1, Real><<<blocks, 256, 0, str>>>(q, S); break;
+    case 2: k_el_spec<DIM, 2, Real><<<blocks, 256, 0, str>>>(q, S); break;
+    case 3: k_el_spec<DIM, 3, Real><<<blocks, 256, 0, str>>>(q, S); break;
+    case 4: k_el_spec<DIM, 4, Real><<<blocks, 256, 0, str>>>(q, S); break;
+    case 5: k_el_spec<DIM, 5, Real><<<blocks, 256, 0, str>>>(q, S); break;
+    case 6: k_el_spec<DIM, 6, Real><<<blocks, 256, 0, str>>>(q, S); break;
     default: return cudaErrorInvalidValue;
   }
+  return cudaGetLastError();
 }
 
 template <class Real>
-cudaError_t solve(const HostModel& m, const void* st, ElasticState& s, cudaStream_t str) {
+cudaError_t solve(const HostModel& m, const void* st, const uint8_t* codes, ElasticState& s, cudaStream_t str) {
   const FftApi& f = fft_api();
   const ElConst<Real> q = make_const<Real>(m);
-  cudaError_t e = m.dim == 3 ? launch_el_np<3, Real>(m.N, q, st, s, 0, str) : launch_el_np<2, Real>(m.N, q, st, s, 0, str);
+  if (q.rank == 0) return cudaSuccess;   // no eigenstrain: no stress
+  cudaError_t e = m.dim == 3 ? launch_eig<3, Real>(m.N, q, st, codes, s, str) : launch_eig<2, Real>(m.N, q, st, codes, s, str);
   if (e != cudaSuccess) return e;
   const bool dbl = sizeof(Real) == 8;
   cufftResult r = dbl ? f.d2z(s.plan_r2c, static_cast<cufftDoubleReal*>(s.E), static_cast<cufftDoubleComplex*>(s.spec))
                       : f.r2c(s.plan_r2c, static_cast<cufftReal*>(s.E), static_cast<cufftComplex*>(s.spec));
   if (r != CUFFT_SUCCESS) return cudaErrorUnknown;
-  const int blocks = (int)((q.ncplx + 255) / 256);
-  if (m.dim == 3)
-    k_el_spec<3, Real><<<blocks, 256, 0, str>>>(q, static_cast<Cplx<Real>*>(s.spec));
-  else
-    k_el_spec<2, Real><<<blocks, 256, 0, str>>>(q, static_cast<Cplx<Real>*>(s.spec));
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  r = dbl ? f.z2d(s.plan_c2r, static_cast<cufftDoubleComplex*>(s.spec), static_cast<cufftDoubleReal*>(s.eps))
-          : f.c2r(s.plan_c2r, static_cast<cufftComplex*>(s.spec), static_cast<cufftReal*>(s.eps));
-  if (r != CUFFT_SUCCESS) return cudaErrorUnknown;
-  return m.dim == 3 ? launch_el_np<3, Real>(m.N, q, st, s, 1, str) : launch_el_np<2, Real>(m.N, q, st, s, 1, str);
+  e = m.dim == 3 ? launch_spec<3, Real>(q, s, str) : launch_spec<2, Real>(q, s, str);
+  if (e != cudaSuccess) return e;
+  r = dbl ? f.z2d(s.plan_c2r, static_cast<cufftDoubleComplex*>(s.spec), static_cast<cufftDoubleReal*>(s.E))
+          : f.c2r(s.plan_c2r, static_cast<cufftComplex*>(s.spec), static_cast<cufftReal*>(s.E));
+  return r == CUFFT_SUCCESS ? cudaSuccess : cudaErrorUnknown;
 }
 
 }  // namespace
 
 bool elastic_available() { return fft_api().ok; }
+
+ElasticBasis elastic_basis(const HostModel& m) {
+  // Gram-Schmidt with the largest remainder next; a remainder below 1e-12 of
+  // the largest eigenstrain is rounding
+  ElasticBasis b;
+  double rem[kNMax][3][3] = {}, top = 0.0;
+  auto norm2 = [&](const double (*t)[3]) {
+    double s = 0.0;
+    for (int i = 0; i < m.dim; ++i)
+      for (int j = 0; j < m.dim; ++j) s += t[i][j] * t[i][j];
+    return s;
+  };
+  for (int a = 0; a < m.N; ++a) {
+    for (int i = 0; i < m.dim; ++i)
+      for (int j = 0; j < m.dim; ++j) rem[a][i][j] = m.eig[a][std::max(i, j)][std::min(i, j)];   // symmetric
+    top = std::max(top, norm2(rem[a]));
+  }
+  while (b.rank < kElRank) {
+    int pick = 0;
+    for (int a = 1; a < m.N; ++a)
+      if (norm2(rem[a]) > norm2(rem[pick])) pick = a;
+    const double n2 = norm2(rem[pick]);
+    if (!(n2 > 1e-24 * top)) break;
+    double (*B)[3] = b.B[b.rank];
+    for (int i = 0; i < m.dim; ++i)
+      for (int j = 0; j < m.dim; ++j) B[i][j] = rem[pick][i][j] / std::sqrt(n2);
+    for (int a = 0; a < m.N; ++a) {
+      double c = 0.0;
+      for (int i = 0; i < m.dim; ++i)
+        for (int j = 0; j < m.dim; ++j) c += rem[a][i][j] * B[i][j];
+      b.c[a][b.rank] = c;
+      for (int i = 0; i < m.dim; ++i)
+        for (int j = 0; j < m.dim; ++j) rem[a][i][j] -= c * B[i][j];
+    }
+    ++b.rank;
+  }
+  return b;
+}
 
 namespace {
 void release_state(ms_ctx* c, ElasticState& s) {
@@ -316,10 +368,13 @@ void release_state(ms_ctx* c, ElasticState& s) {
     if (s.has_c2r) f.destroy(s.plan_c2r);
   }
   dev_free(c->hook, s.E);
-  dev_free(c->hook, s.eps);
   dev_free(c->hook, s.spec);
-  dev_free(c->hook, s.W);
   s = ElasticState{};
+}
+// The context's buffers and plans of another rank, once the stream is done with them.
+void drop_state(ms_ctx* c) {
+  if (c->el.E) cudaStreamSynchronize(c->stream);
+  release_state(c, c->el);
 }
 }  // namespace
 
@@ -331,10 +386,11 @@ bool elastic_grid_fits(const HostModel& m) {
 
 ms_status elastic_setup(ms_ctx* c) {
   const HostModel& m = c->m;
-  // the step kernels read the elastic potentials only while elasticity is on
-  // (ms_update_params may turn it on or off)
-  c->lg.elw = m.el && c->el.ready ? c->el.W : nullptr;
-  if (!m.el || c->el.ready) return MS_OK;
+  // the step kernels read the elastic fields only while elasticity is on
+  // (ms_update_params may turn it on or off, or change the eigenstrains' rank)
+  const int rank_now = m.el ? elastic_basis(m).rank : 0;
+  c->lg.elw = m.el && c->el.ready && c->el.rank == rank_now ? c->el.E : nullptr;
+  if (!m.el || (c->el.ready && c->el.rank == rank_now)) return MS_OK;
   const FftApi& f = fft_api();
   if (!f.ok) return fail(c, MS_ERR_UNSUPPORTED, "elasticity needs cuFFT (libcufft.so.12), which could not be opened");
   if (m.N != 2 && m.N != 3 && m.N != 8) return fail(c, MS_ERR_UNSUPPORTED, "elasticity: phases must be 2, 3 or 8");
@@ -342,16 +398,20 @@ ms_status elastic_setup(ms_ctx* c) {
   // everything is built in a local state and handed to the context only when
   // every buffer and both plans exist; a failure part-way frees what was made
   ElasticState s;
+  s.rank = rank_now;
+  if (rank_now == 0) {   // no eigenstrain in the plane of the grid: nothing to transform
+    s.ready = true;
+    drop_state(c);
+    c->el = s;
+    return MS_OK;
+  }
   const int nz = m.dim == 3 ? m.nz : 1;
   const long long cells = (long long)m.nx * m.ny * nz;
   const long long ncplx = (long long)(m.nx / 2 + 1) * m.ny * nz;
-  s.ncomp = m.dim == 3 ? 6 : 3;
   const size_t real = m.dtype == MS_F64 ? 8 : 4;
-  s.E = dev_alloc(c->hook, s.ncomp * cells * real);
-  s.eps = dev_alloc(c->hook, s.ncomp * cells * real);
-  s.spec = dev_alloc(c->hook, s.ncomp * ncplx * 2 * real);
-  s.W = dev_alloc(c->hook, (size_t)m.N * cells * real);
-  if (!s.E || !s.eps || !s.spec || !s.W) {
+  s.E = dev_alloc(c->hook, s.rank * cells * real);
+  s.spec = dev_alloc(c->hook, s.rank * ncplx * 2 * real);
+  if (!s.E || !s.spec) {
     release_state(c, s);
     return fail(c, MS_ERR_OOM, "elasticity buffers");
   }
@@ -364,14 +424,14 @@ ms_status elastic_setup(ms_ctx* c) {
   int* onb = m.dim == 3 ? onr : onr + 1;
   const bool dbl = m.dtype == MS_F64;
   cufftHandle p1 = 0, p2 = 0;
-  const bool ok1 = f.plan_many(&p1, rank, n, inb, 1, idist, onb, 1, odist, dbl ? CUFFT_D2Z : CUFFT_R2C, s.ncomp) ==
+  const bool ok1 = f.plan_many(&p1, rank, n, inb, 1, idist, onb, 1, odist, dbl ? CUFFT_D2Z : CUFFT_R2C, s.rank) ==
                    CUFFT_SUCCESS;
   if (ok1) {
     s.plan_r2c = p1;
     s.has_r2c = true;
   }
   const bool ok2 = ok1 && f.plan_many(&p2, rank, n, onb, 1, odist, inb, 1, idist, dbl ? CUFFT_Z2D : CUFFT_C2R,
-                                      s.ncomp) == CUFFT_SUCCESS;
+                                      s.rank) == CUFFT_SUCCESS;
   if (ok2) {
     s.plan_c2r = p2;
     s.has_c2r = true;
@@ -385,14 +445,15 @@ ms_status elastic_setup(ms_ctx* c) {
     return fail(c, MS_ERR_CUDA, "cuFFT stream");
   }
   s.ready = true;
+  drop_state(c);
   c->el = s;
-  c->lg.elw = s.W;
+  c->lg.elw = s.E;
   return MS_OK;
 }
 
-ms_status elastic_solve(ms_ctx* c, const void* state) {
-  cudaError_t e = c->m.dtype == MS_F64 ? solve<double>(c->m, state, c->el, c->stream)
-                                       : solve<float>(c->m, state, c->el, c->stream);
+ms_status elastic_solve(ms_ctx* c, const void* state, const uint8_t* codes) {
+  cudaError_t e = c->m.dtype == MS_F64 ? solve<double>(c->m, state, codes, c->el, c->stream)
+                                       : solve<float>(c->m, state, codes, c->el, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "elastic equilibrium");
   return MS_OK;
 }

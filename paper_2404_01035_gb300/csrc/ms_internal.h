@@ -12,6 +12,7 @@ namespace msgb {
 
 constexpr int kNMax = 8;
 constexpr int kKMax = 3;
+constexpr int kElRank = 6;   // independent eigenstrains at most (symmetric tensors)
 
 // Boundary code of an internal cut whose ghost plane is filled by a halo
 // exchange (same value as MS_BC_HALO in the public header).
@@ -60,6 +61,15 @@ struct HostModel {
   double eig[kNMax][3][3] = {};            // eigenstrain of each phase
 };
 
+// Basis of the phases' eigenstrains (in-plane components in 2-D): tensors
+// B[s], orthonormal, and E^a = sum_s c[a][s] B[s].  rank = number of tensors.
+struct ElasticBasis {
+  int rank = 0;
+  double B[kElRank][3][3] = {};
+  double c[kNMax][kElRank] = {};
+};
+ElasticBasis elastic_basis(const HostModel& m);
+
 // Launch geometry of one step.
 struct LaunchGeom {
   int tiles = 0;       // gridDim.x
@@ -71,7 +81,7 @@ struct LaunchGeom {
   int iface_blocks = 0;            // SMs: the interface grid is this x resident CTAs per SM
   int sms = 0;                     // multiprocessors of the device
   unsigned int* at_list = nullptr; // anti-trapping work list (see StepArgs)
-  const void* elw = nullptr;       // elastic part of the phase potentials (see StepArgs)
+  const void* elw = nullptr;       // fields of the elastic phase potentials (see StepArgs)
   unsigned int at_cap = 0;
   int reuse_prev = 1;              // output buffer = state one step before the input (see StepArgs)
   long long step = 0;              // step index of the input state (phi-noise counter)

@@ -57,6 +57,12 @@ void fill_args(void* blob, const HostModel& m, int zchunk, int* status) {
       for (int k = 0; k < 9; ++k) g.rot[p][k] = (Real)m.rot[a][b][k];
     }
   g.n_apairs = 0;
+  if (m.el) {
+    const ElasticBasis eb = elastic_basis(m);
+    g.el_rank = eb.rank;
+    for (int a = 0; a < NP; ++a)
+      for (int s = 0; s < eb.rank; ++s) g.elc[a][s] = (Real)-eb.c[a][s];
+  }
   for (int b = 1; b < NP; ++b)
     for (int a = 0; a < b; ++a) {
       const int q = pair_index<NP>(a, b);

@@ -304,8 +304,7 @@ __global__ void __launch_bounds__(RowsShape<NP, NM>::THREADS, RowsShape<NP, NM>:
       if (g.elw) {
         const unsigned long long cells = (unsigned long long)g.nx * g.ny * g.nz;
         const unsigned long long cell = ((unsigned long long)z * g.ny + y) * g.nx + min(x, g.nx - 1);
-#pragma unroll
-        for (int a = 0; a < NP; ++a) psi[a] += g.elw[a * cells + cell];
+        add_elastic<NP, NM, float, float>(g, cell, cells, psi);
       }
 #pragma unroll
       for (int a = 0; a < NP; ++a) {

@@ -38,11 +38,10 @@ struct AdjointStore {
 
 // Elasticity buffers and FFT plans (allocated while elasticity is on).
 struct ElasticState {
-  void* E = nullptr;      // eigenstrain components, dense
-  void* eps = nullptr;    // periodic strain components, dense
+  void* E = nullptr;      // rank fields, dense: eigenstrain amplitudes, then the potentials p_s
   void* spec = nullptr;   // their half spectra
-  void* W = nullptr;      // -sigma : eps*^b per phase, dense [N][cells]
-  int plan_r2c = 0, plan_c2r = 0, ncomp = 0;
+  int plan_r2c = 0, plan_c2r = 0;
+  int rank = 0;           // independent eigenstrains
   bool has_r2c = false, has_c2r = false;   // the plan handles hold created plans
   bool ready = false;   // every buffer and both plans exist (set only when complete)
 };
@@ -97,7 +96,7 @@ bool parse_fault_spec(const char* spec, int64_t* step, int* code);
 bool elastic_available();                         // cuFFT could be opened
 ms_status elastic_setup(ms_ctx* c);               // buffers and plans, when elasticity is on
 bool elastic_grid_fits(const HostModel& m);       // the FFT plans take the grid's cell count
-ms_status elastic_solve(ms_ctx* c, const void* state);   // w per phase from the state's phi
+ms_status elastic_solve(ms_ctx* c, const void* state, const uint8_t* codes);   // from the state's phi and codes
 void elastic_free(ms_ctx* c);
 // Tiled map of a padded state: box of (tx + 2H) x (ty + 2) x bz planes x nf fields.
 bool encode_state_map(CUtensorMap* tm, void* base, const HostModel& m, int nf, int tx, int ty, int bz = 1);

@@ -535,7 +535,7 @@ ms_status launch_one_step(ms_ctx* c) {
   c->lg.step = c->step;
   if (c->m.el) {   // elastic potentials of phi^n before the step
     if (!c->el.ready) return fail(c, MS_ERR_STATE, "elasticity is on but its buffers and FFT plans do not exist");
-    ms_status es = elastic_solve(c, c->buf[src]);
+    ms_status es = elastic_solve(c, c->buf[src], c->codes[src]);
     if (es != MS_OK) return es;
   }
   cudaError_t e = c->kern->launch(&c->tm[src], &c->tmi[src], c->buf[src], c->args.data(), c->m, c->t, c->buf[dst],
