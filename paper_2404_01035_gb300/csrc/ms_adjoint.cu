@@ -942,7 +942,12 @@ ms_status ms_grad(ms_ctx* c, const void* dphi_T, const void* dmu_T, double* dpar
     char* slots = static_cast<char*>(A.seg);
     e = cudaMemcpyAsync(slots, A.snaps[seg], c->state_bytes, cudaMemcpyDeviceToDevice, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "segment restore");
-    if (len > 1) {
+    const bool multi = multi_steps(c);
+    if (multi && len > 1) {   // as the forward steps went
+      ms_status ms = launch_multi_steps(c, len - 1, slots, c->state_bytes, m.t0 + (double)s0 * m.dt);
+      if (ms != MS_OK) return ms;
+    }
+    if (!multi && len > 1) {
       e = c->kern->codes(slots, m, c->codes[1 - cur_state], st);
       if (e != cudaSuccess) return cuda_fail(c, e, "segment codes");
     }
@@ -950,7 +955,7 @@ ms_status ms_grad(ms_ctx* c, const void* dphi_T, const void* dmu_T, double* dpar
     LaunchGeom lg = c->lg;
     lg.reuse_prev = 0;
     int cs = 1 - cur_state;
-    for (int k = 1; k < len; ++k) {
+    for (int k = 1; k < len && !multi; ++k) {
       CUtensorMap tm, tmi;
       char* src = slots + (size_t)(k - 1) * c->state_bytes;
       if (!encode_step_maps(*c->kern, &tm, &tmi, src, m)) return fail(c, MS_ERR_CUDA, "cuTensorMapEncodeTiled failed");
@@ -974,7 +979,7 @@ ms_status ms_grad(ms_ctx* c, const void* dphi_T, const void* dmu_T, double* dpar
   if (e != cudaSuccess) return cuda_fail(c, e, "gradient reduction");
   // the recompute used both code buffers: restore the current state's codes
   {
-    ms_status rs = refresh_codes(c);
+    ms_status rs = state_replaced(c);
     if (rs != MS_OK) return rs;
   }
   if (dphi0) {

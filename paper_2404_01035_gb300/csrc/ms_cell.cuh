@@ -605,6 +605,13 @@ __device__ __forceinline__ void mu_update(const StepArgs<Real, NP, NM>& g, const
   for (int i = 0; i < NM; ++i) mn[i] = mc[i] + dmu[i];
 }
 
+// T - T_ref at the origin of the last axis at the time of the input state: a
+// launch argument, unless the accessor carries it (several steps per launch).
+template <class Acc, class Real, int NP, int NM>
+__device__ __forceinline__ Real origin_temperature(const Acc&, const StepArgs<Real, NP, NM>& g) {
+  return g.tz0;
+}
+
 // The full cell update.  kz = cell index along the last axis (for T).
 template <int DIM, int NP, int NM, class Real, class S, class Acc, int FEAT = kFeatAll>
 __device__ __forceinline__ void gp_cell(const Acc& A, const StepArgs<Real, NP, NM>& g,
@@ -623,7 +630,7 @@ __device__ __forceinline__ void gp_cell(const Acc& A, const StepArgs<Real, NP, N
     for (int a = 0; a < NP; ++a)
       if (a == l) bulk = (val(ph[a]) == Real(1));
   }
-  const Real s = g.tz0 + g.tzg * (Real(kz) + Real(0.5));   // T^n - T_ref
+  const Real s = origin_temperature(A, g) + g.tzg * (Real(kz) + Real(0.5));   // T^n - T_ref
   S mc[NM];
 #pragma unroll
   for (int i = 0; i < NM; ++i) mc[i] = A.mu(i, 0, 0, 0);

@@ -87,6 +87,18 @@ struct LaunchGeom {
   long long step = 0;              // step index of the input state (phi-noise counter)
 };
 
+// Where the states of a run live: state k at slots + k slot_bytes, or, without
+// slots, alternating between two buffers (state 0 in buf[0]).
+struct MultiRun {
+  void* buf[2];
+  char* slots;
+  size_t slot_bytes;
+  int nsteps;
+  double t;                    // time of state 0
+  double off, G, V, dt;        // T - T_ref = off - G V t at the origin of the last axis
+  unsigned int* counters;      // [0] barrier arrivals, [1] exit tickets; zero between launches
+};
+
 // One compiled forward-step instantiation.
 struct StepKernel {
   int dim, np, nm, dtype, tx, ty;
@@ -103,6 +115,9 @@ struct StepKernel {
   cudaError_t (*launch)(const CUtensorMap* tm, const CUtensorMap* tmi, const void* in, void* blob, const HostModel& m,
                         double t, void* out, const uint8_t* codes_in, uint8_t* codes_out, const LaunchGeom& lg,
                         cudaStream_t st);
+  // Several steps in one persistent launch (2-D; NULL otherwise); segment
+  // codes are neither read nor written.
+  cudaError_t (*multi)(const void* blob, const MultiRun& run, int sms, cudaStream_t st);
   // Recompute the segment codes of a state loaded from outside.
   cudaError_t (*codes)(const void* state, const HostModel& m, uint8_t* codes, cudaStream_t st);
   // Anti-trapping correction of the mu just written by launch (same
@@ -110,6 +125,15 @@ struct StepKernel {
   cudaError_t (*at)(const void* in, void* blob, const HostModel& m, double t, void* out, const uint8_t* codes_in,
                     uint8_t* codes_out, const LaunchGeom& lg, cudaStream_t st);
 };
+
+// Cells up to which a 2-D grid is stepped by the persistent multi-step kernel
+// (FP32, FP64): us a step on a GB300, one launch a step / multi-step: FP32
+// binary 128^2 6.2 / 3.9, 256^2 6.2 / 5.0, 384^2 6.2 / 8.8, ternary 200^2
+// 10.3 / 9.4, 400^2 18.7 / 23.7; FP64 binary 128^2 30.9 / 16.4, 512^2 62 / 41,
+// 900^2 99 / 116, ternary 512^2 424 / 408.
+constexpr long long kMultiMaxCells[2] = {80000, 300000};
+// Steps of one multi-step launch at most (the barrier counts steps x CTAs in 32 bits).
+constexpr int kMultiMaxSteps = 1 << 16;
 
 // Number of 32-cell segments per row.
 inline int segments(const HostModel& m) { return (m.nx + 31) / 32; }

@@ -9,6 +9,7 @@
 #include "ms_at.cuh"
 #include "ms_diag.cuh"
 #include "ms_internal.h"
+#include "ms_multi.cuh"
 #include "ms_rows.cuh"
 #include "ms_split.cuh"
 #include "ms_step.cuh"
@@ -56,13 +57,13 @@ void fill_args(void* blob, const HostModel& m, int zchunk, int* status) {
       g.rotated[p] = m.rotated[a][b];
       for (int k = 0; k < 9; ++k) g.rot[p][k] = (Real)m.rot[a][b][k];
     }
-  g.n_apairs = 0;
   if (m.el) {
     const ElasticBasis eb = elastic_basis(m);
     g.el_rank = eb.rank;
     for (int a = 0; a < NP; ++a)
       for (int s = 0; s < eb.rank; ++s) g.elc[a][s] = (Real)-eb.c[a][s];
   }
+  g.n_apairs = 0;
   for (int b = 1; b < NP; ++b)
     for (int a = 0; a < b; ++a) {
       const int q = pair_index<NP>(a, b);
@@ -213,6 +214,36 @@ cudaError_t launch_step(const CUtensorMap* tm, const CUtensorMap*, const void*, 
   return cudaGetLastError();
 }
 
+// Several steps of a 2-D grid in one cooperative launch (k_gp_multi): a warp
+// per row segment where the grid is small, each SM with a CTA before a second
+// warp of one has work.
+template <int NP, int NM, class Real>
+cudaError_t launch_multi(const void* blob, const MultiRun& run, int sms, cudaStream_t st) {
+  using Sh = MultiShape<NP, NM, Real>;
+  const auto& g = *reinterpret_cast<const StepArgs<Real, NP, NM>*>(blob);
+  auto k = k_gp_multi<NP, NM, Real>;
+  static int per_sm = 0;   // resident CTAs per SM
+  if (per_sm == 0) {
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, Sh::THREADS, 0);
+    if (e != cudaSuccess) return e;
+    per_sm = per_sm < 1 ? 1 : per_sm;
+  }
+  const long long units = (long long)g.segs * g.ny;
+  long long ctas = (units + Sh::WARPS - 1) / Sh::WARPS;
+  if (ctas < sms) ctas = units < sms ? units : sms;
+  if (ctas > (long long)sms * per_sm) ctas = (long long)sms * per_sm;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)ctas);
+  cfg.blockDim = dim3(Sh::THREADS);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, g, run);
+}
+
 // Split 3-D FP32 step: the bulk streaming kernel (tm = mu-only tile map),
 // then the interface kernel over the rows it listed (tmi = interface boxes).
 template <int NP, int NM, int TY>
@@ -324,6 +355,8 @@ StepKernel make_step_kernel() {
   k.args_bytes = sizeof(StepArgs<Real, NP, NM>);
   k.fill = &fill_args<DIM, NP, NM, Real>;
   k.launch = &launch_step<DIM, NP, NM, Real, TX, TY>;
+  k.multi = nullptr;
+  if constexpr (DIM == 2) k.multi = &launch_multi<NP, NM, Real>;
   k.codes = &launch_codes<DIM, NP, Real>;
   k.at = &launch_at<DIM, NP, NM, Real>;
   return k;
@@ -344,6 +377,7 @@ StepKernel make_split_kernel() {
   k.args_bytes = sizeof(StepArgs<float, NP, NM>);
   k.fill = &fill_args<3, NP, NM, float>;
   k.launch = &launch_split<NP, NM, TY>;
+  k.multi = nullptr;
   k.codes = &launch_codes<3, NP, float>;
   k.at = &launch_at<3, NP, NM, float, true>;
   return k;

@@ -58,6 +58,7 @@ struct ms_ctx {
   CUtensorMap tmi[2];   // interface-box maps of buf[0] / buf[1] (split variants)
   void* buf[2] = {nullptr, nullptr};
   uint8_t* codes[2] = {nullptr, nullptr};   // segment codes of buf[0] / buf[1]
+  bool codes_stale = false;                 // the codes do not describe the current state (refresh_codes)
   unsigned int* iface = nullptr;            // work list of the split step (lazily allocated)
   unsigned int* at_list = nullptr;          // anti-trapping work list (allocated while it is on)
   size_t state_bytes = 0;
@@ -69,6 +70,7 @@ struct ms_ctx {
   msgb::AllocHook hook;
   char* small = nullptr;        // status word + diag output + diag partials
   int* status = nullptr;
+  unsigned int* counters = nullptr;   // of the multi-step kernel
   double* diag_out = nullptr;
   double* diag_partials = nullptr;
   int diag_blocks = 0;
@@ -90,6 +92,12 @@ ms_status launch_one_step(ms_ctx* c);
 ms_status apply_launch(ms_ctx* c, const StepKernel* k, int zchunk);
 ms_status ensure_at_list(ms_ctx* c);   // the anti-trapping work list, when the current is on
 ms_status refresh_codes(ms_ctx* c);   // segment codes of the current state
+bool multi_steps(const ms_ctx* c);    // ms_step advances this context by the persistent multi-step kernel
+// n steps by that kernel: between the context's two buffers, or (slots not
+// NULL) from state 0 at slots, time t, to states 1 .. n at slots + k slot_bytes.
+ms_status launch_multi_steps(ms_ctx* c, int n, char* slots, size_t slot_bytes, double t);
+// The current state was replaced: its codes now, or when they are next read.
+ms_status state_replaced(ms_ctx* c);
 // Parse a fault-injection spec "step:K,code:X" (K >= 0, X a non-zero
 // ms_status); false for a malformed one.  NULL or empty = no fault (step -1).
 bool parse_fault_spec(const char* spec, int64_t* step, int* code);

@@ -530,7 +530,44 @@ ms_status apply_launch(ms_ctx* c, const StepKernel* k, int zchunk) {
   return MS_OK;
 }
 
+bool multi_steps(const ms_ctx* c) {
+  return c->kern->multi && !c->m.at && !c->m.el && c->m.noise_amp == 0.0 &&
+         (long long)c->m.nx * c->m.ny <= kMultiMaxCells[c->m.dtype == MS_F64 ? 1 : 0];
+}
+
+ms_status launch_multi_steps(ms_ctx* c, int n, char* slots, size_t slot_bytes, double t) {
+  MultiRun r = {};
+  r.buf[0] = c->buf[c->cur];
+  r.buf[1] = c->buf[1 - c->cur];
+  r.slots = slots;
+  r.slot_bytes = slot_bytes;
+  r.nsteps = n;
+  r.t = t;
+  r.off = c->m.T0 - c->m.T_ref - c->m.G * c->m.z0;
+  r.G = c->m.G;
+  r.V = c->m.V;
+  r.dt = c->m.dt;
+  r.counters = c->counters;
+  cudaError_t e = c->kern->multi(c->args.data(), r, c->lg.sms, c->stream);
+  if (e != cudaSuccess) return cuda_fail(c, e, "multi-step launch");
+  if (slots) return MS_OK;
+  c->cur = (c->cur + n) & 1;
+  c->step += n;
+  c->t = c->m.t0 + (double)c->step * c->m.dt;
+  c->codes_stale = true;
+  return MS_OK;
+}
+
+ms_status state_replaced(ms_ctx* c) {
+  c->codes_stale = true;
+  return multi_steps(c) ? MS_OK : refresh_codes(c);
+}
+
 ms_status launch_one_step(ms_ctx* c) {
+  if (c->codes_stale) {
+    ms_status rs = refresh_codes(c);
+    if (rs != MS_OK) return rs;
+  }
   const int src = c->cur, dst = 1 - c->cur;
   c->lg.step = c->step;
   if (c->m.el) {   // elastic potentials of phi^n before the step
@@ -557,6 +594,7 @@ ms_status refresh_codes(ms_ctx* c) {
   // must not let the next step keep phi there
   e = cudaMemsetAsync(c->codes[1 - c->cur], 0, code_bytes(c->m), c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "segment codes");
+  c->codes_stale = false;
   return MS_OK;
 }
 
@@ -659,6 +697,7 @@ ms_status ms_create(const ms_grid* grid, int n_phases, int n_components, const m
   }
   c->status = reinterpret_cast<int*>(c->small);
   c->diag_out = reinterpret_cast<double*>(c->small + 256);
+  c->counters = reinterpret_cast<unsigned int*>(c->small + 2048);
   c->diag_partials = reinterpret_cast<double*>(c->small + 4096);
   if (cudaMallocHost(&c->diag_host, 4096) != cudaSuccess) {
     ms_destroy(c);
@@ -760,7 +799,7 @@ ms_status ms_set_fields(ms_ctx* c, const void* phi, const void* mu, int on_devic
   MS_CUDA(c, copy_fields(c->m, c->buf[c->cur], 0, c->m.N, phi, nullptr, on_device, c->stream));
   MS_CUDA(c, copy_fields(c->m, c->buf[c->cur], c->m.N, c->m.NM, mu, nullptr, on_device, c->stream));
   MS_CUDA(c, fill_ghosts(c->m, c->buf[c->cur], c->m.N + c->m.NM, c->stream));
-  ms_status rs = refresh_codes(c);
+  ms_status rs = state_replaced(c);
   if (rs != MS_OK) return rs;
   c->step = 0;
   c->t = c->m.t0;
@@ -796,13 +835,25 @@ ms_status ms_step(ms_ctx* c, int64_t n) {
   TraceRange trace("ms_step");
   if (!c) return fail(nullptr, MS_ERR_ARG, "ctx is NULL");
   if (n < 0) return fail(c, MS_ERR_ARG, "n must be >= 0");
-  for (int64_t i = 0; i < n; ++i) {
+  for (int64_t i = 0; i < n;) {
     if (c->fault_step >= 0 && c->step == c->fault_step) c->host_status = c->fault_code;
     if (c->host_status) return fail(c, (ms_status)c->host_status, "injected fault (MS_FAULT)");
     ms_status s = ms_before_step(c);
     if (s != MS_OK) return s;
-    s = launch_one_step(c);
+    int64_t k = 1;
+    if (multi_steps(c)) {
+      // up to the next thing that is due between steps: a snapshot, the
+      // diagnostics, an injected fault
+      k = std::min<int64_t>(n - i, kMultiMaxSteps);
+      if (c->adj.every > 0) k = std::min<int64_t>(k, c->adj.every - (c->step - c->adj.first_step) % c->adj.every);
+      if (c->diag_every > 0) k = std::min<int64_t>(k, c->diag_every - c->step % c->diag_every);
+      if (c->fault_step > c->step) k = std::min<int64_t>(k, c->fault_step - c->step);
+      s = launch_multi_steps(c, (int)k, nullptr, 0, c->t);
+    } else {
+      s = launch_one_step(c);
+    }
     if (s != MS_OK) return s;
+    i += k;
     if (c->diag_every > 0 && c->step % c->diag_every == 0) {
       s = launch_diag_now(c);
       if (s != MS_OK) return s;
@@ -899,7 +950,7 @@ ms_status ms_restore(ms_ctx* c, const void* host_buf, size_t bytes) {
     return fail(c, MS_ERR_ARG, "checkpoint does not match this context");
   MS_CUDA(c, cudaMemcpyAsync(c->buf[c->cur], (const char*)host_buf + sizeof h, c->state_bytes,
                              cudaMemcpyHostToDevice, c->stream));
-  ms_status rs = refresh_codes(c);
+  ms_status rs = state_replaced(c);
   if (rs != MS_OK) return rs;
   MS_CUDA(c, cudaStreamSynchronize(c->stream));
   c->step = h.step;

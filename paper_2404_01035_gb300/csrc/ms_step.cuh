@@ -200,10 +200,10 @@ __device__ __forceinline__ int image_coord(int v, int c, int n, int bc, bool cut
 }
 
 template <int DIM, int NP, int NM, class Real>
-__device__ __forceinline__ void store_cell(const StepArgs<Real, NP, NM>& g, int x, int y, int z,
-                                           const Real* pn, const Real* mn, bool write_phi = true) {
+__device__ __forceinline__ void store_cell_to(const StepArgs<Real, NP, NM>& g, Real* out, int x, int y, int z,
+                                              const Real* pn, const Real* mn, bool write_phi = true) {
   const long long plane = (long long)g.nyp * g.pitch;
-  Real* base = g.out + (long long)(z + g.zoff) * plane + (long long)(y + 1) * g.pitch + x + g.xoff;
+  Real* base = out + (long long)(z + g.zoff) * plane + (long long)(y + 1) * g.pitch + x + g.xoff;
   if (write_phi) {
 #pragma unroll
     for (int a = 0; a < NP; ++a) base[a * g.fstride] = pn[a];
@@ -227,7 +227,7 @@ __device__ __forceinline__ void store_cell(const StepArgs<Real, NP, NM>& g, int 
         if ((ix | iy | iz) == 0) continue;
         const int xi = image_coord(ix, x, g.nx, g.bc[0], false);
         if (xi == kNoImage) continue;
-        Real* p = g.out + (long long)(zi + g.zoff) * plane + (long long)(yi + 1) * g.pitch + xi + g.xoff;
+        Real* p = out + (long long)(zi + g.zoff) * plane + (long long)(yi + 1) * g.pitch + xi + g.xoff;
         if (write_phi) {
 #pragma unroll
           for (int a = 0; a < NP; ++a) p[a * g.fstride] = pn[a];
@@ -237,6 +237,12 @@ __device__ __forceinline__ void store_cell(const StepArgs<Real, NP, NM>& g, int 
       }
     }
   }
+}
+
+template <int DIM, int NP, int NM, class Real>
+__device__ __forceinline__ void store_cell(const StepArgs<Real, NP, NM>& g, int x, int y, int z,
+                                           const Real* pn, const Real* mn, bool write_phi = true) {
+  store_cell_to<DIM>(g, g.out, x, y, z, pn, mn, write_phi);
 }
 
 // Minimum CTAs per SM the register allocation must allow: two for the
