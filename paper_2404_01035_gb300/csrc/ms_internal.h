@@ -79,6 +79,7 @@ struct LaunchGeom {
   unsigned int* iface2 = nullptr;
   unsigned int iface_cap = 0;
   int iface_blocks = 0;            // SMs: the interface grid is this x resident CTAs per SM
+  void* cells = nullptr;           // scratch of the cell-list step (ms_cells.cuh)
   int sms = 0;                     // multiprocessors of the device
   unsigned int* at_list = nullptr; // anti-trapping work list (see StepArgs)
   const void* elw = nullptr;       // fields of the elastic phase potentials (see StepArgs)
@@ -102,7 +103,8 @@ struct MultiRun {
 // One compiled forward-step instantiation.
 struct StepKernel {
   int dim, np, nm, dtype, tx, ty;
-  int split;   // 1: streaming kernel for bulk rows + interface kernel for the rest
+  int split;   // 1: the bulk and the rest by kernels of their own (FP32: streaming kernel and interface rows;
+               // FP64: cell list, ms_cells.cuh), 0: one fused kernel
   int smem_bytes;
   size_t args_bytes;
   // Fill the launch-argument blob from the model (all constants).
@@ -157,6 +159,10 @@ struct DiagKernel {
   cudaError_t (*launch)(const void* state, const HostModel& m, double t, double* partials,
                         int nblocks, double* out, int* status, cudaStream_t st);
 };
+
+size_t cells_scratch_bytes(const HostModel& m);   // of the cell-list step
+// The cell-list step indexes cells with 32 bits.
+inline bool cells_fit(const HostModel& m) { return (long long)m.nx * m.ny * m.nz < 0xFFFFFFF0ll; }
 
 std::vector<StepKernel>& step_registry();
 std::vector<DiagKernel>& diag_registry();

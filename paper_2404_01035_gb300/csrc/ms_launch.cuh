@@ -7,6 +7,7 @@
 #include <cstring>
 
 #include "ms_at.cuh"
+#include "ms_cells.cuh"
 #include "ms_diag.cuh"
 #include "ms_internal.h"
 #include "ms_multi.cuh"
@@ -301,6 +302,34 @@ cudaError_t launch_split(const CUtensorMap* tm, const CUtensorMap* tmi, const vo
   return cudaGetLastError();
 }
 
+// Cell-list 3-D step (FP64): scan, upper faces, update.
+template <int NP, int NM, class Real>
+cudaError_t launch_cells(const CUtensorMap*, const CUtensorMap*, const void* in, void* blob, const HostModel& m,
+                         double t, void* out, const uint8_t* codes_in, uint8_t* codes_out, const LaunchGeom& lg,
+                         cudaStream_t st) {
+  if (!lg.cells || lg.sms < 1) return cudaErrorInvalidValue;
+  auto& g = *reinterpret_cast<StepArgs<Real, NP, NM>*>(blob);
+  set_launch_args(g, m, t, out, codes_in, codes_out, lg);
+  const CellsScratch<Real> c = cells_layout<Real>(lg.cells, m);
+  const Real* p = reinterpret_cast<const Real*>(in);
+  auto kf = k_c_faces<NP, NM, Real>;
+  auto ku = k_c_update<NP, NM, Real>;
+  static int faces_per_sm = 0, update_per_sm = 0;   // resident CTAs per SM
+  if (update_per_sm == 0) {
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&faces_per_sm, kf, 64, 0);
+    int u = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&u, ku, 64, 0);
+    if (e != cudaSuccess) return e;
+    faces_per_sm = faces_per_sm < 1 ? 1 : faces_per_sm;
+    update_per_sm = u < 1 ? 1 : u;
+  }
+  const long long nseg = (long long)segments(m) * m.ny * m.nz;
+  k_c_scan<NP, NM, Real><<<(unsigned)((nseg + 3) / 4), 128, 0, st>>>(g, p, c);
+  kf<<<lg.sms * faces_per_sm, 64, 0, st>>>(g, p, c);
+  ku<<<lg.sms * update_per_sm, 64, 0, st>>>(g, p, c);
+  return cudaGetLastError();
+}
+
 // The anti-trapping correction after a step.  LISTED: the step's interface
 // kernel has already listed the segments (split step), so the listing pass
 // is skipped.
@@ -380,6 +409,27 @@ StepKernel make_split_kernel() {
   k.multi = nullptr;
   k.codes = &launch_codes<3, NP, float>;
   k.at = &launch_at<3, NP, NM, float, true>;
+  return k;
+}
+
+// Cell-list 3-D variant.
+template <int NP, int NM, class Real>
+StepKernel make_cells_kernel() {
+  StepKernel k;
+  k.dim = 3;
+  k.np = NP;
+  k.nm = NM;
+  k.dtype = sizeof(Real) == 8 ? 1 : 0;
+  k.tx = 32;
+  k.ty = 1;
+  k.split = 1;
+  k.smem_bytes = 0;
+  k.args_bytes = sizeof(StepArgs<Real, NP, NM>);
+  k.fill = &fill_args<3, NP, NM, Real>;
+  k.launch = &launch_cells<NP, NM, Real>;
+  k.multi = nullptr;
+  k.codes = &launch_codes<3, NP, Real>;
+  k.at = &launch_at<3, NP, NM, Real>;
   return k;
 }
 

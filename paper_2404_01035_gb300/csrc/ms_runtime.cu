@@ -341,6 +341,7 @@ bool encode_state_map(CUtensorMap* tm, void* base, const HostModel& m, int nf, i
 bool encode_step_maps(const StepKernel& k, CUtensorMap* tm, CUtensorMap* tmi, void* base, const HostModel& m) {
   const int nf = m.N + m.NM;
   if (!k.split) return encode_state_map(tm, base, m, nf, k.tx, k.ty);
+  if (m.dtype == MS_F64) return true;   // the cell-list step reads the state itself
   const size_t s = m.dtype == MS_F64 ? 8 : 4;
   char* mu = static_cast<char*>(base) + (size_t)m.N * m.fstride * s;
   return encode_state_map(tm, mu, m, m.NM, k.tx, k.ty) && encode_state_map(tmi, base, m, nf, 32, 1, 3);
@@ -490,6 +491,12 @@ ms_status ensure_at_list(ms_ctx* c) {
   return MS_OK;
 }
 
+size_t cells_scratch_bytes(const HostModel& m) {
+  const size_t cells = (size_t)m.nx * m.ny * m.nz, s = m.dtype == MS_F64 ? 8 : 4;
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  return up((cells + 2) * 4) + 2 * up(cells) + up(3 * m.N * cells * s) + up((size_t)m.NM * m.NM * cells * s);
+}
+
 ms_status apply_launch(ms_ctx* c, const StepKernel* k, int zchunk) {
   if (c->lg.sms < 1) {
     int dev = 0, sms = 152;
@@ -499,7 +506,14 @@ ms_status apply_launch(ms_ctx* c, const StepKernel* k, int zchunk) {
   }
   ms_status as = ensure_at_list(c);
   if (as != MS_OK) return as;
-  if (k->split && !c->iface) {
+  if (k->split && c->m.dtype == MS_F64 && !c->lg.cells) {
+    if (!cells_fit(c->m)) return fail(c, MS_ERR_UNSUPPORTED, "grid too large for the cell-list step");
+    c->lg.cells = dev_alloc(c->hook, cells_scratch_bytes(c->m));
+    if (!c->lg.cells) return fail(c, MS_ERR_OOM, "cell-list scratch allocation failed");
+    cudaError_t e = cudaMemsetAsync(c->lg.cells, 0, 2 * sizeof(unsigned int), c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "cell-list reset");
+  }
+  if (k->split && c->m.dtype == MS_F32 && !c->iface) {
     // work list of the split step: count, ticket and one entry per warp row
     // (two lists: the second takes the rows left for a second launch)
     const size_t cap = (size_t)segments(c->m) * c->m.ny * c->m.nz;
@@ -713,14 +727,13 @@ ms_status ms_create(const ms_grid* grid, int n_phases, int n_components, const m
     ms_destroy(c);
     return r;
   }
-  // the split step where one is compiled (3-D FP32): faster than the fused
-  // kernels at every size measured on a GB300 (us a step, fused / split:
+  // the split step where one is compiled (3-D): faster than the fused
+  // kernels at every size measured on a GB300 (us a step, fused / split, FP32:
   // eutectic 24^3 87 / 17, 150x133x97 158 / 80, 256^3 769 / 196; 8-phase
   // multigrain 24^3 329 / 19, 128^3 1733 / 231, 384^3 3646 / 389).  A grid too
-  // large for its work-list entries, or without memory for the lists, gets the
-  // fused kernel.
+  // large for its work lists, or without memory for them, gets the fused kernel.
   const StepKernel* split = nullptr;
-  if (c->m.dim == 3 && list_entry_fits(c->m))
+  if (c->m.dim == 3 && (c->m.dtype == MS_F64 ? cells_fit(c->m) : list_entry_fits(c->m)))
     for (auto* v : step_variants(c->m.dim, c->m.N, c->m.NM, c->m.dtype))
       if (v->split) split = v;
   s = MS_ERR_UNSUPPORTED;
@@ -748,6 +761,7 @@ void ms_destroy(ms_ctx* c) {
   }
   dev_free(c->hook, c->small);
   dev_free(c->hook, c->iface);
+  dev_free(c->hook, c->lg.cells);
   dev_free(c->hook, c->at_list);
   if (c->diag_host) cudaFreeHost(c->diag_host);
   delete c;
