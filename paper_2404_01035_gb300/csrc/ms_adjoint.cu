@@ -27,6 +27,7 @@
 //      differences that read the position, and the transposed mu flux
 //      (written out by hand: div is linear in mu and in the cell mobilities,
 //      chained through M(phi_j) once).
+// The 2-D FP32 adjoint runs the three in one launch (k_adj_fused).
 // Parameter partials are reduced per block in FP64, summed over the reverse
 // steps in place and over the blocks in a fixed order at the end.
 #include <cuda_runtime.h>
@@ -105,23 +106,6 @@ struct ValAcc {
   __device__ __forceinline__ uint32_t mask() const { return (1u << NP) - 1u; }
 };
 
-// Stencil accessor yielding phases as Dual<Real, NP> with slot a = 1 for
-// phase a at the padded index `seed`.
-template <int NP, int NM, class Real>
-struct SeedAcc {
-  using D = Dual<Real, NP>;
-  const Real* st;
-  long long fstride, plane, base, seed;
-  int pitch;
-  __device__ __forceinline__ D phi(int a, int dx, int dy, int dz) const {
-    const long long idx = base + dz * plane + (long long)dy * pitch + dx;
-    D v(st[a * fstride + idx]);
-    if (idx == seed) v.d[a] = Real(1);
-    return v;
-  }
-  __device__ __forceinline__ uint32_t mask() const { return (1u << NP) - 1u; }
-};
-
 template <int DIM, class Real, int NP, int NM>
 __device__ __forceinline__ bool in_grid(const StepArgs<Real, NP, NM>& g, int x, int y, int z) {
   return x >= 0 && x < g.nx && y >= 0 && y < g.ny && z >= 0 && z < (DIM == 3 ? g.nz : 1);
@@ -139,6 +123,196 @@ __device__ __forceinline__ bool any_aniso(const unsigned char* aniso, int P) {
   return r;
 }
 
+// The cell pass (see the file comment) for the cell at padded index `base`:
+// its CellStore entries from lam = dL/d(its phi^{n+1}, mu^{n+1}), and its
+// parameter gradient.  kz: lab index along the last axis, lab: lab cell index.
+template <int DIM, int NP, int NM, class Real>
+__device__ __forceinline__ void adj_cell(const Real* __restrict__ st, long long base, int kz, unsigned long long lab,
+                                         const StepArgs<Real, NP, NM>& g, const AdjExtra<Real, NP, NM>& ex,
+                                         const Real* lam, Real* out, double* gpar) {
+  constexpr int P = NP * (NP - 1) / 2;
+  constexpr int ND = NP * NM * NM;
+  using TS = TailSlots<NP, NM>;
+  using DP = Dual<Real, P>;
+  using DD = Dual<Real, ND>;
+  using DT = Dual<Real, TS::T>;
+  const long long plane = (long long)g.nyp * g.pitch;
+  // stencil part: divJ, Gc with delta slots
+  DP divJ[NP], Gc[NP];
+  {
+    ValAcc<NP, NM, Real, DP> A{st, g.fstride, plane, base, g.pitch};
+    DiffPrm<DP, P> dp;
+    dp.mob = DP(g.mob);
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      dp.delta[p] = DP(g.delta[p]);
+      dp.delta[p].d[p] = Real(1);
+    }
+    DP ph[NP];
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+      ph[a] = A.phi(a, 0, 0, 0);
+      divJ[a] = DP(Real(0));
+      Gc[a] = DP(Real(0));
+    }
+    gradient_terms<DIM, NP, NM, Real, DP, ValAcc<NP, NM, Real, DP>, kFeatAll, false>(
+        A, g, dp, ph, A.mask(), any_aniso<DIM>(g.aniso, P), divJ, Gc);
+  }
+  // stencil part: div with D slots (M = sum_a h_a D^a chi^a)
+  DD div[NM];
+  {
+    ValAcc<NP, NM, Real, DD> B{st, g.fstride, plane, base, g.pitch};
+    DD DXd[NP][NM * NM];
+#pragma unroll
+    for (int a = 0; a < NP; ++a)
+#pragma unroll
+      for (int r = 0; r < NM; ++r)
+#pragma unroll
+        for (int c = 0; c < NM; ++c) {
+          DD sum(Real(0));
+#pragma unroll
+          for (int m = 0; m < NM; ++m) {
+            DD Dm(ex.D[a][r * NM + m]);
+            Dm.d[(a * NM + r) * NM + m] = Real(1);
+            sum += Dm * DD(g.chi[a][m * NM + c]);
+          }
+          DXd[a][r * NM + c] = sum;
+        }
+    DD ph[NP], mc[NM], Mc[NM * NM];
+#pragma unroll
+    for (int a = 0; a < NP; ++a) ph[a] = B.phi(a, 0, 0, 0);
+#pragma unroll
+    for (int k = 0; k < NM; ++k) {
+      mc[k] = B.mu(k, 0, 0, 0);
+      div[k] = DD(Real(0));
+    }
+    cell_mobility<NP, NM>(ph, DXd, Mc);
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+#pragma unroll
+      for (int sd = -1; sd <= 1; sd += 2) {
+        const Off<DIM> o = unit<DIM>(d, sd);
+        DD pn[NP], Mn[NM * NM];
+#pragma unroll
+        for (int a = 0; a < NP; ++a) pn[a] = B.phi(a, o.x, o.y, o.z);
+        cell_mobility<NP, NM>(pn, DXd, Mn);
+#pragma unroll
+        for (int r = 0; r < NM; ++r)
+#pragma unroll
+          for (int c = 0; c < NM; ++c) {
+            DD Mf = Real(0.5) * (Mc[r * NM + c] + Mn[r * NM + c]);
+            div[r] += Mf * ((B.mu(c, o.x, o.y, o.z) - mc[c]) * g.inv_dx2);
+          }
+      }
+    }
+  }
+  // the tail, one slot per input
+  Real tb[TS::T];
+  {
+    DT in[TS::T];
+#pragma unroll
+    for (int k = 0; k < TS::T; ++k) in[k] = DT(Real(0));
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+      in[TS::PH + a] = DT(st[a * g.fstride + base]);
+      in[TS::DJ + a] = DT(divJ[a].v);
+      in[TS::GC + a] = DT(Gc[a].v);
+    }
+#pragma unroll
+    for (int k = 0; k < NM; ++k) {
+      in[TS::MC + k] = DT(st[(NP + k) * g.fstride + base]);
+      in[TS::DIV + k] = DT(div[k].v);
+    }
+    in[TS::MOB] = DT(g.mob);
+#pragma unroll
+    for (int k = 0; k < TS::T; ++k) in[k].d[k] = Real(1);
+    DiffPrm<DT, P> dp;
+    dp.mob = in[TS::MOB];
+#pragma unroll
+    for (int p = 0; p < P; ++p) dp.delta[p] = DT(g.delta[p]);
+    const Real s = g.tz0 + g.tzg * (Real(kz) + Real(0.5));
+    DT pn[NP], mn[NM];
+    phase_update<DIM, NP, NM, Real, DT, kFeatAll>(g, dp, in + TS::PH, in + TS::MC, in + TS::DJ, in + TS::GC, s,
+                                                  lab, pn);
+    mu_update<NP, NM, Real, DT>(g, in + TS::PH, pn, in + TS::MC, in + TS::DIV, s, false, mn);
+#pragma unroll
+    for (int k = 0; k < TS::T; ++k) tb[k] = Real(0);
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+      const Real l = lam[a];
+#pragma unroll
+      for (int k = 0; k < TS::T; ++k) tb[k] += l * pn[a].d[k];
+    }
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+      const Real l = lam[NP + m];
+#pragma unroll
+      for (int k = 0; k < TS::T; ++k) tb[k] += l * mn[m].d[k];
+    }
+  }
+  // centre term transposed: slots on the cell's phi and the unscaled
+  // central differences gcr[a][d] it reads
+  {
+    using CS = CellStore<DIM, NP, NM>;
+    constexpr int WC = NP * (1 + DIM);
+    using DC = Dual<Real, WC>;
+    ValAcc<NP, NM, Real, Real> V{st, g.fstride, plane, base, g.pitch};
+    DiffPrm<DC, P> dp;
+    dp.mob = DC(g.mob);
+#pragma unroll
+    for (int p = 0; p < P; ++p) dp.delta[p] = DC(g.delta[p]);
+    DC ph[NP], gcr[NP][DIM], Gcd[NP];
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+      ph[a] = DC(V.phi(a, 0, 0, 0));
+      ph[a].d[a] = Real(1);
+      gcr[a][0] = DC(V.phi(a, 1, 0, 0) - V.phi(a, -1, 0, 0));
+      gcr[a][1] = DC(V.phi(a, 0, 1, 0) - V.phi(a, 0, -1, 0));
+      if constexpr (DIM == 3) gcr[a][2] = DC(V.phi(a, 0, 0, 1) - V.phi(a, 0, 0, -1));
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) gcr[a][d].d[NP + a * DIM + d] = Real(1);
+      Gcd[a] = DC(Real(0));
+    }
+    centre_term<DIM, NP, NM, Real, DC, kFeatAll, false>(g, dp, ph, gcr, V.mask(), Gcd);
+    Real sb[WC];
+#pragma unroll
+    for (int k = 0; k < WC; ++k) sb[k] = Real(0);
+#pragma unroll
+    for (int a = 0; a < NP; ++a)
+#pragma unroll
+      for (int k = 0; k < WC; ++k) sb[k] += tb[TS::GC + a] * Gcd[a].d[k];
+#pragma unroll
+    for (int a = 0; a < NP; ++a) out[CS::PH + a] = tb[TS::PH + a] + sb[a];
+#pragma unroll
+    for (int k = 0; k < NM; ++k) {
+      out[CS::MC + k] = tb[TS::MC + k];
+      out[CS::DIV + k] = tb[TS::DIV + k];
+    }
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+      out[CS::DJ + a] = tb[TS::DJ + a];
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) out[CS::GCR + a * DIM + d] = sb[NP + a * DIM + d];
+    }
+  }
+  // parameter gradient of the cell's update
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    Real sp = Real(0);
+#pragma unroll
+    for (int a = 0; a < NP; ++a) sp += tb[TS::DJ + a] * divJ[a].d[p] + tb[TS::GC + a] * Gc[a].d[p];
+    gpar[p] += (double)sp;
+  }
+  gpar[P] += (double)tb[TS::MOB];
+#pragma unroll
+  for (int k = 0; k < ND; ++k) {
+    Real sd = Real(0);
+#pragma unroll
+    for (int m = 0; m < NM; ++m) sd += tb[TS::DIV + m] * div[m].d[k];
+    gpar[P + 1 + k] += (double)sd;
+  }
+}
+
 // Pass 1 (see the file comment).  tbar: [TB][cells], dense cell order.
 template <int DIM, int NP, int NM, class Real>
 __global__ void __launch_bounds__(128) k_adj_cell(const Real* __restrict__ st, const Real* __restrict__ lam_in,
@@ -146,197 +320,22 @@ __global__ void __launch_bounds__(128) k_adj_cell(const Real* __restrict__ st, c
                                                   const __grid_constant__ StepArgs<Real, NP, NM> g,
                                                   const __grid_constant__ AdjExtra<Real, NP, NM> ex,
                                                   double* __restrict__ partials) {
-  constexpr int P = NP * (NP - 1) / 2;
-  constexpr int ND = NP * NM * NM;
   constexpr int NPRM = ParamCount<NP, NM>::value;
-  using TS = TailSlots<NP, NM>;
-  using DP = Dual<Real, P>;
-  using DD = Dual<Real, ND>;
-  using DT = Dual<Real, TS::T>;
+  constexpr int TB = CellStore<DIM, NP, NM>::TB;
   const long long cells = (long long)g.nx * g.ny * g.nz;
-  const long long plane = (long long)g.nyp * g.pitch;
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   double gpar[NPRM];
 #pragma unroll
   for (int k = 0; k < NPRM; ++k) gpar[k] = 0.0;
   if (i < cells) {
     const int x = (int)(i % g.nx), y = (int)((i / g.nx) % g.ny), z = (int)(i / ((long long)g.nx * g.ny));
-    const long long base = padded_index<DIM>(g, x, y, z);
-    // stencil part: divJ, Gc with delta slots
-    DP divJ[NP], Gc[NP];
-    {
-      ValAcc<NP, NM, Real, DP> A{st, g.fstride, plane, base, g.pitch};
-      DiffPrm<DP, P> dp;
-      dp.mob = DP(g.mob);
+    Real lam[NP + NM], out[TB];
 #pragma unroll
-      for (int p = 0; p < P; ++p) {
-        dp.delta[p] = DP(g.delta[p]);
-        dp.delta[p].d[p] = Real(1);
-      }
-      DP ph[NP];
+    for (int f = 0; f < NP + NM; ++f) lam[f] = lam_in[f * cells + i];
+    adj_cell<DIM, NP, NM, Real>(st, padded_index<DIM>(g, x, y, z), (DIM == 3 ? z : y) + g.zorg, lab_cell<DIM>(g, x, y, z),
+                                g, ex, lam, out, gpar);
 #pragma unroll
-      for (int a = 0; a < NP; ++a) {
-        ph[a] = A.phi(a, 0, 0, 0);
-        divJ[a] = DP(Real(0));
-        Gc[a] = DP(Real(0));
-      }
-      gradient_terms<DIM, NP, NM, Real, DP, ValAcc<NP, NM, Real, DP>, kFeatAll, false>(
-          A, g, dp, ph, A.mask(), any_aniso<DIM>(g.aniso, P), divJ, Gc);
-    }
-    // stencil part: div with D slots (M = sum_a h_a D^a chi^a)
-    DD div[NM];
-    {
-      ValAcc<NP, NM, Real, DD> B{st, g.fstride, plane, base, g.pitch};
-      DD DXd[NP][NM * NM];
-#pragma unroll
-      for (int a = 0; a < NP; ++a)
-#pragma unroll
-        for (int r = 0; r < NM; ++r)
-#pragma unroll
-          for (int c = 0; c < NM; ++c) {
-            DD sum(Real(0));
-#pragma unroll
-            for (int m = 0; m < NM; ++m) {
-              DD Dm(ex.D[a][r * NM + m]);
-              Dm.d[(a * NM + r) * NM + m] = Real(1);
-              sum += Dm * DD(g.chi[a][m * NM + c]);
-            }
-            DXd[a][r * NM + c] = sum;
-          }
-      DD ph[NP], mc[NM], Mc[NM * NM];
-#pragma unroll
-      for (int a = 0; a < NP; ++a) ph[a] = B.phi(a, 0, 0, 0);
-#pragma unroll
-      for (int k = 0; k < NM; ++k) {
-        mc[k] = B.mu(k, 0, 0, 0);
-        div[k] = DD(Real(0));
-      }
-      cell_mobility<NP, NM>(ph, DXd, Mc);
-#pragma unroll
-      for (int d = 0; d < DIM; ++d) {
-#pragma unroll
-        for (int sd = -1; sd <= 1; sd += 2) {
-          const Off<DIM> o = unit<DIM>(d, sd);
-          DD pn[NP], Mn[NM * NM];
-#pragma unroll
-          for (int a = 0; a < NP; ++a) pn[a] = B.phi(a, o.x, o.y, o.z);
-          cell_mobility<NP, NM>(pn, DXd, Mn);
-#pragma unroll
-          for (int r = 0; r < NM; ++r)
-#pragma unroll
-            for (int c = 0; c < NM; ++c) {
-              DD Mf = Real(0.5) * (Mc[r * NM + c] + Mn[r * NM + c]);
-              div[r] += Mf * ((B.mu(c, o.x, o.y, o.z) - mc[c]) * g.inv_dx2);
-            }
-        }
-      }
-    }
-    // the tail, one slot per input
-    Real tb[TS::T];
-    {
-      DT in[TS::T];
-#pragma unroll
-      for (int k = 0; k < TS::T; ++k) in[k] = DT(Real(0));
-#pragma unroll
-      for (int a = 0; a < NP; ++a) {
-        in[TS::PH + a] = DT(st[a * g.fstride + base]);
-        in[TS::DJ + a] = DT(divJ[a].v);
-        in[TS::GC + a] = DT(Gc[a].v);
-      }
-#pragma unroll
-      for (int k = 0; k < NM; ++k) {
-        in[TS::MC + k] = DT(st[(NP + k) * g.fstride + base]);
-        in[TS::DIV + k] = DT(div[k].v);
-      }
-      in[TS::MOB] = DT(g.mob);
-#pragma unroll
-      for (int k = 0; k < TS::T; ++k) in[k].d[k] = Real(1);
-      DiffPrm<DT, P> dp;
-      dp.mob = in[TS::MOB];
-#pragma unroll
-      for (int p = 0; p < P; ++p) dp.delta[p] = DT(g.delta[p]);
-      const int kz = (DIM == 3 ? z : y) + g.zorg;
-      const Real s = g.tz0 + g.tzg * (Real(kz) + Real(0.5));
-      DT pn[NP], mn[NM];
-      phase_update<DIM, NP, NM, Real, DT, kFeatAll>(g, dp, in + TS::PH, in + TS::MC, in + TS::DJ, in + TS::GC, s,
-                                                    lab_cell<DIM>(g, x, y, z), pn);
-      mu_update<NP, NM, Real, DT>(g, in + TS::PH, pn, in + TS::MC, in + TS::DIV, s, false, mn);
-#pragma unroll
-      for (int k = 0; k < TS::T; ++k) tb[k] = Real(0);
-#pragma unroll
-      for (int a = 0; a < NP; ++a) {
-        const Real l = lam_in[a * cells + i];
-#pragma unroll
-        for (int k = 0; k < TS::T; ++k) tb[k] += l * pn[a].d[k];
-      }
-#pragma unroll
-      for (int m = 0; m < NM; ++m) {
-        const Real l = lam_in[(NP + m) * cells + i];
-#pragma unroll
-        for (int k = 0; k < TS::T; ++k) tb[k] += l * mn[m].d[k];
-      }
-    }
-    // centre term transposed: slots on the cell's phi and the unscaled
-    // central differences gcr[a][d] it reads
-    {
-      using CS = CellStore<DIM, NP, NM>;
-      constexpr int WC = NP * (1 + DIM);
-      using DC = Dual<Real, WC>;
-      ValAcc<NP, NM, Real, Real> V{st, g.fstride, plane, base, g.pitch};
-      DiffPrm<DC, P> dp;
-      dp.mob = DC(g.mob);
-#pragma unroll
-      for (int p = 0; p < P; ++p) dp.delta[p] = DC(g.delta[p]);
-      DC ph[NP], gcr[NP][DIM], Gcd[NP];
-#pragma unroll
-      for (int a = 0; a < NP; ++a) {
-        ph[a] = DC(V.phi(a, 0, 0, 0));
-        ph[a].d[a] = Real(1);
-        gcr[a][0] = DC(V.phi(a, 1, 0, 0) - V.phi(a, -1, 0, 0));
-        gcr[a][1] = DC(V.phi(a, 0, 1, 0) - V.phi(a, 0, -1, 0));
-        if constexpr (DIM == 3) gcr[a][2] = DC(V.phi(a, 0, 0, 1) - V.phi(a, 0, 0, -1));
-#pragma unroll
-        for (int d = 0; d < DIM; ++d) gcr[a][d].d[NP + a * DIM + d] = Real(1);
-        Gcd[a] = DC(Real(0));
-      }
-      centre_term<DIM, NP, NM, Real, DC, kFeatAll, false>(g, dp, ph, gcr, V.mask(), Gcd);
-      Real sb[WC];
-#pragma unroll
-      for (int k = 0; k < WC; ++k) sb[k] = Real(0);
-#pragma unroll
-      for (int a = 0; a < NP; ++a)
-#pragma unroll
-        for (int k = 0; k < WC; ++k) sb[k] += tb[TS::GC + a] * Gcd[a].d[k];
-#pragma unroll
-      for (int a = 0; a < NP; ++a) tbar[(CS::PH + a) * cells + i] = tb[TS::PH + a] + sb[a];
-#pragma unroll
-      for (int k = 0; k < NM; ++k) {
-        tbar[(CS::MC + k) * cells + i] = tb[TS::MC + k];
-        tbar[(CS::DIV + k) * cells + i] = tb[TS::DIV + k];
-      }
-#pragma unroll
-      for (int a = 0; a < NP; ++a) {
-        tbar[(CS::DJ + a) * cells + i] = tb[TS::DJ + a];
-#pragma unroll
-        for (int d = 0; d < DIM; ++d) tbar[(CS::GCR + a * DIM + d) * cells + i] = sb[NP + a * DIM + d];
-      }
-    }
-    // parameter gradient of cell i's update
-#pragma unroll
-    for (int p = 0; p < P; ++p) {
-      Real sp = Real(0);
-#pragma unroll
-      for (int a = 0; a < NP; ++a) sp += tb[TS::DJ + a] * divJ[a].d[p] + tb[TS::GC + a] * Gc[a].d[p];
-      gpar[p] += (double)sp;
-    }
-    gpar[P] += (double)tb[TS::MOB];
-#pragma unroll
-    for (int k = 0; k < ND; ++k) {
-      Real sd = Real(0);
-#pragma unroll
-      for (int m = 0; m < NM; ++m) sd += tb[TS::DIV + m] * div[m].d[k];
-      gpar[P + 1 + k] += (double)sd;
-    }
+    for (int k = 0; k < TB; ++k) tbar[k * cells + i] = out[k];
   }
   if (partials) {
     // per warp by a fixed shuffle tree, then the 4 warps in order
@@ -357,87 +356,19 @@ __global__ void __launch_bounds__(128) k_adj_cell(const Real* __restrict__ st, c
   }
 }
 
-// Face fluxes along axis D whose stencil contains position (px, py, pz):
-// acc[a'] += sum_a Jbar_f[a] dJ_f[a]/dphi_a'(p).  A face is named by its
-// lower cell L (upper R = L + e_D); its stencil is L, R and, with
-// anisotropy, L +- e_t, R +- e_t for t != D.
+// Adjoint of the face flux along axis D at the face whose lower cell has
+// padded index `base`: the flux is differentiated in forward mode with one
+// slot per face value pf_a and face gradient component gr_a,d, contracted with
+// Jbar, and given per stencil position class (FaceStore).
 template <int DIM, int D, int NP, int NM, class Real>
-__device__ __forceinline__ void gather_faces(const Real* __restrict__ st, const Real* __restrict__ tbar,
-                                             const StepArgs<Real, NP, NM>& g, bool need_tan, int px, int py, int pz,
-                                             long long seed, Real* acc) {
-  constexpr int P = NP * (NP - 1) / 2;
-  using TS = TailSlots<NP, NM>;
-  using DN = Dual<Real, NP>;
-  const long long cells = (long long)g.nx * g.ny * g.nz;
-  const long long plane = (long long)g.nyp * g.pitch;
-  DiffPrm<DN, P> dp;
-  dp.mob = DN(g.mob);
-#pragma unroll
-  for (int p = 0; p < P; ++p) dp.delta[p] = DN(g.delta[p]);
-  const int ncand = 2 + (need_tan ? 4 * (DIM - 1) : 0);
-#pragma unroll 1
-  for (int c = 0; c < ncand; ++c) {
-    // offset of L from p
-    int o[3] = {0, 0, 0};
-    if (c == 0) {
-      o[D] = -1;   // p is R
-    } else if (c > 1) {
-      const int k = c - 2;
-      const int t = DIM == 2 ? 1 - D : (D + 1 + (k >> 2)) % 3;   // a tangential axis of D
-      const int sgn = (k & 1) ? 1 : -1;
-      o[t] = -sgn;                  // p = L + sgn e_t, or
-      if ((k >> 1) & 1) o[D] = -1;  // p = R + sgn e_t
-    }
-    const int lx = px + o[0], ly = py + o[1], lz = pz + o[2];
-    const int rx = lx + (D == 0), ry = ly + (D == 1), rz = lz + (D == 2);
-    const bool inL = in_grid<DIM>(g, lx, ly, lz), inR = in_grid<DIM>(g, rx, ry, rz);
-    if (!inL && !inR) continue;
-    Real Jbar[NP];
-    const long long li = ((long long)lz * g.ny + ly) * g.nx + lx, ri = ((long long)rz * g.ny + ry) * g.nx + rx;
-#pragma unroll
-    for (int a = 0; a < NP; ++a) {
-      const Real bl = inL ? tbar[(TS::DJ + a) * cells + li] : Real(0);
-      const Real br = inR ? tbar[(TS::DJ + a) * cells + ri] : Real(0);
-      Jbar[a] = (bl - br) * g.inv_dx;
-    }
-    SeedAcc<NP, NM, Real> A{st, g.fstride, plane, padded_index<DIM>(g, lx, ly, lz), seed, g.pitch};
-    DN J[NP];
-    face_flux<DIM, D, NP, NM, Real, DN, SeedAcc<NP, NM, Real>, kFeatAll>(A, g, dp, A.mask(), 1, need_tan, J);
-#pragma unroll
-    for (int a = 0; a < NP; ++a)
-#pragma unroll
-      for (int b = 0; b < NP; ++b) acc[b] += Jbar[a] * J[a].d[b];
-  }
-}
-
-// Pass 2 for the faces along axis D of one cell i: the face with lower cell
-// L = i and, at the lower domain end, the face with L = i - e_D.  The flux
-// adjoint is Jbar = (tbar_divJ(L) - tbar_divJ(R)) / dx over the cells of the
-// grid among L, R; the face flux is differentiated in forward mode with one
-// slot per face value pf_a and face gradient component gr_a,d, and the result
-// is written per stencil position class (FaceStore).
-template <int DIM, int D, int NP, int NM, class Real>
-__device__ __forceinline__ void face_adjoint(const Real* __restrict__ st, const Real* __restrict__ tbar,
-                                             Real* __restrict__ frec, const StepArgs<Real, NP, NM>& g,
-                                             bool need_tan, int lx, int ly, int lz) {
+__device__ __forceinline__ void face_records(const Real* __restrict__ st, long long base, const StepArgs<Real, NP, NM>& g,
+                                             bool need_tan, const Real* Jbar, Real* rec) {
   constexpr int P = NP * (NP - 1) / 2;
   constexpr int W = NP * (1 + DIM);
-  using CS = CellStore<DIM, NP, NM>;
   using FS = FaceStore<DIM, NP>;
   using DW = Dual<Real, W>;
-  const long long cells = (long long)g.nx * g.ny * g.nz;
   const long long plane = (long long)g.nyp * g.pitch;
-  const int rx = lx + (D == 0), ry = ly + (D == 1), rz = lz + (D == 2);
-  const bool inL = in_grid<DIM>(g, lx, ly, lz), inR = in_grid<DIM>(g, rx, ry, rz);
-  const long long li = ((long long)lz * g.ny + ly) * g.nx + lx, ri = ((long long)rz * g.ny + ry) * g.nx + rx;
-  Real Jbar[NP];
-#pragma unroll
-  for (int a = 0; a < NP; ++a) {
-    const Real bl = inL ? tbar[(CS::DJ + a) * cells + li] : Real(0);
-    const Real br = inR ? tbar[(CS::DJ + a) * cells + ri] : Real(0);
-    Jbar[a] = (bl - br) * g.inv_dx;
-  }
-  ValAcc<NP, NM, Real, Real> V{st, g.fstride, plane, padded_index<DIM>(g, lx, ly, lz), g.pitch};
+  ValAcc<NP, NM, Real, Real> V{st, g.fstride, plane, base, g.pitch};
   DW pf[NP], gr[NP][DIM];
 #pragma unroll
   for (int a = 0; a < NP; ++a) {
@@ -475,21 +406,46 @@ __device__ __forceinline__ void face_adjoint(const Real* __restrict__ st, const 
   for (int a = 0; a < NP; ++a)
 #pragma unroll
     for (int k = 0; k < W; ++k) sb[k] += Jbar[a] * J[a].d[k];
-  const long long fid = face_id<DIM, D>(g, lx, ly, lz);
-  const long long nfaces = (long long)(g.nx + (D == 0)) * (g.ny + (D == 1)) * ((DIM == 3 ? g.nz : 1) + (D == 2));
 #pragma unroll
   for (int a = 0; a < NP; ++a) {
     const Real gn = sb[NP + a * DIM + D] * g.inv_dx;
-    frec[(FS::AL + a) * nfaces + fid] = Real(0.5) * sb[a] - gn;
-    frec[(FS::AR + a) * nfaces + fid] = Real(0.5) * sb[a] + gn;
+    rec[FS::AL + a] = Real(0.5) * sb[a] - gn;
+    rec[FS::AR + a] = Real(0.5) * sb[a] + gn;
     int tt = 0;
 #pragma unroll
     for (int t = 0; t < DIM; ++t) {
       if (t == D) continue;
-      frec[(FS::TG + a * (DIM - 1) + tt) * nfaces + fid] = sb[NP + a * DIM + t] * g.quarter_inv_dx;
+      rec[FS::TG + a * (DIM - 1) + tt] = sb[NP + a * DIM + t] * g.quarter_inv_dx;
       ++tt;
     }
   }
+}
+
+// Pass 2 for the face along axis D with lower cell L = (lx, ly, lz): the flux
+// adjoint is Jbar = (tbar_divJ(L) - tbar_divJ(R)) / dx over the cells of the
+// grid among L, R.
+template <int DIM, int D, int NP, int NM, class Real>
+__device__ __forceinline__ void face_adjoint(const Real* __restrict__ st, const Real* __restrict__ tbar,
+                                             Real* __restrict__ frec, const StepArgs<Real, NP, NM>& g,
+                                             bool need_tan, int lx, int ly, int lz) {
+  using CS = CellStore<DIM, NP, NM>;
+  using FS = FaceStore<DIM, NP>;
+  const long long cells = (long long)g.nx * g.ny * g.nz;
+  const int rx = lx + (D == 0), ry = ly + (D == 1), rz = lz + (D == 2);
+  const bool inL = in_grid<DIM>(g, lx, ly, lz), inR = in_grid<DIM>(g, rx, ry, rz);
+  const long long li = ((long long)lz * g.ny + ly) * g.nx + lx, ri = ((long long)rz * g.ny + ry) * g.nx + rx;
+  Real Jbar[NP], rec[FS::N];
+#pragma unroll
+  for (int a = 0; a < NP; ++a) {
+    const Real bl = inL ? tbar[(CS::DJ + a) * cells + li] : Real(0);
+    const Real br = inR ? tbar[(CS::DJ + a) * cells + ri] : Real(0);
+    Jbar[a] = (bl - br) * g.inv_dx;
+  }
+  face_records<DIM, D, NP, NM, Real>(st, padded_index<DIM>(g, lx, ly, lz), g, need_tan, Jbar, rec);
+  const long long fid = face_id<DIM, D>(g, lx, ly, lz);
+  const long long nfaces = (long long)(g.nx + (D == 0)) * (g.ny + (D == 1)) * ((DIM == 3 ? g.nz : 1) + (D == 2));
+#pragma unroll
+  for (int k = 0; k < FS::N; ++k) frec[k * nfaces + fid] = rec[k];
 }
 
 template <int DIM, int NP, int NM, class Real>
@@ -711,6 +667,244 @@ __global__ void __launch_bounds__(GatherShape<DIM>::THREADS)
   }
 }
 
+// The three passes in one kernel for 2-D FP32: a CTA covers 30 x TY cells and
+// computes the cell pass for them and the ring around them, the face records of
+// every face that touches them, and the gather, with everything in between in
+// shared memory (a thread per cell of the ringed tile).  The three launches of a
+// 256^2 reverse step were latency and traffic through L2 (cell 10.0, faces 4.6,
+// gather 11.1 us); one launch of 288 CTAs, two per SM, redoes a third of the
+// cell pass instead: 15.0 us.  FP64 keeps the three passes: its cell pass is bound by
+// the FP64 pipe, where redoing costs what it computes.
+// Local cell (lx, ly) of the tile, ring included, is the grid cell at x0 + lx,
+// y0 + ly, wrapped where the axis is periodic; past a no-flux boundary there is
+// none (its entries are zero), and a boundary cell also collects what reads its
+// ghost image.
+constexpr int kFusedTX = 30, kFusedTY = 8;
+template <int NP, int NM>
+struct FusedShape {
+  static constexpr int W = kFusedTX + 2, H = kFusedTY + 2;
+  static constexpr int THREADS = W * H;
+  using FS = FaceStore<2, NP>;
+  // per local cell: adjoints of divJ, of the central differences and of div,
+  // M, mu, the records of its upper x and y faces
+  static constexpr int DJ = 0, GCR = NP, DIV = GCR + 2 * NP, M = DIV + NM, MU = M + NM * NM, FX = MU + NM,
+                       FY = FX + FS::N, N = FY + FS::N;
+};
+inline dim3 fused_grid(const HostModel& m) {
+  return dim3((unsigned)((m.nx + kFusedTX - 1) / kFusedTX), (unsigned)((m.ny + kFusedTY - 1) / kFusedTY));
+}
+
+template <int NP, int NM, class Real>
+__global__ void __launch_bounds__(FusedShape<NP, NM>::THREADS, 2)
+    k_adj_fused(const Real* __restrict__ st, const Real* __restrict__ lam_in, Real* __restrict__ lam_out,
+                const __grid_constant__ StepArgs<Real, NP, NM> g, const __grid_constant__ AdjExtra<Real, NP, NM> ex,
+                double* __restrict__ partials) {
+  using Fu = FusedShape<NP, NM>;
+  using FS = FaceStore<2, NP>;
+  using CS = CellStore<2, NP, NM>;
+  using DN = Dual<Real, NP>;
+  constexpr int NPRM = ParamCount<NP, NM>::value;
+  constexpr int P = NP * (NP - 1) / 2;
+  constexpr int NW = Fu::THREADS / 32;
+  __shared__ Real sm[Fu::N][Fu::THREADS];
+  __shared__ double red[NW][NPRM];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int lx = lane - 1, ly = (tid >> 5) - 1;
+  const int gx = (int)blockIdx.x * kFusedTX + lx, gy = (int)blockIdx.y * kFusedTY + ly;
+  const long long cells = (long long)g.nx * g.ny;
+  // the grid cell (vx, vy: there is one) and the padded position to read at
+  auto wrap = [](int i, int n, int bc, int& w) {
+    w = i;
+    if (i >= 0 && i < n) return true;
+    if (bc != 3 || i < -1 || i > n) return false;
+    w = i < 0 ? n - 1 : 0;
+    return true;
+  };
+  int wx, wy;
+  const bool vx = wrap(gx, g.nx, g.bc[0], wx), vy = wrap(gy, g.ny, g.bc[1], wy);
+  const bool valid = vx && vy;
+  const bool inner = lx >= 0 && lx < kFusedTX && ly >= 0 && ly < kFusedTY && gx < g.nx && gy < g.ny;
+  const long long base = padded_index<2>(g, wx, wy, 0);   // read only at cells and at the lower ghosts
+  const bool need_tan = any_aniso<2>(g.aniso, P);
+  double gpar[NPRM];
+#pragma unroll
+  for (int k = 0; k < NPRM; ++k) gpar[k] = 0.0;
+  Real own[NP + NM], Mj[NM * NM], muj[NM], phj[NP];
+#pragma unroll
+  for (int f = 0; f < NP + NM; ++f) own[f] = Real(0);
+  // ---- cell pass
+  if (valid) {
+    Real lam[NP + NM], out[CS::TB];
+    const long long i = (long long)wy * g.nx + wx;
+#pragma unroll
+    for (int f = 0; f < NP + NM; ++f) lam[f] = lam_in[f * cells + i];
+    adj_cell<2, NP, NM, Real>(st, base, wy + g.zorg, 0ull, g, ex, lam, out, gpar);
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+      own[a] = out[CS::PH + a];
+      sm[Fu::DJ + a][tid] = out[CS::DJ + a];
+      phj[a] = st[a * g.fstride + base];
+    }
+#pragma unroll
+    for (int k = 0; k < 2 * NP; ++k) sm[Fu::GCR + k][tid] = out[CS::GCR + k];
+    cell_mobility<NP, NM>(phj, g.DX, Mj);
+#pragma unroll
+    for (int k = 0; k < NM; ++k) {
+      own[NP + k] = out[CS::MC + k];
+      sm[Fu::DIV + k][tid] = out[CS::DIV + k];
+      muj[k] = st[(NP + k) * g.fstride + base];
+      sm[Fu::MU + k][tid] = muj[k];
+    }
+#pragma unroll
+    for (int k = 0; k < NM * NM; ++k) sm[Fu::M + k][tid] = Mj[k];
+  } else {
+#pragma unroll
+    for (int k = 0; k < Fu::FX; ++k) sm[k][tid] = Real(0);
+  }
+  __syncthreads();
+  // ---- face pass: this cell's upper x and y faces (of a cell past the lower
+  // boundary: the boundary face)
+  {
+    const bool rvx = lane < 31 && ((gx + 1 >= 0 && gx + 1 < g.nx) || (g.bc[0] == 3 && gx + 1 <= g.nx));
+    const bool rvy = ly <= kFusedTY - 1 && ((gy + 1 >= 0 && gy + 1 < g.ny) || (g.bc[1] == 3 && gy + 1 <= g.ny));
+    Real Jbar[NP], rec[FS::N];
+    if (lane < 31 && vy && (vx || (gx == -1 && rvx))) {
+#pragma unroll
+      for (int a = 0; a < NP; ++a) Jbar[a] = (sm[Fu::DJ + a][tid] - sm[Fu::DJ + a][tid + 1]) * g.inv_dx;
+      face_records<2, 0, NP, NM, Real>(st, base, g, need_tan, Jbar, rec);
+    } else {
+#pragma unroll
+      for (int k = 0; k < FS::N; ++k) rec[k] = Real(0);
+    }
+#pragma unroll
+    for (int k = 0; k < FS::N; ++k) sm[Fu::FX + k][tid] = rec[k];
+    if (ly < kFusedTY && vx && (vy || (gy == -1 && rvy))) {
+#pragma unroll
+      for (int a = 0; a < NP; ++a) Jbar[a] = (sm[Fu::DJ + a][tid] - sm[Fu::DJ + a][tid + 32]) * g.inv_dx;
+      face_records<2, 1, NP, NM, Real>(st, base, g, need_tan, Jbar, rec);
+    } else {
+#pragma unroll
+      for (int k = 0; k < FS::N; ++k) rec[k] = Real(0);
+    }
+#pragma unroll
+    for (int k = 0; k < FS::N; ++k) sm[Fu::FY + k][tid] = rec[k];
+  }
+  __syncthreads();
+  // ---- gather
+  if (inner) {
+    Real acc[NP + NM], Mbar[NM * NM];
+#pragma unroll
+    for (int f = 0; f < NP + NM; ++f) acc[f] = own[f];
+#pragma unroll
+    for (int k = 0; k < NM * NM; ++k) Mbar[k] = Real(0);
+    // local positions holding this cell's value: itself and, at no-flux
+    // boundaries, its ghost images (a periodic image is a wrapped neighbour's)
+    int xs[3], ys[3], nxs = 1, nys = 1;
+    xs[0] = lx;
+    ys[0] = ly;
+    if (g.bc[0] != 3 && gx == 0) xs[nxs++] = lx - 1;
+    if (g.bc[0] != 3 && gx == g.nx - 1) xs[nxs++] = lx + 1;
+    if (g.bc[1] != 3 && gy == 0) ys[nys++] = ly - 1;
+    if (g.bc[1] != 3 && gy == g.ny - 1) ys[nys++] = ly + 1;
+    auto at = [](int x, int y) { return (y + 1) * Fu::W + x + 1; };
+    auto in = [](int x, int y) { return x >= -1 && x <= kFusedTX && y >= -1 && y <= kFusedTY; };
+#pragma unroll 1
+    for (int iy = 0; iy < nys; ++iy)
+#pragma unroll 1
+      for (int ix = 0; ix < nxs; ++ix) {
+        const int px = xs[ix], py = ys[iy];
+        // face records that read the position
+        auto face = [&](int F, int slot, int x, int y, Real sgn, int as) {
+          if (!in(x, y)) return;
+          const int l = at(x, y);
+#pragma unroll
+          for (int a = 0; a < NP; ++a) acc[a] += sgn * sm[F + slot + a * as][l];
+        };
+        face(Fu::FX, FS::AR, px - 1, py, Real(1), 1);
+        face(Fu::FX, FS::AL, px, py, Real(1), 1);
+        face(Fu::FY, FS::AR, px, py - 1, Real(1), 1);
+        face(Fu::FY, FS::AL, px, py, Real(1), 1);
+        if (need_tan) {
+#pragma unroll
+          for (int s = -1; s <= 1; s += 2) {
+            face(Fu::FX, FS::TG, px, py - s, Real(s), 1);       // p = L + s e_y
+            face(Fu::FX, FS::TG, px - 1, py - s, Real(s), 1);   // p = R + s e_y
+            face(Fu::FY, FS::TG, px - s, py, Real(s), 1);
+            face(Fu::FY, FS::TG, px - s, py - 1, Real(s), 1);
+          }
+        }
+        // centre-term differences and mu fluxes of the four neighbours of the position
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int d = c >> 1, s = (c & 1) ? 1 : -1;
+          const int qx = px - (d == 0 ? s : 0), qy = py - (d == 1 ? s : 0);
+          if (!in(qx, qy)) continue;
+          const int l = at(qx, qy);
+#pragma unroll
+          for (int a = 0; a < NP; ++a) acc[a] += Real(s) * sm[Fu::GCR + a * 2 + d][l];
+#pragma unroll
+          for (int r = 0; r < NM; ++r) {
+            const Real db = sm[Fu::DIV + r][l];
+#pragma unroll
+            for (int q = 0; q < NM; ++q) {
+              acc[NP + q] += db * (Real(0.5) * (sm[Fu::M + r * NM + q][l] + Mj[r * NM + q])) * g.inv_dx2;
+              Mbar[r * NM + q] += db * (Real(0.5) * (muj[q] - sm[Fu::MU + q][l])) * g.inv_dx2;
+            }
+          }
+        }
+      }
+    // mu flux of the cell itself
+    Real db[NM];
+#pragma unroll
+    for (int r = 0; r < NM; ++r) db[r] = sm[Fu::DIV + r][tid];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const long long nb = base + ((c >> 1) == 0 ? 1 : (long long)g.pitch) * ((c & 1) ? 1 : -1);
+      Real phn[NP], Mn[NM * NM];
+#pragma unroll
+      for (int a = 0; a < NP; ++a) phn[a] = st[a * g.fstride + nb];
+      cell_mobility<NP, NM>(phn, g.DX, Mn);
+#pragma unroll
+      for (int r = 0; r < NM; ++r)
+#pragma unroll
+        for (int q = 0; q < NM; ++q) {
+          const Real mun = st[(NP + q) * g.fstride + nb];
+          acc[NP + q] -= db[r] * (Real(0.5) * (Mj[r * NM + q] + Mn[r * NM + q])) * g.inv_dx2;
+          Mbar[r * NM + q] += db[r] * (Real(0.5) * (mun - muj[q])) * g.inv_dx2;
+        }
+    }
+    // M(phi_j): chain the mobility adjoint to the phases
+    DN ph[NP], M[NM * NM];
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+      ph[a] = DN(phj[a]);
+      ph[a].d[a] = Real(1);
+    }
+    cell_mobility<NP, NM>(ph, g.DX, M);
+#pragma unroll
+    for (int k = 0; k < NM * NM; ++k)
+#pragma unroll
+      for (int b = 0; b < NP; ++b) acc[b] += Mbar[k] * M[k].d[b];
+    const long long j = (long long)gy * g.nx + gx;
+#pragma unroll
+    for (int f = 0; f < NP + NM; ++f) lam_out[f * cells + j] = acc[f];
+  }
+  // parameter partials of the CTA's own cells: a fixed shuffle tree per warp, the warps in order
+#pragma unroll
+  for (int k = 0; k < NPRM; ++k) {
+    double v = inner ? gpar[k] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) red[tid >> 5][k] = v;
+  }
+  __syncthreads();
+  if (tid < NPRM) {
+    double v = 0.0;
+    for (int w = 0; w < NW; ++w) v += red[w][tid];
+    partials[((long long)blockIdx.y * gridDim.x + blockIdx.x) * NPRM + tid] += v;   // summed over the reverse steps
+  }
+}
+
 // gsum[k] += sum over blocks of partials[b][k]: one warp per parameter, lane
 // l summing blocks l, l + 32, ... in order, then a fixed shuffle tree
 // (deterministic).
@@ -731,6 +925,7 @@ constexpr int kMaxGradParams = 64;
 
 struct AdjKernel {
   int dim, np, nm, dtype, nprm;
+  int fused;   // 1: one launch per reverse step (k_adj_fused), tbar unused
   cudaError_t (*launch)(const void* state, const void* lam_in, void* lam_out, void* tbar, const void* blob,
                         const HostModel& m, double t, double* partials, cudaStream_t st);
 };
@@ -776,16 +971,43 @@ cudaError_t launch_adjoint(const void* state, const void* lam_in, void* lam_out,
   return cudaGetLastError();
 }
 
+// Parameter partials of a reverse step: one set per block of its cell pass.
+inline long long adjoint_blocks(const AdjKernel& k, const HostModel& m) {
+  if (k.fused) return (long long)fused_grid(m).x * fused_grid(m).y;
+  return ((long long)m.nx * m.ny * m.nz + 127) / 128;
+}
+
+template <int NP, int NM, class Real>
+cudaError_t launch_adjoint_fused(const void* state, const void* lam_in, void* lam_out, void*, const void* blob,
+                                 const HostModel& m, double t, double* partials, cudaStream_t st) {
+  StepArgs<Real, NP, NM> g = *reinterpret_cast<const StepArgs<Real, NP, NM>*>(blob);
+  g.tz0 = (Real)temp_offset(m, t);
+  AdjExtra<Real, NP, NM> ex;
+  for (int a = 0; a < NP; ++a)
+    for (int k = 0; k < NM * NM; ++k) ex.D[a][k] = (Real)m.D[a][k];
+  k_adj_fused<NP, NM, Real><<<fused_grid(m), FusedShape<NP, NM>::THREADS, 0, st>>>(
+      reinterpret_cast<const Real*>(state), reinterpret_cast<const Real*>(lam_in), reinterpret_cast<Real*>(lam_out), g,
+      ex, partials);
+  return cudaGetLastError();
+}
+
+template <int NP, int NM, class Real>
+AdjKernel make_adjoint_fused() {
+  static_assert(ParamCount<NP, NM>::value <= kMaxGradParams, "gradient scratch too small");
+  return AdjKernel{2, NP, NM, sizeof(Real) == 8 ? 1 : 0, ParamCount<NP, NM>::value, 1,
+                   &launch_adjoint_fused<NP, NM, Real>};
+}
+
 template <int DIM, int NP, int NM, class Real>
 AdjKernel make_adjoint() {
   static_assert(ParamCount<NP, NM>::value <= kMaxGradParams, "gradient scratch too small");
-  return AdjKernel{DIM, NP, NM, sizeof(Real) == 8 ? 1 : 0, ParamCount<NP, NM>::value,
+  return AdjKernel{DIM, NP, NM, sizeof(Real) == 8 ? 1 : 0, ParamCount<NP, NM>::value, 0,
                    &launch_adjoint<DIM, NP, NM, Real>};
 }
 
 const std::vector<AdjKernel>& adjoint_registry() {
   static const std::vector<AdjKernel> r = {
-      make_adjoint<2, 2, 1, float>(),
+      make_adjoint_fused<2, 1, float>(),
       make_adjoint<2, 2, 1, double>(),
       make_adjoint<2, 3, 2, double>(),
       make_adjoint<3, 2, 1, double>(),
@@ -895,7 +1117,7 @@ ms_status ms_grad(ms_ctx* c, const void* dphi_T, const void* dmu_T, double* dpar
   const long long cells = (long long)m.nx * m.ny * m.nz;
   const size_t lam_bytes = (size_t)NF * cells * s;
   const int nprm = ak->nprm;
-  const int blocks = (int)((cells + 127) / 128);   // blocks of the cell pass (parameter partials)
+  const int blocks = (int)adjoint_blocks(*ak, m);   // sets of parameter partials
   if (nprm > kMaxGradParams) return fail(c, MS_ERR_UNSUPPORTED, "too many parameters for the gradient scratch");
   // lazily sized work buffers, each allocated while it is missing: a failed
   // allocation leaves its pointer null and the next call retries it
@@ -904,7 +1126,7 @@ ms_status ms_grad(ms_ctx* c, const void* dphi_T, const void* dmu_T, double* dpar
       A.adj[b] = dev_alloc(c->hook, lam_bytes);
       if (!A.adj[b]) return fail(c, MS_ERR_OOM, "adjoint state allocation failed");
     }
-  if (!A.tbar) {
+  if (!ak->fused && !A.tbar) {
     A.tbar = dev_alloc(c->hook, (size_t)adjoint_work_elems(m) * s);
     if (!A.tbar) return fail(c, MS_ERR_OOM, "adjoint tail buffer allocation failed");
   }
