@@ -158,7 +158,6 @@ __device__ __forceinline__ void at_face(const StepArgs<Real, NP, NM>& g, const A
 template <int DIM, int NP, int NM, class Real>
 __global__ void __launch_bounds__(256) k_at_list(const __grid_constant__ StepArgs<Real, NP, NM> g) {
   const long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
   const int nzi = DIM == 3 ? g.nz : 1;
   const long long nseg = (long long)g.segs * g.ny * nzi;
   bool need = false;
@@ -177,16 +176,8 @@ __global__ void __launch_bounds__(256) k_at_list(const __grid_constant__ StepArg
           pure = pure && (load_code_from(g.codes_in, g, s + ds, y + dy, z + dz) & kCodePhase) == c0;
     need = !pure;
   }
-  const unsigned int m = __ballot_sync(0xffffffffu, need);
-  if (m == 0u) return;
-  const int first = __ffs(m) - 1;
-  unsigned int base = 0;
-  if (lane == first) base = atomicAdd(&g.at_list[0], (unsigned int)__popc(m));
-  base = __shfl_sync(0xffffffffu, base, first);
-  if (need) {
-    const unsigned int i = base + __popc(m & ((1u << lane) - 1u));
-    if (i < g.at_cap) g.at_list[2 + i] = (unsigned int)w;
-  }
+  const unsigned int i = block_append<256>(&g.at_list[0], need);
+  if (need && i < g.at_cap) g.at_list[2 + i] = (unsigned int)w;
 }
 
 // Warps over the listed segments: stage the block, correct mu.  The last CTA

@@ -71,16 +71,16 @@ struct PadAcc {
 };
 
 template <int NP, int NM, class Real>
-__global__ void __launch_bounds__(128) k_c_scan(const __grid_constant__ StepArgs<Real, NP, NM> g,
+__global__ void __launch_bounds__(256) k_c_scan(const __grid_constant__ StepArgs<Real, NP, NM> g,
                                                 const Real* __restrict__ in,
                                                 const __grid_constant__ CellsScratch<Real> c) {
   const int lane = threadIdx.x & 31;
-  const unsigned int w = (blockIdx.x * 128u + threadIdx.x) >> 5;
-  const unsigned int nseg = (unsigned int)g.segs * g.ny * g.nz;
-  if (w >= nseg) return;
+  const unsigned int nseg = (unsigned int)g.segs * g.ny * g.nz, w0 = (blockIdx.x * 256u + threadIdx.x) >> 5;
+  const bool live = w0 < nseg;   // (warps past the end redo the last segment and list nothing)
+  const unsigned int w = live ? w0 : nseg - 1;
   const int sg = (int)(w % g.segs), y = (int)((w / g.segs) % g.ny), z = (int)(w / ((unsigned int)g.segs * g.ny));
   const int x = 32 * sg + lane;
-  const bool active = x < g.nx;
+  const bool active = live && x < g.nx;
   const long long plane = (long long)g.nyp * g.pitch;
   const Real* s = in + (long long)(z + g.zoff) * plane + (long long)(y + 1) * g.pitch + g.xoff;
   // the 27 segment codes around: all one pure phase = the whole segment is bulk
@@ -139,18 +139,13 @@ __global__ void __launch_bounds__(128) k_c_scan(const __grid_constant__ StepArgs
   // code of the output segment: pure where every cell is bulk in one phase
   const int ref = __shfl_sync(0xffffffffu, bulk, 0);
   const bool same = __all_sync(0xffffffffu, !active || bulk == ref);
-  if (lane == 0) g.codes_out[((long long)(z + g.zoff) * g.ny + y) * g.segs + sg] = same ? (uint8_t)ref : (uint8_t)0;
-  const unsigned int need = __ballot_sync(0xffffffffu, active && bulk == 0);
-  if (need) {
-    const int first = __ffs(need) - 1;
-    unsigned int base = 0;
-    if (lane == first) base = atomicAdd(&c.list[0], (unsigned int)__popc(need));
-    base = __shfl_sync(0xffffffffu, base, first);
-    if ((need >> lane) & 1u) {
-      const unsigned int k = base + __popc(need & ((1u << lane) - 1u));
-      c.list[2 + k] = cell;
-      c.mask[k] = (uint8_t)present;
-    }
+  if (live && lane == 0)
+    g.codes_out[((long long)(z + g.zoff) * g.ny + y) * g.segs + sg] = same ? (uint8_t)ref : (uint8_t)0;
+  const bool want = active && bulk == 0;
+  const unsigned int k = block_append<256>(&c.list[0], want);
+  if (want) {
+    c.list[2 + k] = cell;
+    c.mask[k] = (uint8_t)present;
   }
 }
 

@@ -104,51 +104,71 @@ __device__ __forceinline__ void cell_of(const GgsArgs<Real>& g, unsigned int i, 
   y = (int)(r - (unsigned int)z * (unsigned int)g.ny);
 }
 
+// Each block takes 1024 consecutive cells and its places in the list with one
+// atomic (one per warp serialised on the counter: 37 us at 128^3 on a GB300).
+constexpr int kClassifyRounds = 4;
 template <class Real>
 __global__ void __launch_bounds__(256) k_ggs_classify(const __grid_constant__ GgsArgs<Real> g) {
-  const long long li = blockIdx.x * 256ll + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  bool listed = false;
-  const unsigned int i = (unsigned int)li;
-  if (li < g.cells) {
-    int x, y, z;
-    cell_of(g, i, x, y, z);
-    const uint8_t c0 = g.code_in[i];
-    bool bulk = c0 != 0;
-    if (bulk) {
-      // (every neighbour's code at once: the loads are in flight together)
-      uint8_t nb[6];
+  __shared__ unsigned int s_place[8 * kClassifyRounds + 1];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const long long first = blockIdx.x * (256ll * kClassifyRounds) + threadIdx.x;
+  unsigned int need[kClassifyRounds];
 #pragma unroll
-      for (int d = 0; d < 3; ++d)
+  for (int rnd = 0; rnd < kClassifyRounds; ++rnd) {
+    const long long li = first + 256 * rnd;
+    const unsigned int i = (unsigned int)li;
+    bool listed = false;
+    if (li < g.cells) {
+      int x, y, z;
+      cell_of(g, i, x, y, z);
+      const uint8_t c0 = g.code_in[i];
+      bool bulk = c0 != 0;
+      if (bulk) {
+        // (every neighbour's code at once: the loads are in flight together)
+        uint8_t nb[6];
 #pragma unroll
-        for (int s = 0; s < 2; ++s) nb[2 * d + s] = d < g.dim ? g.code_in[nb_index(g, x, y, z, d, s ? 1 : -1)] : c0;
+        for (int d = 0; d < 3; ++d)
 #pragma unroll
-      for (int k = 0; k < 6; ++k) bulk = bulk && nb[k] == c0;
-    }
-    if (bulk) {
-      // the destination holds the state one step back: rewrite only when it differs
-      if (g.code_out[i] != c0 || g.cnt_out[i] != 1) {
-        g.cnt_out[i] = 1;
-        g.idx_out[i] = (uint8_t)(c0 - 1);
-        g.val_out[i] = Real(1);
-        g.code_out[i] = c0;
+          for (int s = 0; s < 2; ++s) nb[2 * d + s] = d < g.dim ? g.code_in[nb_index(g, x, y, z, d, s ? 1 : -1)] : c0;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) bulk = bulk && nb[k] == c0;
       }
-    } else {
-      listed = true;
+      if (bulk) {
+        // the destination holds the state one step back: rewrite only when it differs
+        if (g.code_out[i] != c0 || g.cnt_out[i] != 1) {
+          g.cnt_out[i] = 1;
+          g.idx_out[i] = (uint8_t)(c0 - 1);
+          g.val_out[i] = Real(1);
+          g.code_out[i] = c0;
+        }
+      } else {
+        listed = true;
+      }
     }
+    need[rnd] = __ballot_sync(0xffffffffu, listed);
+    if (lane == 0) s_place[rnd * 8 + wid] = __popc(need[rnd]);
   }
-  const unsigned int need = __ballot_sync(0xffffffffu, listed);
-  if (need) {
-    const int first = __ffs(need) - 1;
-    unsigned int base = 0;
-    if (lane == first) base = atomicAdd(&g.list[0], (unsigned int)__popc(need));
-    base = __shfl_sync(0xffffffffu, base, first);
-    if (listed) {
-      const unsigned int k = base + __popc(need & ((1u << lane) - 1u));
-      if (k < g.list_cap) g.list[1 + k] = i;
+  __syncthreads();
+  if (wid == 0) {   // exclusive sums of the 32 warp counts, in cell order
+    const unsigned int c = s_place[lane];
+    unsigned int t = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned int u = __shfl_up_sync(0xffffffffu, t, o);
+      if (lane >= o) t += u;
     }
+    s_place[lane] = t - c;
+    if (lane == 31) s_place[32] = t ? atomicAdd(&g.list[0], t) : 0u;
   }
+  __syncthreads();
+#pragma unroll
+  for (int rnd = 0; rnd < kClassifyRounds; ++rnd)
+    if ((need[rnd] >> lane) & 1u) {
+      const unsigned int k = s_place[32] + s_place[rnd * 8 + wid] + __popc(need[rnd] & ((1u << lane) - 1u));
+      if (k < g.list_cap) g.list[1 + k] = (unsigned int)(first + 256 * rnd);
+    }
 }
+static_assert(8 * kClassifyRounds == 32, "one warp sums the counts");
 
 // Simplex projection (Held-Wolfe-Crowder 1974; Duchi et al. 2008) of the
 // first n <= kUnion values: the threshold theta (phi = max(v - theta, 0)).
@@ -581,7 +601,7 @@ GgsArgs<Real> make_args(const ms_ggs* s, int src) {
 template <class Real>
 cudaError_t step_once(ms_ggs* s) {
   const GgsArgs<Real> g = make_args<Real>(s, s->cur);
-  k_ggs_classify<Real><<<(unsigned int)((s->cells + 255) / 256), 256, 0, s->stream>>>(g);
+  k_ggs_classify<Real><<<(unsigned int)((s->cells + 1023) / 1024), 256, 0, s->stream>>>(g);
   if (s->uniform) {
     k_ggs_update<Real, kUnionSmall, true><<<s->upd_blocks, UpdShape<Real, kUnionSmall>::THREADS, 0, s->stream>>>(g);
     k_ggs_update<Real, kUnion, true><<<s->upd_blocks, UpdShape<Real, kUnion>::THREADS, 0, s->stream>>>(g);

@@ -324,7 +324,7 @@ cudaError_t launch_cells(const CUtensorMap*, const CUtensorMap*, const void* in,
     update_per_sm = u < 1 ? 1 : u;
   }
   const long long nseg = (long long)segments(m) * m.ny * m.nz;
-  k_c_scan<NP, NM, Real><<<(unsigned)((nseg + 3) / 4), 128, 0, st>>>(g, p, c);
+  k_c_scan<NP, NM, Real><<<(unsigned)((nseg + 7) / 8), 256, 0, st>>>(g, p, c);
   kf<<<lg.sms * faces_per_sm, 64, 0, st>>>(g, p, c);
   ku<<<lg.sms * update_per_sm, 64, 0, st>>>(g, p, c);
   return cudaGetLastError();

@@ -95,6 +95,30 @@ __device__ __forceinline__ uint32_t stencil_mask(const Acc& A) {
   return m;
 }
 
+// Position in a work list for each thread of a block whose `want` is true: the
+// block takes its places with one atomic on the list's counter (same-address
+// atomics serialise: about one a nanosecond).  Every thread of the block calls.
+template <int THREADS>
+__device__ __forceinline__ unsigned int block_append(unsigned int* counter, bool want) {
+  __shared__ unsigned int s_place[THREADS / 32 + 1];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const unsigned int m = __ballot_sync(0xffffffffu, want);
+  __syncthreads();   // the places of an earlier call have been read
+  if (lane == 0) s_place[wid] = __popc(m);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned int t = 0;
+    for (int k = 0; k < THREADS / 32; ++k) {
+      const unsigned int c = s_place[k];
+      s_place[k] = t;
+      t += c;
+    }
+    s_place[THREADS / 32] = t ? atomicAdd(counter, t) : 0u;
+  }
+  __syncthreads();
+  return s_place[THREADS / 32] + s_place[wid] + __popc(m & ((1u << lane) - 1u));
+}
+
 // Stencil accessor over the shared-memory ring (planes k-1, k, k+1).
 template <int DIM, int NP, int NM, class Real, int TX, int TY>
 struct SmemAcc {
@@ -245,15 +269,17 @@ __device__ __forceinline__ void store_cell(const StepArgs<Real, NP, NM>& g, int 
   store_cell_to<DIM>(g, g.out, x, y, z, pn, mn, write_phi);
 }
 
-// Minimum CTAs per SM the register allocation must allow: two for the
-// few-phase kernels of up to 256 consumer threads, else one.
-template <int NP, int NT>
+// Minimum CTAs per SM the register allocation must allow: four for the binary
+// 2-D FP32 kernels (56 registers; at 59 three fit and a 1537x1411 step took 35
+// instead of 29 us on a GB300), two for the other few-phase kernels of up to
+// 256 consumer threads, else one.
+template <int DIM, int NP, class Real, int NT>
 struct MinBlocks {
-  static constexpr int value = (NP <= 4 && NT <= 256) ? 2 : 1;
+  static constexpr int value = NP <= 4 && NT <= 256 ? (DIM == 2 && NP == 2 && sizeof(Real) == 4 ? 4 : 2) : 1;
 };
 
 template <int DIM, int NP, int NM, class Real, int TX, int TY>
-__global__ void __launch_bounds__(TX* TY + 32, MinBlocks<NP, TX * TY>::value)
+__global__ void __launch_bounds__(TX* TY + 32, MinBlocks<DIM, NP, Real, TX * TY>::value)
     k_gp_step(const __grid_constant__ CUtensorMap tm, const __grid_constant__ StepArgs<Real, NP, NM> g) {
   using Sh = StepShape<DIM, NP, NM, Real, TX, TY>;
   constexpr int NST = Sh::NST;
