@@ -458,28 +458,41 @@ __device__ __forceinline__ void pair_grad(const S* q, Real gam2, const S& del, b
   }
 }
 
-// Interpolation h_a (Eq. hphi) through e1 = sum phi, e2 = sum_{b<c} phi_b phi_c:
-// sum_{b<c; b,c != a} phi_b phi_c = e2 - phi_a (e1 - phi_a).
+// sum_{b<c; b,c != a} phi_b phi_c for every a: nothing for two phases, the
+// product of the others for three, else through e1 = sum phi and e2 =
+// sum_{b<c} phi_b phi_c as e2 - phi_a (e1 - phi_a).
+template <int NP, class S>
+__device__ __forceinline__ void other_products(const S* ph, S* rest) {
+  if constexpr (NP == 3) {
+    rest[0] = ph[1] * ph[2];
+    rest[1] = ph[0] * ph[2];
+    rest[2] = ph[0] * ph[1];
+  } else if constexpr (NP > 3) {
+    S e1 = ph[0];
+#pragma unroll
+    for (int a = 1; a < NP; ++a) e1 += ph[a];
+    S run = ph[0], e2 = ph[1] * run;
+#pragma unroll
+    for (int a = 2; a < NP; ++a) {
+      run += ph[a - 1];
+      e2 += ph[a] * run;
+    }
+#pragma unroll
+    for (int a = 0; a < NP; ++a) rest[a] = e2 - ph[a] * (e1 - ph[a]);
+  }
+}
+
+// Interpolation h_a = phi_a^2 (3 - 2 phi_a) + 2 phi_a sum_{b<c; b,c != a} phi_b phi_c (Eq. hphi).
 template <int NP, class S>
 __device__ __forceinline__ void interp_h(const S* ph, S* h) {
-  S e1 = ph[0];
-#pragma unroll
-  for (int a = 1; a < NP; ++a) e1 += ph[a];
-  S e2 = S(0.0f * val(e1));
-  {
-    S run = ph[0];
-#pragma unroll
-    for (int a = 1; a < NP; ++a) {
-      e2 += ph[a] * run;
-      run += ph[a];
-    }
-  }
+  using R = decltype(val(ph[0]));
+  S rest[NP];
+  other_products<NP>(ph, rest);
 #pragma unroll
   for (int a = 0; a < NP; ++a) {
-    S rest = e2 - ph[a] * (e1 - ph[a]);
-    S p2 = ph[a] * ph[a];
-    h[a] = decltype(val(e1))(3) * p2 - decltype(val(e1))(2) * p2 * ph[a] +
-           decltype(val(e1))(2) * ph[a] * rest;
+    const S p2 = ph[a] * ph[a];
+    h[a] = R(3) * p2 - R(2) * p2 * ph[a];
+    if constexpr (NP > 2) h[a] = h[a] + R(2) * ph[a] * rest[a];
   }
 }
 

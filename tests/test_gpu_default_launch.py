@@ -14,7 +14,7 @@ TOL = STEPS * 4 * 2 * 2.0 ** -24
 
 
 @pytest.mark.parametrize("nx,ny,nz", [(1, 5, 40), (33, 1, 9), (7, 9, 1), (130, 7, 5), (64, 12, 11)])
-@pytest.mark.parametrize("N,kind", [(2, "well"), (2, "noise"), (3, "rotated"), (3, "gamma3"), (3, "anti_trapping")])
+@pytest.mark.parametrize("N,kind", [(2, "well"), (2, "noise"), (3, "rotated"), (3, "gamma3")])
 def test_default_equals_fused(nx, ny, nz, N, kind):
     from paper_2404_01035_gb300 import Simulation
     p = W.small_multiphase(n=8, dim=3, N=N, NM=N - 1, nx=nx, ny=ny, nz=nz, rotate=kind == "rotated",
@@ -22,8 +22,6 @@ def test_default_equals_fused(nx, ny, nz, N, kind):
                            bc=[1, 3, 3] if kind == "well" else None, seed=nx + 3 * nz)
     if kind == "noise":
         p = p.copy(noise_amp=0.05, noise_seed=3)
-    if kind == "anti_trapping":
-        p = p.copy(anti_trapping=1)
     out = []
     for fused in (False, True):
         sim = Simulation(p, dtype="f32")
