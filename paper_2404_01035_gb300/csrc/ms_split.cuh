@@ -16,46 +16,55 @@
 namespace msgb {
 
 // ---------------------------------------------------------------- streaming
-// Each consumer thread updates 4 consecutive cells of one row (16-byte shared
-// loads and global stores), a warp one 128-cell row of the tile; one producer
-// warp streams the mu planes of the tile through a TMA ring and derives the
-// per-segment bulk flags from the segment codes.
+// A CTA takes a tile of 128 x TY cells through `zchunk` planes, a warp per row
+// and 4 consecutive cells per lane; a producer warp streams the mu planes of
+// the tile through a TMA ring.  While the first planes are on their way the CTA
+// reads the segment codes of its block (its planes, rows and segments with one
+// of each on either side) and derives a flag per segment: the pure phase + 1
+// when the 3 x 3 x 3 segments around it hold that phase alone, else 0, in which
+// case the segment goes on the interface list.  Then each warp with bulk
+// segments marches in z: the plane below and the plane itself stay in
+// registers, the plane above and the two rows beside come from the ring, the x
+// neighbours by shuffle.
+//
+// What bounds it: DRAM (mu in and out) and instruction issue.  Measured on a
+// GB300, with flags, list places and ghost images in the march / here: 66 / 66 us
+// at 256^3 with 3 phases and 2 solutes, 374 / 330 us at 512^3 and 64 / 21 us at
+// 192^3 (all interface) with 8 phases and 1 solute.  The same march on plain
+// loads one plane ahead in registers, without the ring: 75, 331 and 17 us.
 template <int NP, int NM, int TY>
 struct StreamShape {
-  static constexpr int VEC = 4;                   // cells per thread (float4)
+  static constexpr int VEC = 4;                   // cells per lane (float4)
   static constexpr int TX = 32 * VEC;             // cells per warp row
   static constexpr int WCS = TX / 32;             // 32-cell segments per warp row
   static constexpr int H = 4;                     // 16-byte halo of the TMA box
   static constexpr int SX = TX + 2 * H;
   static constexpr int SY = TY + 2;
-  static constexpr int NCW = TY;                  // consumer warps, one per row
-  static constexpr int NT = 32 * NCW;
+  static constexpr int NT = 32 * TY;              // consumer threads
   static constexpr int NTHREADS = NT + 32;
   static constexpr int FSTRIDE = SY * SX;         // elements per field in a stage
   static constexpr int STAGE_BYTES = NM * FSTRIDE * 4;
   static constexpr int STAGE_STRIDE = (STAGE_BYTES + 127) / 128 * 128;
   static constexpr int NST_RAW = (44 * 1024) / STAGE_STRIDE;   // 4 CTAs per SM
   static constexpr int NST = NST_RAW < 4 ? 4 : (NST_RAW > 12 ? 12 : NST_RAW);
-  static constexpr int NFL = SY * WCS;            // row flags per entry (one per producer lane)
-  static constexpr int NWF = TY * WCS;            // combined flags per entry
   static constexpr int CSEG = WCS + 2;
-  static constexpr int CODE_ENTRIES = (kMaxZChunk + 2) * SY * CSEG;
-  static constexpr int OFF_FLAG = NST * STAGE_STRIDE;
-  static constexpr int OFF_CODE = OFF_FLAG + (NST * NWF + 15) / 16 * 16;
-  static constexpr int NCOEF = NM * NM + NM;     // Kb_l and eb_l of one phase
-  static constexpr int OFF_COEF = OFF_CODE + (CODE_ENTRIES + 15) / 16 * 16;
+  static constexpr int MAXE = kMaxZChunk + 2;     // ring entries at most
+  static constexpr int NCOEF = NM * NM + NM;      // Kb_l and eb_l of one phase
+  static constexpr int OFF_CODE = NST * STAGE_STRIDE;
+  static constexpr int OFF_ROW = OFF_CODE + (MAXE * SY * CSEG + 15) / 16 * 16;
+  static constexpr int OFF_FLAG = OFF_ROW + (MAXE * SY * WCS + 15) / 16 * 16;
+  static constexpr int OFF_COEF = OFF_FLAG + (kMaxZChunk * TY * WCS + 15) / 16 * 16;
   static constexpr int OFF_BAR = OFF_COEF + (NP * NCOEF * 4 + 15) / 16 * 16;
   static constexpr int OFF_ABORT = OFF_BAR + 2 * NST * 8;
   static constexpr int SMEM_BYTES = OFF_ABORT + 16 + 128;
   static constexpr int MIN_BLOCKS = 4;
-  static_assert(NFL <= 32, "the producer warp holds one row flag per lane");
 };
 
 // Four cells' worth of one field.
-__device__ __forceinline__ float4 lds4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ void stg4(float* p, float a, float b, float c, float d) {
   *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
 }
+__device__ __forceinline__ float4 lds4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
 template <int NP, int NM, int TY>
 __global__ void __launch_bounds__(StreamShape<NP, NM, TY>::NTHREADS, StreamShape<NP, NM, TY>::MIN_BLOCKS)
@@ -65,60 +74,45 @@ __global__ void __launch_bounds__(StreamShape<NP, NM, TY>::NTHREADS, StreamShape
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
-  uint8_t* rowflag = smem + Sh::OFF_FLAG;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + Sh::OFF_BAR);
-  uint64_t* empty = full + NST;
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + Sh::OFF_ABORT);
-  auto stage = [&](int s) { return reinterpret_cast<float*>(smem + s * Sh::STAGE_STRIDE); };
-
-  const int tid = threadIdx.x, lane = tid & 31;
+  uint8_t* const s_code = smem + Sh::OFF_CODE;
+  uint8_t* const s_row = smem + Sh::OFF_ROW;
+  uint8_t* const s_flag = smem + Sh::OFF_FLAG;
+  float* const s_coef = reinterpret_cast<float*>(smem + Sh::OFF_COEF);
+  uint64_t* const full = reinterpret_cast<uint64_t*>(smem + Sh::OFF_BAR);
+  uint64_t* const empty = full + NST;
+  volatile int* const abort_flag = reinterpret_cast<volatile int*>(smem + Sh::OFF_ABORT);
+  auto stage = [&](int i) { return reinterpret_cast<float*>(smem + i * Sh::STAGE_STRIDE); };
+  const int tid = threadIdx.x, lane = tid & 31, ty = tid >> 5;
   const int tiles_x = (g.nx + Sh::TX - 1) / Sh::TX;
   const int x0 = (blockIdx.x % tiles_x) * Sh::TX;
   const int y0 = (blockIdx.x / tiles_x) * TY;
   const int zb = blockIdx.y * g.zchunk;
-  const int ze = min(g.nz, zb + g.zchunk);
-  const int nplanes = ze - zb + 2;   // ring entries j <-> plane zb - 1 + j
-  const int nk = ze - zb;
-  if (nplanes > kMaxZChunk + 2) {   // the host clamps z-chunks; never touch smem beyond its size
+  const int nk = min(g.nz, zb + g.zchunk) - zb;   // planes of this CTA
+  const int nplanes = nk + 2;                     // ring entries j <-> plane zb - 1 + j
+  if (nk > kMaxZChunk) {   // the host clamps z-chunks; never touch smem beyond its size
     if (tid == 0) atomicOr(g.status, kStatusLaunch);
     return;
   }
-  const int seg0 = x0 >> 5;
-
-  if (tid == 0) {
-    for (int s = 0; s < NST; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], Sh::NCW);
-    }
+  // the first ring entries
+  const int npre = nplanes < NST ? nplanes : NST;
+  auto load = [&](int j) {   // by one thread
+    const int i = j % NST;
+    mbar_expect_tx(&full[i], Sh::STAGE_BYTES);
+    tma_load_4d(stage(i), &tm, &full[i], x0 + g.xoff - Sh::H, y0, zb - 1 + j + g.zoff, 0);
+  };
+  if (tid == Sh::NT) {
+    for (int i = 0; i < NST; ++i) mbar_init(&full[i], 1);
     *abort_flag = 0;
     mbar_fence_init();
-  }
-  // bulk coefficients of every phase (indexed by the flag below)
-  float* scoef = reinterpret_cast<float*>(smem + Sh::OFF_COEF);
-  if (tid < NP * Sh::NCOEF) {
-    const int a = tid / Sh::NCOEF, r = tid % Sh::NCOEF;
-    scoef[tid] = r < NM * NM ? g.Kb[a][r] : g.eb[a][r - NM * NM];
-  }
-  __syncthreads();
-
-  // The producer starts the first ring entries (their flags are published by
-  // a plain arrive later); every thread loads the segment codes the CTA needs
-  // (input state, with halo).
-  const int npre = nplanes < NST ? nplanes : NST;
-  if (tid == Sh::NT) {
     prefetch_tensormap(&tm);
-    for (int j = 0; j < npre; ++j) {
-      mbar_expect_tx_only(&full[j], Sh::STAGE_BYTES);
-      tma_load_4d(stage(j), &tm, &full[j], x0 + g.xoff - Sh::H, y0, zb - 1 + j + g.zoff, 0);
-    }
+    for (int j = 0; j < npre; ++j) load(j);
   }
+  const int seg0 = x0 >> 5;
+  // codes: thread (row, segment), boundary-mapped once, for planes zb - 1 + j
   {
-    // thread (pair, group): segment k of row ay (boundary-mapped once), for
-    // the entries j = group, group + GROUPS, ... of this CTA's planes
     constexpr int PAIRS = Sh::SY * Sh::CSEG;
     constexpr int GROUPS = Sh::NTHREADS / PAIRS;
     static_assert(GROUPS >= 1, "the code preload needs one thread per (row, segment)");
-    uint8_t* scode = smem + Sh::OFF_CODE;
     if (tid < GROUPS * PAIRS) {
       const int pr = tid % PAIRS, j0 = tid / PAIRS;
       const int k = pr % Sh::CSEG, ay = pr / Sh::CSEG;
@@ -126,7 +120,7 @@ __global__ void __launch_bounds__(StreamShape<NP, NM, TY>::NTHREADS, StreamShape
           (long long)bc_map(y0 - 1 + ay, g.ny, g.bc[1]) * g.segs + bc_map(seg0 - 1 + k, g.segs, g.bc[0]);
       const long long pstride = (long long)g.ny * g.segs;
 #pragma unroll 4
-      for (int j = j0; j < nplanes; j += GROUPS) {
+      for (int j = j0; j < nk + 2; j += GROUPS) {
         const int z = zb - 1 + j;
         int zz;   // as load_code: ghost code planes at internal cuts
         if (z >= 0 && z < g.nz)
@@ -135,95 +129,122 @@ __global__ void __launch_bounds__(StreamShape<NP, NM, TY>::NTHREADS, StreamShape
           zz = z < 0 ? 0 : g.nz + 1;
         else
           zz = bc_map(z, g.nz, g.bc[2]) + g.zoff;
-        scode[(j * Sh::SY + ay) * Sh::CSEG + k] = __ldg(g.codes_in + zz * pstride + rowoff);
+        s_code[j * PAIRS + pr] = __ldg(g.codes_in + zz * pstride + rowoff);
       }
     }
+    // bulk coefficients of every phase (indexed by the flag)
+    for (int e = tid; e < NP * Sh::NCOEF; e += Sh::NTHREADS) {
+      const int a = e / Sh::NCOEF, r = e % Sh::NCOEF;
+      s_coef[e] = r < NM * NM ? g.Kb[a][r] : g.eb[a][r - NM * NM];
+    }
+  }
+  __syncthreads();
+  // rows: three adjacent segments of one pure phase.  A segment cut by the end
+  // of a ragged row is never bulk (it is listed), so that bulk groups are always
+  // 4 whole cells.
+  for (int e = tid; e < (nk + 2) * Sh::SY * Sh::WCS; e += Sh::NTHREADS) {
+    const int wc = e % Sh::WCS, ja = e / Sh::WCS;
+    s_row[e] = (seg0 + wc + 1) * 32 <= g.nx ? (uint8_t)combine_codes(s_code + ja * Sh::CSEG + wc) : (uint8_t)0;
+  }
+  __syncthreads();
+  const int reuse = g.reuse_prev ? kCodeReuse : 0;
+  for (int e0 = 0; e0 < nk * TY * Sh::WCS; e0 += Sh::NTHREADS) {
+    const int e = e0 + tid, wc = e % Sh::WCS, row = e / Sh::WCS % TY, k = e / (Sh::WCS * TY);
+    const int y = y0 + row, seg = seg0 + wc;
+    const bool inside = e < nk * TY * Sh::WCS && y < g.ny && seg < g.segs;
+    int f = 0;
+    if (inside) {
+      const uint8_t* r = s_row + (k * Sh::SY + row) * Sh::WCS + wc;
+      f = r[0];
+#pragma unroll
+      for (int q = 1; q < 9; ++q) f = r[((q / 3) * Sh::SY + q % 3) * Sh::WCS] == f ? f : 0;
+    }
+    if (e < nk * TY * Sh::WCS) {
+      // bit kCodeReuse of the flag: the output buffer holds phi already (the
+      // state before the input held the phase there too)
+      const int reused = f != 0 ? s_code[((k + 1) * Sh::SY + row + 1) * Sh::CSEG + wc + 1] & reuse : 0;
+      s_flag[e] = (uint8_t)(f | reused);
+    }
+    const long long ci = ((long long)(zb + k + g.zoff) * g.ny + y) * g.segs + seg;
+    if (f != 0) g.codes_out[ci] = (uint8_t)(f | kCodeReuse);   // input and output pure phase l
+    const bool want = inside && f == 0;
+    const unsigned int i = block_append<Sh::NTHREADS>(&g.iface[0], want);
+    if (want && i < g.iface_cap)
+      g.iface[2 + i] = ((unsigned int)(zb + k) << (g.seg_bits + g.y_bits)) | ((unsigned int)y << g.seg_bits) |
+                       (unsigned int)seg;
+  }
+  __syncthreads();
+  // a row without bulk segments has nothing to stream; the others share the ring
+  uint32_t any = 0u;
+  if (tid < Sh::NT) {
+    for (int k = lane; k < nk; k += 32) any |= *reinterpret_cast<const uint32_t*>(s_flag + (k * TY + ty) * Sh::WCS);
+    any = __reduce_or_sync(0xffffffffu, any);
+  }
+  const int streaming = __syncthreads_count(lane == 0 && any != 0u);   // warps
+  if (tid == 0) {
+    for (int i = 0; i < NST; ++i) mbar_init(&empty[i], streaming);
+    mbar_fence_init();
   }
   __syncthreads();   // the last CTA-wide barrier: roles split below
 
   if (tid >= Sh::NT) {
-    // ---------------- producer warp: TMA loads + bulk flags of every entry
-    const int f_ay = lane / Sh::WCS, f_wc = lane % Sh::WCS;
-    // a segment cut by the end of a ragged row is never bulk: it goes to the
-    // interface list, so that bulk groups are always 4 whole cells
-    const bool fl = lane < Sh::NFL && (seg0 + f_wc + 1) * 32 <= g.nx;
-    const uint8_t* scode = smem + Sh::OFF_CODE;
-    int issued = npre, arrived = 0;
+    // ---------------- producer
+    if (lane != 0) return;
+    int issued = npre;
     bool ok = true;
-    int rf2 = 0, rf1 = 0, rf0 = 0;   // row flags of entries j-2, j-1, j
-    for (int j = 0; j < nplanes; ++j) {
-      const int s = j % NST;
-      if (j >= NST) {
-        ok = ok && mbar_wait_bounded(&empty[s], ((j / NST) - 1) & 1);
-        ok = ok && *abort_flag == 0;
-        if (__any_sync(0xffffffffu, !ok)) break;
-        if (lane == 0) {
-          mbar_expect_tx_only(&full[s], Sh::STAGE_BYTES);
-          tma_load_4d(stage(s), &tm, &full[s], x0 + g.xoff - Sh::H, y0, zb - 1 + j + g.zoff, 0);
-        }
-        issued = j + 1;
-      }
-      rf2 = rf1;
-      rf1 = rf0;
-      rf0 = fl ? combine_codes(scode + (j * Sh::SY + f_ay) * Sh::CSEG + f_wc) : 0;
-      // flag of segment wc of row ty at the centre entry j-1: the pure phase
-      // + 1 when the 3 x 3 x 3 segments around it all hold that phase
-      const int pc = (rf2 == rf1 && rf1 == rf0) ? rf1 : 0;
-      const int up = __shfl_down_sync(0xffffffffu, pc, Sh::WCS);
-      const int up2 = __shfl_down_sync(0xffffffffu, pc, 2 * Sh::WCS);
-      if (lane < Sh::NWF && j >= 1)
-        rowflag[((j - 1) % NST) * Sh::NWF + lane] = (uint8_t)((pc == up && up == up2) ? pc : 0);
-      __syncwarp();
-      if (lane == 0) {
-        __threadfence_block();
-        mbar_arrive(&full[s]);   // publishes the flags; the data lands by complete_tx
-      }
-      arrived = j + 1;
+    for (int j = npre; j < nplanes && streaming > 0; ++j) {
+      ok = mbar_wait_bounded(&empty[j % NST], ((j / NST) - 1) & 1) && *abort_flag == 0;
+      if (!ok) break;
+      load(j);
+      issued = j + 1;
     }
-    if (!ok && lane == 0) {
+    if (!ok) {
       atomicOr(g.status, kStatusTimeout);
       *abort_flag = 1;
-      for (int j = arrived; j < issued; ++j) mbar_arrive(&full[j % NST]);
-      for (int s = 0; s < NST; ++s) {
-        if (issued <= s) continue;
-        const int j = s + ((issued - 1 - s) / NST) * NST;
-        mbar_wait_bounded(&full[s], (j / NST) & 1);
-      }
     }
+    // nobody may be left to wait for the copies in flight (no streaming warp, or
+    // an abort): see them land before this warp leaves
+    if (!ok || streaming == 0)
+      for (int i = 0; i < NST; ++i) {
+        if (issued <= i) continue;
+        const int j = i + ((issued - 1 - i) / NST) * NST;
+        mbar_wait_bounded(&full[i], (j / NST) & 1);
+      }
     return;
   }
+  if (any == 0u) return;
 
-  // -------------------- consumer warps: 4 cells per thread, one plane at a time
-  const int ty = tid >> 5;
-  const int wc = lane >> 3;              // segment of this thread within the row
-  const int seg = seg0 + wc;
-  const int xs = x0 + 4 * lane;          // first of this thread's cells
-  const int y = y0 + ty;
-  const bool have = y < g.ny && xs < g.nx;
-  // a bulk flag implies 4 whole cells (x ghost images of the first / last
-  // cell of the row are added as single stores)
-  const long long oxl = xs == 0 ? (g.bc[0] == 3 ? g.nx : -1) : 0;                // image of cell q = 0
-  const long long oxr = xs + 3 == g.nx - 1 ? (g.bc[0] == 3 ? -g.nx : 1) : 0;     // image of cell q = 3
-  const bool leader = (lane & 7) == 0 && y < g.ny && seg < g.segs;
-  const long long plane = (long long)g.nyp * g.pitch;
-  float* const out0 = g.out + (long long)(zb + g.zoff) * plane + (long long)(y + 1) * g.pitch + xs + g.xoff;
-  const long long oy0 = y == 0 ? (long long)(g.bc[1] == 3 ? g.ny : -1) * g.pitch : 0;
-  const long long oy1 = y == g.ny - 1 ? (long long)(g.bc[1] == 3 ? -g.ny : 1) * g.pitch : 0;
-  const long long cplane = (long long)g.ny * g.segs;
-  // z image offsets of the first / last plane of the grid (internal cuts get
-  // their ghost planes from the exchange)
-  const long long oz_first = g.bc[2] == kBcHalo ? 0 : (g.bc[2] == 3 ? g.nz : -1) * plane;
-  const long long oz_last = g.bc[2] == kBcHalo ? 0 : (g.bc[2] == 3 ? -g.nz : 1) * plane;
-  uint8_t* const code0 = g.codes_out + ((long long)(zb + g.zoff) * g.ny + y) * g.segs + seg;
-  // input code of this thread's segment at plane k: entry k + 1, row ty + 1,
-  // segment wc + 1 of the shared copy
-  const uint8_t* const scentre = smem + Sh::OFF_CODE + (Sh::SY + ty + 1) * Sh::CSEG + wc + 1;
-  const int reuse = g.reuse_prev ? kCodeReuse : 0;
-  const int sidx = (ty + 1) * Sh::SX + Sh::H + 4 * lane;
+  // -------------------- consumer warps: 4 cells per lane, one plane at a time
+  const int xs = x0 + 4 * lane, y = y0 + ty;
+  const bool last = xs + 3 == g.nx - 1;
+  const long long plane = (long long)g.nyp * g.pitch, fs = g.fstride;
+  const int pitch = g.pitch;
+  float* o = g.out + (long long)(zb + g.zoff) * plane + (long long)(y + 1) * pitch + xs + g.xoff;
+  const bool first = xs == 0;
+  const long long oxl = g.bc[0] == 3 ? g.nx : -1, oxr = 3 + (g.bc[0] == 3 ? -g.nx : 1);   // images of their cells
+  const bool yend = y == 0 || y == g.ny - 1;
+  const bool zcut = g.bc[2] == kBcHalo;                 // internal cuts get their ghost planes from the exchange
+  const int sidx = (ty + 1) * Sh::SX + Sh::H + 4 * lane;   // this lane's cells in a stage
+  float4 d[NM], c[NM];
   bool ok = mbar_wait_bounded(&full[0], 0) && mbar_wait_bounded(&full[1], 0);
-  int s0 = 0, s1 = 1, s2 = 2 % NST;
+  if (__all_sync(0xffffffffu, ok)) {
+#pragma unroll
+    for (int i = 0; i < NM; ++i) {
+      d[i] = lds4(stage(0) + i * Sh::FSTRIDE + sidx);
+      c[i] = lds4(stage(1) + i * Sh::FSTRIDE + sidx);
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&empty[0]);
+  }
+  int s1 = 1, s2 = 2 % NST;
   uint32_t par2 = (2 / NST) & 1;
-  for (int k = 0; k < nk; ++k) {
+  int lk = 0;              // phase + 1 whose coefficients are loaded
+  float kb[NM * NM], eb[NM];
+#pragma unroll
+  for (int q = 0; q < NM * NM; ++q) kb[q] = 0.0f;
+#pragma unroll
+  for (int q = 0; q < NM; ++q) eb[q] = 0.0f;
+  for (int k = 0; k < nk; ++k, o += plane) {
     ok = ok && mbar_wait_bounded(&full[s2], par2) && *abort_flag == 0;
     if (!__all_sync(0xffffffffu, ok)) {   // the warp leaves together (shuffles below)
       if (lane == 0) {
@@ -233,131 +254,118 @@ __global__ void __launch_bounds__(StreamShape<NP, NM, TY>::NTHREADS, StreamShape
       return;
     }
     const int z = zb + k;
-    const int flag = rowflag[s1 * Sh::NWF + ty * Sh::WCS + wc];
-    // stencil sums of every lane (warp-uniform: the x neighbours come by
-    // shuffle; lanes outside the grid read zero-filled box cells)
-    float L[NM][4], mc[NM][4];
-    {
-      const float* c0 = stage(s0) + sidx;
-      const float* c1 = stage(s1) + sidx;
-      const float* c2 = stage(s2) + sidx;
+    float4 u[NM], n[NM], s[NM];
+    float xm[NM], xp[NM];
 #pragma unroll
-      for (int i = 0; i < NM; ++i) {
-        const int fo = i * Sh::FSTRIDE;
-        const float4 c = lds4(c1 + fo);
-        // x neighbours of the group: from the adjacent lanes, the box halo at the ends
-        float xm = __shfl_up_sync(0xffffffffu, c.w, 1), xp = __shfl_down_sync(0xffffffffu, c.x, 1);
-        if (lane == 0) xm = c1[fo - 1];
-        if (lane == 31) xp = c1[fo + 4];
-        const float4 n = lds4(c1 + fo - Sh::SX), sN = lds4(c1 + fo + Sh::SX);
-        const float4 d = lds4(c0 + fo), u = lds4(c2 + fo);
-        const float cv[4] = {c.x, c.y, c.z, c.w};
-        const float lv[4] = {xm, c.x, c.y, c.z}, rv[4] = {c.y, c.z, c.w, xp};
-        const float nv[4] = {n.x, n.y, n.z, n.w}, sv[4] = {sN.x, sN.y, sN.z, sN.w};
-        const float dv[4] = {d.x, d.y, d.z, d.w}, uv[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          mc[i][q] = cv[q];
-          float sum = (lv[q] + rv[q]) + (nv[q] + sv[q]);
-          sum += dv[q] + uv[q];
-          L[i][q] = sum - 6.0f * cv[q];
-        }
-      }
+    for (int i = 0; i < NM; ++i) {
+      const float* const q = stage(s1) + i * Sh::FSTRIDE + sidx;
+      u[i] = lds4(stage(s2) + i * Sh::FSTRIDE + sidx);
+      n[i] = lds4(q - Sh::SX);
+      s[i] = lds4(q + Sh::SX);
+      xm[i] = __shfl_up_sync(0xffffffffu, c[i].w, 1);
+      xp[i] = __shfl_down_sync(0xffffffffu, c[i].x, 1);
+      if (lane == 0) xm[i] = q[-1];
+      if (lane == 31) xp[i] = q[4];
     }
-    if (flag != 0 && have) {
-      const int l = flag - 1;
-      const float* cf = scoef + l * Sh::NCOEF;
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&empty[s1]);   // entry k + 1 is read: the rest of it is in registers
+    const int fl = s_flag[(k * TY + ty) * Sh::WCS + (lane >> 3)];
+    float L[NM][4];
+#pragma unroll
+    for (int i = 0; i < NM; ++i) {
+      L[i][0] = (xm[i] + c[i].y) + (n[i].x + s[i].x) + (d[i].x + u[i].x) - 6.0f * c[i].x;
+      L[i][1] = (c[i].x + c[i].z) + (n[i].y + s[i].y) + (d[i].y + u[i].y) - 6.0f * c[i].y;
+      L[i][2] = (c[i].y + c[i].w) + (n[i].z + s[i].z) + (d[i].z + u[i].z) - 6.0f * c[i].z;
+      L[i][3] = (c[i].z + xp[i]) + (n[i].w + s[i].w) + (d[i].w + u[i].w) - 6.0f * c[i].w;
+    }
+    if (fl != 0) {
+      const int l1 = fl & kCodePhase;
+      if (l1 != lk) {
+        lk = l1;
+        const float* cf = s_coef + (l1 - 1) * Sh::NCOEF;
+#pragma unroll
+        for (int q = 0; q < NM * NM; ++q) kb[q] = cf[q];
+#pragma unroll
+        for (int q = 0; q < NM; ++q) eb[q] = cf[NM * NM + q];
+      }
       float mn[NM][4];
 #pragma unroll
       for (int i = 0; i < NM; ++i) {
-        const float eb = cf[NM * NM + i];
-        float kb[NM];
-#pragma unroll
-        for (int j = 0; j < NM; ++j) kb[j] = cf[i * NM + j];
+        const float cv[4] = {c[i].x, c[i].y, c[i].z, c[i].w};
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          float dd = mc[i][q] - eb;
+          float t = cv[q] - eb[i];
 #pragma unroll
-          for (int j = 0; j < NM; ++j) dd += kb[j] * L[j][q];
-          mn[i][q] = dd;
+          for (int j = 0; j < NM; ++j) t += kb[i * NM + j] * L[j][q];
+          mn[i][q] = t;
         }
       }
-      // a bulk flag implies that the input held phase l here; the output
-      // buffer (the state before it) also did when the input's reuse bit is set
-      const bool write_phi = (scentre[k * Sh::SY * Sh::CSEG] & reuse) == 0;
-      float* p = out0 + k * plane;
-      const long long fs = g.fstride;
-      // the cell row
+      const bool write_phi = (fl & kCodeReuse) == 0;
+      // the cells and the x ghost images of the row's first and last
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        float* const r = o + (NP + i) * fs;
+        stg4(r, mn[i][0], mn[i][1], mn[i][2], mn[i][3]);
+        if (first) r[oxl] = mn[i][0];
+        if (last) r[oxr] = mn[i][3];
+      }
       if (write_phi) {
-#pragma unroll
+#pragma unroll 1
         for (int a = 0; a < NP; ++a) {
-          const float v = a == l ? 1.0f : 0.0f;
-          stg4(p + a * fs, v, v, v, v);
+          const float v = a == l1 - 1 ? 1.0f : 0.0f;
+          float* const r = o + a * fs;
+          stg4(r, v, v, v, v);
+          if (first) r[oxl] = v;
+          if (last) r[oxr] = v;
         }
       }
+      if (yend || (!zcut && (z == 0 || z == g.nz - 1))) {
+        // ghost images of the whole row (with those) on y and z boundaries: a
+        // loop over (iz, iy), not unrolled
+#pragma unroll 1
+        for (int v = 1; v < 9; ++v) {
+          const int iz = v / 3, iy = v % 3;
+          long long off = 0;
+          if (iy == 1) {
+            if (y != 0) continue;
+            off += (long long)(g.bc[1] == 3 ? g.ny : -1) * pitch;
+          } else if (iy == 2) {
+            if (y != g.ny - 1) continue;
+            off += (long long)(g.bc[1] == 3 ? -g.ny : 1) * pitch;
+          }
+          if (iz == 1) {
+            if (zcut || z != 0) continue;
+            off += (g.bc[2] == 3 ? g.nz : -1) * plane;
+          } else if (iz == 2) {
+            if (zcut || z != g.nz - 1) continue;
+            off += (g.bc[2] == 3 ? -g.nz : 1) * plane;
+          }
+          float* const q = o + off;
 #pragma unroll
-      for (int i = 0; i < NM; ++i) stg4(p + (NP + i) * fs, mn[i][0], mn[i][1], mn[i][2], mn[i][3]);
-      // x ghost images of the row's first / last cell (lanes 0 and 31 of the
-      // tiles at the x ends)
-      if (oxl | oxr) {
-#pragma unroll
-        for (int a = 0; a < NP + NM; ++a) {
-          if (a < NP && !write_phi) continue;
-          const float v0 = a < NP ? (a == l ? 1.0f : 0.0f) : mn[a < NP ? 0 : a - NP][0];
-          const float v3 = a < NP ? (a == l ? 1.0f : 0.0f) : mn[a < NP ? 0 : a - NP][3];
-          if (oxl) p[oxl + a * fs] = v0;
-          if (oxr) p[3 + oxr + a * fs] = v3;
-        }
-      }
-      // rows at a y or z boundary (rare): their y / z images, with x images
-      const long long oz0 = z == 0 ? oz_first : 0, oz1 = z == g.nz - 1 ? oz_last : 0;
-      if ((oy0 | oy1 | oz0 | oz1) != 0) {
-        // (the loops are unrolled so that every array index is a constant
-        // and nothing lives in local memory)
-        const long long oy[3] = {0, oy0, oy1}, oz[3] = {0, oz0, oz1};
-#pragma unroll
-        for (int iz = 0; iz < 3; ++iz)
-#pragma unroll
-          for (int iy = 0; iy < 3; ++iy) {
-            if ((iy | iz) == 0 || (iy && !oy[iy]) || (iz && !oz[iz])) continue;
-            float* q = p + oy[iy] + oz[iz];
-#pragma unroll
-            for (int a = 0; a < NP + NM; ++a) {
-              if (a < NP && !write_phi) continue;
-              float c4[4];
-              if (a < NP) {
-                const float v = a == l ? 1.0f : 0.0f;
-                c4[0] = c4[1] = c4[2] = c4[3] = v;
-              } else {
-#pragma unroll
-                for (int u = 0; u < 4; ++u) c4[u] = mn[a - NP][u];
-              }
-              stg4(q + a * fs, c4[0], c4[1], c4[2], c4[3]);
-              if (oxl) q[oxl + a * fs] = c4[0];
-              if (oxr) q[3 + oxr + a * fs] = c4[3];
+          for (int i = 0; i < NM; ++i) {
+            float* const r = q + (NP + i) * fs;
+            stg4(r, mn[i][0], mn[i][1], mn[i][2], mn[i][3]);
+            if (first) r[oxl] = mn[i][0];
+            if (last) r[oxr] = mn[i][3];
+          }
+          if (write_phi) {
+#pragma unroll 1
+            for (int a = 0; a < NP; ++a) {
+              const float f = a == l1 - 1 ? 1.0f : 0.0f;
+              float* const r = q + a * fs;
+              stg4(r, f, f, f, f);
+              if (first) r[oxl] = f;
+              if (last) r[oxr] = f;
             }
           }
+        }
       }
     }
-    // segment codes of bulk segments (input and output pure phase l: reuse
-    // bit set); the others go to the interface list
-    if (leader && flag != 0) code0[k * cplane] = (uint8_t)(flag | kCodeReuse);
-    const unsigned int need = __ballot_sync(0xffffffffu, leader && flag == 0);
-    if (need) {
-      const int first = __ffs(need) - 1;
-      unsigned int base = 0;
-      if (lane == first) base = atomicAdd(&g.iface[0], (unsigned int)__popc(need));
-      base = __shfl_sync(0xffffffffu, base, first);
-      if ((need >> lane) & 1u) {
-        const unsigned int i = base + __popc(need & ((1u << lane) - 1u));
-        if (i < g.iface_cap)
-          g.iface[2 + i] = ((unsigned int)z << (g.seg_bits + g.y_bits)) | ((unsigned int)y << g.seg_bits) |
-                           (unsigned int)seg;
-      }
+#pragma unroll
+    for (int i = 0; i < NM; ++i) {
+      d[i] = c[i];
+      c[i] = u[i];
     }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&empty[s0]);   // this warp is done with entry k
-    s0 = s1;
     s1 = s2;
     if (++s2 == NST) {
       s2 = 0;
