@@ -182,10 +182,10 @@ inline bool uniform_gamma(const HostModel& m) {
 }
 
 // The interface rows of the split step by k_gp_rows (many phases, one boundary energy).
-template <int NP, int NM, bool ANISO>
+template <int NP, int NM, bool ANISO, bool GG>
 cudaError_t launch_rows(const StepArgs<float, NP, NM>& g, const void* in, int sms, cudaStream_t st) {
-  using Sh = RowsShape<NP, NM>;
-  auto k = k_gp_rows<NP, NM, ANISO>;
+  using Sh = RowsShape<NP, NM, ANISO, GG>;
+  auto k = k_gp_rows<NP, NM, ANISO, GG>;
   static int per_sm = 0;   // resident CTAs per SM
   if (per_sm == 0) {
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, Sh::THREADS, 0);
@@ -294,9 +294,12 @@ cudaError_t launch_split(const CUtensorMap* tm, const CUtensorMap* tmi, const vo
   const int v = plain ? 1 : 0;
   ks<<<dim3(lg.tiles, lg.zchunks), Ss::NTHREADS, Ss::SMEM_BYTES, st>>>(*tm, g);
   if constexpr (two)
-    if (uniform_gamma(m))
-      return g.n_apairs ? launch_rows<NP, NM, true>(g, in, lg.iface_blocks, st)
-                        : launch_rows<NP, NM, false>(g, in, lg.iface_blocks, st);
+    if (uniform_gamma(m)) {
+      if (g.n_apairs) return m.gg ? launch_rows<NP, NM, true, true>(g, in, lg.iface_blocks, st)
+                                  : launch_rows<NP, NM, true, false>(g, in, lg.iface_blocks, st);
+      return m.gg ? launch_rows<NP, NM, false, true>(g, in, lg.iface_blocks, st)
+                  : launch_rows<NP, NM, false, false>(g, in, lg.iface_blocks, st);
+    }
   ki<<<lg.iface_blocks * iface_per_sm[v], Si::THREADS, Si::SMEM_BYTES, st>>>(*tmi, g);
   if constexpr (two) kf<<<lg.iface_blocks * full_per_sm[v], Si::THREADS, Si::SMEM_BYTES, st>>>(*tmi, g);
   return cudaGetLastError();

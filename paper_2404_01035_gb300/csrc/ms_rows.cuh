@@ -10,28 +10,74 @@
 //   Gc_a = sum_b g_ab . grad phi_b = 2 gamma (phi_a T - grad phi_a . S1),
 //          T = sum_b |grad phi_b|^2,
 // and likewise the obstacle and well derivatives and the driving force, so a
-// cell costs O(N) instead of O(N^2); an anisotropic pair adds the difference
-// of its g to 2 gamma q.  Without the triple term gamma_abc the multi-obstacle
-// potential puts every phase on every boundary, so a listed row of an 8-phase
-// grid usually holds all 8 phases and the pair form pays for all 28 pairs (and
-// spills: 255 registers).  Measured on a GB300, interface rows of one step: 8
-// grains filling 192^3 (isotropic) 5846 us by pairs, 351 us here; 7 rotated
-// grains in 512^3 698 us by pairs, 115 us here.  What bounds it: instruction
-// issue (about 700 instructions a row without anisotropy) and the latency of
-// its loads at 16 warps per SM.  Models with unequal gamma or the triple term
-// keep the pair form (k_gp_iface).
+// cell costs O(N) instead of O(N^2).  With the face values and differences of
+// the discretisation written out in the cell's value c and the neighbours' n,
+// the two faces of an axis and its part of the centre term need the sums N2 =
+// sum n^2, X = sum n c, Y = sum n_- n_+ over the phases and C2 = sum c^2:
+//   dx^2 (div J - Gc)_a = gamma [ n_-a (C2 + X_- - V/2) + n_+a (C2 + X_+ + V/2)
+//                                 - c_a (N2_- + X_- + N2_+ + X_+ + T/2) ],
+//   V = X_+ - X_-, T = N2_- + N2_+ - 2 Y.
+// An anisotropic pair adds the difference of its g to 2 gamma q.
+//
+// Without the triple term gamma_abc the multi-obstacle potential puts every
+// phase on every boundary, so a listed row of an 8-phase grid usually holds all
+// 8 phases and the pair form pays for all 28 pairs (and spills: 255 registers).
+// What bounds it: instruction issue, the latency of its loads, and with
+// anisotropic pairs the instruction cache (so one code path for rotated and
+// unrotated pairs, and builds of their own for grain growth).  Measured on a
+// GB300, interface rows of one step, by pairs / with the sums taken face by
+// face / here: 8 grains filling 192^3 (isotropic) 5846 / 340 / 233 us; 7 rotated
+// grains in 128^3 with an eigenstrain - / 141 / 109 us; in 512^3 (few interface
+// rows) 698 / 186 / 142 us.  Models with unequal gamma or the triple term keep
+// the pair form (k_gp_iface).
 #pragma once
 
 #include "ms_split.cuh"
 
 namespace msgb {
 
-template <int NP, int NM>
+template <int NP, int NM, bool ANISO, bool GG>
 struct RowsShape {
   static constexpr int WARPS = 4;
   static constexpr int THREADS = 32 * WARPS;
-  static constexpr int MIN_BLOCKS = 4;
+  static constexpr int MIN_BLOCKS = ANISO ? 4 : GG ? 8 : 6;   // 16 / 32 / 24 warps per SM
 };
+
+// Threshold of the simplex projection (phi = max(v - theta, 0)): sorted values,
+// running sums (project's rule).  Eight values go through Batcher's odd-even
+// merge network (19 exchanges of two instructions; insertion takes 28 of three).
+template <int NP>
+__device__ __forceinline__ float simplex_shift(const float* v) {
+  float u[NP];
+#pragma unroll
+  for (int a = 0; a < NP; ++a) u[a] = v[a];
+  auto order = [&](int i, int j) {   // u[i] >= u[j]
+    const float hi = fmaxf(u[i], u[j]), lo = fminf(u[i], u[j]);
+    u[i] = hi;
+    u[j] = lo;
+  };
+  if constexpr (NP == 8) {
+    order(0, 1), order(2, 3), order(4, 5), order(6, 7);
+    order(0, 2), order(1, 3), order(4, 6), order(5, 7);
+    order(1, 2), order(5, 6);
+    order(0, 4), order(1, 5), order(2, 6), order(3, 7);
+    order(2, 4), order(3, 5);
+    order(1, 2), order(3, 4), order(5, 6);
+  } else {
+#pragma unroll
+    for (int i = 1; i < NP; ++i)
+#pragma unroll
+      for (int j = i; j > 0; --j) order(j - 1, j);
+  }
+  float csum = u[0], theta = u[0] - 1.0f;
+#pragma unroll
+  for (int j = 1; j < NP; ++j) {
+    csum += u[j];
+    const float t = (csum - 1.0f) * float(1.0 / (j + 1));
+    theta = u[j] - t > 0.0f ? t : theta;
+  }
+  return theta;
+}
 
 // g = dA/dq of an anisotropic pair minus its isotropic part 2 gamma q, for the
 // two faces of an axis (or, in both halves, one cell) in paired FP32: the
@@ -39,13 +85,13 @@ struct RowsShape {
 // 1e-12 (pair_grad's rule; the isotropic part is then taken off as well).
 // ONLY >= 0: that component alone.
 template <int ONLY>
-__device__ __forceinline__ void aniso_excess(const F2* q, float gam2, float del, bool rotated, const float* R, F2* out) {
-  F2 r[3] = {q[0], q[1], q[2]};
-  if (rotated) {
+__device__ __forceinline__ void aniso_excess(const F2* q, float gam2, float del, const float* R, F2* out) {
+  // (unrotated pairs too: R is the identity then, and one code path keeps the
+  // kernel nearer the instruction cache's size)
+  F2 r[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-      r[i] = fma2(f2s(R[i * 3 + 2]), q[2], fma2(f2s(R[i * 3 + 1]), q[1], f2s(R[i * 3]) * q[0]));
-  }
+  for (int i = 0; i < 3; ++i)
+    r[i] = fma2(f2s(R[i * 3 + 2]), q[2], fma2(f2s(R[i * 3 + 1]), q[1], f2s(R[i * 3]) * q[0]));
   F2 r2[3], Q = q[0] * q[0];
   Q = fma2(q[2], q[2], fma2(q[1], q[1], Q));
 #pragma unroll
@@ -63,8 +109,7 @@ __device__ __forceinline__ void aniso_excess(const F2* q, float gam2, float del,
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
     if (ONLY >= 0 && j != ONLY) continue;
-    F2 v = g[j];
-    if (rotated) v = fma2(f2s(R[6 + j]), g[2], fma2(f2s(R[3 + j]), g[1], f2s(R[j]) * g[0]));
+    F2 v = fma2(f2s(R[6 + j]), g[2], fma2(f2s(R[3 + j]), g[1], f2s(R[j]) * g[0]));
     v = f2(tl ? 0.0f : f2lo(v), th ? 0.0f : f2hi(v));
     out[j] = fma2(f2s(-gam2), q[j], v);
   }
@@ -108,8 +153,8 @@ __device__ __forceinline__ F2 edge_diff(const Edge19& v) {
 // Excess flux of the pair through the two faces along D: adds its divergence
 // to (da, db).
 template <int D>
-__device__ __forceinline__ void pair_faces(const Edge19& va, const Edge19& vb, float gam2, float del, bool rotated,
-                                           const float* R, float inv_dx, float qdx, float& da, float& db) {
+__device__ __forceinline__ void pair_faces(const Edge19& va, const Edge19& vb, float gam2, float del, const float* R,
+                                           float inv_dx, float qdx, float& da, float& db) {
   constexpr int T = (D + 1) % 3, U = (D + 2) % 3;
   auto grads = [&](const Edge19& v, F2& pf, F2* gr) {
     const F2 l = f2(v.m[D], v.c), r = f2(v.c, v.p[D]);
@@ -123,7 +168,7 @@ __device__ __forceinline__ void pair_faces(const Edge19& va, const Edge19& vb, f
   grads(vb, pb, gb);
 #pragma unroll
   for (int i = 0; i < 3; ++i) q[i] = pa * gb[i] - pb * ga[i];
-  aniso_excess<D>(q, gam2, del, rotated, R, x);
+  aniso_excess<D>(q, gam2, del, R, x);
   const F2 ja = pb * x[D], jb = pa * x[D];   // J_a = -ja, J_b = jb
   da -= (f2hi(ja) - f2lo(ja)) * inv_dx;
   db += (f2hi(jb) - f2lo(jb)) * inv_dx;
@@ -133,10 +178,10 @@ __device__ __forceinline__ void pair_faces(const Edge19& va, const Edge19& vb, f
 // plain loads (a warp's loads are whole rows, and neighbouring list entries
 // share them through L1 and L2), which leaves shared memory and the registers
 // of a staging ring to more warps.
-template <int NP, int NM, bool ANISO>
-__global__ void __launch_bounds__(RowsShape<NP, NM>::THREADS, RowsShape<NP, NM>::MIN_BLOCKS)
+template <int NP, int NM, bool ANISO, bool GG>
+__global__ void __launch_bounds__(RowsShape<NP, NM, ANISO, GG>::THREADS, RowsShape<NP, NM, ANISO, GG>::MIN_BLOCKS)
     k_gp_rows(const __grid_constant__ StepArgs<float, NP, NM> g, const float* __restrict__ in) {
-  using Sh = RowsShape<NP, NM>;
+  using Sh = RowsShape<NP, NM, ANISO, GG>;
   __shared__ unsigned int s_count;
   __shared__ float s_dg[ANISO ? Sh::WARPS : 1][ANISO ? NP : 1][32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -161,7 +206,7 @@ __global__ void __launch_bounds__(RowsShape<NP, NM>::THREADS, RowsShape<NP, NM>:
     const bool active = x < g.nx;
     // lanes past the end of a ragged row repeat its last cell (in bounds)
     const float* s = in + (long long)(z + g.zoff) * plane + (long long)(y + 1) * g.pitch + min(x, g.nx - 1) + g.xoff;
-    float ph[NP], dg[NP], gc[NP][3];
+    float ph[NP], dg[NP];
     float e1 = 0.0f, p2s = 0.0f;
 #pragma unroll
     for (int a = 0; a < NP; ++a) {
@@ -178,29 +223,27 @@ __global__ void __launch_bounds__(RowsShape<NP, NM>::THREADS, RowsShape<NP, NM>:
       dv[k] = f2s(0.0f);
     }
     float Mc[NM * NM];
-    if (!g.gg) cell_mobility<NP, NM>(ph, g.DX, Mc);
-    // isotropic part, axis by axis: outward differences d = nb - c and sums
-    // t = nb + c = 2 phi_face on both faces; sum of the two outward fluxes
-    const float kf = 0.25f * gam2 * g.inv_dx * g.inv_dx;
+    if constexpr (!GG) cell_mobility<NP, NM>(ph, g.DX, Mc);
+    // isotropic part, axis by axis (see the file comment)
+    const float kf = 0.5f * gam2 * g.inv_dx * g.inv_dx;
 #pragma unroll
     for (int D = 0; D < 3; ++D) {
-      F2 nb[NP], S1 = f2s(0.0f), S2 = f2s(0.0f);
+      F2 nb[NP], N2 = f2s(0.0f);
+      float Xm = 0.0f, Xp = 0.0f, Y = 0.0f;
 #pragma unroll
       for (int a = 0; a < NP; ++a) {
         nb[a] = f2(s[a * fs - o[D]], s[a * fs + o[D]]);
-        const F2 d = nb[a] - f2s(ph[a]), t = nb[a] + f2s(ph[a]);
-        S1 = fma2(t, d, S1);
-        S2 = fma2(t, t, S2);
-        gc[a][D] = f2hi(nb[a]) - f2lo(nb[a]);
+        N2 = fma2(nb[a], nb[a], N2);
+        Xm += f2lo(nb[a]) * ph[a];
+        Xp += f2hi(nb[a]) * ph[a];
+        Y += f2lo(nb[a]) * f2hi(nb[a]);
       }
-      const F2 nS1 = f2s(-1.0f) * S1;
+      const float V = 0.5f * (Xp - Xm), T = 0.5f * (f2lo(N2) + f2hi(N2)) - Y;
+      const float wm = kf * ((p2s + Xm) - V), wp = kf * ((p2s + Xp) + V);
+      const float wc = -kf * (((f2lo(N2) + Xm) + (f2hi(N2) + Xp)) + T);
 #pragma unroll
-      for (int a = 0; a < NP; ++a) {
-        const F2 d = nb[a] - f2s(ph[a]), t = nb[a] + f2s(ph[a]);
-        const F2 J = fma2(t, nS1, d * S2);
-        dg[a] += kf * (f2lo(J) + f2hi(J));
-      }
-      if (!g.gg) {
+      for (int a = 0; a < NP; ++a) dg[a] += f2lo(nb[a]) * wm + (f2hi(nb[a]) * wp + ph[a] * wc);
+      if constexpr (!GG) {
         // mu fluxes through the two faces (mobility_pair's form)
         F2 e1n = nb[0], e2n = f2s(0.0f), run = nb[0], Mn[NM * NM];
 #pragma unroll
@@ -227,20 +270,6 @@ __global__ void __launch_bounds__(RowsShape<NP, NM>::THREADS, RowsShape<NP, NM>:
           }
       }
     }
-    {
-      float T = 0.0f, V[3] = {0.0f, 0.0f, 0.0f};
-#pragma unroll
-      for (int a = 0; a < NP; ++a)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          T += gc[a][d] * gc[a][d];
-          V[d] += ph[a] * gc[a][d];
-        }
-      const float kc = gam2 * g.half_inv_dx * g.half_inv_dx;
-#pragma unroll
-      for (int a = 0; a < NP; ++a)
-        dg[a] -= kc * (ph[a] * T - (gc[a][0] * V[0] + gc[a][1] * V[1] + gc[a][2] * V[2]));
-    }
     if constexpr (ANISO) {
       // anisotropic pairs: a run-time loop (indices of phases are data, so the
       // sums live in shared memory, one column per lane)
@@ -263,11 +292,10 @@ __global__ void __launch_bounds__(RowsShape<NP, NM>::THREADS, RowsShape<NP, NM>:
         const bool ha = load19(s + a * fs, o, va);
         if (!__any_sync(0xffffffffu, ha)) continue;
         float da = 0.0f, db = 0.0f;
-        const bool rot = g.rotated[p] != 0;
         const float del = g.delta[p];
-        pair_faces<0>(va, vb, gam2, del, rot, g.rot[p], g.inv_dx, g.quarter_inv_dx, da, db);
-        pair_faces<1>(va, vb, gam2, del, rot, g.rot[p], g.inv_dx, g.quarter_inv_dx, da, db);
-        pair_faces<2>(va, vb, gam2, del, rot, g.rot[p], g.inv_dx, g.quarter_inv_dx, da, db);
+        pair_faces<0>(va, vb, gam2, del, g.rot[p], g.inv_dx, g.quarter_inv_dx, da, db);
+        pair_faces<1>(va, vb, gam2, del, g.rot[p], g.inv_dx, g.quarter_inv_dx, da, db);
+        pair_faces<2>(va, vb, gam2, del, g.rot[p], g.inv_dx, g.quarter_inv_dx, da, db);
         float Ga = 0.0f, Gb = 0.0f;
         {
           float ca[3], cb[3];
@@ -278,7 +306,7 @@ __global__ void __launch_bounds__(RowsShape<NP, NM>::THREADS, RowsShape<NP, NM>:
             cb[d] = (vb.p[d] - vb.m[d]) * g.half_inv_dx;
             q[d] = f2s(va.c * cb[d] - vb.c * ca[d]);
           }
-          aniso_excess<-1>(q, gam2, del, rot, g.rot[p], xs);
+          aniso_excess<-1>(q, gam2, del, g.rot[p], xs);
 #pragma unroll
           for (int d = 0; d < 3; ++d) {
             Ga += f2lo(xs[d]) * cb[d];
@@ -299,41 +327,57 @@ __global__ void __launch_bounds__(RowsShape<NP, NM>::THREADS, RowsShape<NP, NM>:
     {
       const float cw = g.cw[0][1];
       float psi[NP], A1 = 0.0f, A2 = 0.0f;
+      if constexpr (!GG) {
 #pragma unroll
-      for (int a = 0; a < NP; ++a) psi[a] = g.gg ? 0.0f : grand_potential<NP, NM, float>(g, a, mc, sT);
-      if (g.elw) {
-        const unsigned long long cells = (unsigned long long)g.nx * g.ny * g.nz;
-        const unsigned long long cell = ((unsigned long long)z * g.ny + y) * g.nx + min(x, g.nx - 1);
-        add_elastic<NP, NM, float, float>(g, cell, cells, psi);
-      }
+        for (int a = 0; a < NP; ++a) psi[a] = grand_potential<NP, NM, float>(g, a, mc, sT);
+        if (g.elw) {
+          const unsigned long long cells = (unsigned long long)g.nx * g.ny * g.nz;
+          const unsigned long long cell = ((unsigned long long)z * g.ny + y) * g.nx + min(x, g.nx - 1);
+          add_elastic<NP, NM, float, float>(g, cell, cells, psi);
+        }
 #pragma unroll
-      for (int a = 0; a < NP; ++a) {
-        A1 += psi[a] * ph[a];
-        A2 += psi[a] * (ph[a] * ph[a]);
+        for (int a = 0; a < NP; ++a) {
+          A1 += psi[a] * ph[a];
+          A2 += psi[a] * (ph[a] * ph[a]);
+        }
       }
       float e2 = 0.0f, run = ph[0];
+      if constexpr (!GG) {
 #pragma unroll
-      for (int a = 1; a < NP; ++a) {
-        e2 += ph[a] * run;
-        run += ph[a];
+        for (int a = 1; a < NP; ++a) {
+          e2 += ph[a] * run;
+          run += ph[a];
+        }
       }
       float v[NP];
 #pragma unroll
       for (int a = 0; a < NP; ++a) {
         const float q2 = ph[a] * ph[a], others = e1 - ph[a];
         const float W = g.potential == 1 ? cw * others : cw * (ph[a] * (p2s - q2));
-        const float rest = e2 - ph[a] * others;
-        float P = psi[a] * (6.0f * ph[a] - 6.0f * q2 + 2.0f * rest);
-        P += 2.0f * (others * (A1 - psi[a] * ph[a]) - (A2 - psi[a] * q2));
+        float P = 0.0f;
+        if constexpr (!GG) {
+          const float rest = e2 - ph[a] * others;
+          P = psi[a] * (6.0f * ph[a] - 6.0f * q2 + 2.0f * rest);
+          P += 2.0f * (others * (A1 - psi[a] * ph[a]) - (A2 - psi[a] * q2));
+        }
         const float rate = g.mob * ((g.eps * dg[a] - W * g.inv_eps - P) * g.inv_eps);
         v[a] = ph[a] + g.dt * rate;
         if (g.noise_amp != 0.0f && ph[a] > 0.0f && ph[a] < 1.0f)
           v[a] += g.dt * g.noise_amp *
                   noise_variate<float>(g.noise_seed, g.step, lab_cell<3>(g, min(x, g.nx - 1), y, z) * NP + a);
       }
-      project<NP>(g.potential, v, pn);
+      if (g.potential == 1) {
+        const float theta = simplex_shift<NP>(v);
+#pragma unroll
+        for (int a = 0; a < NP; ++a) {
+          const float d = v[a] - theta;
+          pn[a] = d > 0.0f ? d : 0.0f;
+        }
+      } else {
+        project<NP>(g.potential, v, pn);
+      }
     }
-    if (g.gg) {   // grain growth: mu held
+    if constexpr (GG) {   // grain growth: mu held
 #pragma unroll
       for (int k = 0; k < NM; ++k) mn[k] = mc[k];
     } else {
