@@ -115,6 +115,12 @@ bool encode_step_maps(const StepKernel& k, CUtensorMap* tm, CUtensorMap* tmi, vo
 void set_layout(HostModel& m);   // padded layout of one state buffer
 std::vector<const StepKernel*> step_variants(int dim, int np, int nm, int dtype);
 cudaError_t fill_ghosts(const HostModel& m, void* buf, int nf, cudaStream_t st);
+// Dense device-resident fields to a padded state with its ghosts and segment
+// codes (codes may be NULL), and back (phi or mu may be NULL); ms_fields.cu.
+bool field_kernels_fit(const HostModel& m);
+cudaError_t load_fields(const HostModel& m, void* padded, const void* phi, const void* mu, uint8_t* codes,
+                        cudaStream_t st);
+cudaError_t unload_fields(const HostModel& m, const void* padded, void* phi, void* mu, cudaStream_t st);
 cudaError_t copy_fields(const HostModel& m, void* padded, int f0, int nf, const void* dense, void* dense_out,
                         int on_device, cudaStream_t st);
 }  // namespace msgb

@@ -810,11 +810,19 @@ ms_status ms_update_params(ms_ctx* c, const ms_params* p) {
 
 ms_status ms_set_fields(ms_ctx* c, const void* phi, const void* mu, int on_device) {
   if (!c || !phi || !mu) return fail(c, MS_ERR_ARG, "ctx, phi and mu are required");
-  MS_CUDA(c, copy_fields(c->m, c->buf[c->cur], 0, c->m.N, phi, nullptr, on_device, c->stream));
-  MS_CUDA(c, copy_fields(c->m, c->buf[c->cur], c->m.N, c->m.NM, mu, nullptr, on_device, c->stream));
-  MS_CUDA(c, fill_ghosts(c->m, c->buf[c->cur], c->m.N + c->m.NM, c->stream));
-  ms_status rs = state_replaced(c);
-  if (rs != MS_OK) return rs;
+  if (on_device && field_kernels_fit(c->m)) {
+    // (the multi-step kernel keeps no codes: they wait for a reader)
+    c->codes_stale = multi_steps(c);
+    MS_CUDA(c, load_fields(c->m, c->buf[c->cur], phi, mu, c->codes_stale ? nullptr : c->codes[c->cur], c->stream));
+    // as refresh_codes: the other buffer's codes must not let a step keep phi there
+    if (!c->codes_stale) MS_CUDA(c, cudaMemsetAsync(c->codes[1 - c->cur], 0, code_bytes(c->m), c->stream));
+  } else {
+    MS_CUDA(c, copy_fields(c->m, c->buf[c->cur], 0, c->m.N, phi, nullptr, on_device, c->stream));
+    MS_CUDA(c, copy_fields(c->m, c->buf[c->cur], c->m.N, c->m.NM, mu, nullptr, on_device, c->stream));
+    MS_CUDA(c, fill_ghosts(c->m, c->buf[c->cur], c->m.N + c->m.NM, c->stream));
+    ms_status rs = state_replaced(c);
+    if (rs != MS_OK) return rs;
+  }
   c->step = 0;
   c->t = c->m.t0;
   ms_reset_extra(c);
@@ -823,8 +831,12 @@ ms_status ms_set_fields(ms_ctx* c, const void* phi, const void* mu, int on_devic
 
 ms_status ms_get_fields(ms_ctx* c, void* phi, void* mu, int on_device) {
   if (!c) return fail(nullptr, MS_ERR_ARG, "ctx is NULL");
-  if (phi) MS_CUDA(c, copy_fields(c->m, c->buf[c->cur], 0, c->m.N, nullptr, phi, on_device, c->stream));
-  if (mu) MS_CUDA(c, copy_fields(c->m, c->buf[c->cur], c->m.N, c->m.NM, nullptr, mu, on_device, c->stream));
+  if (on_device && field_kernels_fit(c->m)) {
+    MS_CUDA(c, unload_fields(c->m, c->buf[c->cur], phi, mu, c->stream));
+  } else {
+    if (phi) MS_CUDA(c, copy_fields(c->m, c->buf[c->cur], 0, c->m.N, nullptr, phi, on_device, c->stream));
+    if (mu) MS_CUDA(c, copy_fields(c->m, c->buf[c->cur], c->m.N, c->m.NM, nullptr, mu, on_device, c->stream));
+  }
   MS_CUDA(c, cudaStreamSynchronize(c->stream));
   return MS_OK;
 }
