@@ -156,7 +156,8 @@ inline size_t code_bytes(const HostModel& m) { return (size_t)segments(m) * m.ny
 // One compiled FP64 diagnostics instantiation.
 struct DiagKernel {
   int dim, np, nm, dtype;
-  cudaError_t (*launch)(const void* state, const HostModel& m, double t, double* partials,
+  // codes: the state's segment codes, or NULL where they do not describe it
+  cudaError_t (*launch)(const void* state, const uint8_t* codes, const HostModel& m, double t, double* partials,
                         int nblocks, double* out, int* status, cudaStream_t st);
 };
 

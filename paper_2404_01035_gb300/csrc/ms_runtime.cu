@@ -626,8 +626,8 @@ bool parse_fault_spec(const char* spec, int64_t* step, int* code) {
 }
 
 ms_status launch_diag_now(ms_ctx* c) {
-  cudaError_t e = c->diagk->launch(c->buf[c->cur], c->m, c->t, c->diag_partials, c->diag_blocks,
-                                   c->diag_out, c->status, c->stream);
+  cudaError_t e = c->diagk->launch(c->buf[c->cur], c->codes_stale ? nullptr : c->codes[c->cur], c->m, c->t,
+                                   c->diag_partials, c->diag_blocks, c->diag_out, c->status, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "diag launch");
   return MS_OK;
 }
