@@ -19,9 +19,12 @@
 //   3. k_el_spec: p_s(k) in place
 //   4. cuFFT C2R: p_s(x), which the step reads where it needs them.
 // What bounds it: memory passes.  7 grains with one dilatation, 128^3 FP32 on
-// a GB300, without the step: 230 us with one transform per component and
-// w_b stored per phase, see the figures at k_el_spec for this form.  cuFFT is
-// opened at run time, so the library loads (and everything else runs) without it.
+// a GB300, without the step: 235 us with one transform per component and
+// w_b stored per phase, 53 us here (k_el_eig 12.0, k_el_spec 11.2; 16 and 16
+// with 64-bit index arithmetic and the stiffness contracted over all 81
+// products per wavevector).
+// cuFFT is opened at run time, so the library loads (and everything else runs)
+// without it.
 #include <cuda_runtime.h>
 #include <cufft.h>
 #include <dlfcn.h>
@@ -76,7 +79,7 @@ struct ElConst {
   Real Pl[kElRank][3][3];          // B_ij C_ijkl
   Real Pr[kElRank][3][3];          // C_ijkl B_kl
   Real Q[kElRank][kElRank];        // B^s : C : B^s'
-  Real C[3][3][3][3];
+  Real D[3][3][6];                 // A_ik = C_ijkl k_j k_l over the products k_j k_l, j <= l
   Real kstep[3];                   // 2 pi / (n dx) per axis
   int rank, nx, ny, nz, nxh, pitch, nyp, xoff, zoff, segs;
   long long fstride, cells, ncplx;
@@ -86,10 +89,11 @@ struct ElConst {
 template <int DIM, int NP, class Real>
 __global__ void __launch_bounds__(256) k_el_eig(const __grid_constant__ ElConst<Real> q, const Real* __restrict__ st,
                                                 const uint8_t* __restrict__ codes, Real* __restrict__ E) {
-  const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  // (32-bit indices: elastic_grid_fits bounds the cells by 2^31)
+  const unsigned w = blockIdx.x * 8u + (threadIdx.x >> 5), row = w / (unsigned)q.segs;
   const int lane = threadIdx.x & 31;
-  if (w >= (long long)q.segs * q.ny * q.nz) return;
-  const int sg = (int)(w % q.segs), y = (int)((w / q.segs) % q.ny), z = (int)(w / ((long long)q.segs * q.ny));
+  const int sg = (int)(w - row * q.segs), z = (int)(row / (unsigned)q.ny), y = (int)(row - (unsigned)z * q.ny);
+  if (z >= q.nz) return;
   const int x = 32 * sg + lane;
   if (x >= q.nx) return;
   const long long idx = ((long long)z * q.ny + y) * q.nx + x;
@@ -126,9 +130,9 @@ __device__ __forceinline__ Real wavenumber(int i, int n, Real step) {
 // One thread per wavevector, all fields of it in place.
 template <int DIM, int RANK, class Real>
 __global__ void __launch_bounds__(256) k_el_spec(const __grid_constant__ ElConst<Real> q, Cplx<Real>* __restrict__ S) {
-  const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= q.ncplx) return;
-  const int mx = (int)(idx % q.nxh), my = (int)((idx / q.nxh) % q.ny), mz = (int)(idx / ((long long)q.nxh * q.ny));
+  const unsigned idx = blockIdx.x * 256u + threadIdx.x, row = idx / (unsigned)q.nxh;
+  if (idx >= (unsigned long long)q.ncplx) return;
+  const int mx = (int)(idx - row * q.nxh), mz = (int)(row / (unsigned)q.ny), my = (int)(row - (unsigned)mz * q.ny);
   Real k[3] = {wavenumber<Real>(mx, q.nx, q.kstep[0]), wavenumber<Real>(my, q.ny, q.kstep[1]),
                DIM == 3 ? wavenumber<Real>(mz, q.nz, q.kstep[2]) : Real(0)};
   Real k2 = Real(0);
@@ -140,17 +144,20 @@ __global__ void __launch_bounds__(256) k_el_spec(const __grid_constant__ ElConst
   // v^s = Pr^s k and y^s = G v^s, G = A^-1 (adjugate over the determinant), A_ik = C_ijkl k_j k_l
   Real yv[RANK][DIM];
   if (k2 != Real(0)) {
-    Real A[DIM][DIM];
+    Real A[DIM][DIM], kk[DIM * (DIM + 1) / 2];
+    int n = 0;
+#pragma unroll
+    for (int j = 0; j < DIM; ++j)
+#pragma unroll
+      for (int l = j; l < DIM; ++l) kk[n++] = k[j] * k[l];
 #pragma unroll
     for (int i = 0; i < DIM; ++i)
 #pragma unroll
-      for (int kk = 0; kk < DIM; ++kk) {
+      for (int j = 0; j < DIM; ++j) {
         Real a = Real(0);
 #pragma unroll
-        for (int j = 0; j < DIM; ++j)
-#pragma unroll
-          for (int l = 0; l < DIM; ++l) a += q.C[i][j][kk][l] * k[j] * k[l];
-        A[i][kk] = a;
+        for (int p = 0; p < DIM * (DIM + 1) / 2; ++p) a += q.D[i][j][p] * kk[p];
+        A[i][j] = a;
       }
     Real adj[DIM][DIM], det;
     if constexpr (DIM == 2) {
@@ -225,10 +232,13 @@ ElConst<Real> make_const(const HostModel& m) {
   for (int a = 0; a < m.N; ++a)
     for (int s = 0; s < eb.rank; ++s) q.c[a][s] = (Real)eb.c[a][s];
   const int dim = m.dim;
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j)
-      for (int k = 0; k < 3; ++k)
-        for (int l = 0; l < 3; ++l) q.C[i][j][k][l] = (Real)m.elC[i][j][k][l];
+  for (int i = 0; i < dim; ++i)
+    for (int k = 0; k < dim; ++k) {
+      int n = 0;
+      for (int j = 0; j < dim; ++j)
+        for (int l = j; l < dim; ++l)
+          q.D[i][k][n++] = (Real)(j == l ? m.elC[i][j][k][j] : m.elC[i][j][k][l] + m.elC[i][l][k][j]);
+    }
   for (int s = 0; s < eb.rank; ++s) {
     for (int k = 0; k < dim; ++k)
       for (int l = 0; l < dim; ++l) {
