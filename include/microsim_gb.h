@@ -372,9 +372,9 @@ ms_status ms_batch_get_fields(ms_batch* b, int sim, void* phi, void* mu, int on_
 ms_status ms_batch_step(ms_batch* b, int64_t n);
 ms_status ms_batch_sync(ms_batch* b);
 int64_t ms_batch_cells(const ms_batch* b);   /* total cells over all simulations */
-/* Tile height of the batched work list: the persistent kernel is compiled for
- * 32 x 4, 32 x 8 (the default) and 32 x 16 tiles; a change rebuilds the work
- * list and the tensor maps (synchronous) and recaptures the graph at the next
+/* Strip height of the batched work list: the persistent kernel is compiled for
+ * strips of 128 x 4, 128 x 8 (the default) and 128 x 16 cells; a change rebuilds
+ * the work list (synchronous) and recaptures the graph at the next
  * ms_batch_step.  MS_ERR_ARG for another height. */
 ms_status ms_batch_set_tile(ms_batch* b, int tile_height);
 int ms_batch_tile(const ms_batch* b);        /* current tile height, 0 for NULL */

@@ -77,7 +77,7 @@ class Batch:
         return lib().ms_batch_cells(self.h)
 
     def set_tile(self, tile_height: int):
-        """Tile height of the work list (4, 8 or 16 rows of 32 cells)."""
+        """Strip height of the work list (4, 8 or 16 rows of 128 cells)."""
         self._c(lib().ms_batch_set_tile(self.h, int(tile_height)))
 
     def tile_height(self) -> int:

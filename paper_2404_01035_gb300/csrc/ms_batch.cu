@@ -2,18 +2,19 @@
 // and parameters advanced by ONE persistent, cooperative kernel launch
 // (captured once into a CUDA graph and replayed).
 //
-// Work list: every (simulation, 32 x TY tile) pair, as precomputed
-// descriptors.  Each CTA takes a contiguous range of it every step; a producer
-// warp reads the descriptors 32 at a time (one coalesced load, the next chunk
-// in flight) and TMA-loads the items' halo'ed tiles (each simulation has its
-// own tensor map, kept in global memory) into a shared-memory ring, while the
-// consumer warps compute the current one with the same cell update as the
-// single-simulation kernel.  A consumer warp takes the bulk update when the
-// three halo rows around its row, its 32 columns and the column on each side,
-// hold one pure phase in the staged data itself (the exact condition of the
-// bulk shortcut; no segment codes are kept).  A grid-wide barrier (atomic
-// counter, bounded spin on %globaltimer) separates time steps, because a step
-// reads the ghost cells its neighbours wrote in the previous step.
+// A step has two phases with a grid-wide barrier (atomic counter, bounded spin
+// on %globaltimer) after each.  In the first, a warp per strip of 128 x R cells
+// (work list of precomputed descriptors, a contiguous range per CTA) updates
+// the segments whose 3 x 3 block of segment codes is one pure phase, which
+// touches mu alone (PlaneStrip, as in the split 2-D step), and lists the others.
+// In the second, a warp per listed 32-cell segment of any simulation stages its
+// 3 x 34 cells and takes the full cell update.  The list spreads the interface
+// rows, which cost many times a bulk row, over all warps.  Reads go past L1:
+// the rows are other SMs' stores of the previous phase.
+//
+// What bounds it: the two barriers and the latency of each phase.  32 simulations
+// of 64^2 .. 512^2 (3.2 M cells) on a GB300: 19.6 us a step; 60 us with every tile
+// staged through a TMA ring, a cell per thread, and phi tested cell by cell.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -25,6 +26,7 @@
 #include "../../include/microsim_gb.h"
 #include "ms_launch.cuh"
 #include "ms_rt.h"
+#include "ms_strip.cuh"
 #include "ms_trace.h"
 
 namespace msgb {
@@ -36,197 +38,170 @@ ms_status build_model(ms_ctx* c, const ms_grid* g, int N, int K, const ms_params
 template <class Real, int NP, int NM>
 struct alignas(64) BatchSim {
   StepArgs<Real, NP, NM> g[2];   // [parity of the source buffer]
+  const Real* in[2];             // the source buffer
 };
 
-// One work item: simulation, tile origin, TMA x coordinate of its box.
+// One work item: simulation, strip (128 cells wide) and first row.
 struct alignas(16) BatchItem {
-  int sim, x0, y0, bx;
+  int sim, sx, y0, pad;
 };
 
-__device__ __forceinline__ bool grid_barrier(unsigned int* counter, unsigned int target) {
-  __threadfence();
-  fence_proxy_async_global();   // generic stores of this step -> TMA loads of the next
-  atomicAdd(counter, 1u);
-  const unsigned long long t0 = globaltimer();
-  while (atomicAdd(counter, 0u) < target) {
-    if (globaltimer() - t0 > kWaitLimitNs) return false;
-    __nanosleep(64);
-  }
-  __threadfence();
-  fence_proxy_async_global();
-  return true;
-}
+// A listed row segment: simulation, (y << seg_bits) | segment.
+struct alignas(8) BatchRow {
+  unsigned int sim, row;
+};
 
-template <int NP, int NM, class Real, int TX, int TY>
-__global__ void __launch_bounds__(TX* TY + 32, TY <= 8 ? 3 : 1)
-    k_batch(const BatchSim<Real, NP, NM>* __restrict__ sims, const CUtensorMap* __restrict__ maps,
-            const BatchItem* __restrict__ items, int nitems, int nsteps, int parity0,
-            unsigned int* barrier, int* status) {
-  using Sh = StepShape<2, NP, NM, Real, TX, TY>;
-  static_assert(TX == 32, "one warp per tile row");
-  constexpr int NST = 8;
-  extern __shared__ unsigned char smem_raw[];
-  unsigned char* smem =
-      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
-  int4* sitem = reinterpret_cast<int4*>(smem + NST * Sh::STAGE_STRIDE);
-  uint64_t* full = reinterpret_cast<uint64_t*>(sitem + NST);
-  uint64_t* empty = full + NST;
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + NST);
-  auto stage = [&](int s) { return reinterpret_cast<Real*>(smem + s * Sh::STAGE_STRIDE); };
-  const int tid = threadIdx.x, lane = tid & 31;
-  if (tid == 0) {
-    for (int s = 0; s < NST; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], Sh::NCW);
-    }
-    *abort_flag = 0;
-    mbar_fence_init();
-  }
-  __syncthreads();
-  // contiguous item range: consecutive tiles of one simulation share its constants
+// What a strip reads of a simulation's arguments, copied to shared memory (the
+// arguments themselves lie in global memory, where every store might alias them).
+template <int NP, int NM>
+struct StripArgs {
+  long long fstride;
+  const uint8_t* codes_in;
+  uint8_t* codes_out;
+  float* out;
+  const float* in;
+  int nx, ny, pitch, xoff, segs, reuse_prev, seg_bits;
+  int bc[3];
+  float Kb[NP][NM * NM], eb[NP][NM];
+};
+
+template <int R>
+struct BatchShape {
+  static constexpr int WARPS = 4;
+  static constexpr int THREADS = 32 * WARPS;
+  static constexpr int MIN_BLOCKS = R <= 8 ? 5 : 4;
+};
+
+// counters: [0] barrier arrivals, [1 + (step & 1)] rows listed by the step;
+// all zero at the launch.
+template <int NP, int NM, int R>
+__global__ void __launch_bounds__(BatchShape<R>::THREADS, BatchShape<R>::MIN_BLOCKS)
+    k_batch(const BatchSim<float, NP, NM>* __restrict__ sims, const BatchItem* __restrict__ items, int nitems,
+            BatchRow* rows, int nsteps, int parity0, unsigned int* counters, int* status) {
+  using Bs = BatchShape<R>;
+  using Strip = PlaneStrip<NP, NM, R, true>;
+  using Ms = MultiShape<NP, NM, float>;
+  __shared__ StripArgs<NP, NM> s_args[Bs::WARPS];
+  __shared__ uint8_t s_code[Bs::WARPS][Strip::CODES];
+  __shared__ float s_box[Bs::WARPS][Ms::BOX];
+  __shared__ int s_ok;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  StripArgs<NP, NM>& a = s_args[wid];
+  float* const box = s_box[wid];
   const int per = (nitems + (int)gridDim.x - 1) / (int)gridDim.x;
-  const int ibeg = min(nitems, (int)blockIdx.x * per);
-  const int my_items = min(nitems, ibeg + per) - ibeg;
-  long long seq = 0;      // ring position (continues across steps)
-  long long issued = 0;   // loads issued (producer lane 0)
+  const int ibeg = min(nitems, (int)blockIdx.x * per), iend = min(nitems, ibeg + per);
+  auto barrier = [&](unsigned int round) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      s_ok = multi_barrier(&counters[0], round * gridDim.x) ? 1 : 0;
+      if (!s_ok) atomicOr(status, kStatusTimeout);
+    }
+    __syncthreads();
+    return s_ok != 0;
+  };
   for (int step = 0; step < nsteps; ++step) {
     const int par = (parity0 + step) & 1;
-    if (tid >= Sh::NT) {
-      // ---------------- producer warp: descriptors 32 at a time, one TMA per item
-      auto fetch = [&](int k0) {
-        int4 d = make_int4(0, 0, 0, 0);
-        if (k0 + lane < my_items) {
-          const BatchItem it = items[ibeg + k0 + lane];
-          d = make_int4(it.sim, it.x0, it.y0, it.bx);
-        }
-        return d;
-      };
-      int4 cur = fetch(0), nxt = fetch(32);
-      bool ok = true;
-      for (int k = 0; k < my_items; ++k) {
-        if ((k & 31) == 0 && k > 0) {
-          cur = nxt;
-          nxt = fetch(k + 32);
-        }
-        const long long q = seq + k;
-        const int s = (int)(q % NST);
-        if (q >= NST) ok = ok && mbar_wait_bounded(&empty[s], (uint32_t)(((q / NST) - 1) & 1));
-        ok = ok && *abort_flag == 0;
-        if (__any_sync(0xffffffffu, !ok)) {
-          if (lane == 0) {
-            atomicOr(status, kStatusTimeout);
-            *abort_flag = 1;
-          }
-          break;
-        }
-        const int j = k & 31;
-        const int sim = __shfl_sync(0xffffffffu, cur.x, j);
-        const int x0 = __shfl_sync(0xffffffffu, cur.y, j);
-        const int y0 = __shfl_sync(0xffffffffu, cur.z, j);
-        const int bx = __shfl_sync(0xffffffffu, cur.w, j);
+    unsigned int* const listed = &counters[1 + (step & 1)];
+    // ---- bulk
+    int cur = -1;
+    for (int k = ibeg + wid; k < iend; k += Bs::WARPS) {
+      const BatchItem it = items[k];
+      if (it.sim != cur) {
+        cur = it.sim;
+        __syncwarp();
         if (lane == 0) {
-          sitem[s] = make_int4(sim, x0, y0, 0);
-          __threadfence_block();
-          mbar_expect_tx(&full[s], Sh::STAGE_BYTES);   // arrive (release) + expected bytes
-          tma_load_4d(stage(s), &maps[2 * sim + par], &full[s], bx, y0, 0, 0);
-          issued = q + 1;
-        }
-      }
-    } else {
-      // ---------------- consumer warps: one tile row each
-      const int tx = tid % TX, ty = tid / TX;
-      for (int k = 0; k < my_items; ++k) {
-        const long long q = seq + k;
-        const int s = (int)(q % NST);
-        const bool ok = mbar_wait_bounded(&full[s], (uint32_t)((q / NST) & 1)) && *abort_flag == 0;
-        if (!__all_sync(0xffffffffu, ok)) {   // the warp leaves together (votes below)
-          if (lane == 0) {
-            atomicOr(status, kStatusTimeout);
-            *abort_flag = 1;
-          }
-          break;
-        }
-        const int4 it = sitem[s];
-        const StepArgs<Real, NP, NM>& g = sims[it.x].g[par];
-        const int x0 = it.y, y0 = it.z;
-        const int x = x0 + tx, y = y0 + ty;
-        const bool active = x < g.nx && y < g.ny;
-        // bulk test on the staged phi: rows ty..ty+2 (halo'ed) of this lane's
-        // column, and of the columns beside the row for lanes 0 and 31
-        const Real* st = stage(s);
-        auto column_code = [&](int col) {
-          int c = -1;
+          const StepArgs<float, NP, NM>& g = sims[cur].g[par];
+          a.fstride = g.fstride;
+          a.codes_in = g.codes_in;
+          a.codes_out = g.codes_out;
+          a.out = g.out;
+          a.in = sims[cur].in[par];
+          a.nx = g.nx;
+          a.ny = g.ny;
+          a.pitch = g.pitch;
+          a.xoff = g.xoff;
+          a.segs = g.segs;
+          a.reuse_prev = g.reuse_prev;
+          a.seg_bits = g.seg_bits;
 #pragma unroll
-          for (int r = 0; r < 3; ++r) {
-            uint32_t nz = 0, one = 0;
+          for (int d = 0; d < 3; ++d) a.bc[d] = g.bc[d];
 #pragma unroll
-            for (int a = 0; a < NP; ++a) {
-              const Real v = st[a * Sh::SY * Sh::SX + (ty + r) * Sh::SX + col];
-              nz |= (v != Real(0) ? 1u : 0u) << a;
-              one |= (v == Real(1) ? 1u : 0u) << a;
-            }
-            const int pc = (__popc(nz) == 1 && nz == one) ? __ffs(nz) : 0;
-            c = (c == -1 || c == pc) ? pc : 0;
-          }
-          return c;
-        };
-        int mine = column_code(Sh::H + tx);
-        if (tx == 0 || tx == TX - 1) {
-          const int side = column_code(tx == 0 ? Sh::H - 1 : Sh::H + TX);
-          mine = mine == side ? mine : 0;
-        }
-        const int ref = __shfl_sync(0xffffffffu, mine, 0);
-        const int flag = __all_sync(0xffffffffu, mine == ref) ? ref : 0;
-        if (active) {
-          SmemAcc<2, NP, NM, Real, TX, TY> acc;
-          acc.st[0] = acc.st[1] = acc.st[2] = st;
-          acc.g = &g;
-          acc.sidx = (ty + 1) * Sh::SX + tx + Sh::H;
-          Real pn[NP], mn[NM];
-          if (flag != 0) {
-            bulk_cell<2, NP, NM, Real>(acc, g, flag - 1, pn, mn);
-          } else {
-            DiffPrm<Real, StepArgs<Real, NP, NM>::P> dp;
-            dp.mob = g.mob;
+          for (int p = 0; p < NP; ++p) {
 #pragma unroll
-            for (int p = 0; p < StepArgs<Real, NP, NM>::P; ++p) dp.delta[p] = g.delta[p];
-            gp_cell<2, NP, NM, Real, Real>(acc, g, dp, y + g.zorg, lab_cell<2>(g, x, y, 0), pn, mn);
+            for (int q = 0; q < NM * NM; ++q) a.Kb[p][q] = g.Kb[p][q];
+#pragma unroll
+            for (int q = 0; q < NM; ++q) a.eb[p][q] = g.eb[p][q];
           }
-          store_cell<2>(g, x, y, 0, pn, mn);
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[s]);
       }
+      Strip st;
+      st.flags(a, it.sx, it.y0, lane, s_code[wid]);
+      st.list(listed, lane, [&](unsigned int at, int r) {
+        __stcg(reinterpret_cast<uint2*>(rows) + at,
+               make_uint2((unsigned int)it.sim,
+                          ((unsigned int)(it.y0 + r) << a.seg_bits) | (unsigned int)(4 * it.sx + (lane >> 3))));
+      });
+      st.update(a, a.in, it.sx, it.y0, lane, s_code[wid]);
+      __syncwarp();
     }
-    seq += my_items;
-    __syncthreads();
-    // grid-wide barrier between steps
-    if (tid == 0) {
-      if (*abort_flag || !grid_barrier(barrier, (unsigned int)(step + 1) * gridDim.x)) {
-        atomicOr(status, kStatusTimeout);
-        *abort_flag = 1;
+    if (!barrier(2u * step + 1u)) break;
+    // ---- interface rows
+    if (blockIdx.x == 0 && threadIdx.x == 0) counters[1 + ((step + 1) & 1)] = 0u;   // last read a phase ago
+    const unsigned int count = __ldcg(listed);
+    for (unsigned int k = wid * gridDim.x + blockIdx.x; k < count; k += gridDim.x * Bs::WARPS) {
+      const uint2 e = __ldcg(reinterpret_cast<const uint2*>(rows) + k);
+      const StepArgs<float, NP, NM>& g = sims[e.x].g[par];
+      const float* in = sims[e.x].in[par];
+      const int nx = g.nx, sg = (int)(e.y & ((1u << g.seg_bits) - 1u)), y = (int)(e.y >> g.seg_bits);
+      const int x = 32 * sg + lane;
+      const bool active = x < nx;
+      // columns 32 sg - 1 .. 32 sg + 32 (never past the ghost column nx)
+      const float* row = in + (long long)y * g.pitch + 32 * sg - 1 + g.xoff;
+      const int c0 = min(lane, nx - 32 * sg + 1), c1 = min(lane + 32, nx - 32 * sg + 1);
+#pragma unroll
+      for (int f = 0; f < Ms::NF; ++f)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const float* p = row + f * g.fstride + (long long)q * g.pitch;
+          box[(f * 3 + q) * Ms::BX + lane] = __ldcg(p + c0);
+          if (lane < 2) box[(f * 3 + q) * Ms::BX + 32 + lane] = __ldcg(p + c1);
+        }
+      __syncwarp();
+      int code = 0;
+      if (active) {
+        MultiAcc<NP, NM, float> acc;
+        acc.s = box + Ms::BX + lane + 1;
+        acc.g = &g;
+        acc.tz0 = g.tz0;
+        DiffPrm<float, StepArgs<float, NP, NM>::P> dp;
+        dp.mob = g.mob;
+#pragma unroll
+        for (int p = 0; p < StepArgs<float, NP, NM>::P; ++p) dp.delta[p] = g.delta[p];
+        float pn[NP], mn[NM];
+        gp_cell<2, NP, NM, float, float>(acc, g, dp, y + g.zorg, 0ull, pn, mn);
+        uint32_t nzm = 0, one = 0;
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+          nzm |= (pn[q] != 0.0f ? 1u : 0u) << q;
+          one |= (pn[q] == 1.0f ? 1u : 0u) << q;
+        }
+        code = (__popc(nzm) == 1 && nzm == one) ? __ffs(nzm) : 0;
+        store_cell<2>(g, x, y, 0, pn, mn);
       }
+      const int ref = __shfl_sync(0xffffffffu, code, 0);
+      const bool same = __all_sync(0xffffffffu, !active || code == ref);
+      if (lane == 0) {
+        const long long ci = (long long)y * g.segs + sg;
+        int c = same ? ref : 0;
+        if (c != 0 && (__ldcg(g.codes_in + ci) & kCodePhase) == c) c |= kCodeReuse;   // pure before and after
+        g.codes_out[ci] = (uint8_t)c;
+      }
+      __syncwarp();
     }
-    __syncthreads();
-    if (*abort_flag) break;
-  }
-  // drain: every issued load was consumed in a complete run; after an abort,
-  // wait (bounded) for the loads still in flight before the CTA exits
-  if (*abort_flag && tid == Sh::NT) {
-    for (int s = 0; s < NST; ++s) {
-      if (issued <= s) continue;
-      const long long q = s + ((issued - 1 - s) / NST) * NST;   // last load issued into stage s
-      mbar_wait_bounded(&full[s], (uint32_t)((q / NST) & 1));
-    }
+    if (step + 1 < nsteps && !barrier(2u * step + 2u)) break;
   }
 }
-
-template <int NP, int NM, class Real, int TX, int TY>
-struct BatchShape {
-  using Sh = StepShape<2, NP, NM, Real, TX, TY>;
-  static constexpr int NST = 8;
-  static constexpr int SMEM = NST * Sh::STAGE_STRIDE + NST * 16 + 2 * NST * 8 + 16 + 128;
-};
 
 }  // namespace msgb
 
@@ -237,19 +212,21 @@ struct ms_batch {
   std::vector<HostModel> models;
   std::vector<size_t> off;              // byte offset of each simulation's two state buffers
   std::vector<size_t> sbytes;           // state bytes per simulation (one buffer)
-  void* state = nullptr;                // all state buffers
+  std::vector<size_t> coff;             // byte offset of its two segment-code arrays
+  size_t total = 0;                     // bytes of states and codes
+  void* state = nullptr;                // all state buffers, then all codes
   void* sims = nullptr;                 // BatchSim array (device)
-  CUtensorMap* maps = nullptr;          // [nsims][2] (device)
   BatchItem* items = nullptr;
   int nitems = 0;
-  unsigned int* barrier = nullptr;
+  BatchRow* rows = nullptr;             // interface rows of a step (room for every row segment)
+  unsigned int* barrier = nullptr;      // counters of the kernel (see k_batch)
   int* status = nullptr;
   int parity = 0;                       // buffer holding the current state
   int64_t steps_done = 0;
   cudaStream_t stream = nullptr;
   AllocHook hook;
-  int grid = 0, smem = 0;
-  int ty = 0;                           // tile height of the work list (kBTYs)
+  int grid = 0;
+  int ty = 0;                           // rows of a strip (kBTYs)
   cudaGraphExec_t graph = nullptr;
   int64_t graph_n = -1;
   std::string err;
@@ -257,22 +234,20 @@ struct ms_batch {
 
 namespace {
 
-// Tiles are 32 cells (one warp row) wide; their height is chosen at run time
-// among the compiled ones (ms_batch_set_tile / ms_batch_tune).
-constexpr int kBTX = 32, kBTY = 8;
+// Strips are 128 cells wide; their height is chosen at run time among the
+// compiled ones (ms_batch_set_tile / ms_batch_tune).
+constexpr int kBTY = 8;
 constexpr int kBTYs[] = {4, 8, 16};
 constexpr int kNBTY = 3;
 
-template <int TY>
-void* batch_kernel() {
-  return reinterpret_cast<void*>(k_batch<2, 1, float, kBTX, TY>);
-}
 void* batch_kernel_for(int ty) {
-  return ty == 4 ? batch_kernel<4>() : ty == 16 ? batch_kernel<16>() : batch_kernel<8>();
+  return ty == 4    ? reinterpret_cast<void*>(k_batch<2, 1, 4>)
+         : ty == 16 ? reinterpret_cast<void*>(k_batch<2, 1, 16>)
+                    : reinterpret_cast<void*>(k_batch<2, 1, 8>);
 }
-int batch_smem_for(int ty) {
-  return ty == 4 ? BatchShape<2, 1, float, kBTX, 4>::SMEM
-                 : ty == 16 ? BatchShape<2, 1, float, kBTX, 16>::SMEM : BatchShape<2, 1, float, kBTX, 8>::SMEM;
+
+uint8_t* codes_of(const ms_batch* b, int sim, int par) {
+  return static_cast<uint8_t*>(b->state) + b->coff[sim] + par * code_bytes(b->models[sim]);
 }
 
 ms_status bfail(ms_batch* b, ms_status s, const std::string& m) {
@@ -286,19 +261,18 @@ void batch_free(ms_batch* b) {
   if (b->graph) cudaGraphExecDestroy(b->graph);
   dev_free(b->hook, b->state);
   dev_free(b->hook, b->sims);
-  dev_free(b->hook, b->maps);
   dev_free(b->hook, b->items);
+  dev_free(b->hook, b->rows);
   dev_free(b->hook, b->barrier);
   delete b;
 }
 
 cudaError_t launch_batch(ms_batch* b, int64_t n) {
-  cudaError_t e = cudaMemsetAsync(b->barrier, 0, sizeof(unsigned int), b->stream);
+  cudaError_t e = cudaMemsetAsync(b->barrier, 0, 4 * sizeof(unsigned int), b->stream);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(b->grid);
-  cfg.blockDim = dim3(kBTX * b->ty + 32);
-  cfg.dynamicSmemBytes = b->smem;
+  cfg.blockDim = dim3(BatchShape<kBTY>::THREADS);
   cfg.stream = b->stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
@@ -306,32 +280,19 @@ cudaError_t launch_batch(ms_batch* b, int64_t n) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const BatchSim<float, 2, 1>* sims = (const BatchSim<float, 2, 1>*)b->sims;
-  const CUtensorMap* maps = (const CUtensorMap*)b->maps;
-  const BatchItem* items = (const BatchItem*)b->items;
-  if (b->ty == 4)
-    return cudaLaunchKernelEx(&cfg, k_batch<2, 1, float, kBTX, 4>, sims, maps, items, b->nitems, (int)n, b->parity,
-                              b->barrier, b->status);
-  if (b->ty == 16)
-    return cudaLaunchKernelEx(&cfg, k_batch<2, 1, float, kBTX, 16>, sims, maps, items, b->nitems, (int)n, b->parity,
-                              b->barrier, b->status);
-  return cudaLaunchKernelEx(&cfg, k_batch<2, 1, float, kBTX, 8>, sims, maps, items, b->nitems, (int)n, b->parity,
-                            b->barrier, b->status);
+  const BatchItem* items = b->items;
+  auto kern = b->ty == 4 ? k_batch<2, 1, 4> : b->ty == 16 ? k_batch<2, 1, 16> : k_batch<2, 1, 8>;
+  return cudaLaunchKernelEx(&cfg, kern, sims, items, b->nitems, b->rows, (int)n, b->parity, b->barrier, b->status);
 }
 
-// Work list, tensor maps and persistent grid for tile height ty (one of
-// kBTYs): items are (simulation, 32 x ty tile) pairs in simulation order,
-// the maps' boxes are the tiles with their halo.  Drops the captured graph.
+// Work list and persistent grid for strips of ty rows (one of kBTYs): items are
+// (simulation, strip) pairs in simulation order.  Drops the captured graph.
 cudaError_t batch_set_tiles(ms_batch* b, int ty) {
-  std::vector<CUtensorMap> hm(2 * b->nsims);
   std::vector<BatchItem> items;
   for (int i = 0; i < b->nsims; ++i) {
     const HostModel& m = b->models[i];
-    const size_t half = (b->sbytes[i] + 255) / 256 * 256;
-    char* base = static_cast<char*>(b->state) + b->off[i];
-    for (int par = 0; par < 2; ++par)
-      if (!encode_state_map(&hm[2 * i + par], base + par * half, m, 3, kBTX, ty)) return cudaErrorInvalidValue;
     for (int y0 = 0; y0 < m.ny; y0 += ty)
-      for (int x0 = 0; x0 < m.nx; x0 += kBTX) items.push_back(BatchItem{i, x0, y0, x0 + m.xoff - 16 / 4});
+      for (int sx = 0; 128 * sx < m.nx; ++sx) items.push_back(BatchItem{i, sx, y0, 0});
   }
   cudaError_t e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return e;
@@ -340,21 +301,14 @@ cudaError_t batch_set_tiles(ms_batch* b, int ty) {
   if (!b->items) return cudaErrorMemoryAllocation;
   b->nitems = (int)items.size();
   e = cudaMemcpyAsync(b->items, items.data(), sizeof(BatchItem) * items.size(), cudaMemcpyHostToDevice, b->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(b->maps, hm.data(), sizeof(CUtensorMap) * hm.size(), cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-  void* kern = batch_kernel_for(ty);
-  const int smem = batch_smem_for(ty);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   int per_sm = 0, dev = 0, sms = 0;
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBTX * ty + 32, smem);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel_for(ty), BatchShape<kBTY>::THREADS, 0);
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   b->ty = ty;
-  b->smem = smem;
   b->grid = std::max(1, per_sm) * sms;
   if (b->graph) {
     cudaGraphExecDestroy(b->graph);
@@ -408,20 +362,30 @@ ms_status ms_batch_create(int nsims, const ms_grid* grids, int n_phases, int n_c
   b->N = 2;
   b->NM = 1;
   b->dtype = MS_F32;
-  // one allocation for all states (2 buffers each)
-  size_t tot = 0;
+  // one allocation for all states (2 buffers each) and segment codes
+  size_t tot = 0, nrows = 0;
   for (int i = 0; i < nsims; ++i) {
     const HostModel& m = b->models[i];
+    if (!list_entry_fits(m)) {
+      batch_free(b);
+      return bfail(nullptr, MS_ERR_UNSUPPORTED, "grid too large for the batched work list");
+    }
     const size_t sb = (size_t)m.fstride * (m.N + m.NM) * 4;
     b->sbytes.push_back(sb);
     b->off.push_back(tot);
     tot += 2 * ((sb + 255) / 256 * 256);
+    nrows += (size_t)segments(m) * m.ny;
   }
+  for (int i = 0; i < nsims; ++i) {
+    b->coff.push_back(tot);
+    tot += (2 * code_bytes(b->models[i]) + 15) / 16 * 16;
+  }
+  b->total = tot;
   b->state = dev_alloc(b->hook, tot);
   b->sims = dev_alloc(b->hook, sizeof(BatchSim<float, 2, 1>) * nsims);
-  b->maps = static_cast<CUtensorMap*>(dev_alloc(b->hook, sizeof(CUtensorMap) * 2 * nsims));
+  b->rows = static_cast<BatchRow*>(dev_alloc(b->hook, sizeof(BatchRow) * nrows));
   b->barrier = static_cast<unsigned int*>(dev_alloc(b->hook, 256));
-  if (!b->state || !b->sims || !b->maps || !b->barrier) {
+  if (!b->state || !b->sims || !b->rows || !b->barrier) {
     batch_free(b);
     return bfail(nullptr, MS_ERR_OOM, "batch allocation failed");
   }
@@ -430,9 +394,7 @@ ms_status ms_batch_create(int nsims, const ms_grid* grids, int n_phases, int n_c
   if (e == cudaSuccess) e = cudaMemsetAsync(b->barrier, 0, 256, b->stream);
   // per-simulation constants
   std::vector<BatchSim<float, 2, 1>> hs(nsims);
-  const StepKernel* k = nullptr;
-  for (auto& sk : step_registry())
-    if (sk.dim == 2 && sk.np == 2 && sk.nm == 1 && sk.dtype == 0 && sk.tx == kBTX && sk.ty == kBTY) k = &sk;
+  const StepKernel* k = step_variants(2, 2, 1, 0).front();
   for (int i = 0; i < nsims && e == cudaSuccess; ++i) {
     const HostModel& m = b->models[i];
     const size_t half = (b->sbytes[i] + 255) / 256 * 256;
@@ -442,10 +404,14 @@ ms_status ms_batch_create(int nsims, const ms_grid* grids, int n_phases, int n_c
       k->fill(&g, m, 1, b->status);
       g.out = reinterpret_cast<float*>(base + (1 - par) * half);
       g.tz0 = (float)temp_offset(m, m.t0);
+      g.codes_in = codes_of(b, i, par);
+      g.codes_out = codes_of(b, i, 1 - par);
+      g.reuse_prev = 1;
+      hs[i].in[par] = reinterpret_cast<const float*>(base + par * half);
     }
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->sims, hs.data(), sizeof(hs[0]) * nsims, cudaMemcpyHostToDevice, b->stream);
-  // work list, tensor maps and persistent grid (every CTA resident at once)
+  // work list and persistent grid (every CTA resident at once)
   if (e == cudaSuccess) e = batch_set_tiles(b, kBTY);
   if (e != cudaSuccess) {
     std::string m = std::string("batch set-up: ") + cudaGetErrorString(e);
@@ -468,6 +434,7 @@ ms_status ms_batch_set_fields(ms_batch* b, int sim, const void* phi, const void*
   cudaError_t e = copy_fields(m, buf, 0, m.N, phi, nullptr, on_device, b->stream);
   if (e == cudaSuccess) e = copy_fields(m, buf, m.N, m.NM, mu, nullptr, on_device, b->stream);
   if (e == cudaSuccess) e = fill_ghosts(m, buf, m.N + m.NM, b->stream);
+  if (e == cudaSuccess) e = step_variants(2, 2, 1, 0).front()->codes(buf, m, codes_of(b, sim, b->parity), b->stream);
   if (e == cudaSuccess && !on_device) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bfail(b, MS_ERR_CUDA, std::string("batch set fields: ") + cudaGetErrorString(e));
   return MS_OK;
@@ -490,7 +457,7 @@ ms_status ms_batch_step(ms_batch* b, int64_t n) {
   TraceRange trace("ms_batch_step");
   if (!b || n < 0) return bfail(b, MS_ERR_ARG, "bad argument");
   if (n == 0) return MS_OK;
-  // the grid barrier counts (steps x CTAs) in 32 bits: at most 2^20 steps per launch
+  // the grid barrier counts (2 steps x CTAs) in 32 bits: at most 2^20 steps per launch
   if (n > ((int64_t)1 << 20)) return bfail(b, MS_ERR_BOUNDS, "at most 1048576 steps per ms_batch_step call");
   // the launch (barrier reset + cooperative kernel) is captured once per
   // (n, parity) and replayed
@@ -555,8 +522,7 @@ int ms_batch_tile(const ms_batch* b) { return b ? b->ty : 0; }
 ms_status ms_batch_tune(ms_batch* b, int steps_per_trial, double* best_ms_per_step) {
   TraceRange trace("ms_batch_tune");
   if (!b || steps_per_trial < 1) return bfail(b, MS_ERR_ARG, "bad argument");
-  size_t tot = 0;
-  for (int i = 0; i < b->nsims; ++i) tot = std::max(tot, b->off[i] + 2 * ((b->sbytes[i] + 255) / 256 * 256));
+  const size_t tot = b->total;
   void* save = dev_alloc(b->hook, tot);
   if (!save) return bfail(b, MS_ERR_OOM, "batch tuner: state copy allocation failed");
   const int parity0 = b->parity;
