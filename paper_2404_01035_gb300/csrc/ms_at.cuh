@@ -10,9 +10,9 @@
 // is linear in its right-hand side).  Two kernels: k_at_list lists the 32-cell
 // row segments whose 3 x 3 (x 3) block of segments is not one pure phase in
 // phi^n (elsewhere every phase gradient at every face of the segment's cells
-// is zero, so no face has a normal and the current vanishes); k_at_work stages
-// the block around each listed segment in shared memory (phi^n and mu^n from
-// the input, phi^{n+1} from the output) and corrects mu, one lane per cell.
+// is zero, so no face has a normal and the current vanishes); k_at_work
+// corrects mu on the listed segments (phi^n and mu^n from the input, phi^{n+1}
+// from the output), one lane per cell.
 #pragma once
 
 #include "ms_step.cuh"
@@ -37,47 +37,27 @@ __device__ __forceinline__ Real at_coefficient(int potential, Real eps, Real p) 
   return Real(0.78539816339744830962) * eps * p * (Real(1) - h) * inv_sqrt(p * (Real(1) - p));   // pi / 4
 }
 
-// Shape of the staged block of one row segment: fields [phi^n (NP), mu^n
-// (NM), phi^{n+1} (NP)] x planes (3 in 3-D, 1 in 2-D) x 3 rows x 34 cells
-// (x0 - 1 .. x0 + 32).
-template <int DIM, int NP, int NM, class Real>
-struct AtShape {
-  static constexpr int NF = 2 * NP + NM;
-  static constexpr int BX = 34;
-  static constexpr int NPL = DIM == 3 ? 3 : 1;
-  static constexpr int ROWS = NF * NPL * 3;
-  static constexpr int WARP_ELEMS = ROWS * BX;
-  static constexpr int WARP_BYTES = WARP_ELEMS * (int)sizeof(Real);
-  static constexpr int WARPS_RAW = (160 * 1024) / WARP_BYTES;
-  static constexpr int WARPS = WARPS_RAW < 1 ? 1 : (WARPS_RAW > 8 ? 8 : WARPS_RAW);
-  static constexpr int THREADS = 32 * WARPS;
-  static constexpr int SMEM_BYTES = WARPS * WARP_BYTES;
-};
-
-// Asynchronous copy of one element from global to shared memory (cp.async
-// through L1, bypassing registers), and the wait for this thread's copies.
-template <class Real>
-__device__ __forceinline__ void cp_async_elem(Real* dst, const Real* src) {
-  if constexpr (sizeof(Real) == 8)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
-// Reads of the staged block relative to the lane's cell: field f, offsets
-// dx, dy, dz in [-1, 1] (dz = 0 in 2-D).
+// Reads relative to a cell: phi^n and mu^n from the input state, phi^{n+1} from
+// the output (whose phi the correction does not write), offsets in [-1, 1].
 template <int DIM, int NP, int NM, class Real>
 struct AtBox {
-  using Sh = AtShape<DIM, NP, NM, Real>;
-  const Real* s;   // the warp's block
-  int lane;
-  __device__ __forceinline__ Real at(int f, int dx, int dy, int dz) const {
-    return s[((f * Sh::NPL + (DIM == 3 ? dz + 1 : 0)) * 3 + dy + 1) * Sh::BX + lane + 1 + dx];
+  const Real* in;    // the cell in field 0 of the input
+  const Real* out;   // and of the output
+  long long fs, plane;
+  int pitch;
+  __device__ __forceinline__ long long off(int f, int dx, int dy, int dz) const {
+    return f * fs + (DIM == 3 ? dz * plane : 0) + (long long)dy * pitch + dx;
   }
-  __device__ __forceinline__ Real phi(int a, int dx, int dy, int dz) const { return at(a, dx, dy, dz); }
-  __device__ __forceinline__ Real mu(int i, int dx, int dy, int dz) const { return at(NP + i, dx, dy, dz); }
-  __device__ __forceinline__ Real phin(int a, int dx, int dy, int dz) const { return at(NP + NM + a, dx, dy, dz); }
+  __device__ __forceinline__ Real phi(int a, int dx, int dy, int dz) const { return __ldg(in + off(a, dx, dy, dz)); }
+  __device__ __forceinline__ Real mu(int i, int dx, int dy, int dz) const { return __ldg(in + off(NP + i, dx, dy, dz)); }
+  __device__ __forceinline__ Real phin(int a, int dx, int dy, int dz) const { return __ldg(out + off(a, dx, dy, dz)); }
+};
+
+template <class Real>
+struct AtShape {
+  static constexpr int THREADS = 128;
+  static constexpr int WARPS = THREADS / 32;
+  static constexpr int MIN_BLOCKS = sizeof(Real) == 4 ? 4 : 2;
 };
 
 // dt times the normal component along axis d of j_at_i (the rates are taken
@@ -153,6 +133,84 @@ __device__ __forceinline__ void at_face(const StepArgs<Real, NP, NM>& g, const A
   }
 }
 
+// dt times (j_at on the upper face along axis D minus on the lower one), FP32:
+// at_face's arithmetic for both faces at once in paired registers.  gcr: the
+// cell's unscaled central differences, whose sum with a neighbour's is the
+// 4-point tangential average.  A face without a normal has a zero unit normal,
+// so its current vanishes without a test.  lanes: the warp's lanes that call.
+template <int DIM, int D, int NP, int NM>
+__device__ __forceinline__ void at_axis(const StepArgs<float, NP, NM>& g, const AtBox<DIM, NP, NM, float>& A,
+                                        const float (*gcr)[DIM], int k, uint32_t lanes, float* dJ) {
+  constexpr int L = NP - 1;   // the liquid
+  constexpr int X = D == 0, Y = D == 1, Z = D == 2;
+  F2 nL[DIM], cl[NM], mf[NM], J[NM], sf;
+  // unit normal of phase a on both faces; false where no lane has one
+  auto normal = [&](int a, F2 lr, F2* n) {
+    F2 gr[DIM], g2 = f2s(0.0f);
+#pragma unroll
+    for (int t = 0; t < DIM; ++t) {
+      if (t == D) {
+        gr[t] = lr * f2s(g.inv_dx);
+      } else {
+        const int tx = t == 0, ty = t == 1, tz = t == 2;
+        const F2 nb = f2(A.phi(a, tx - X, ty - Y, tz - Z), A.phi(a, tx + X, ty + Y, tz + Z)) -
+                      f2(A.phi(a, -tx - X, -ty - Y, -tz - Z), A.phi(a, X - tx, Y - ty, Z - tz));
+        gr[t] = (nb + f2s(gcr[a][t])) * f2s(g.quarter_inv_dx);
+      }
+      g2 = fma2(gr[t], gr[t], g2);
+    }
+    const float lo = f2lo(g2), hi = f2hi(g2);
+    const F2 inv = f2(lo >= 1e-12f ? inv_sqrt(lo) : 0.0f, hi >= 1e-12f ? inv_sqrt(hi) : 0.0f);
+#pragma unroll
+    for (int t = 0; t < DIM; ++t) n[t] = gr[t] * inv;
+    return lo >= 1e-12f || hi >= 1e-12f;
+  };
+#pragma unroll
+  for (int i = 0; i < NM; ++i) J[i] = f2s(0.0f);
+  const bool hasL = normal(L, f2(A.phi(L, 0, 0, 0), A.phi(L, X, Y, Z)) - f2(A.phi(L, -X, -Y, -Z), A.phi(L, 0, 0, 0)), nL);
+  if (__any_sync(lanes, hasL)) {
+    // T - T_ref: the mean of the two cells' temperatures (after the boundary mapping)
+    const int n = DIM == 3 ? g.nz : g.ny, bc = g.bc[DIM - 1];
+    const float zo = (float)g.zorg + 0.5f;
+    const int kl = bc_map(k - (D == DIM - 1), n, bc), kh = bc_map(k + (D == DIM - 1), n, bc);
+    sf = f2(g.tz0 + g.tzg * (0.5f * (float)(kl + k) + zo), g.tz0 + g.tzg * (0.5f * (float)(k + kh) + zo));
+#pragma unroll
+    for (int i = 0; i < NM; ++i)
+      mf[i] = f2s(0.5f) * (f2(A.mu(i, -X, -Y, -Z), A.mu(i, 0, 0, 0)) + f2(A.mu(i, 0, 0, 0), A.mu(i, X, Y, Z)));
+    auto conc = [&](int a, F2* c) {
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        c[i] = f2s(0.0f);
+#pragma unroll
+        for (int j = 0; j < NM; ++j)
+          c[i] = fma2(f2s(g.chi[a][i * NM + j]), mf[j] - fma2(f2s(g.B1[a][j]), sf, f2s(g.B0[a][j])), c[i]);
+      }
+    };
+    conc(L, cl);
+#pragma unroll
+    for (int a = 0; a < L; ++a) {
+      const float vm = A.phi(a, -X, -Y, -Z), v0 = A.phi(a, 0, 0, 0), vp = A.phi(a, X, Y, Z);
+      const F2 l = f2(vm, v0), r = f2(v0, vp);
+      F2 na[DIM];
+      if (!__any_sync(lanes, normal(a, r - l, na))) continue;
+      const F2 pf = f2s(0.5f) * (l + r);
+      const float d0 = A.phin(a, 0, 0, 0) - v0;
+      const F2 rate = f2s(0.5f) * (f2(A.phin(a, -X, -Y, -Z) - vm, d0) + f2(d0, A.phin(a, X, Y, Z) - vp));
+      F2 proj = f2s(0.0f);   // n_alpha . n_liq
+#pragma unroll
+      for (int t = 0; t < DIM; ++t) proj = fma2(na[t], nL[t], proj);
+      const F2 co = f2(at_coefficient<float>(g.potential, g.eps, f2lo(pf)), at_coefficient<float>(g.potential, g.eps, f2hi(pf)));
+      const F2 w = f2s(-1.0f) * co * rate * na[D] * proj;
+      F2 ca[NM];
+      conc(a, ca);
+#pragma unroll
+      for (int i = 0; i < NM; ++i) J[i] = fma2(w, ca[i] - cl[i], J[i]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NM; ++i) dJ[i] = f2hi(J[i]) - f2lo(J[i]);
+}
+
 // One thread per row segment: append the segments whose block of segments is
 // not one pure phase in phi^n to the work list ([0] count, [1] ticket).
 template <int DIM, int NP, int NM, class Real>
@@ -180,58 +238,73 @@ __global__ void __launch_bounds__(256) k_at_list(const __grid_constant__ StepArg
   if (need && i < g.at_cap) g.at_list[2 + i] = (unsigned int)w;
 }
 
-// Warps over the listed segments: stage the block, correct mu.  The last CTA
-// to finish clears the list (ticket), so the launches replay from a graph.
+// Warps over the listed segments, a lane per cell, the stencil by plain loads
+// (whole rows; L1 holds what the offsets share).  The last CTA to finish clears
+// the list (ticket), so the launches replay from a graph.  FP32 evaluates the
+// two faces of an axis together.  What bounds it: the latency of its loads (16
+// warps per SM at 128 registers).  eutectic 150x133x97 on a GB300: 53 us a step; 63
+// us with the block staged element by element in shared memory, every face on its
+// own and the rows without a current corrected too.
 template <int DIM, int NP, int NM, class Real>
-__global__ void __launch_bounds__(AtShape<DIM, NP, NM, Real>::THREADS)
+__global__ void __launch_bounds__(AtShape<Real>::THREADS, AtShape<Real>::MIN_BLOCKS)
     k_at_work(const __grid_constant__ StepArgs<Real, NP, NM> g, const Real* __restrict__ in) {
-  using Sh = AtShape<DIM, NP, NM, Real>;
-  extern __shared__ unsigned char smem_raw[];
-  __shared__ unsigned int s_count;
+  using Sh = AtShape<Real>;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  Real* const box = reinterpret_cast<Real*>(smem_raw) + wid * Sh::WARP_ELEMS;
-  if (threadIdx.x == 0) s_count = min(*(volatile unsigned int*)&g.at_list[0], g.at_cap);
-  __syncthreads();
-  const unsigned int count = s_count;
+  const unsigned int count = min(*(volatile unsigned int*)&g.at_list[0], g.at_cap);
   const long long plane = (long long)g.nyp * g.pitch;
-  const AtBox<DIM, NP, NM, Real> A{box, lane};
   for (unsigned int i = blockIdx.x * Sh::WARPS + wid; i < count; i += gridDim.x * Sh::WARPS) {
     const unsigned int r = g.at_list[2 + i];
     const int s = (int)(r % (unsigned int)g.segs);
     const unsigned int zy = r / (unsigned int)g.segs;
     const int y = (int)(zy % (unsigned int)g.ny), z = (int)(zy / (unsigned int)g.ny);
-    const int x0 = 32 * s;
-    // stage: rows (field, plane, row) of 34 cells x0 - 1 .. x0 + 32, all
-    // copies in flight at once; cells past the +x ghost (x > nx) are never
-    // read by an active lane and stay unset.  mu^n and phi^{n+1} are read
-    // only at the two cells of a face, never on the four corner rows (a
-    // y and a z offset together), which are left unset for them.
-    const int xa = x0 - 1 + lane, xb = x0 + 31 + lane;
-    for (int row = 0; row < Sh::ROWS; ++row) {
-      const int f = row / (3 * Sh::NPL), pl = (row / 3) % Sh::NPL, ry = row % 3;
-      if (DIM == 3 && f >= NP && pl != 1 && ry != 1) continue;
-      const int zz = DIM == 3 ? z + pl - 1 : 0, yy = y + ry - 1;
-      const Real* src = f < NP + NM ? in + (long long)f * g.fstride : g.out + (long long)(f - NP - NM) * g.fstride;
-      src += (long long)(DIM == 3 ? zz + g.zoff : 0) * plane + (long long)(yy + 1) * g.pitch + g.xoff;
-      if (xa <= g.nx) cp_async_elem(box + row * Sh::BX + lane, src + xa);
-      if (lane < 2 && xb <= g.nx) cp_async_elem(box + row * Sh::BX + 32 + lane, src + xb);
-    }
-    cp_async_wait_all();
-    __syncwarp();
-    const int x = x0 + lane;
+    const int x = 32 * s + lane;
+    const uint32_t lanes = __ballot_sync(0xffffffffu, x < g.nx);
+    // (a split step also lists rows for their cut end alone: k_at_list's criterion)
+    int code = -1;
+    if (lane < (DIM == 3 ? 27 : 9))
+      code = load_code_from(g.codes_in, g, s + lane % 3 - 1, y + lane / 3 % 3 - 1, DIM == 3 ? z + lane / 9 - 1 : z) & kCodePhase;
+    const int c0 = __shfl_sync(0xffffffffu, code, 0);
+    if (__all_sync(0xffffffffu, c0 != 0 && (code == -1 || code == c0))) continue;
     if (x < g.nx) {
+      const long long o = (long long)(DIM == 3 ? z + g.zoff : 0) * plane + (long long)(y + 1) * g.pitch + x + g.xoff;
+      const AtBox<DIM, NP, NM, Real> A{in + o, g.out + o, g.fstride, plane, g.pitch};
       const int k = DIM == 3 ? z : y;   // index along the last axis
       Real div[NM];
 #pragma unroll
       for (int q = 0; q < NM; ++q) div[q] = Real(0);
+      if constexpr (sizeof(Real) == 4) {
+        Real gcr[NP][DIM], dJ[NM];
 #pragma unroll
-      for (int d = 0; d < DIM; ++d) {
-        Real Jp[NM], Jm[NM];
-        at_face<DIM, NP, NM, Real>(g, A, 0, 0, 0, d, k, Jp);
-        at_face<DIM, NP, NM, Real>(g, A, -(d == 0), -(d == 1), -(d == 2), d, k - (d == DIM - 1), Jm);
+        for (int a = 0; a < NP; ++a) {
+          gcr[a][0] = A.phi(a, 1, 0, 0) - A.phi(a, -1, 0, 0);
+          gcr[a][1] = A.phi(a, 0, 1, 0) - A.phi(a, 0, -1, 0);
+          if constexpr (DIM == 3) gcr[a][2] = A.phi(a, 0, 0, 1) - A.phi(a, 0, 0, -1);
+        }
+        at_axis<DIM, 0, NP, NM>(g, A, gcr, k, lanes, dJ);
 #pragma unroll
-        for (int q = 0; q < NM; ++q) div[q] += (Jp[q] - Jm[q]) * g.inv_dx;
+        for (int q = 0; q < NM; ++q) div[q] += dJ[q] * g.inv_dx;
+        at_axis<DIM, 1, NP, NM>(g, A, gcr, k, lanes, dJ);
+#pragma unroll
+        for (int q = 0; q < NM; ++q) div[q] += dJ[q] * g.inv_dx;
+        if constexpr (DIM == 3) {
+          at_axis<DIM, 2, NP, NM>(g, A, gcr, k, lanes, dJ);
+#pragma unroll
+          for (int q = 0; q < NM; ++q) div[q] += dJ[q] * g.inv_dx;
+        }
+      } else {
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) {
+          Real Jp[NM], Jm[NM];
+          at_face<DIM, NP, NM, Real>(g, A, 0, 0, 0, d, k, Jp);
+          at_face<DIM, NP, NM, Real>(g, A, -(d == 0), -(d == 1), -(d == 2), d, k - (d == DIM - 1), Jm);
+#pragma unroll
+          for (int q = 0; q < NM; ++q) div[q] += (Jp[q] - Jm[q]) * g.inv_dx;
+        }
       }
+      bool moved = false;   // a row without a current keeps mu*
+#pragma unroll
+      for (int q = 0; q < NM; ++q) moved = moved || div[q] != Real(0);
+      if (!__any_sync(lanes, moved)) continue;
       // mu^{n+1} = mu* + chi(h(phi^{n+1}))^-1 (-dt div j_at)
       Real pn[NP], h[NP];
 #pragma unroll
@@ -247,13 +320,12 @@ __global__ void __launch_bounds__(AtShape<DIM, NP, NM, Real>::THREADS)
 #pragma unroll
       for (int q = 0; q < NM; ++q) rhs[q] = -div[q];   // the rates above carry no 1/dt: dt div j_at
       solve_small<NM>(chi, rhs, dmu);
-      const long long o = (long long)(DIM == 3 ? z + g.zoff : 0) * plane + (long long)(y + 1) * g.pitch + x + g.xoff;
 #pragma unroll
       for (int q = 0; q < NM; ++q) mn[q] = g.out[(long long)(NP + q) * g.fstride + o] + dmu[q];
       store_cell<DIM>(g, x, y, z, pn, mn, false);
     }
-    __syncwarp();   // the block is refilled for the next segment
   }
+  // every CTA read the count before taking its ticket; the last one clears the list
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();

@@ -339,7 +339,7 @@ cudaError_t launch_cells(const CUtensorMap*, const CUtensorMap*, const void* in,
 template <int DIM, int NP, int NM, class Real, bool LISTED = false>
 cudaError_t launch_at(const void* in, void* blob, const HostModel& m, double t, void* out, const uint8_t* codes_in,
                       uint8_t* codes_out, const LaunchGeom& lg, cudaStream_t st) {
-  using Sh = AtShape<DIM, NP, NM, Real>;
+  using Sh = AtShape<Real>;
   if (!lg.at_list || lg.sms < 1) return cudaErrorInvalidValue;
   auto& g = *reinterpret_cast<StepArgs<Real, NP, NM>*>(blob);
   set_launch_args(g, m, t, out, codes_in, codes_out, lg);
@@ -347,10 +347,7 @@ cudaError_t launch_at(const void* in, void* blob, const HostModel& m, double t, 
   static bool configured = false;   // attributes are per function, set once
   static int per_sm = 1;            // resident CTAs per SM
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(kw, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::SMEM_BYTES);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kw, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kw, Sh::THREADS, Sh::SMEM_BYTES);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kw, Sh::THREADS, 0);
     if (e != cudaSuccess) return e;
     per_sm = per_sm < 1 ? 1 : per_sm;
     configured = true;
@@ -359,7 +356,7 @@ cudaError_t launch_at(const void* in, void* blob, const HostModel& m, double t, 
     const long long nseg = (long long)segments(m) * m.ny * (DIM == 3 ? m.nz : 1);
     k_at_list<DIM, NP, NM, Real><<<(int)((nseg + 255) / 256), 256, 0, st>>>(g);
   }
-  kw<<<lg.sms * per_sm, Sh::THREADS, Sh::SMEM_BYTES, st>>>(g, reinterpret_cast<const Real*>(in));
+  kw<<<lg.sms * per_sm, Sh::THREADS, 0, st>>>(g, reinterpret_cast<const Real*>(in));
   return cudaGetLastError();
 }
 
