@@ -259,12 +259,6 @@ __global__ void __launch_bounds__(AtShape<Real>::THREADS, AtShape<Real>::MIN_BLO
     const int y = (int)(zy % (unsigned int)g.ny), z = (int)(zy / (unsigned int)g.ny);
     const int x = 32 * s + lane;
     const uint32_t lanes = __ballot_sync(0xffffffffu, x < g.nx);
-    // (a split step also lists rows for their cut end alone: k_at_list's criterion)
-    int code = -1;
-    if (lane < (DIM == 3 ? 27 : 9))
-      code = load_code_from(g.codes_in, g, s + lane % 3 - 1, y + lane / 3 % 3 - 1, DIM == 3 ? z + lane / 9 - 1 : z) & kCodePhase;
-    const int c0 = __shfl_sync(0xffffffffu, code, 0);
-    if (__all_sync(0xffffffffu, c0 != 0 && (code == -1 || code == c0))) continue;
     if (x < g.nx) {
       const long long o = (long long)(DIM == 3 ? z + g.zoff : 0) * plane + (long long)(y + 1) * g.pitch + x + g.xoff;
       const AtBox<DIM, NP, NM, Real> A{in + o, g.out + o, g.fstride, plane, g.pitch};

@@ -263,14 +263,18 @@ cudaError_t launch_split(const CUtensorMap* tm, const CUtensorMap* tmi, const vo
   // the interface kernels in two builds: every optional path of the cell
   // update, and none of them (when the model uses none: the common case)
   const bool plain = plain_model(m);
-  auto ks = k_gp_stream<NP, NM, TY>;
+  const bool ragged = m.nx % 4 != 0;
+  auto ks = ragged ? k_gp_stream<NP, NM, TY, true> : k_gp_stream<NP, NM, TY, false>;
   auto ki = plain ? k_gp_iface<3, NP, NM, float, 0, 0> : k_gp_iface<3, NP, NM, float, 0, kFeatAll>;
   auto kf = plain ? k_gp_iface<3, NP, NM, float, two ? 1 : 0, 0>   // only launched when two
                   : k_gp_iface<3, NP, NM, float, two ? 1 : 0, kFeatAll>;
   static bool configured = false;   // attributes are per function, set once
   static int iface_per_sm[2] = {0, 0}, full_per_sm[2] = {0, 0};   // resident CTAs per SM (all, plain)
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, Ss::SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(k_gp_stream<NP, NM, TY, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         Ss::SMEM_BYTES);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_gp_stream<NP, NM, TY, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Ss::SMEM_BYTES);
     for (int v = 0; v < 2 && e == cudaSuccess; ++v) {
       auto vi = v ? k_gp_iface<3, NP, NM, float, 0, 0> : k_gp_iface<3, NP, NM, float, 0, kFeatAll>;
       auto vf = v ? k_gp_iface<3, NP, NM, float, two ? 1 : 0, 0> : k_gp_iface<3, NP, NM, float, two ? 1 : 0, kFeatAll>;

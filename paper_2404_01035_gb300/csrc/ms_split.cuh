@@ -66,7 +66,12 @@ __device__ __forceinline__ void stg4(float* p, float a, float b, float c, float 
 }
 __device__ __forceinline__ float4 lds4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
-template <int NP, int NM, int TY>
+//
+// RAGGED: rows that are no multiple of 4 cells, whose last lane stores cell by
+// cell (the others keep the shorter code: 66 against 69 us at 256^3).  Listing
+// every segment cut by a row's end instead cost the interface kernel 11 of 54 us
+// at 150x133x97.
+template <int NP, int NM, int TY, bool RAGGED>
 __global__ void __launch_bounds__(StreamShape<NP, NM, TY>::NTHREADS, StreamShape<NP, NM, TY>::MIN_BLOCKS)
     k_gp_stream(const __grid_constant__ CUtensorMap tm, const __grid_constant__ StepArgs<float, NP, NM> g) {
   using Sh = StreamShape<NP, NM, TY>;
@@ -139,12 +144,10 @@ __global__ void __launch_bounds__(StreamShape<NP, NM, TY>::NTHREADS, StreamShape
     }
   }
   __syncthreads();
-  // rows: three adjacent segments of one pure phase.  A segment cut by the end
-  // of a ragged row is never bulk (it is listed), so that bulk groups are always
-  // 4 whole cells.
+  // rows: three adjacent segments of one pure phase
   for (int e = tid; e < (nk + 2) * Sh::SY * Sh::WCS; e += Sh::NTHREADS) {
     const int wc = e % Sh::WCS, ja = e / Sh::WCS;
-    s_row[e] = (seg0 + wc + 1) * 32 <= g.nx ? (uint8_t)combine_codes(s_code + ja * Sh::CSEG + wc) : (uint8_t)0;
+    s_row[e] = (uint8_t)combine_codes(s_code + ja * Sh::CSEG + wc);
   }
   __syncthreads();
   const int reuse = g.reuse_prev ? kCodeReuse : 0;
@@ -216,15 +219,28 @@ __global__ void __launch_bounds__(StreamShape<NP, NM, TY>::NTHREADS, StreamShape
 
   // -------------------- consumer warps: 4 cells per lane, one plane at a time
   const int xs = x0 + 4 * lane, y = y0 + ty;
-  const bool last = xs + 3 == g.nx - 1;
+  const int keep = g.nx - xs;                // cells of this lane inside the row (4 and more: all)
+  const bool last = RAGGED ? keep >= 1 && keep <= 4 : keep == 4;
   const long long plane = (long long)g.nyp * g.pitch, fs = g.fstride;
   const int pitch = g.pitch;
   float* o = g.out + (long long)(zb + g.zoff) * plane + (long long)(y + 1) * pitch + xs + g.xoff;
   const bool first = xs == 0;
-  const long long oxl = g.bc[0] == 3 ? g.nx : -1, oxr = 3 + (g.bc[0] == 3 ? -g.nx : 1);   // images of their cells
+  const long long oxl = g.bc[0] == 3 ? g.nx : -1, oxr = g.bc[0] == 3 ? -xs - 1 : RAGGED ? keep : 4;   // images of their cells
   const bool yend = y == 0 || y == g.ny - 1;
   const bool zcut = g.bc[2] == kBcHalo;                 // internal cuts get their ghost planes from the exchange
   const int sidx = (ty + 1) * Sh::SX + Sh::H + 4 * lane;   // this lane's cells in a stage
+  // a lane's cells of a row, and the x ghost images of the row's first and last
+  auto put = [&](float* r, float a, float b, float e, float f) {
+    if (!RAGGED || keep >= 4) {
+      stg4(r, a, b, e, f);
+    } else {   // the end of a ragged row
+      r[0] = a;
+      if (keep >= 2) r[1] = b;
+      if (keep >= 3) r[2] = e;
+    }
+    if (first) r[oxl] = a;
+    if (last) r[oxr] = !RAGGED || keep == 4 ? f : keep == 3 ? e : keep == 2 ? b : a;
+  };
   float4 d[NM], c[NM];
   bool ok = mbar_wait_bounded(&full[0], 0) && mbar_wait_bounded(&full[1], 0);
   if (__all_sync(0xffffffffu, ok)) {
@@ -278,7 +294,7 @@ __global__ void __launch_bounds__(StreamShape<NP, NM, TY>::NTHREADS, StreamShape
       L[i][2] = (c[i].y + c[i].w) + (n[i].z + s[i].z) + (d[i].z + u[i].z) - 6.0f * c[i].z;
       L[i][3] = (c[i].z + xp[i]) + (n[i].w + s[i].w) + (d[i].w + u[i].w) - 6.0f * c[i].w;
     }
-    if (fl != 0) {
+    if (fl != 0 && keep > 0) {
       const int l1 = fl & kCodePhase;
       if (l1 != lk) {
         lk = l1;
@@ -301,22 +317,13 @@ __global__ void __launch_bounds__(StreamShape<NP, NM, TY>::NTHREADS, StreamShape
         }
       }
       const bool write_phi = (fl & kCodeReuse) == 0;
-      // the cells and the x ghost images of the row's first and last
 #pragma unroll
-      for (int i = 0; i < NM; ++i) {
-        float* const r = o + (NP + i) * fs;
-        stg4(r, mn[i][0], mn[i][1], mn[i][2], mn[i][3]);
-        if (first) r[oxl] = mn[i][0];
-        if (last) r[oxr] = mn[i][3];
-      }
+      for (int i = 0; i < NM; ++i) put(o + (NP + i) * fs, mn[i][0], mn[i][1], mn[i][2], mn[i][3]);
       if (write_phi) {
 #pragma unroll 1
         for (int a = 0; a < NP; ++a) {
           const float v = a == l1 - 1 ? 1.0f : 0.0f;
-          float* const r = o + a * fs;
-          stg4(r, v, v, v, v);
-          if (first) r[oxl] = v;
-          if (last) r[oxr] = v;
+          put(o + a * fs, v, v, v, v);
         }
       }
       if (yend || (!zcut && (z == 0 || z == g.nz - 1))) {
@@ -342,20 +349,12 @@ __global__ void __launch_bounds__(StreamShape<NP, NM, TY>::NTHREADS, StreamShape
           }
           float* const q = o + off;
 #pragma unroll
-          for (int i = 0; i < NM; ++i) {
-            float* const r = q + (NP + i) * fs;
-            stg4(r, mn[i][0], mn[i][1], mn[i][2], mn[i][3]);
-            if (first) r[oxl] = mn[i][0];
-            if (last) r[oxr] = mn[i][3];
-          }
+          for (int i = 0; i < NM; ++i) put(q + (NP + i) * fs, mn[i][0], mn[i][1], mn[i][2], mn[i][3]);
           if (write_phi) {
 #pragma unroll 1
             for (int a = 0; a < NP; ++a) {
               const float f = a == l1 - 1 ? 1.0f : 0.0f;
-              float* const r = q + a * fs;
-              stg4(r, f, f, f, f);
-              if (first) r[oxl] = f;
-              if (last) r[oxr] = f;
+              put(q + a * fs, f, f, f, f);
             }
           }
         }
@@ -611,9 +610,8 @@ __global__ void __launch_bounds__(IfaceShape<NP, NM, Real>::THREADS, IfaceShape<
     const int sg = (int)(r & seg_mask);
     const int y = (int)((r >> g.seg_bits) & y_mask), z = (int)(r >> zshift);
     // with the anti-trapping current on, its correction works on the same
-    // segments (a block of segments that is not one pure phase in phi^n, plus
-    // cut segments, where the current vanishes): the list is copied, by
-    // linear segment index, at the same positions
+    // segments (those whose block of segments is not one pure phase in phi^n):
+    // the list is copied, by linear segment index, at the same positions
     if (MODE == 0 && g.at_list && lane == 0 && i < g.at_cap)
       g.at_list[2 + i] = (unsigned int)(((long long)z * g.ny + y) * g.segs + sg);
     const int x = 32 * sg + lane;
