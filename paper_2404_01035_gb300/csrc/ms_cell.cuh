@@ -643,7 +643,7 @@ __device__ __forceinline__ void gp_cell(const Acc& A, const StepArgs<Real, NP, N
     const int l = __ffs(mask) - 1;
 #pragma unroll
     for (int a = 0; a < NP; ++a)
-      if (a == l) bulk = (val(ph[a]) == Real(1));
+      if (a == l) bulk = is_one(val(ph[a]));
   }
   const Real s = origin_temperature(A, g) + g.tzg * (Real(kz) + Real(0.5));   // T^n - T_ref
   S mc[NM];

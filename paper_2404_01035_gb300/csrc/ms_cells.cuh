@@ -16,8 +16,8 @@
 // A flux stored by no cell is zero: a face below a listed cell whose lower cell
 // is not listed has its whole stencil inside that cell's pure block.
 // eutectic 67x50x61 on a GB300: 894 us a step in the fused kernel, whose tiles
-// put the interface planes on 63 CTAs, 182 us in this form (scan 45, faces 53,
-// update 83).
+// put the interface planes on 63 CTAs, 145 us in this form (scan 15, faces 53,
+// update 77).
 #pragma once
 
 #include "ms_step.cuh"
@@ -102,8 +102,8 @@ __global__ void __launch_bounds__(256) k_c_scan(const __grid_constant__ StepArgs
 #pragma unroll
         for (int a = 0; a < NP; ++a) {
           const Real v = p[a * g.fstride];
-          nz |= (v != Real(0) ? 1u : 0u) << a;
-          one |= (v == Real(1) ? 1u : 0u) << a;
+          nz |= (nonzero(v) ? 1u : 0u) << a;
+          one |= (is_one(v) ? 1u : 0u) << a;
         }
         nzm |= nz;
         const int pc = (__popc(nz) == 1 && nz == one) ? __ffs(nz) : 0;

@@ -109,8 +109,8 @@ __global__ void __launch_bounds__(MultiShape<NP, NM, Real>::THREADS)
 #pragma unroll
           for (int a = 0; a < NP; ++a) {
             const Real v = box[(a * 3 + q) * Sh::BX + col];
-            nz |= (v != Real(0) ? 1u : 0u) << a;
-            one |= (v == Real(1) ? 1u : 0u) << a;
+            nz |= (nonzero(v) ? 1u : 0u) << a;
+            one |= (is_one(v) ? 1u : 0u) << a;
           }
           const int pc = (__popc(nz) == 1 && nz == one) ? __ffs(nz) : 0;
           c = (c == -1 || c == pc) ? pc : 0;

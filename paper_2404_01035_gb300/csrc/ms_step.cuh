@@ -83,12 +83,12 @@ __device__ __forceinline__ uint32_t stencil_mask(const Acc& A) {
 #pragma unroll
     for (int dy = -1; dy <= 1; ++dy)
 #pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) any = any || A.phi(a, dx, dy, 0) != 0;
+      for (int dx = -1; dx <= 1; ++dx) any = any || nonzero(A.phi(a, dx, dy, 0));
     if constexpr (DIM == 3) {
 #pragma unroll
       for (int dz = -1; dz <= 1; dz += 2)
-        any = any || A.phi(a, 0, 0, dz) != 0 || A.phi(a, -1, 0, dz) != 0 || A.phi(a, 1, 0, dz) != 0 ||
-              A.phi(a, 0, -1, dz) != 0 || A.phi(a, 0, 1, dz) != 0;
+        any = any || nonzero(A.phi(a, 0, 0, dz)) || nonzero(A.phi(a, -1, 0, dz)) || nonzero(A.phi(a, 1, 0, dz)) ||
+              nonzero(A.phi(a, 0, -1, dz)) || nonzero(A.phi(a, 0, 1, dz));
     }
     m |= (any ? 1u : 0u) << a;
   }
@@ -481,8 +481,8 @@ __global__ void __launch_bounds__(TX* TY + 32, MinBlocks<DIM, NP, Real, TX * TY>
         uint32_t nzm = 0, one = 0;
 #pragma unroll
         for (int a = 0; a < NP; ++a) {
-          nzm |= (pn[a] != Real(0) ? 1u : 0u) << a;
-          one |= (pn[a] == Real(1) ? 1u : 0u) << a;
+          nzm |= (nonzero(pn[a]) ? 1u : 0u) << a;
+          one |= (is_one(pn[a]) ? 1u : 0u) << a;
         }
         code = (__popc(nzm) == 1 && nzm == one) ? __ffs(nzm) : 0;
       }
@@ -530,8 +530,8 @@ __global__ void __launch_bounds__(256) k_codes(const Real* __restrict__ st, int 
 #pragma unroll
     for (int a = 0; a < NP; ++a) {
       const Real v = st[a * fstride + i0];
-      nzm |= (v != Real(0) ? 1u : 0u) << a;
-      one |= (v == Real(1) ? 1u : 0u) << a;
+      nzm |= (nonzero(v) ? 1u : 0u) << a;
+      one |= (is_one(v) ? 1u : 0u) << a;
     }
     code = (__popc(nzm) == 1 && nzm == one) ? __ffs(nzm) : 0;
   }
