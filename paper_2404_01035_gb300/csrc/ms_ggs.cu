@@ -15,14 +15,13 @@
 // (grain index, value) pairs sorted by grain index (slot-major arrays), and a
 // code byte (grain + 1 when the cell is that grain alone with value 1, else 0).
 // One step = two launches:
-//   k_ggs_classify: one thread per cell; a cell whose 7 codes name one grain
-//     keeps it (written only when the destination buffer, which holds the
-//     state one step back, does not already hold it); the others are appended
-//     to a work list (warp-aggregated).
+//   k_ggs_classify: a cell whose 7 codes name one grain keeps it (written only
+//     when the destination buffer, which holds the state one step back, does
+//     not already hold it); the others are appended to a work list (one atomic
+//     per 1024 cells).
 //   k_ggs_update: grid-stride over the list (a build for unions of up to 4
-//     grains, which defers larger ones to a second list and build); the grains of the 7 stencil cells
-//     (a 64-bit union mask), their values gathered into per-thread shared
-//     memory, the face fluxes, centre term, potential derivative and rate over
+//     grains, which defers larger ones to a second list and build); the grains
+//     of the 7 stencil cells (a 64-bit union mask), their values, the face fluxes, centre term, potential derivative and rate over
 //     that union in increasing grain order (the order of the dense sums, whose
 //     other terms are exact zeros), the projection over the union, and the
 //     non-zero results stored.
@@ -170,6 +169,71 @@ __global__ void __launch_bounds__(256) k_ggs_classify(const __grid_constant__ Gg
 }
 static_assert(8 * kClassifyRounds == 32, "one warp sums the counts");
 
+// The same for rows of a multiple of 4 cells, 4 consecutive cells of a row per
+// thread: the codes of a cell's six neighbours are compared four at a time (at
+// 128^3 on a GB300: 7.8 us against 17 for a cell per thread and round).
+template <class Real>
+__global__ void __launch_bounds__(256) k_ggs_classify4(const __grid_constant__ GgsArgs<Real> g) {
+  __shared__ unsigned int s_place[9];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const long long first = blockIdx.x * 1024ll + 4 * threadIdx.x;
+  unsigned int listed = 0u;   // by bit
+  if (first < g.cells) {
+    const unsigned int i = (unsigned int)first;
+    int x, y, z;
+    cell_of(g, i, x, y, z);
+    auto word = [&](const uint8_t* p, unsigned int at) { return *reinterpret_cast<const unsigned int*>(p + at); };
+    const unsigned int c = word(g.code_in, i);
+    const unsigned int left = g.code_in[nb_index(g, x, y, z, 0, -1)], right = g.code_in[nb_index(g, x + 3, y, z, 0, 1)];
+    const unsigned int ym = word(g.code_in, nb_index(g, x, y, z, 1, -1)), yp = word(g.code_in, nb_index(g, x, y, z, 1, 1));
+    unsigned int zm = c, zp = c;
+    if (g.dim == 3) {
+      zm = word(g.code_in, nb_index(g, x, y, z, 2, -1));
+      zp = word(g.code_in, nb_index(g, x, y, z, 2, 1));
+    }
+    const unsigned int co = word(g.code_out, i), no = word(g.cnt_out, i);
+    const unsigned int bulk = __vcmpeq4(c, (c << 8) | left) & __vcmpeq4(c, (c >> 8) | (right << 24)) & __vcmpeq4(c, ym) &
+                              __vcmpeq4(c, yp) & __vcmpeq4(c, zm) & __vcmpeq4(c, zp) & ~__vcmpeq4(c, 0u);
+    // the destination holds the state one step back: rewrite only what differs
+    const unsigned int stale = bulk & ~(__vcmpeq4(c, co) & __vcmpeq4(no, 0x01010101u));
+    if (stale) {
+      for (int k = 0; k < 4; ++k) {
+        if (!((stale >> (8 * k)) & 1u)) continue;
+        const uint8_t ck = (uint8_t)(c >> (8 * k));
+        g.cnt_out[i + k] = 1;
+        g.idx_out[i + k] = (uint8_t)(ck - 1);
+        g.val_out[i + k] = Real(1);
+        g.code_out[i + k] = ck;
+      }
+    }
+    const unsigned int l = ~bulk & 0x01010101u;
+    listed = (l | (l >> 7) | (l >> 14) | (l >> 21)) & 15u;
+  }
+  const unsigned int mine = __popc(listed);
+  unsigned int t = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned int u = __shfl_up_sync(0xffffffffu, t, o);
+    if (lane >= o) t += u;
+  }
+  if (lane == 31) s_place[wid] = t;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned int sum = 0u;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+      const unsigned int n = s_place[w];
+      s_place[w] = sum;
+      sum += n;
+    }
+    s_place[8] = sum ? atomicAdd(&g.list[0], sum) : 0u;
+  }
+  __syncthreads();
+  unsigned int at = s_place[8] + s_place[wid] + t - mine;
+  for (unsigned int m = listed; m; m &= m - 1u, ++at)
+    if (at < g.list_cap) g.list[1 + at] = (unsigned int)first + __ffs(m) - 1;
+}
+
 // Simplex projection (Held-Wolfe-Crowder 1974; Duchi et al. 2008) of the
 // first n <= kUnion values: the threshold theta (phi = max(v - theta, 0)).
 template <class Real, int K>
@@ -177,16 +241,27 @@ __device__ __forceinline__ Real simplex_theta(const Real* v, int n) {
   Real u[K];
 #pragma unroll
   for (int a = 0; a < K; ++a) u[a] = a < n ? v[a] : Real(-INFINITY);
-  // insertion sort, descending (a fixed network over K entries)
+  // descending, by Batcher's odd-even merge network (5 and 19 exchanges)
+  auto order = [&](int i, int j) {
+    if (u[j] > u[i]) {
+      const Real t = u[j];
+      u[j] = u[i];
+      u[i] = t;
+    }
+  };
+  static_assert(K == 2 || K == 4 || K == 8, "networks of 2, 4 and 8");
+  if constexpr (K == 2) order(0, 1);
 #pragma unroll
-  for (int i = 1; i < K; ++i)
-#pragma unroll
-    for (int j = i; j > 0; --j)
-      if (u[j] > u[j - 1]) {
-        const Real t = u[j];
-        u[j] = u[j - 1];
-        u[j - 1] = t;
-      }
+  for (int h = 0; h + 4 <= K; h += 4) {
+    order(h, h + 1), order(h + 2, h + 3);
+    order(h, h + 2), order(h + 1, h + 3);
+    order(h + 1, h + 2);
+  }
+  if constexpr (K == 8) {
+    order(0, 4), order(1, 5), order(2, 6), order(3, 7);
+    order(2, 4), order(3, 5);
+    order(1, 2), order(3, 4), order(5, 6);
+  }
   Real csum = Real(0), theta = Real(0);
 #pragma unroll
   for (int j = 0; j < K; ++j) {
@@ -206,27 +281,132 @@ struct UpdShape {
   static constexpr int MIN_BLOCKS = sizeof(Real) * KU > 16 ? 8 : 6;   // registers for 16 / 24 warps per SM
 };
 
+// Projection of the values v of the union's grains over the union, and the cell's
+// new slots.
+template <class Real, int K>
+__device__ __forceinline__ void store_union(const GgsArgs<Real>& g, unsigned int i, const Real* v, const int* uid, int nu) {
+  // projection over the locally active grains (the union)
+  const Real theta = simplex_theta<Real, K>(v, nu);
+  int n_out = 0;
+  uint8_t code = 0;
+#pragma unroll
+  for (int a = 0; a < K; ++a) {
+    if (a >= nu) break;
+    const Real dd = v[a] - theta;
+    const Real pn = dd > Real(0) ? dd : Real(0);
+    if (pn > Real(0)) {
+      if (n_out < kSlots) {
+        g.idx_out[(size_t)n_out * g.cells + i] = (uint8_t)uid[a];
+        g.val_out[(size_t)n_out * g.cells + i] = pn;
+        if (pn == Real(1)) code = (uint8_t)(uid[a] + 1);
+      }
+      ++n_out;
+    }
+  }
+  if (n_out > kSlots) {
+    atomicOr(g.status, kStatusOverflow);
+    n_out = kSlots;
+  }
+  g.cnt_out[i] = (uint8_t)n_out;
+  g.code_out[i] = n_out == 1 ? code : 0;
+}
+
+// One gamma: the update of cell i, whose stencil (cells ci, their first PRE slots
+// in pidx / pval, cntc stored) holds the nu <= K grains uid.
+template <class Real, int K, int PRE>
+__device__ __forceinline__ void update_uniform(const GgsArgs<Real>& g, unsigned int i, const unsigned int* ci,
+                                               const int* cntc, const int (*pidx)[PRE], const Real (*pval)[PRE],
+                                               const int* uid, int nu, int most) {
+  Real v[K];
+  // a stencil cell's values of the union's grains
+  auto gather = [&](int c, Real* out) {
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+      Real r = Real(0);
+#pragma unroll
+      for (int k = 0; k < PRE; ++k) r = pidx[c][k] == uid[u] ? pval[c][k] : r;
+      out[u] = u < nu ? r : Real(0);
+    }
+    for (int k = PRE; k < most; ++k) {
+      if (k >= cntc[c]) continue;
+      const int a = g.idx_in[(size_t)k * g.cells + ci[c]];
+      const Real r = g.val_in[(size_t)k * g.cells + ci[c]];
+#pragma unroll
+      for (int u = 0; u < K; ++u) out[u] = u < nu && a == uid[u] ? r : out[u];
+    }
+  };
+  Real ph[K], dg[K];
+  Real e1 = Real(0), e2 = Real(0), C2 = Real(0);
+  gather(0, ph);
+#pragma unroll
+  for (int a = 0; a < K; ++a) {
+    dg[a] = Real(0);
+    e2 += ph[a] * e1;
+    e1 += ph[a];
+    C2 += ph[a] * ph[a];
+  }
+  const Real kf = Real(0.5) * g.gam2_0 * g.inv_dx * g.inv_dx;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    if (d >= g.dim) continue;
+    Real nm[K], np[K];
+    gather(1 + 2 * d, nm);
+    gather(2 + 2 * d, np);
+    Real N2m = Real(0), N2p = Real(0), Xm = Real(0), Xp = Real(0), Y = Real(0);
+#pragma unroll
+    for (int a = 0; a < K; ++a) {
+      N2m += nm[a] * nm[a];
+      N2p += np[a] * np[a];
+      Xm += nm[a] * ph[a];
+      Xp += np[a] * ph[a];
+      Y += nm[a] * np[a];
+    }
+    const Real V = Real(0.5) * (Xp - Xm), Tt = Real(0.5) * (N2m + N2p) - Y;
+    const Real wm = kf * ((C2 + Xm) - V), wp = kf * ((C2 + Xp) + V);
+    const Real wc = -kf * (((N2m + Xm) + (N2p + Xp)) + Tt);
+#pragma unroll
+    for (int a = 0; a < K; ++a) dg[a] += nm[a] * wm + (np[a] * wp + ph[a] * wc);
+  }
+#pragma unroll
+  for (int a = 0; a < K; ++a) {
+    // S4 potential derivative (obstacle, with the triple term), S5 rate and explicit Euler
+    const Real others = e1 - ph[a];
+    Real W = g.cw_0 * others;
+    if (g.has_g3) W += g.g3 * (e2 - ph[a] * others);
+    const Real r = g.mob * (g.eps * dg[a] - W * g.inv_eps) * g.inv_eps;
+    v[a] = ph[a] + g.dt * r;
+  }
+  store_union<Real, K>(g, i, v, uid, nu);
+}
+
 // Two builds: KU = kUnionSmall takes the cells of the first list whose
 // stencil holds at most that many grains (nearly all) and moves the others to
 // the second list, which the KU = kUnion build then updates (each build's
 // registers fit its own union size).
 //
 // UNI: one gamma for every pair (the rule; a table of gammas takes the other
-// build).  The sums over pairs then factorise, with S1 = sum_b phi_b grad
-// phi_b, S2 = sum_b phi_b^2 on a face and T = sum_b |grad phi_b|^2 at the cell:
-//   J_a = 2 gamma (grad phi_a S2 - phi_a S1),
-//   Gc_a = 2 gamma (phi_a T - grad phi_a . sum_b phi_b grad phi_b),
-// O(grains) instead of O(grains^2) per face and straight-line (absent slots of
-// the union hold zeros).  The gathered values lie [cell][slot][thread] in
-// shared memory, so that a warp's accesses never share a bank.  8 grains in
-// 128^3, FP32, GB300: 144 -> 61 us (KU = 4) and 23 -> 16 us (KU = 8) a step.
+// build).  The sums over pairs then factorise: with a cell's values c and its
+// neighbours' n along an axis, N2 = sum n^2, X = sum n c, Y = sum n_- n_+, C2 =
+// sum c^2, V = X_+ - X_- and T = N2_- + N2_+ - 2 Y,
+//   dx^2 (div J - Gc)_a = gamma [ n_-a (C2 + X_- - V/2) + n_+a (C2 + X_+ + V/2)
+//                                 - c_a (N2_- + X_- + N2_+ + X_+ + T/2) ]
+// summed over the axes: O(grains) instead of O(grains^2), and straight-line
+// (absent grains of the union hold zeros); warps whose stencils hold two grains at
+// most, as most of a boundary does, take a build of the update for two.  What
+// bounds it is integer and FP32 instruction issue (gathering the values of the
+// seven cells by grain is two thirds of it).  The first kPre slots of the seven
+// cells are loaded at once, before their counts are known (a stale slot is then
+// ignored), and matched to the union in registers.  8 grains in 128^3, FP32, GB300,
+// KU = 4 / KU = 8 a step: 144 / 23 us by pairs, 61 / 17 us with the sums face by face
+// and the values scattered to shared memory, 55 / 12 us here.
 template <class Real, int KU, bool UNI>
 __global__ void __launch_bounds__(UpdShape<Real, KU>::THREADS, UpdShape<Real, KU>::MIN_BLOCKS)
     k_ggs_update(const __grid_constant__ GgsArgs<Real> g) {
   constexpr int T = UpdShape<Real, KU>::THREADS;
   constexpr bool kFirst = KU < kUnion;
   unsigned int* list = kFirst ? g.list : g.list2;
-  __shared__ Real s_val[7 * KU][T];
+  constexpr int kPre = kFirst ? 2 : 3;
+  __shared__ Real s_val[UNI ? 1 : 7 * KU][T];   // by pairs: [cell][slot][thread], a warp never shares a bank
   const int tid = threadIdx.x;
   auto sv = [&](int c, int u) -> Real& { return s_val[c * KU + u][tid]; };
   const unsigned int count = min(*(volatile const unsigned int*)&list[0], g.list_cap);
@@ -241,25 +421,63 @@ __global__ void __launch_bounds__(UpdShape<Real, KU>::THREADS, UpdShape<Real, KU
     int x, y, z;
     cell_of(g, i, x, y, z);
     ci[0] = i;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      ci[1 + 2 * d] = d < g.dim ? nb_index(g, x, y, z, d, -1) : i;
-      ci[2 + 2 * d] = d < g.dim ? nb_index(g, x, y, z, d, 1) : i;
-    }
+    auto neighbours = [&](int d, int pos, int n, int bc, unsigned int step) {
+      const unsigned int wrap = (unsigned int)(n - 1) * step;
+      ci[1 + 2 * d] = pos > 0 ? i - step : bc == 3 ? i + wrap : i;
+      ci[2 + 2 * d] = pos < n - 1 ? i + step : bc == 3 ? i - wrap : i;
+    };
+    neighbours(0, x, g.nx, g.bc[0], 1u);
+    neighbours(1, y, g.ny, g.bc[1], (unsigned int)g.nx);
+    ci[5] = ci[6] = i;
+    if (g.dim == 3) neighbours(2, z, g.nz, g.bc[2], (unsigned int)g.nx * (unsigned int)g.ny);
     int most = 0;
+    int pidx[7][kPre];
+    Real pval[7][kPre];
 #pragma unroll
     for (int c = 0; c < 7; ++c) {
       cntc[c] = live && c < nst ? (int)g.cnt_in[ci[c]] : 0;
+#pragma unroll
+      for (int k = 0; k < kPre; ++k) {
+        pidx[c][k] = g.idx_in[(size_t)k * g.cells + ci[c]];
+        if constexpr (UNI) pval[c][k] = g.val_in[(size_t)k * g.cells + ci[c]];
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 7; ++c) {
       most = max(most, cntc[c]);
+#pragma unroll
+      for (int k = 0; k < kPre; ++k)
+        if (k >= cntc[c]) pidx[c][k] = kMaxGrains;   // no grain
     }
     most = __reduce_max_sync(0xffffffffu, most);   // slots in use anywhere in the warp
     // union of the grains present on the stencil
-    unsigned long long mask = 0ull;
-    for (int k = 0; k < most; ++k) {
+    uint32_t lo = 0u, hi = 0u;
+    // bit a (bits past 31 and 63 shift out: lshift clamps)
+    auto lshift = [](int a) {
+      uint32_t r;
+      asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(a));
+      return r;
+    };
+#pragma unroll
+    for (int c = 0; c < 7; ++c)
+#pragma unroll
+      for (int k = 0; k < kPre; ++k) lo |= lshift(pidx[c][k]);
+    if (g.N > 32) {
 #pragma unroll
       for (int c = 0; c < 7; ++c)
-        if (k < cntc[c]) mask |= 1ull << g.idx_in[(size_t)k * g.cells + ci[c]];
+#pragma unroll
+        for (int k = 0; k < kPre; ++k) hi |= lshift(pidx[c][k] - 32);
     }
+    for (int k = kPre; k < most; ++k) {
+#pragma unroll
+      for (int c = 0; c < 7; ++c)
+        if (k < cntc[c]) {
+          const int a = g.idx_in[(size_t)k * g.cells + ci[c]];
+          lo |= lshift(a);
+          hi |= lshift(a - 32);
+        }
+    }
+    const unsigned long long mask = ((unsigned long long)hi << 32) | lo;
     const int nu = __popcll(mask);
     if (live && nu > KU) {
       if constexpr (kFirst) {
@@ -269,85 +487,42 @@ __global__ void __launch_bounds__(UpdShape<Real, KU>::THREADS, UpdShape<Real, KU
         atomicOr(g.status, kStatusOverflow);
       }
     }
+    const bool two = __all_sync(0xffffffffu, !live || nu <= 2);   // anywhere in the warp
     if (!live || nu > KU) continue;
     int uid[KU];
     {
       unsigned long long m = mask;
 #pragma unroll
       for (int u = 0; u < KU; ++u) {
-        uid[u] = m ? __ffsll((long long)m) - 1 : 0;
+        uid[u] = m ? __ffsll((long long)m) - 1 : 0;   // (the entries past nu are not used)
         m &= m - 1ull;
       }
     }
-#pragma unroll
-    for (int c = 0; c < 7; ++c)
-#pragma unroll
-      for (int u = 0; u < KU; ++u) sv(c, u) = Real(0);
-    for (int k = 0; k < most; ++k) {
-#pragma unroll
-      for (int c = 0; c < 7; ++c)
-        if (k < cntc[c]) {
-          const int a = g.idx_in[(size_t)k * g.cells + ci[c]];
-          sv(c, __popcll(mask & ((1ull << a) - 1ull))) = g.val_in[(size_t)k * g.cells + ci[c]];
-        }
-    }
     // S1-S3: divergence of the face fluxes (isotropic: the normal component
     // of g = 2 gamma q needs the normal differences only) and the centre term
-    Real v[KU];
     if constexpr (UNI) {
-      Real ph[KU], dg[KU], gc[KU][3];
-      Real e1 = Real(0), e2 = Real(0);
-#pragma unroll
-      for (int a = 0; a < KU; ++a) {
-        ph[a] = sv(0, a);
-        dg[a] = Real(0);
-        e2 += ph[a] * e1;
-        e1 += ph[a];
-      }
-      const Real kf = Real(0.25) * g.gam2_0 * g.inv_dx * g.inv_dx;
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-#pragma unroll
-        for (int a = 0; a < KU; ++a) gc[a][d] = Real(0);
-        if (d >= g.dim) continue;
-        // outward differences and sums (twice the face values) of both faces
-        Real nb[2][KU], S1[2] = {Real(0), Real(0)}, S2[2] = {Real(0), Real(0)};
-#pragma unroll
-        for (int a = 0; a < KU; ++a) {
-#pragma unroll
-          for (int s = 0; s < 2; ++s) {
-            nb[s][a] = sv(1 + 2 * d + s, a);
-            const Real t = nb[s][a] + ph[a];
-            S1[s] += t * (nb[s][a] - ph[a]);
-            S2[s] += t * t;
-          }
-          gc[a][d] = nb[1][a] - nb[0][a];
-        }
-#pragma unroll
-        for (int a = 0; a < KU; ++a)
-#pragma unroll
-          for (int s = 0; s < 2; ++s) dg[a] += kf * ((nb[s][a] - ph[a]) * S2[s] - (nb[s][a] + ph[a]) * S1[s]);
-      }
-      Real Tt = Real(0), V[3] = {Real(0), Real(0), Real(0)};
-#pragma unroll
-      for (int a = 0; a < KU; ++a)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          Tt += gc[a][d] * gc[a][d];
-          V[d] += ph[a] * gc[a][d];
-        }
-      const Real kc = g.gam2_0 * g.half_inv_dx * g.half_inv_dx;
-#pragma unroll
-      for (int a = 0; a < KU; ++a) {
-        const Real Gc = kc * (ph[a] * Tt - (gc[a][0] * V[0] + gc[a][1] * V[1] + gc[a][2] * V[2]));
-        // S4 potential derivative (obstacle, with the triple term), S5 rate and explicit Euler
-        const Real others = e1 - ph[a];
-        Real W = g.cw_0 * others;
-        if (g.has_g3) W += g.g3 * (e2 - ph[a] * others);
-        const Real r = g.mob * (g.eps * (dg[a] - Gc) - W * g.inv_eps) * g.inv_eps;
-        v[a] = ph[a] + g.dt * r;
+      if constexpr (kFirst) {   // two grains: most cells of a boundary
+        if (two)
+          update_uniform<Real, 2, kPre>(g, i, ci, cntc, pidx, pval, uid, nu, 0);
+        else
+          update_uniform<Real, KU, kPre>(g, i, ci, cntc, pidx, pval, uid, nu, most);
+      } else {
+        update_uniform<Real, KU, kPre>(g, i, ci, cntc, pidx, pval, uid, nu, most);
       }
     } else {
+      Real v[KU];
+#pragma unroll
+      for (int c = 0; c < 7; ++c)
+#pragma unroll
+        for (int u = 0; u < KU; ++u) sv(c, u) = Real(0);
+      for (int k = 0; k < most; ++k) {
+#pragma unroll
+        for (int c = 0; c < 7; ++c)
+          if (k < cntc[c]) {
+            const int a = g.idx_in[(size_t)k * g.cells + ci[c]];
+            sv(c, __popcll(mask & ((1ull << a) - 1ull))) = g.val_in[(size_t)k * g.cells + ci[c]];
+          }
+      }
       Real divJ[KU], Gc[KU];
 #pragma unroll
       for (int u = 0; u < KU; ++u) {
@@ -435,31 +610,8 @@ __global__ void __launch_bounds__(UpdShape<Real, KU>::THREADS, UpdShape<Real, KU
         const Real r = g.mob * (g.eps * (divJ[a] - Gc[a]) - W * g.inv_eps) * g.inv_eps;
         v[a] = sv(0, a) + g.dt * r;
       }
+      store_union<Real, KU>(g, i, v, uid, nu);
     }
-    // projection over the locally active grains (the union)
-    const Real theta = simplex_theta<Real, KU>(v, nu);
-    int n_out = 0;
-    uint8_t code = 0;
-#pragma unroll
-    for (int a = 0; a < KU; ++a) {
-      if (a >= nu) break;
-      const Real dd = v[a] - theta;
-      const Real pn = dd > Real(0) ? dd : Real(0);
-      if (pn > Real(0)) {
-        if (n_out < kSlots) {
-          g.idx_out[(size_t)n_out * g.cells + i] = (uint8_t)uid[a];
-          g.val_out[(size_t)n_out * g.cells + i] = pn;
-          if (pn == Real(1)) code = (uint8_t)(uid[a] + 1);
-        }
-        ++n_out;
-      }
-    }
-    if (n_out > kSlots) {
-      atomicOr(g.status, kStatusOverflow);
-      n_out = kSlots;
-    }
-    g.cnt_out[i] = (uint8_t)n_out;
-    g.code_out[i] = n_out == 1 ? code : 0;
   }
   if constexpr (!kFirst) {
     // the last CTA of the step's last kernel keeps the listed count and
@@ -529,7 +681,7 @@ struct ms_ggs {
   int* status = nullptr;
   int cur = 0;
   int64_t step = 0;
-  int upd_blocks = 0;
+  int sms = 0;
   bool uniform = false;                // one gamma for every pair
   double gamma0 = 0.0;                 // gamma of the first pair
   double g3 = 0.0;
@@ -601,14 +753,17 @@ GgsArgs<Real> make_args(const ms_ggs* s, int src) {
 template <class Real>
 cudaError_t step_once(ms_ggs* s) {
   const GgsArgs<Real> g = make_args<Real>(s, s->cur);
-  k_ggs_classify<Real><<<(unsigned int)((s->cells + 1023) / 1024), 256, 0, s->stream>>>(g);
-  if (s->uniform) {
-    k_ggs_update<Real, kUnionSmall, true><<<s->upd_blocks, UpdShape<Real, kUnionSmall>::THREADS, 0, s->stream>>>(g);
-    k_ggs_update<Real, kUnion, true><<<s->upd_blocks, UpdShape<Real, kUnion>::THREADS, 0, s->stream>>>(g);
-  } else {
-    k_ggs_update<Real, kUnionSmall, false><<<s->upd_blocks, UpdShape<Real, kUnionSmall>::THREADS, 0, s->stream>>>(g);
-    k_ggs_update<Real, kUnion, false><<<s->upd_blocks, UpdShape<Real, kUnion>::THREADS, 0, s->stream>>>(g);
-  }
+  const unsigned int blocks = (unsigned int)((s->cells + 1023) / 1024);
+  if (g.nx % 4 == 0)   // (rows, and the code array behind the counts, start on words then)
+    k_ggs_classify4<Real><<<blocks, 256, 0, s->stream>>>(g);
+  else
+    k_ggs_classify<Real><<<blocks, 256, 0, s->stream>>>(g);
+  const auto small = s->uniform ? k_ggs_update<Real, kUnionSmall, true> : k_ggs_update<Real, kUnionSmall, false>;
+  const auto large = s->uniform ? k_ggs_update<Real, kUnion, true> : k_ggs_update<Real, kUnion, false>;
+  using Ss = UpdShape<Real, kUnionSmall>;
+  using Sl = UpdShape<Real, kUnion>;
+  small<<<s->sms * Ss::MIN_BLOCKS, Ss::THREADS, 0, s->stream>>>(g);
+  large<<<s->sms * Sl::MIN_BLOCKS, Sl::THREADS, 0, s->stream>>>(g);
   return cudaGetLastError();
 }
 
@@ -775,7 +930,7 @@ ms_status ms_ggs_create(const ms_grid* grid, int n_grains, const ms_params* p, v
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  s->upd_blocks = 8 * sms;
+  s->sms = sms;
   if (e != cudaSuccess) {
     std::string m = std::string("sparse grain growth set-up: ") + cudaGetErrorString(e);
     ms_ggs_destroy(s);
