@@ -673,7 +673,7 @@ __global__ void __launch_bounds__(GatherShape<DIM>::THREADS)
 // shared memory (a thread per cell of the ringed tile).  The three launches of a
 // 256^2 reverse step were latency and traffic through L2 (cell 10.0, faces 4.6,
 // gather 11.1 us); one launch of 288 CTAs, two per SM, redoes a third of the
-// cell pass instead: 15.0 us.  FP64 keeps the three passes: its cell pass is bound by
+// cell pass instead: 13.7 us.  FP64 keeps the three passes: its cell pass is bound by
 // the FP64 pipe, where redoing costs what it computes.
 // Local cell (lx, ly) of the tile, ring included, is the grid cell at x0 + lx,
 // y0 + ly, wrapped where the axis is periodic; past a no-flux boundary there is
@@ -794,7 +794,7 @@ __global__ void __launch_bounds__(FusedShape<NP, NM>::THREADS, 2)
   if (inner) {
     Real acc[NP + NM], Mbar[NM * NM];
 #pragma unroll
-    for (int f = 0; f < NP + NM; ++f) acc[f] = own[f];
+    for (int f = 0; f < NP + NM; ++f) acc[f] = Real(0);   // (the small terms first, own last: one rounding at its size)
 #pragma unroll
     for (int k = 0; k < NM * NM; ++k) Mbar[k] = Real(0);
     // local positions holding this cell's value: itself and, at no-flux
@@ -887,7 +887,7 @@ __global__ void __launch_bounds__(FusedShape<NP, NM>::THREADS, 2)
       for (int b = 0; b < NP; ++b) acc[b] += Mbar[k] * M[k].d[b];
     const long long j = (long long)gy * g.nx + gx;
 #pragma unroll
-    for (int f = 0; f < NP + NM; ++f) lam_out[f * cells + j] = acc[f];
+    for (int f = 0; f < NP + NM; ++f) lam_out[f * cells + j] = own[f] + acc[f];
   }
   // parameter partials of the CTA's own cells: a fixed shuffle tree per warp, the warps in order
 #pragma unroll
