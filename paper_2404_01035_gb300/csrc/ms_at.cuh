@@ -57,7 +57,7 @@ template <class Real>
 struct AtShape {
   static constexpr int THREADS = 128;
   static constexpr int WARPS = THREADS / 32;
-  static constexpr int MIN_BLOCKS = sizeof(Real) == 4 ? 4 : 2;
+  static constexpr int MIN_BLOCKS = sizeof(Real) == 4 ? 6 : 2;   // FP32: 80 registers, 24 warps per SM
 };
 
 // dt times the normal component along axis d of j_at_i (the rates are taken
@@ -241,10 +241,10 @@ __global__ void __launch_bounds__(256) k_at_list(const __grid_constant__ StepArg
 // Warps over the listed segments, a lane per cell, the stencil by plain loads
 // (whole rows; L1 holds what the offsets share).  The last CTA to finish clears
 // the list (ticket), so the launches replay from a graph.  FP32 evaluates the
-// two faces of an axis together.  What bounds it: the latency of its loads (16
-// warps per SM at 128 registers).  eutectic 150x133x97 on a GB300: 53 us a step; 63
-// us with the block staged element by element in shared memory, every face on its
-// own and the rows without a current corrected too.
+// two faces of an axis together.  What bounds it: the latency of its loads, so 24
+// warps per SM: eutectic 150x133x97 on a GB300 takes 40 us a step, 53 with 16
+// warps, 63 with the block staged element by element in shared memory, every face
+// on its own and the rows without a current corrected too.
 template <int DIM, int NP, int NM, class Real>
 __global__ void __launch_bounds__(AtShape<Real>::THREADS, AtShape<Real>::MIN_BLOCKS)
     k_at_work(const __grid_constant__ StepArgs<Real, NP, NM> g, const Real* __restrict__ in) {
