@@ -21,10 +21,11 @@
 //     per 1024 cells).
 //   k_ggs_update: grid-stride over the list (a build for unions of up to 4
 //     grains, which defers larger ones to a second list and build); the grains
-//     of the 7 stencil cells (a 64-bit union mask), their values, the face fluxes, centre term, potential derivative and rate over
-//     that union in increasing grain order (the order of the dense sums, whose
-//     other terms are exact zeros), the projection over the union, and the
-//     non-zero results stored.
+//     of the 7 stencil cells (a 64-bit union mask), their values, the face
+//     fluxes, centre term, potential derivative and rate over that union in
+//     increasing grain order (the order of the dense sums, whose other terms
+//     are exact zeros), the projection over the union, and the non-zero results
+//     stored.
 // A cell that would need more than kSlots grains (or a stencil union above
 // kUnion) sets the sticky status MS_ERR_BOUNDS instead of losing a grain.
 #include <cuda_runtime.h>
@@ -278,7 +279,7 @@ __device__ __forceinline__ Real simplex_theta(const Real* v, int n) {
 template <class Real, int KU>
 struct UpdShape {
   static constexpr int THREADS = sizeof(Real) * KU > 16 ? 64 : 128;
-  static constexpr int MIN_BLOCKS = sizeof(Real) * KU > 16 ? 8 : 6;   // registers for 16 / 24 warps per SM
+  static constexpr int MIN_BLOCKS = 8;   // registers for 16 / 32 warps per SM
 };
 
 // Projection of the values v of the union's grains over the union, and the cell's
@@ -398,7 +399,8 @@ __device__ __forceinline__ void update_uniform(const GgsArgs<Real>& g, unsigned 
 // cells are loaded at once, before their counts are known (a stale slot is then
 // ignored), and matched to the union in registers.  8 grains in 128^3, FP32, GB300,
 // KU = 4 / KU = 8 a step: 144 / 23 us by pairs, 61 / 17 us with the sums face by face
-// and the values scattered to shared memory, 55 / 12 us here.
+// and the values scattered to shared memory, 53 / 12 us here (55 with 24 warps per
+// SM instead of 32).
 template <class Real, int KU, bool UNI>
 __global__ void __launch_bounds__(UpdShape<Real, KU>::THREADS, UpdShape<Real, KU>::MIN_BLOCKS)
     k_ggs_update(const __grid_constant__ GgsArgs<Real> g) {
