@@ -203,11 +203,51 @@ __global__ void __launch_bounds__(BatchShape<R>::THREADS, BatchShape<R>::MIN_BLO
   }
 }
 
+// The same steps for batches whose strips would be few: a warp per 32-cell
+// segment of any simulation (item: simulation, segment, row), as k_gp_multi, with
+// one barrier a step and no codes.
+template <int NP, int NM>
+__global__ void __launch_bounds__(MultiShape<NP, NM, float>::THREADS)
+    k_batch_units(const BatchSim<float, NP, NM>* __restrict__ sims, const BatchItem* __restrict__ items, int nitems,
+                  int nsteps, int parity0, unsigned int* counters, int* status) {
+  using Sh = MultiShape<NP, NM, float>;
+  __shared__ float s_box[Sh::WARPS][Sh::BOX];
+  __shared__ int s_ok;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  float* const box = s_box[wid];
+  for (int step = 0; step < nsteps; ++step) {
+    const int par = (parity0 + step) & 1;
+    for (int k = wid * gridDim.x + blockIdx.x; k < nitems; k += gridDim.x * Sh::WARPS) {
+      const BatchItem it = items[k];
+      const StepArgs<float, NP, NM>& g = sims[it.sim].g[par];
+      MultiAcc<NP, NM, float> acc;
+      acc.g = &g;
+      acc.tz0 = g.tz0;
+      DiffPrm<float, StepArgs<float, NP, NM>::P> dp;
+      dp.mob = g.mob;
+#pragma unroll
+      for (int p = 0; p < StepArgs<float, NP, NM>::P; ++p) dp.delta[p] = g.delta[p];
+      const int flag = stage_unit<NP, NM, float>(g, sims[it.sim].in[par], box, lane, it.sx, it.y0);
+      update_unit(g, acc, dp, box, g.out, lane, it.sx, it.y0, flag);
+      __syncwarp();
+    }
+    if (step + 1 == nsteps) break;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      s_ok = multi_barrier(&counters[0], (unsigned int)(step + 1) * gridDim.x) ? 1 : 0;
+      if (!s_ok) atomicOr(status, kStatusTimeout);
+    }
+    __syncthreads();
+    if (!s_ok) break;
+  }
+}
+
 }  // namespace msgb
 
 using namespace msgb;
 
 struct ms_batch {
+  bool units = false;                   // steps by k_batch_units
   int nsims = 0, N = 0, NM = 0, dtype = 0;
   std::vector<HostModel> models;
   std::vector<size_t> off;              // byte offset of each simulation's two state buffers
@@ -240,8 +280,15 @@ constexpr int kBTY = 8;
 constexpr int kBTYs[] = {4, 8, 16};
 constexpr int kNBTY = 3;
 
-void* batch_kernel_for(int ty) {
-  return ty == 4    ? reinterpret_cast<void*>(k_batch<2, 1, 4>)
+// Cells of all simulations up to which a batch steps by units: below, the strips'
+// two phases and barriers dominate (us a step on a GB300, units / strips: 8 x 64^2
+// 4.7 / 14.0, 30 x 77^2 10.8 / 15.9, 8 x 200^2 11.5 / 13.9, 2 x 512^2 14.6 / 13.1,
+// 4 x 400^2 17.8 / 13.5, 64 x 128^2 31.0 / 20.8).
+constexpr long long kBatchUnitCells = 400000;
+
+void* batch_kernel_for(const ms_batch* b, int ty) {
+  return b->units  ? reinterpret_cast<void*>(k_batch_units<2, 1>)
+         : ty == 4    ? reinterpret_cast<void*>(k_batch<2, 1, 4>)
          : ty == 16 ? reinterpret_cast<void*>(k_batch<2, 1, 16>)
                     : reinterpret_cast<void*>(k_batch<2, 1, 8>);
 }
@@ -281,6 +328,8 @@ cudaError_t launch_batch(ms_batch* b, int64_t n) {
   cfg.numAttrs = 1;
   const BatchSim<float, 2, 1>* sims = (const BatchSim<float, 2, 1>*)b->sims;
   const BatchItem* items = b->items;
+  if (b->units)
+    return cudaLaunchKernelEx(&cfg, k_batch_units<2, 1>, sims, items, b->nitems, (int)n, b->parity, b->barrier, b->status);
   auto kern = b->ty == 4 ? k_batch<2, 1, 4> : b->ty == 16 ? k_batch<2, 1, 16> : k_batch<2, 1, 8>;
   return cudaLaunchKernelEx(&cfg, kern, sims, items, b->nitems, b->rows, (int)n, b->parity, b->barrier, b->status);
 }
@@ -291,8 +340,8 @@ cudaError_t batch_set_tiles(ms_batch* b, int ty) {
   std::vector<BatchItem> items;
   for (int i = 0; i < b->nsims; ++i) {
     const HostModel& m = b->models[i];
-    for (int y0 = 0; y0 < m.ny; y0 += ty)
-      for (int sx = 0; 128 * sx < m.nx; ++sx) items.push_back(BatchItem{i, sx, y0, 0});
+    for (int y0 = 0; y0 < m.ny; y0 += b->units ? 1 : ty)
+      for (int sx = 0; (b->units ? 32 : 128) * sx < m.nx; ++sx) items.push_back(BatchItem{i, sx, y0, 0});
   }
   cudaError_t e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return e;
@@ -304,12 +353,13 @@ cudaError_t batch_set_tiles(ms_batch* b, int ty) {
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   int per_sm = 0, dev = 0, sms = 0;
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel_for(ty), BatchShape<kBTY>::THREADS, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel_for(b, ty), BatchShape<kBTY>::THREADS, 0);
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   b->ty = ty;
   b->grid = std::max(1, per_sm) * sms;
+  if (b->units) b->grid = std::min(b->grid, std::max(sms, (b->nitems + BatchShape<kBTY>::WARPS - 1) / BatchShape<kBTY>::WARPS));
   if (b->graph) {
     cudaGraphExecDestroy(b->graph);
     b->graph = nullptr;
@@ -376,6 +426,7 @@ ms_status ms_batch_create(int nsims, const ms_grid* grids, int n_phases, int n_c
     tot += 2 * ((sb + 255) / 256 * 256);
     nrows += (size_t)segments(m) * m.ny;
   }
+  b->units = ms_batch_cells(b) <= kBatchUnitCells;
   for (int i = 0; i < nsims; ++i) {
     b->coff.push_back(tot);
     tot += (2 * code_bytes(b->models[i]) + 15) / 16 * 16;

@@ -48,6 +48,67 @@ __device__ __forceinline__ Real origin_temperature(const MultiAcc<NP, NM, Real>&
   return A.tz0;
 }
 
+// One unit, by a warp: stages the 3 x 34 cells of every field around segment sg
+// of row y in box and tells the pure phase + 1 that they all hold, or 0.
+template <int NP, int NM, class Real>
+__device__ __forceinline__ int stage_unit(const StepArgs<Real, NP, NM>& g, const Real* in, Real* box, int lane, int sg,
+                                          int y) {
+  using Sh = MultiShape<NP, NM, Real>;
+  // columns 32 sg - 1 .. 32 sg + 32 (never past the ghost column nx)
+  const Real* row = in + (long long)y * g.pitch + 32 * sg - 1 + g.xoff;
+  const int c0 = min(lane, g.nx - 32 * sg + 1), c1 = min(lane + 32, g.nx - 32 * sg + 1);
+#pragma unroll
+  for (int f = 0; f < Sh::NF; ++f)
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const Real* p = row + f * g.fstride + (long long)q * g.pitch;
+      box[(f * 3 + q) * Sh::BX + lane] = __ldcg(p + c0);
+      if (lane < 2) box[(f * 3 + q) * Sh::BX + 32 + lane] = __ldcg(p + c1);
+    }
+  __syncwarp();
+  // one pure phase on this column's three rows (l + 1), 0 otherwise
+  auto column = [&](int col) {
+    int c = -1;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      uint32_t nz = 0, one = 0;
+#pragma unroll
+      for (int a = 0; a < NP; ++a) {
+        const Real v = box[(a * 3 + q) * Sh::BX + col];
+        nz |= (nonzero(v) ? 1u : 0u) << a;
+        one |= (is_one(v) ? 1u : 0u) << a;
+      }
+      const int pc = (__popc(nz) == 1 && nz == one) ? __ffs(nz) : 0;
+      c = (c == -1 || c == pc) ? pc : 0;
+    }
+    return c;
+  };
+  int mine = column(min(lane + 1, g.nx - 32 * sg + 1));
+  if (lane == 0 || lane == 31) {
+    const int side = column(lane == 0 ? 0 : min(33, g.nx - 32 * sg + 1));
+    mine = mine == side ? mine : 0;
+  }
+  const int ref = __shfl_sync(0xffffffffu, mine, 0);
+  return __all_sync(0xffffffffu, mine == ref) ? ref : 0;
+}
+
+// The staged unit's new cells (flag as stage_unit's).
+template <int NP, int NM, class Real, class DP>
+__device__ __forceinline__ void update_unit(const StepArgs<Real, NP, NM>& g, MultiAcc<NP, NM, Real>& acc, const DP& dp,
+                                            const Real* box, Real* out, int lane, int sg, int y, int flag) {
+  using Sh = MultiShape<NP, NM, Real>;
+  const int x = 32 * sg + lane;
+  if (x < g.nx) {
+    acc.s = box + Sh::BX + lane + 1;
+    Real pn[NP], mn[NM];
+    if (flag != 0)
+      bulk_cell<2, NP, NM, Real>(acc, g, flag - 1, pn, mn);
+    else
+      gp_cell<2, NP, NM, Real, Real>(acc, g, dp, y + g.zorg, 0ull, pn, mn);
+    store_cell_to<2>(g, out, x, y, 0, pn, mn);
+  }
+}
+
 // Arrive and wait until `target` arrivals are in; false after the time limit.
 __device__ __forceinline__ bool multi_barrier(unsigned int* counter, unsigned int target) {
   asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
@@ -86,53 +147,9 @@ __global__ void __launch_bounds__(MultiShape<NP, NM, Real>::THREADS)
     acc.g = &g;
     acc.tz0 = (Real)(r.off - r.G * (r.V * (r.t + (double)k * r.dt)));
     for (int u = wid * gridDim.x + blockIdx.x; u < units; u += total) {
-      const int y = u / g.segs, sg = u - y * g.segs, x = 32 * sg + lane;
-      const bool active = x < g.nx;
-      // columns 32 sg - 1 .. 32 sg + 32 (never past the ghost column nx)
-      const Real* row = in + (long long)y * g.pitch + 32 * sg - 1 + g.xoff;
-      const int c0 = min(lane, g.nx - 32 * sg + 1), c1 = min(lane + 32, g.nx - 32 * sg + 1);
-#pragma unroll
-      for (int f = 0; f < Sh::NF; ++f)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          const Real* p = row + f * g.fstride + (long long)q * g.pitch;
-          box[(f * 3 + q) * Sh::BX + lane] = __ldcg(p + c0);
-          if (lane < 2) box[(f * 3 + q) * Sh::BX + 32 + lane] = __ldcg(p + c1);
-        }
-      __syncwarp();
-      // one pure phase on this column's three rows (l + 1), 0 otherwise
-      auto column = [&](int col) {
-        int c = -1;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          uint32_t nz = 0, one = 0;
-#pragma unroll
-          for (int a = 0; a < NP; ++a) {
-            const Real v = box[(a * 3 + q) * Sh::BX + col];
-            nz |= (nonzero(v) ? 1u : 0u) << a;
-            one |= (is_one(v) ? 1u : 0u) << a;
-          }
-          const int pc = (__popc(nz) == 1 && nz == one) ? __ffs(nz) : 0;
-          c = (c == -1 || c == pc) ? pc : 0;
-        }
-        return c;
-      };
-      int mine = column(min(lane + 1, g.nx - 32 * sg + 1));
-      if (lane == 0 || lane == 31) {
-        const int side = column(lane == 0 ? 0 : min(33, g.nx - 32 * sg + 1));
-        mine = mine == side ? mine : 0;
-      }
-      const int ref = __shfl_sync(0xffffffffu, mine, 0);
-      const int flag = __all_sync(0xffffffffu, mine == ref) ? ref : 0;
-      if (active) {
-        acc.s = box + Sh::BX + lane + 1;
-        Real pn[NP], mn[NM];
-        if (flag != 0)
-          bulk_cell<2, NP, NM, Real>(acc, g, flag - 1, pn, mn);
-        else
-          gp_cell<2, NP, NM, Real, Real>(acc, g, dp, y + g.zorg, 0ull, pn, mn);
-        store_cell_to<2>(g, out, x, y, 0, pn, mn);
-      }
+      const int y = u / g.segs, sg = u - y * g.segs;
+      const int flag = stage_unit<NP, NM, Real>(g, in, box, lane, sg, y);
+      update_unit(g, acc, dp, box, out, lane, sg, y, flag);
       __syncwarp();
     }
     if (k + 1 == r.nsteps) break;

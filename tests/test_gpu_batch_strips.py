@@ -1,5 +1,5 @@
 """Batched runs at the edges of the 128-cell strips and of the 32-cell segments,
-for each strip height: every simulation matches its own single run."""
+for each strip height and by units: every simulation matches its own single run."""
 import numpy as np
 import pytest
 
@@ -13,21 +13,24 @@ STEPS = 6
 TOL = STEPS * 4 * 2 * 2.0 ** -24
 
 
-@pytest.mark.parametrize("tile", [4, 8, 16])
+@pytest.mark.parametrize("tile", [4, 8, 16, 0])   # 0: few cells in all, stepped by units
 def test_strip_edges(tile):
     from paper_2404_01035_gb300 import Simulation
     from paper_2404_01035_gb300.batch import Batch
     probs = []
     for i, (nx, ny, bc) in enumerate([(1, 40, [3, 3, 3]), (40, 1, [1, 1, 3]), (31, 17, [3, 1, 3]), (32, 16, [1, 3, 3]),
                                       (64, 15, [3, 3, 3]), (127, 9, [1, 1, 3]), (128, 8, [3, 3, 3]), (129, 7, [1, 3, 3]),
-                                      (256, 33, [1, 1, 3]), (260, 31, [3, 3, 3])]):
+                                      (256, 33, [1, 1, 3]), (260, 31, [3, 3, 3])] +
+                                     ([(1111, 400, [3, 1, 3])] if tile else [])):
         probs.append(W.small_multiphase(n=8, dim=2, N=2, NM=1, nx=nx, ny=ny, bc=bc, seed=nx + ny).copy(V=0.0))
     phi = []
-    for p in probs:   # pure regions beside interfaces of a few cells
-        f = np.clip(3.0 * np.asarray(p.phi0)[0] - 1.0, 0.0, 1.0)
+    for p in probs:   # stripes of one phase, 75 cells wide, with boundaries of 15 cells
+        x, y = np.arange(p.nx)[None, :], np.arange(p.ny)[:, None]
+        t = np.mod((x + 0.4 * y + 4.0 * np.sin(y / 9.0)) / 75.0, 2)
+        f = np.clip(5.0 * (0.6 - np.abs(np.mod(t + 1.0, 2.0) - 1.0)), 0.0, 1.0)[None]
         phi.append(np.stack([f, 1.0 - f]))
     b = Batch(probs)
-    b.set_tile(tile)
+    b.set_tile(tile or 8)
     for i, p in enumerate(probs):
         b.set_fields(i, phi[i], p.mu0)
     b.step(STEPS)
