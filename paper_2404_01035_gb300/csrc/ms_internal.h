@@ -134,6 +134,11 @@ struct StepKernel {
 // 10.3 / 9.4, 400^2 18.7 / 23.7; FP64 binary 128^2 30.9 / 16.4, 512^2 62 / 41,
 // 900^2 99 / 116, ternary 512^2 424 / 408.
 constexpr long long kMultiMaxCells[2] = {80000, 300000};
+// Cells from which a binary 2-D FP32 context starts with the split step: its two
+// launches cost 14 us however small the grid (us a step on a GB300, fused / split,
+// a dendrite: 290^2 6.2 / 14.4, 700^2 10.3 / 15.4, 1000^2 16.4 / 16.4, 1537x1411
+// 28.9 / 18.6, 2048^2 51.4 / 28.3).
+constexpr long long kPlaneMinCells = 1200000;
 // Steps of one multi-step launch at most (the barrier counts steps x CTAs in 32 bits).
 constexpr int kMultiMaxSteps = 1 << 16;
 

@@ -11,6 +11,7 @@
 #include "ms_diag.cuh"
 #include "ms_internal.h"
 #include "ms_multi.cuh"
+#include "ms_plane.cuh"
 #include "ms_rows.cuh"
 #include "ms_split.cuh"
 #include "ms_step.cuh"
@@ -309,6 +310,33 @@ cudaError_t launch_split(const CUtensorMap* tm, const CUtensorMap* tmi, const vo
   return cudaGetLastError();
 }
 
+// Split 2-D FP32 step: bulk strips, then the segments they listed.
+template <int NP, int NM>
+cudaError_t launch_plane(const CUtensorMap*, const CUtensorMap*, const void* in, void* blob, const HostModel& m,
+                         double t, void* out, const uint8_t* codes_in, uint8_t* codes_out, const LaunchGeom& lg,
+                         cudaStream_t st) {
+  using Sh = PlaneShape<NM>;
+  if (!lg.iface || lg.iface_blocks < 1) return cudaErrorInvalidValue;
+  auto& g = *reinterpret_cast<StepArgs<float, NP, NM>*>(blob);
+  set_launch_args(g, m, t, out, codes_in, codes_out, lg);
+  const bool plain = plain_model(m);
+  auto ki = plain ? k_plane_iface<NP, NM, 0> : k_plane_iface<NP, NM, kFeatAll>;
+  static int per_sm[2] = {0, 0};   // resident CTAs per SM (all, plain)
+  if (per_sm[1] == 0) {
+    int a = 0, b = 0;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_plane_iface<NP, NM, kFeatAll>, 128, 0);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_plane_iface<NP, NM, 0>, 128, 0);
+    if (e != cudaSuccess) return e;
+    per_sm[0] = a < 1 ? 1 : a;
+    per_sm[1] = b < 1 ? 1 : b;
+  }
+  const float* p = reinterpret_cast<const float*>(in);
+  const long long strips = (long long)((m.nx + Sh::TX - 1) / Sh::TX) * ((m.ny + Sh::R - 1) / Sh::R);
+  k_plane_stream<NP, NM><<<(unsigned)((strips + Sh::WARPS - 1) / Sh::WARPS), Sh::THREADS, 0, st>>>(g, p);
+  ki<<<lg.iface_blocks * per_sm[plain ? 1 : 0], 128, 0, st>>>(g, p);
+  return cudaGetLastError();
+}
+
 // Cell-list 3-D step (FP64): scan, upper faces, update.
 template <int NP, int NM, class Real>
 cudaError_t launch_cells(const CUtensorMap*, const CUtensorMap*, const void* in, void* blob, const HostModel& m,
@@ -413,6 +441,27 @@ StepKernel make_split_kernel() {
   k.multi = nullptr;
   k.codes = &launch_codes<3, NP, float>;
   k.at = &launch_at<3, NP, NM, float, true>;
+  return k;
+}
+
+// Split 2-D FP32 variant; strips are 128 x R cells.
+template <int NP, int NM>
+StepKernel make_plane_kernel() {
+  StepKernel k;
+  k.dim = 2;
+  k.np = NP;
+  k.nm = NM;
+  k.dtype = 0;
+  k.tx = PlaneShape<NM>::TX;
+  k.ty = PlaneShape<NM>::R;
+  k.split = 1;
+  k.smem_bytes = 0;
+  k.args_bytes = sizeof(StepArgs<float, NP, NM>);
+  k.fill = &fill_args<2, NP, NM, float>;
+  k.launch = &launch_plane<NP, NM>;
+  k.multi = &launch_multi<NP, NM, float>;
+  k.codes = &launch_codes<2, NP, float>;
+  k.at = &launch_at<2, NP, NM, float>;
   return k;
 }
 

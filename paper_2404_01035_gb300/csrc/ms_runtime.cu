@@ -341,7 +341,7 @@ bool encode_state_map(CUtensorMap* tm, void* base, const HostModel& m, int nf, i
 bool encode_step_maps(const StepKernel& k, CUtensorMap* tm, CUtensorMap* tmi, void* base, const HostModel& m) {
   const int nf = m.N + m.NM;
   if (!k.split) return encode_state_map(tm, base, m, nf, k.tx, k.ty);
-  if (m.dtype == MS_F64) return true;   // the cell-list step reads the state itself
+  if (m.dtype == MS_F64 || m.dim == 2) return true;   // the cell-list and the split 2-D step read the state itself
   const size_t s = m.dtype == MS_F64 ? 8 : 4;
   char* mu = static_cast<char*>(base) + (size_t)m.N * m.fstride * s;
   return encode_state_map(tm, mu, m, m.NM, k.tx, k.ty) && encode_state_map(tmi, base, m, nf, 32, 1, 3);
@@ -733,7 +733,8 @@ ms_status ms_create(const ms_grid* grid, int n_phases, int n_components, const m
   // multigrain 24^3 329 / 19, 128^3 1733 / 231, 384^3 3646 / 389).  A grid too
   // large for its work lists, or without memory for them, gets the fused kernel.
   const StepKernel* split = nullptr;
-  if (c->m.dim == 3 && (c->m.dtype == MS_F64 ? cells_fit(c->m) : list_entry_fits(c->m)))
+  if (c->m.dim == 3 ? (c->m.dtype == MS_F64 ? cells_fit(c->m) : list_entry_fits(c->m))
+                    : c->m.dtype == MS_F32 && list_entry_fits(c->m) && (long long)c->m.nx * c->m.ny >= kPlaneMinCells)
     for (auto* v : step_variants(c->m.dim, c->m.N, c->m.NM, c->m.dtype))
       if (v->split) split = v;
   s = MS_ERR_UNSUPPORTED;

@@ -46,16 +46,14 @@ struct PlaneStrip {
                         bc_map(seg0 - 1 + k, g.segs, g.bc[0]));
     }
     __syncwarp();
-    // a segment cut by the row's end is listed: bulk groups are whole
-    const bool whole = (seg + 1) * 32 <= g.nx;
 #pragma unroll
-    for (int r = 0; r < R + 2; ++r) rf[r] = whole ? combine_codes(code + r * CS + wc) : 0;
+    for (int r = 0; r < R + 2; ++r) rf[r] = combine_codes(code + r * CS + wc);
     bulk = listed = 0u;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const bool inside = y0 + r < g.ny && seg < g.segs;
       const bool b = rf[r] != 0 && rf[r] == rf[r + 1] && rf[r + 1] == rf[r + 2];
-      bulk |= (inside && b ? 1u : 0u) << r;
+      bulk |= (inside && b && 128 * sx + 4 * lane < g.nx ? 1u : 0u) << r;
       listed |= (inside && !b ? 1u : 0u) << r;
     }
   }
@@ -87,11 +85,12 @@ struct PlaneStrip {
                                          const uint8_t* code) const {
     if (!__any_sync(0xffffffffu, bulk != 0u)) return;
     const int wc = lane >> 3, seg = 4 * sx + wc, xs = 128 * sx + 4 * lane;
-    const bool have = xs < g.nx;
-    const bool first = xs == 0, last = xs + 3 == g.nx - 1, sider = lane == 0 || lane == 31 || last;
+    const bool have = xs <= g.nx;   // (the lane past the row's end holds its ghost for its neighbour)
+    const int keep = g.nx - xs;   // cells of this lane inside the row (4 and more: all)
+    const bool first = xs == 0, last = keep >= 1 && keep <= 4, sider = lane == 0 || lane == 31;
     const float* row = in + (long long)NP * g.fstride + (long long)y0 * g.pitch + xs + g.xoff;
     float4 v[NM][R + 2];
-    float e[NM][R + 2];   // the strip's or the row's neighbour in x (lanes 0, 31 and the row's last)
+    float e[NM][R + 2];   // the strip's neighbours in x (lanes 0 and 31)
 #pragma unroll
     for (int r = 0; r < R + 2; ++r)
 #pragma unroll
@@ -102,7 +101,7 @@ struct PlaneStrip {
         e[i][r] = ok && sider && r >= 1 && r <= R ? ld1<L2>(p + (lane == 0 ? -1 : 4)) : 0.0f;
       }
     const int reuse = g.reuse_prev ? kCodeReuse : 0;
-    const long long oxl = g.bc[0] == 3 ? g.nx : -1, oxr = 3 + (g.bc[0] == 3 ? -g.nx : 1);
+    const long long oxl = g.bc[0] == 3 ? g.nx : -1, oxr = g.bc[0] == 3 ? -xs - 1 : keep;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int y = y0 + r, l = rf[r + 1] - 1;
@@ -112,7 +111,7 @@ struct PlaneStrip {
         const float4 c = v[i][r + 1], n = v[i][r], s = v[i][r + 2];
         float xm = __shfl_up_sync(0xffffffffu, c.w, 1), xp = __shfl_down_sync(0xffffffffu, c.x, 1);
         if (lane == 0) xm = e[i][r + 1];
-        if (lane == 31 || last) xp = e[i][r + 1];
+        if (lane == 31) xp = e[i][r + 1];
         L[i][0] = (xm + c.y) + (n.x + s.x) - 4.0f * c.x;
         L[i][1] = (c.x + c.z) + (n.y + s.y) - 4.0f * c.y;
         L[i][2] = (c.y + c.w) + (n.z + s.z) - 4.0f * c.z;
@@ -133,23 +132,29 @@ struct PlaneStrip {
       }
       const bool write_phi = (code[(r + 1) * CS + wc + 1] & reuse) == 0;
       float* const o0 = g.out + (long long)(y + 1) * g.pitch + xs + g.xoff;
+      // the lane's cells and the x ghost images of the row's first and last
+      auto cells = [&](float* q, const float* w) {
+        if (keep >= 4) {
+          stg4(q, w[0], w[1], w[2], w[3]);
+        } else {   // the end of a ragged row
+          q[0] = w[0];
+          if (keep >= 2) q[1] = w[1];
+          if (keep >= 3) q[2] = w[2];
+        }
+        if (first) q[oxl] = w[0];
+        if (last) q[oxr] = keep == 4 ? w[3] : keep == 3 ? w[2] : keep == 2 ? w[1] : w[0];
+      };
       auto put = [&](float* p) {
         if (write_phi) {
 #pragma unroll
           for (int a = 0; a < NP; ++a) {
             const float f = a == l ? 1.0f : 0.0f;
-            stg4(p + a * g.fstride, f, f, f, f);
-            if (first) p[a * g.fstride + oxl] = f;
-            if (last) p[a * g.fstride + oxr] = f;
+            const float w[4] = {f, f, f, f};
+            cells(p + a * g.fstride, w);
           }
         }
 #pragma unroll
-        for (int i = 0; i < NM; ++i) {
-          float* q = p + (NP + i) * g.fstride;
-          stg4(q, mn[i][0], mn[i][1], mn[i][2], mn[i][3]);
-          if (first) q[oxl] = mn[i][0];
-          if (last) q[oxr] = mn[i][3];
-        }
+        for (int i = 0; i < NM; ++i) cells(p + (NP + i) * g.fstride, mn[i]);
       };
       put(o0);
       if (y == 0) put(o0 + (long long)(g.bc[1] == 3 ? g.ny : -1) * g.pitch);
