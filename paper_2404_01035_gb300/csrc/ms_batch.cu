@@ -255,6 +255,8 @@ struct ms_batch {
   std::vector<size_t> coff;             // byte offset of its two segment-code arrays
   size_t total = 0;                     // bytes of states and codes
   void* state = nullptr;                // all state buffers, then all codes
+  void* stage = nullptr;                // dense fields of the largest simulation, on their way to or from the host
+                                        // (NULL: strided copies)
   void* sims = nullptr;                 // BatchSim array (device)
   BatchItem* items = nullptr;
   int nitems = 0;
@@ -307,6 +309,7 @@ void batch_free(ms_batch* b) {
   if (b->stream) cudaStreamSynchronize(b->stream);
   if (b->graph) cudaGraphExecDestroy(b->graph);
   dev_free(b->hook, b->state);
+  dev_free(b->hook, b->stage);
   dev_free(b->hook, b->sims);
   dev_free(b->hook, b->items);
   dev_free(b->hook, b->rows);
@@ -433,6 +436,9 @@ ms_status ms_batch_create(int nsims, const ms_grid* grids, int n_phases, int n_c
   }
   b->total = tot;
   b->state = dev_alloc(b->hook, tot);
+  size_t dense = 0;
+  for (auto& m : b->models) dense = std::max(dense, sizeof(float) * (m.N + m.NM) * (size_t)m.nx * m.ny);
+  b->stage = dev_alloc(b->hook, dense);
   b->sims = dev_alloc(b->hook, sizeof(BatchSim<float, 2, 1>) * nsims);
   b->rows = static_cast<BatchRow*>(dev_alloc(b->hook, sizeof(BatchRow) * nrows));
   b->barrier = static_cast<unsigned int*>(dev_alloc(b->hook, 256));
@@ -482,10 +488,25 @@ ms_status ms_batch_set_fields(ms_batch* b, int sim, const void* phi, const void*
   const HostModel& m = b->models[sim];
   const size_t half = (b->sbytes[sim] + 255) / 256 * 256;
   char* buf = static_cast<char*>(b->state) + b->off[sim] + b->parity * half;
-  cudaError_t e = copy_fields(m, buf, 0, m.N, phi, nullptr, on_device, b->stream);
-  if (e == cudaSuccess) e = copy_fields(m, buf, m.N, m.NM, mu, nullptr, on_device, b->stream);
-  if (e == cudaSuccess) e = fill_ghosts(m, buf, m.N + m.NM, b->stream);
-  if (e == cudaSuccess) e = step_variants(2, 2, 1, 0).front()->codes(buf, m, codes_of(b, sim, b->parity), b->stream);
+  cudaError_t e = cudaSuccess;
+  if (on_device || b->stage) {
+    // (host fields: dense copies; strided ones run at a tenth of their rate)
+    const void *p = phi, *q = mu;
+    if (!on_device) {
+      char* s = static_cast<char*>(b->stage);
+      const size_t np = sizeof(float) * m.N * m.nx * m.ny, nm = sizeof(float) * m.NM * m.nx * m.ny;
+      e = cudaMemcpyAsync(s, phi, np, cudaMemcpyHostToDevice, b->stream);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(s + np, mu, nm, cudaMemcpyHostToDevice, b->stream);
+      p = s;
+      q = s + np;
+    }
+    if (e == cudaSuccess) e = load_fields(m, buf, p, q, codes_of(b, sim, b->parity), b->stream);
+  } else {
+    e = copy_fields(m, buf, 0, m.N, phi, nullptr, on_device, b->stream);
+    if (e == cudaSuccess) e = copy_fields(m, buf, m.N, m.NM, mu, nullptr, on_device, b->stream);
+    if (e == cudaSuccess) e = fill_ghosts(m, buf, m.N + m.NM, b->stream);
+    if (e == cudaSuccess) e = step_variants(2, 2, 1, 0).front()->codes(buf, m, codes_of(b, sim, b->parity), b->stream);
+  }
   if (e == cudaSuccess && !on_device) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bfail(b, MS_ERR_CUDA, std::string("batch set fields: ") + cudaGetErrorString(e));
   return MS_OK;
@@ -497,8 +518,18 @@ ms_status ms_batch_get_fields(ms_batch* b, int sim, void* phi, void* mu, int on_
   const size_t half = (b->sbytes[sim] + 255) / 256 * 256;
   char* buf = static_cast<char*>(b->state) + b->off[sim] + b->parity * half;
   cudaError_t e = cudaSuccess;
-  if (phi) e = copy_fields(m, buf, 0, m.N, nullptr, phi, on_device, b->stream);
-  if (e == cudaSuccess && mu) e = copy_fields(m, buf, m.N, m.NM, nullptr, mu, on_device, b->stream);
+  if (on_device) {
+    e = unload_fields(m, buf, phi, mu, b->stream);
+  } else if (b->stage) {   // as the way in
+    char* s = static_cast<char*>(b->stage);
+    const size_t np = sizeof(float) * m.N * m.nx * m.ny, nm = sizeof(float) * m.NM * m.nx * m.ny;
+    e = unload_fields(m, buf, phi ? s : nullptr, mu ? s + np : nullptr, b->stream);
+    if (e == cudaSuccess && phi) e = cudaMemcpyAsync(phi, s, np, cudaMemcpyDeviceToHost, b->stream);
+    if (e == cudaSuccess && mu) e = cudaMemcpyAsync(mu, s + np, nm, cudaMemcpyDeviceToHost, b->stream);
+  } else {
+    if (phi) e = copy_fields(m, buf, 0, m.N, nullptr, phi, on_device, b->stream);
+    if (e == cudaSuccess && mu) e = copy_fields(m, buf, m.N, m.NM, nullptr, mu, on_device, b->stream);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bfail(b, MS_ERR_CUDA, std::string("batch get fields: ") + cudaGetErrorString(e));
   return MS_OK;
