@@ -208,8 +208,8 @@ ms_status ms_get_fields(ms_ctx* ctx, void* phi, void* mu, int on_device);
  * Valid until the next ms_step / ms_set_fields / ms_destroy. */
 ms_status ms_fields(ms_ctx* ctx, void** phi_dev, void** mu_dev, int64_t strides[4]);
 
-/* Enqueue n explicit steps (each a single fused kernel launch) and, every
- * diag_every steps (ms_set_diag_every), the FP64 diagnostics kernel. */
+/* Enqueue n explicit steps (one to three kernel launches each; small 2-D grids
+ * take many steps per launch) and, every diag_every steps (ms_set_diag_every), the FP64 diagnostics kernel. */
 ms_status ms_step(ms_ctx* ctx, int64_t n);
 
 /* Run FP64 diagnostics of the current state and wait for them:
@@ -290,12 +290,15 @@ ms_status ms_set_launch(ms_ctx* ctx, int tile, int zchunk);
 /* Number of tile shapes compiled for this context and their (tx, ty). */
 int ms_tile_count(const ms_ctx* ctx);
 ms_status ms_tile_shape(const ms_ctx* ctx, int tile, int* tx, int* ty);
-/* 1 when tile variant `tile` is a split step (3-D only): a streaming kernel
- * updates the warp rows whose stencil holds one pure phase and lists the
- * others, which a second kernel then updates with the full Sec. 2.1 cell
- * update; results agree with the fused variant of the same tile to FP
- * rounding.  The split variant allocates work lists of 8 bytes per 32-cell
- * row segment (once, through the context's allocator) when first selected.
+/* 1 when tile variant `tile` is a split step (3-D, and binary 2-D FP32): a
+ * streaming kernel updates the row segments (FP64: the cells) whose stencil
+ * holds one pure phase and lists the others, which further kernels then update
+ * with the full Sec. 2.1 cell update; results agree with the fused variants to
+ * FP rounding.  The split variant allocates its scratch once, through the
+ * context's allocator, when first selected: in FP32 work lists of 8 bytes per
+ * 32-cell row segment, in FP64 per cell a list entry, two bytes, 3 N fluxes and
+ * (K-1)^2 mobilities.  A context starts with the split step in 3-D and for
+ * binary 2-D FP32 grids from 1.2 million cells, where its scratch can be had.
  * 0 for a fused variant, -1 for a bad index. */
 int ms_tile_split(const ms_ctx* ctx, int tile);
 /* Current launch: tile index and z-chunk (either pointer may be NULL). */
@@ -337,7 +340,8 @@ int ms_grad_param_count(const ms_ctx* ctx);
  * dmu0, dense device arrays dL/dphi and dL/dmu of the state at the first
  * recorded step.  Synchronous.  Segments between snapshots are recomputed with
  * the forward kernel; per reverse step three adjoint kernels run (per cell,
- * per face, per cell: a gather, no atomics, deterministic).  The current
+ * per face, per cell: a gather, no atomics, deterministic), or one that does
+ * the three in shared memory (2-D FP32).  The current
  * state is left unchanged.  Work buffers (two adjoint states, the per-face
  * records, one segment of `every` states, FP64 partials) are allocated on
  * first use through the context's allocator and kept until ms_destroy.
@@ -354,10 +358,11 @@ ms_status ms_grad(ms_ctx* ctx, const void* dphi_T, const void* dmu_T, double* dp
  * build compiles the batched kernel for 2-D, N = 2, K = 2, FP32 and
  * time-independent temperature (G V = 0); other combinations return
  * MS_ERR_UNSUPPORTED.  Each simulation keeps its own ping-pong state and
- * its own TMA descriptor in device memory.
+ * its segment codes in device memory.
  * ms_batch_step(b, n): advances every simulation n steps in ONE cooperative,
- * persistent kernel launch that walks a (simulation, tile) work list with a
- * bounded-spin grid barrier between steps; the launch is captured once into a
+ * persistent kernel launch that walks a work list of strips (batches of few
+ * cells: of 32-cell row segments) of the simulations, with bounded-spin grid
+ * barriers; the launch is captured once into a
  * CUDA graph per (n, buffer parity) and replayed.  Asynchronous; a barrier
  * timeout is reported by ms_batch_sync as MS_ERR_TIMEOUT.
  * Field I/O per simulation as in ms_set_fields / ms_get_fields (synchronous
