@@ -25,3 +25,18 @@ def test_rows_match_the_oracle(dim, nx, ny, nz, bc):
     s.close()
     o, _ = oracle.run(p, phi0, np.asarray(p.mu0)[:, :nz, :ny, :nx], steps)
     assert np.abs(g - o).max() <= 1e-10
+
+
+def test_more_than_32_grains_match_the_oracle():
+    # grain indices on both halves of the 64-bit union masks
+    from paper_2404_01035_gb300.sparse_gg import SparseGrainGrowth
+    p = W.sparse_grain_growth(n=132, dim=2, grains=48)
+    steps = 10
+    s = SparseGrainGrowth(p, dtype="f64")
+    s.set_fields(p.phi0)
+    s.step(steps)
+    g = np.asarray(s.get_fields(), dtype=np.float64)
+    s.close()
+    o, _ = oracle.run(p, p.phi0, p.mu0, steps)
+    assert np.abs(g - o).max() <= 1e-10
+    assert (np.asarray(p.phi0)[32:] > 0).any() and np.abs(o - p.phi0).max() > 1e-3
