@@ -88,7 +88,9 @@ extern "C" ms_status ms_tune(ms_ctx* c, const char* cache_path, int steps, doubl
             if (p != std::string::npos) std::sscanf(it->second.c_str() + it->second.find(':', p) + 1, "%lf", &ms);
             *best_ms = ms;
           }
-          return apply_launch(c, v, zc);
+          const ms_status as = apply_launch(c, v, zc);
+          if (as == MS_OK || !v->split) return as;
+          break;   // no scratch for the split step that won elsewhere: time the candidates
         }
     }
   }
@@ -116,7 +118,10 @@ extern "C" ms_status ms_tune(ms_ctx* c, const char* cache_path, int steps, doubl
   ms_status st = MS_OK;
   for (auto* v : variants) {
     for (int zc : zcs) {
-      if ((st = apply_launch(c, v, zc)) != MS_OK) break;
+      if ((st = apply_launch(c, v, zc)) != MS_OK) {
+        if (v->split) st = MS_OK;   // no scratch for it here: not a candidate
+        break;
+      }
       c->cur = cur0;
       e = cudaMemcpyAsync(c->buf[c->cur], saved, c->state_bytes, cudaMemcpyDeviceToDevice, c->stream);
       if ((st = refresh_codes(c)) != MS_OK) break;
