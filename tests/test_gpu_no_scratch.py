@@ -59,3 +59,40 @@ def test_starts_and_tunes_without_the_split_step(tmp_path, dim, dtype, nx, ny, n
     again = sim.get_fields()
     sim.close()
     assert np.isfinite(got[0]).all() and np.abs(got[0] - again[0]).max() <= 1e-5
+
+
+def test_tunes_where_the_scratch_took_the_memory():
+    # room for the state and the FP64 cell list, but not for the tuner's copy of the state as well
+    from paper_2404_01035_gb300 import Simulation
+    from paper_2404_01035_gb300._binding import TorchAllocator
+
+    class Bounded(TorchAllocator):
+        limit, used = None, 0
+
+        def __init__(self):
+            super().__init__()
+            self.sizes = {}
+
+        def _do_alloc(self, nbytes, user):
+            if self.limit is not None and self.used + int(nbytes) > self.limit:
+                return None
+            ptr = super()._do_alloc(nbytes, user)
+            self.sizes[ptr] = int(nbytes)
+            self.used += int(nbytes)
+            return ptr
+
+        def _do_free(self, ptr, user):
+            self.used -= self.sizes.pop(ptr, 0)
+            super()._do_free(ptr, user)
+
+    p = W.small_multiphase(n=8, dim=3, N=3, NM=2, nx=64, ny=40, nz=24, seed=4)
+    alloc = Bounded()
+    sim = Simulation(p, dtype="f64", allocator=alloc)
+    assert sim.tiles()[sim.launch()[0]][2] == 1
+    alloc.limit = alloc.used
+    sim.set_fields(p.phi0, p.mu0)
+    sim.tune(None, steps_per_trial=2)
+    assert sim.tiles()[sim.launch()[0]][2] == 0
+    sim.step(3)
+    assert np.isfinite(sim.get_fields()[0]).all()
+    sim.close()
