@@ -1053,7 +1053,7 @@ ms_status ms_before_step(ms_ctx* c) {
   if (rel < 0 || rel % a.every != 0) return MS_OK;
   const size_t idx = (size_t)(rel / a.every);
   if (idx < a.snaps.size()) return MS_OK;
-  void* p = dev_alloc(c->hook, c->state_bytes);
+  void* p = alloc_with_room(c, c->state_bytes);
   if (!p) return fail(c, MS_ERR_OOM, "adjoint snapshot allocation failed");
   a.snaps.push_back(p);
   cudaError_t e = cudaMemcpyAsync(p, c->buf[c->cur], c->state_bytes, cudaMemcpyDeviceToDevice, c->stream);
@@ -1125,26 +1125,26 @@ ms_status ms_grad(ms_ctx* c, const void* dphi_T, const void* dmu_T, double* dpar
   // allocation leaves its pointer null and the next call retries it
   for (int b = 0; b < 2; ++b)
     if (!A.adj[b]) {
-      A.adj[b] = dev_alloc(c->hook, lam_bytes);
+      A.adj[b] = alloc_with_room(c, lam_bytes);
       if (!A.adj[b]) return fail(c, MS_ERR_OOM, "adjoint state allocation failed");
     }
   if (!ak->fused && !A.tbar) {
-    A.tbar = dev_alloc(c->hook, (size_t)adjoint_work_elems(m) * s);
+    A.tbar = alloc_with_room(c, (size_t)adjoint_work_elems(m) * s);
     if (!A.tbar) return fail(c, MS_ERR_OOM, "adjoint tail buffer allocation failed");
   }
   if (!A.gpart) {
-    A.gpart = static_cast<double*>(dev_alloc(c->hook, sizeof(double) * (size_t)blocks * nprm));
+    A.gpart = static_cast<double*>(alloc_with_room(c, sizeof(double) * (size_t)blocks * nprm));
     if (!A.gpart) return fail(c, MS_ERR_OOM, "gradient scratch allocation failed");
   }
   if (!A.gsum) {
-    A.gsum = static_cast<double*>(dev_alloc(c->hook, sizeof(double) * kMaxGradParams));
+    A.gsum = static_cast<double*>(alloc_with_room(c, sizeof(double) * kMaxGradParams));
     if (!A.gsum) return fail(c, MS_ERR_OOM, "gradient scratch allocation failed");
   }
   const size_t seg_need = (size_t)A.every * c->state_bytes;
   if (!A.seg || A.seg_bytes < seg_need) {
     dev_free(c->hook, A.seg);
     A.seg_bytes = 0;
-    A.seg = dev_alloc(c->hook, seg_need);
+    A.seg = alloc_with_room(c, seg_need);
     if (!A.seg) return fail(c, MS_ERR_OOM, "adjoint segment allocation failed");
     A.seg_bytes = seg_need;
   }

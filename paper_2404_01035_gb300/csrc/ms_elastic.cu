@@ -419,8 +419,8 @@ ms_status elastic_setup(ms_ctx* c) {
   const long long cells = (long long)m.nx * m.ny * nz;
   const long long ncplx = (long long)(m.nx / 2 + 1) * m.ny * nz;
   const size_t real = m.dtype == MS_F64 ? 8 : 4;
-  s.E = dev_alloc(c->hook, s.rank * cells * real);
-  s.spec = dev_alloc(c->hook, s.rank * ncplx * 2 * real);
+  s.E = alloc_with_room(c, s.rank * cells * real);
+  s.spec = alloc_with_room(c, s.rank * ncplx * 2 * real);
   if (!s.E || !s.spec) {
     release_state(c, s);
     return fail(c, MS_ERR_OOM, "elasticity buffers");

@@ -544,6 +544,21 @@ ms_status apply_launch(ms_ctx* c, const StepKernel* k, int zchunk) {
   return MS_OK;
 }
 
+void* alloc_with_room(ms_ctx* c, size_t bytes) {
+  void* p = dev_alloc(c->hook, bytes);
+  if (p || !c->kern || !c->kern->split) return p;
+  for (auto* v : step_variants(c->m.dim, c->m.N, c->m.NM, c->m.dtype)) {
+    if (v->split) continue;
+    if (apply_launch(c, v, 0) != MS_OK || cudaStreamSynchronize(c->stream) != cudaSuccess) return nullptr;
+    dev_free(c->hook, c->lg.cells);
+    dev_free(c->hook, c->iface);
+    c->lg.cells = nullptr;
+    c->iface = c->lg.iface = c->lg.iface2 = nullptr;
+    return dev_alloc(c->hook, bytes);
+  }
+  return nullptr;
+}
+
 bool multi_steps(const ms_ctx* c) {
   return c->kern->multi && !c->m.at && !c->m.el && c->m.noise_amp == 0.0 &&
          (long long)c->m.nx * c->m.ny <= kMultiMaxCells[c->m.dtype == MS_F64 ? 1 : 0];

@@ -95,20 +95,7 @@ extern "C" ms_status ms_tune(ms_ctx* c, const char* cache_path, int steps, doubl
     }
   }
   // save the state, time every candidate from the same state, restore
-  void* saved = dev_alloc(c->hook, c->state_bytes);
-  if (!saved && c->kern->split) {
-    // the split step's own scratch (more than the state in FP64) may be what leaves no room
-    const StepKernel* fused = nullptr;
-    for (auto* v : variants)
-      if (!v->split && !fused) fused = v;
-    if (fused && apply_launch(c, fused, 0) == MS_OK && cudaStreamSynchronize(c->stream) == cudaSuccess) {
-      dev_free(c->hook, c->lg.cells);
-      dev_free(c->hook, c->iface);
-      c->lg.cells = nullptr;
-      c->iface = c->lg.iface = c->lg.iface2 = nullptr;
-      saved = dev_alloc(c->hook, c->state_bytes);
-    }
-  }
+  void* saved = alloc_with_room(c, c->state_bytes);
   if (!saved) return fail(c, MS_ERR_OOM, "tuner scratch allocation failed");
   const int cur0 = c->cur;
   const int64_t step0 = c->step;

@@ -61,9 +61,7 @@ def test_starts_and_tunes_without_the_split_step(tmp_path, dim, dtype, nx, ny, n
     assert np.isfinite(got[0]).all() and np.abs(got[0] - again[0]).max() <= 1e-5
 
 
-def test_tunes_where_the_scratch_took_the_memory():
-    # room for the state and the FP64 cell list, but not for the tuner's copy of the state as well
-    from paper_2404_01035_gb300 import Simulation
+def _bounded():
     from paper_2404_01035_gb300._binding import TorchAllocator
 
     class Bounded(TorchAllocator):
@@ -84,15 +82,32 @@ def test_tunes_where_the_scratch_took_the_memory():
         def _do_free(self, ptr, user):
             self.used -= self.sizes.pop(ptr, 0)
             super()._do_free(ptr, user)
+    return Bounded()
 
-    p = W.small_multiphase(n=8, dim=3, N=3, NM=2, nx=64, ny=40, nz=24, seed=4)
-    alloc = Bounded()
-    sim = Simulation(p, dtype="f64", allocator=alloc)
-    assert sim.tiles()[sim.launch()[0]][2] == 1
-    alloc.limit = alloc.used
-    sim.set_fields(p.phi0, p.mu0)
-    sim.tune(None, steps_per_trial=2)
-    assert sim.tiles()[sim.launch()[0]][2] == 0
-    sim.step(3)
-    assert np.isfinite(sim.get_fields()[0]).all()
-    sim.close()
+
+@pytest.mark.parametrize("what", ["tune", "checkpoints"])
+def test_scratch_makes_room(what):
+    # room for the state and the FP64 cell list, but not for the tuner's copy of the state
+    # or a checkpoint as well
+    from paper_2404_01035_gb300 import Simulation
+    p = W.small_multiphase(n=8, dim=3, N=2, NM=1, nx=64, ny=40, nz=24, seed=4)
+    out = []
+    for bounded in (False, True):
+        alloc = _bounded()
+        sim = Simulation(p, dtype="f64", allocator=alloc)
+        assert sim.tiles()[sim.launch()[0]][2] == 1
+        if bounded:
+            alloc.limit = alloc.used
+        sim.set_fields(p.phi0, p.mu0)
+        sim.step(2)
+        if what == "tune":
+            sim.tune(None, steps_per_trial=2)
+        else:
+            sim.enable_checkpoints(8)   # one: 2.5 MB padded, beside 3.8 MB of scratch
+        sim.step(6)
+        out.append(sim.get_fields())
+        assert not bounded or sim.tiles()[sim.launch()[0]][2] == 0
+        sim.close()
+    # the same step in other kernels: a few roundings of values up to 2 per step
+    assert np.abs(out[0][0] - out[1][0]).max() <= 8 * 32 * 2.0 ** -52
+    assert np.abs(out[0][1] - out[1][1]).max() <= 8 * 32 * 2.0 ** -52
