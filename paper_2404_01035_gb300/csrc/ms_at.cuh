@@ -134,13 +134,14 @@ __device__ __forceinline__ void at_face(const StepArgs<Real, NP, NM>& g, const A
 }
 
 // dt times (j_at on the upper face along axis D minus on the lower one), FP32:
-// at_face's arithmetic for both faces at once in paired registers.  gcr: the
-// cell's unscaled central differences, whose sum with a neighbour's is the
-// 4-point tangential average.  A face without a normal has a zero unit normal,
-// so its current vanishes without a test.  lanes: the warp's lanes that call.
+// at_face's arithmetic for both faces at once in paired registers, in its order:
+// where a trace of a phase puts |grad phi|^2 near the cut-off of the normals, the
+// last bit decides whether the current acts, so every launch takes the same sums.
+// A face without a normal has a zero unit normal, so its current vanishes without a
+// test.  lanes: the warp's lanes that call.
 template <int DIM, int D, int NP, int NM>
 __device__ __forceinline__ void at_axis(const StepArgs<float, NP, NM>& g, const AtBox<DIM, NP, NM, float>& A,
-                                        const float (*gcr)[DIM], int k, uint32_t lanes, float* dJ) {
+                                        int k, uint32_t lanes, float* dJ) {
   constexpr int L = NP - 1;   // the liquid
   constexpr int X = D == 0, Y = D == 1, Z = D == 2;
   F2 nL[DIM], cl[NM], mf[NM], J[NM], sf;
@@ -153,9 +154,10 @@ __device__ __forceinline__ void at_axis(const StepArgs<float, NP, NM>& g, const 
         gr[t] = lr * f2s(g.inv_dx);
       } else {
         const int tx = t == 0, ty = t == 1, tz = t == 2;
-        const F2 nb = f2(A.phi(a, tx - X, ty - Y, tz - Z), A.phi(a, tx + X, ty + Y, tz + Z)) -
-                      f2(A.phi(a, -tx - X, -ty - Y, -tz - Z), A.phi(a, X - tx, Y - ty, Z - tz));
-        gr[t] = (nb + f2s(gcr[a][t])) * f2s(g.quarter_inv_dx);
+        const float u = A.phi(a, tx, ty, tz), d = A.phi(a, -tx, -ty, -tz);
+        gr[t] = ((f2(A.phi(a, tx - X, ty - Y, tz - Z), u) + f2(u, A.phi(a, tx + X, ty + Y, tz + Z))) -
+                 (f2(A.phi(a, -tx - X, -ty - Y, -tz - Z), d) + f2(d, A.phi(a, X - tx, Y - ty, Z - tz)))) *
+                f2s(g.quarter_inv_dx);
       }
       g2 = fma2(gr[t], gr[t], g2);
     }
@@ -267,21 +269,15 @@ __global__ void __launch_bounds__(AtShape<Real>::THREADS, AtShape<Real>::MIN_BLO
 #pragma unroll
       for (int q = 0; q < NM; ++q) div[q] = Real(0);
       if constexpr (sizeof(Real) == 4) {
-        Real gcr[NP][DIM], dJ[NM];
-#pragma unroll
-        for (int a = 0; a < NP; ++a) {
-          gcr[a][0] = A.phi(a, 1, 0, 0) - A.phi(a, -1, 0, 0);
-          gcr[a][1] = A.phi(a, 0, 1, 0) - A.phi(a, 0, -1, 0);
-          if constexpr (DIM == 3) gcr[a][2] = A.phi(a, 0, 0, 1) - A.phi(a, 0, 0, -1);
-        }
-        at_axis<DIM, 0, NP, NM>(g, A, gcr, k, lanes, dJ);
+        Real dJ[NM];
+        at_axis<DIM, 0, NP, NM>(g, A, k, lanes, dJ);
 #pragma unroll
         for (int q = 0; q < NM; ++q) div[q] += dJ[q] * g.inv_dx;
-        at_axis<DIM, 1, NP, NM>(g, A, gcr, k, lanes, dJ);
+        at_axis<DIM, 1, NP, NM>(g, A, k, lanes, dJ);
 #pragma unroll
         for (int q = 0; q < NM; ++q) div[q] += dJ[q] * g.inv_dx;
         if constexpr (DIM == 3) {
-          at_axis<DIM, 2, NP, NM>(g, A, gcr, k, lanes, dJ);
+          at_axis<DIM, 2, NP, NM>(g, A, k, lanes, dJ);
 #pragma unroll
           for (int q = 0; q < NM; ++q) div[q] += dJ[q] * g.inv_dx;
         }

@@ -299,27 +299,18 @@ __device__ __forceinline__ void mobility_pair(const Acc& A, const StepArgs<float
   F2 f[NP];
 #pragma unroll
   for (int a = 0; a < NP; ++a) f[a] = f2(A.phi(a, m.x, m.y, m.z), A.phi(a, p.x, p.y, p.z));
-  F2 rest[NP];
-  if constexpr (NP == 3) {
-    rest[0] = f[1] * f[2];
-    rest[1] = f[0] * f[2];
-    rest[2] = f[0] * f[1];
-  } else if constexpr (NP > 3) {
-    F2 e1 = f[0], e2 = f2s(0.0f), run = f[0];
+  F2 e1 = f[0], e2 = f2s(0.0f), run = f[0];
 #pragma unroll
-    for (int a = 1; a < NP; ++a) {
-      e1 = e1 + f[a];
-      e2 = fma2(f[a], run, e2);
-      run = run + f[a];
-    }
-#pragma unroll
-    for (int a = 0; a < NP; ++a) rest[a] = e2 - f[a] * (e1 - f[a]);
+  for (int a = 1; a < NP; ++a) {
+    e1 = e1 + f[a];
+    e2 = fma2(f[a], run, e2);
+    run = run + f[a];
   }
 #pragma unroll
   for (int a = 0; a < NP; ++a) {
-    // p^2 (3 - 2 p) + 2 p rest
-    F2 h = f[a] * f[a] * fma2(f2s(-2.0f), f[a], f2s(3.0f));
-    if constexpr (NP > 2) h = fma2(f2s(2.0f) * f[a], rest[a], h);
+    const F2 rest = e2 - f[a] * (e1 - f[a]);
+    const F2 p2 = f[a] * f[a];
+    const F2 h = f2s(3.0f) * p2 - f2s(2.0f) * p2 * f[a] + f2s(2.0f) * f[a] * rest;
 #pragma unroll
     for (int k = 0; k < NM * NM; ++k) M[k] = a == 0 ? h * f2s(g.DX[0][k]) : fma2(h, f2s(g.DX[a][k]), M[k]);
   }
@@ -334,16 +325,14 @@ __device__ __forceinline__ void mobility_pair_liquid(const Acc& A, const StepArg
   F2 f[NP];
 #pragma unroll
   for (int a = 0; a < NP; ++a) f[a] = f2(A.phi(a, m.x, m.y, m.z), A.phi(a, p.x, p.y, p.z));
-  F2 h = f[L] * f[L] * fma2(f2s(-2.0f), f[L], f2s(3.0f));
-  if constexpr (NP > 2) {
-    F2 rest = f[0] * f[1], run = f[0] + f[1];
+  F2 rest = f2s(0.0f), run = f[0];
 #pragma unroll
-    for (int b = 2; b < L; ++b) {
-      rest = fma2(f[b], run, rest);
-      run = run + f[b];
-    }
-    h = fma2(f2s(2.0f) * f[L], rest, h);
+  for (int b = 1; b < L; ++b) {
+    rest = fma2(f[b], run, rest);
+    run = run + f[b];
   }
+  const F2 p2 = f[L] * f[L];
+  const F2 h = f2s(3.0f) * p2 - f2s(2.0f) * p2 * f[L] + f2s(2.0f) * f[L] * rest;
 #pragma unroll
   for (int k = 0; k < NM * NM; ++k) M[k] = h * f2s(g.DX[L][k]);
 }
@@ -353,15 +342,26 @@ template <int NP, int NM, class Real>
 __device__ __forceinline__ void mobility_liquid(const Real* ph, const StepArgs<Real, NP, NM>& g, Real* M) {
   constexpr int L = NP - 1;
   const Real p2 = ph[L] * ph[L];
-  Real h = Real(3) * p2 - Real(2) * p2 * ph[L];
-  if constexpr (NP > 2) {
-    Real rest = ph[0] * ph[1], run = ph[0] + ph[1];
+  Real h;
+  if constexpr (WrittenOut<Real>::value) {
+    h = Real(3) * p2 - Real(2) * p2 * ph[L];
+    if constexpr (NP > 2) {
+      Real rest = ph[0] * ph[1], run = ph[0] + ph[1];
 #pragma unroll
-    for (int b = 2; b < L; ++b) {
+      for (int b = 2; b < L; ++b) {
+        rest += ph[b] * run;
+        run += ph[b];
+      }
+      h += Real(2) * ph[L] * rest;
+    }
+  } else {
+    Real rest = Real(0), run = ph[0];
+#pragma unroll
+    for (int b = 1; b < L; ++b) {
       rest += ph[b] * run;
       run += ph[b];
     }
-    h += Real(2) * ph[L] * rest;
+    h = Real(3) * p2 - Real(2) * p2 * ph[L] + Real(2) * ph[L] * rest;
   }
 #pragma unroll
   for (int k = 0; k < NM * NM; ++k) M[k] = h * g.DX[L][k];
@@ -542,21 +542,36 @@ __device__ __forceinline__ void phase_update(const StepArgs<Real, NP, NM>& g, co
   }
   // dh_a/dphi_a = 6 phi_a (1 - phi_a) + 2 rest_a; dh_b/dphi_a = 2 phi_b sum_{c
   // != a, b} phi_c, which two phases do not have and three share as 2 phi_b phi_c
-  S rest[NP], e1 = ph[0];
-  other_products<NP>(ph, rest);
-  if constexpr (NP > 3) {
+  // (written out so where WrittenOut says)
+  S rest[NP], e1 = ph[0], e2 = S(Real(0));
+  if constexpr (WrittenOut<S>::value) {
+    other_products<NP>(ph, rest);
+    if constexpr (NP > 3) {
+#pragma unroll
+      for (int a = 1; a < NP; ++a) e1 += ph[a];
+    }
+  } else {
 #pragma unroll
     for (int a = 1; a < NP; ++a) e1 += ph[a];
+    S run = ph[0];
+#pragma unroll
+    for (int a = 1; a < NP; ++a) {
+      e2 += ph[a] * run;
+      run += ph[a];
+    }
   }
   S v[NP];
 #pragma unroll
   for (int a = 0; a < NP; ++a) {
-    S dh = Real(6) * ph[a] - Real(6) * (ph[a] * ph[a]);
-    if constexpr (NP > 2) dh = dh + Real(2) * rest[a];
-    S P = psi[a] * dh;
-    if constexpr (NP == 3) {
-      P += (psi[(a + 1) % 3] + psi[(a + 2) % 3]) * (Real(2) * rest[a]);
-    } else if constexpr (NP > 3) {
+    S P;
+    if constexpr (WrittenOut<S>::value && NP <= 3) {
+      S dh = Real(6) * ph[a] - Real(6) * (ph[a] * ph[a]);
+      if constexpr (NP > 2) dh = dh + Real(2) * rest[a];
+      P = psi[a] * dh;
+      if constexpr (NP == 3) P += (psi[(a + 1) % 3] + psi[(a + 2) % 3]) * (Real(2) * rest[a]);
+    } else {
+      const S r2 = WrittenOut<S>::value ? rest[a] : e2 - ph[a] * (e1 - ph[a]);
+      P = psi[a] * (Real(6) * ph[a] - Real(6) * (ph[a] * ph[a]) + Real(2) * r2);
 #pragma unroll
       for (int b = 0; b < NP; ++b) {
         if (b == a) continue;

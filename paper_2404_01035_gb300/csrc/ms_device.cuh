@@ -10,6 +10,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "ms_internal.h"
 
 namespace msgb {
@@ -470,6 +472,17 @@ __device__ __forceinline__ void pair_grad(const S* q, Real gam2, const S& del, b
   }
 }
 
+// Scalars whose interpolation and driving force are written out for two and
+// three phases: doubles and dual numbers, whose arithmetic bounds their kernels
+// (FP64 dendrite 128^2 on a GB300 16.4 -> 13.6 us a step, an FP32 reverse step 15.0
+// -> 13.7).  Plain FP32 keeps one form for every phase count: its kernels do not
+// gain, and the anti-trapping current, which switches on at |grad phi|^2 >= 1e-12,
+// makes differences of 1e-2 in single cells out of another rounding of phi.
+template <class S>
+struct WrittenOut {
+  static constexpr bool value = !std::is_same<S, float>::value;
+};
+
 // sum_{b<c; b,c != a} phi_b phi_c for every a: nothing for two phases, the
 // product of the others for three, else through e1 = sum phi and e2 =
 // sum_{b<c} phi_b phi_c as e2 - phi_a (e1 - phi_a).
@@ -498,13 +511,30 @@ __device__ __forceinline__ void other_products(const S* ph, S* rest) {
 template <int NP, class S>
 __device__ __forceinline__ void interp_h(const S* ph, S* h) {
   using R = decltype(val(ph[0]));
-  S rest[NP];
-  other_products<NP>(ph, rest);
+  if constexpr (WrittenOut<S>::value) {
+    S rest[NP];
+    other_products<NP>(ph, rest);
 #pragma unroll
-  for (int a = 0; a < NP; ++a) {
-    const S p2 = ph[a] * ph[a];
-    h[a] = R(3) * p2 - R(2) * p2 * ph[a];
-    if constexpr (NP > 2) h[a] = h[a] + R(2) * ph[a] * rest[a];
+    for (int a = 0; a < NP; ++a) {
+      const S p2 = ph[a] * ph[a];
+      h[a] = R(3) * p2 - R(2) * p2 * ph[a];
+      if constexpr (NP > 2) h[a] = h[a] + R(2) * ph[a] * rest[a];
+    }
+  } else {
+    S e1 = ph[0];
+#pragma unroll
+    for (int a = 1; a < NP; ++a) e1 += ph[a];
+    S e2 = 0.0f * e1, run = ph[0];
+#pragma unroll
+    for (int a = 1; a < NP; ++a) {
+      e2 += ph[a] * run;
+      run += ph[a];
+    }
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+      const S rest = e2 - ph[a] * (e1 - ph[a]), p2 = ph[a] * ph[a];
+      h[a] = R(3) * p2 - R(2) * p2 * ph[a] + R(2) * ph[a] * rest;
+    }
   }
 }
 

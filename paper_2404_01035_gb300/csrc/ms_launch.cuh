@@ -162,7 +162,9 @@ void set_launch_args(StepArgs<Real, NP, NM>& g, const HostModel& m, double t, vo
 
 // A model that uses none of the optional paths of the cell update (rotated
 // pairs, gamma_abc, phi noise, elasticity, grain growth) and in which only
-// the liquid diffuses (the one-sided model: D = 0 in every other phase).
+// the liquid diffuses (the one-sided model: D = 0 in every other phase).  Nor the
+// anti-trapping current: it makes large differences out of the last bits of phi
+// (at_axis), so its models take one form of the update whatever the launch.
 inline bool plain_model(const HostModel& m) {
   for (int a = 0; a < m.N; ++a)
     for (int b = 0; b < m.N; ++b)
@@ -170,7 +172,7 @@ inline bool plain_model(const HostModel& m) {
   for (int a = 0; a + 1 < m.N; ++a)
     for (int k = 0; k < m.NM * m.NM; ++k)
       if (m.DX[a][k] != 0.0) return false;
-  return !m.has_g3 && m.noise_amp == 0.0 && !m.el && !m.gg;
+  return !m.has_g3 && m.noise_amp == 0.0 && !m.el && !m.gg && !m.at;
 }
 
 // One boundary energy for every pair and no triple term: the sums over pairs
@@ -299,7 +301,7 @@ cudaError_t launch_split(const CUtensorMap* tm, const CUtensorMap* tmi, const vo
   const int v = plain ? 1 : 0;
   ks<<<dim3(lg.tiles, lg.zchunks), Ss::NTHREADS, Ss::SMEM_BYTES, st>>>(*tm, g);
   if constexpr (two)
-    if (uniform_gamma(m)) {
+    if (uniform_gamma(m) && !m.at) {   // (with the current, as plain_model: pairs, in the order of the fused kernel)
       if (g.n_apairs) return m.gg ? launch_rows<NP, NM, true, true>(g, in, lg.iface_blocks, st)
                                   : launch_rows<NP, NM, true, false>(g, in, lg.iface_blocks, st);
       return m.gg ? launch_rows<NP, NM, false, true>(g, in, lg.iface_blocks, st)

@@ -28,8 +28,8 @@
 // GB300, interface rows of one step, by pairs / with the sums taken face by
 // face / here: 8 grains filling 192^3 (isotropic) 5846 / 340 / 233 us; 7 rotated
 // grains in 128^3 with an eigenstrain - / 141 / 109 us; in 512^3 (few interface
-// rows) 698 / 186 / 142 us.  Models with unequal gamma or the triple term keep
-// the pair form (k_gp_iface).
+// rows) 698 / 186 / 142 us.  Models with unequal gamma, the triple term or the
+// anti-trapping current keep the pair form (k_gp_iface).
 #pragma once
 
 #include "ms_split.cuh"
@@ -187,8 +187,6 @@ __global__ void __launch_bounds__(RowsShape<NP, NM, ANISO, GG>::THREADS, RowsSha
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   unsigned int* const list = g.iface;
   if (threadIdx.x == 0) s_count = min(*(volatile unsigned int*)&list[0], g.iface_cap);
-  if (g.at_list && blockIdx.x == 0 && threadIdx.x == 0)   // see the copy below
-    g.at_list[0] = min(*(volatile unsigned int*)&list[0], g.at_cap);
   __syncthreads();
   const unsigned int count = s_count;
   const unsigned int seg_mask = (1u << g.seg_bits) - 1u, y_mask = (1u << g.y_bits) - 1u;
@@ -198,10 +196,6 @@ __global__ void __launch_bounds__(RowsShape<NP, NM, ANISO, GG>::THREADS, RowsSha
   for (unsigned int i = blockIdx.x * Sh::WARPS + wid; i < count; i += gridDim.x * Sh::WARPS) {
     const unsigned int r = list[2 + i];
     const int sg = (int)(r & seg_mask), y = (int)((r >> g.seg_bits) & y_mask), z = (int)(r >> (g.seg_bits + g.y_bits));
-    // the anti-trapping correction works on the same segments: the list is
-    // copied, by linear segment index, at the same positions
-    if (g.at_list && lane == 0 && i < g.at_cap)
-      g.at_list[2 + i] = (unsigned int)(((long long)z * g.ny + y) * g.segs + sg);
     const int x = 32 * sg + lane;
     const bool active = x < g.nx;
     // lanes past the end of a ragged row repeat its last cell (in bounds)

@@ -746,10 +746,13 @@ ms_status ms_create(const ms_grid* grid, int n_phases, int n_components, const m
   // kernels at every size measured on a GB300 (us a step, fused / split, FP32:
   // eutectic 24^3 87 / 17, 150x133x97 158 / 80, 256^3 769 / 196; 8-phase
   // multigrain 24^3 329 / 19, 128^3 1733 / 231, 384^3 3646 / 389).  A grid too
-  // large for its work lists, or without memory for them, gets the fused kernel.
+  // large for its work lists, or without memory for them, gets the fused kernel,
+  // and so do many phases with the anti-trapping current in FP32, whose split step
+  // sums the pairs in another order (see at_axis for what that does to the current).
   const StepKernel* split = nullptr;
-  if (c->m.dim == 3 ? (c->m.dtype == MS_F64 ? cells_fit(c->m) : list_entry_fits(c->m))
-                    : c->m.dtype == MS_F32 && list_entry_fits(c->m) && (long long)c->m.nx * c->m.ny >= kPlaneMinCells)
+  const bool fixed_order = c->m.at && c->m.dtype == MS_F32 && c->m.N > 3;
+  if (!fixed_order && (c->m.dim == 3 ? (c->m.dtype == MS_F64 ? cells_fit(c->m) : list_entry_fits(c->m))
+                    : c->m.dtype == MS_F32 && list_entry_fits(c->m) && (long long)c->m.nx * c->m.ny >= kPlaneMinCells))
     for (auto* v : step_variants(c->m.dim, c->m.N, c->m.NM, c->m.dtype))
       if (v->split) split = v;
   s = MS_ERR_UNSUPPORTED;
