@@ -346,27 +346,28 @@ __device__ __forceinline__ void update_uniform(const GgsArgs<Real>& g, unsigned 
     e1 += ph[a];
     C2 += ph[a] * ph[a];
   }
-  const Real kf = Real(0.5) * g.gam2_0 * g.inv_dx * g.inv_dx;
+  const Real kf = g.gam2_0 * g.inv_dx * g.inv_dx;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     if (d >= g.dim) continue;
-    Real nm[K], np[K];
-    gather(1 + 2 * d, nm);
-    gather(2 + 2 * d, np);
-    Real N2m = Real(0), N2p = Real(0), Xm = Real(0), Xp = Real(0), Y = Real(0);
+    Real w[K], u[K];   // differences to the two neighbours (see k_ggs_update)
+    gather(1 + 2 * d, w);
+    gather(2 + 2 * d, u);
+    Real S = Real(0), Xw = Real(0), Xu = Real(0), Y = Real(0);
 #pragma unroll
     for (int a = 0; a < K; ++a) {
-      N2m += nm[a] * nm[a];
-      N2p += np[a] * np[a];
-      Xm += nm[a] * ph[a];
-      Xp += np[a] * ph[a];
-      Y += nm[a] * np[a];
+      w[a] -= ph[a];
+      u[a] -= ph[a];
+      S += w[a] * w[a] + u[a] * u[a];
+      Xw += w[a] * ph[a];
+      Xu += u[a] * ph[a];
+      Y += w[a] * u[a];
     }
-    const Real V = Real(0.5) * (Xp - Xm), Tt = Real(0.5) * (N2m + N2p) - Y;
-    const Real wm = kf * ((C2 + Xm) - V), wp = kf * ((C2 + Xp) + V);
-    const Real wc = -kf * (((N2m + Xm) + (N2p + Xp)) + Tt);
+    const Real V = Real(0.25) * (Xu - Xw), Tt = Real(0.25) * S - Real(0.5) * Y;
+    const Real kw = kf * ((C2 + Real(0.5) * Xw) - V), ku = kf * ((C2 + Real(0.5) * Xu) + V);
+    const Real kc = -kf * (((Xu + Xw) + Real(0.5) * S) + Tt);
 #pragma unroll
-    for (int a = 0; a < K; ++a) dg[a] += nm[a] * wm + (np[a] * wp + ph[a] * wc);
+    for (int a = 0; a < K; ++a) dg[a] += (w[a] * kw + u[a] * ku) + ph[a] * kc;
   }
 #pragma unroll
   for (int a = 0; a < K; ++a) {
@@ -386,12 +387,13 @@ __device__ __forceinline__ void update_uniform(const GgsArgs<Real>& g, unsigned 
 // registers fit its own union size).
 //
 // UNI: one gamma for every pair (the rule; a table of gammas takes the other
-// build).  The sums over pairs then factorise: with a cell's values c and its
-// neighbours' n along an axis, N2 = sum n^2, X = sum n c, Y = sum n_- n_+, C2 =
-// sum c^2, V = X_+ - X_- and T = N2_- + N2_+ - 2 Y,
-//   dx^2 (div J - Gc)_a = gamma [ n_-a (C2 + X_- - V/2) + n_+a (C2 + X_+ + V/2)
-//                                 - c_a (N2_- + X_- + N2_+ + X_+ + T/2) ]
-// summed over the axes: O(grains) instead of O(grains^2), and straight-line
+// build).  The sums over pairs then factorise: with a cell's values c and the
+// differences u = n_+ - c, w = n_- - c to its neighbours along an axis, X = sum u c,
+// S = sum u^2 (of u, of w), Y = sum u w, C2 = sum c^2, V = (X_u - X_w) / 4 and T =
+// (S_u + S_w - 2 Y) / 4,
+//   dx^2 (div J - Gc)_a = 2 gamma [ u_a (C2 + X_u / 2 + V) + w_a (C2 + X_w / 2 - V)
+//                                   - c_a (X_u + X_w + (S_u + S_w) / 2 + T) ]
+// (differences, or terms of order 1 cancel: see k_gp_rows), summed over the axes: O(grains) instead of O(grains^2), and straight-line
 // (absent grains of the union hold zeros); warps whose stencils hold two grains at
 // most, as most of a boundary does, take a build of the update for two.  What
 // bounds it is integer and FP32 instruction issue (gathering the values of the
