@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(256) k_c_scan(const __grid_constant__ StepArgs
                                                 const Real* __restrict__ in,
                                                 const __grid_constant__ CellsScratch<Real> c) {
   const int lane = threadIdx.x & 31;
-  const unsigned int nseg = (unsigned int)g.segs * g.ny * g.nz, w0 = (blockIdx.x * 256u + threadIdx.x) >> 5;
+  const unsigned int nseg = (unsigned int)g.segs * g.ny * g.nz, w0 = blockIdx.x * 8u + (threadIdx.x >> 5);
   const bool live = w0 < nseg;   // (warps past the end redo the last segment and list nothing)
   const unsigned int w = live ? w0 : nseg - 1;
   const int sg = (int)(w % g.segs), y = (int)((w / g.segs) % g.ny), z = (int)(w / ((unsigned int)g.segs * g.ny));

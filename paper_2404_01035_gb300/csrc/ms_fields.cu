@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(256) k_load_fields(const __grid_constant__ Fie
                                                      const Real* __restrict__ mu, Real* __restrict__ out,
                                                      uint8_t* __restrict__ codes) {
   using V = Vec<Real, VEC>;
-  const unsigned int w = (blockIdx.x * 256u + threadIdx.x) >> 5;
+  const unsigned int w = blockIdx.x * 8u + (threadIdx.x >> 5);   // (warps: threads would pass 2^32 with the grid)
   const int lane = threadIdx.x & 31;
   if (w >= (unsigned int)q.pieces * q.ny * q.nz) return;
   const unsigned int r = w / (unsigned int)q.pieces;
@@ -123,7 +123,7 @@ template <class Real, int VEC>
 __global__ void __launch_bounds__(256) k_unload_fields(const __grid_constant__ FieldGeom q, const Real* __restrict__ in,
                                                        Real* __restrict__ phi, Real* __restrict__ mu) {
   using V = Vec<Real, VEC>;
-  const unsigned int w = (blockIdx.x * 256u + threadIdx.x) >> 5;
+  const unsigned int w = blockIdx.x * 8u + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= (unsigned int)q.pieces * q.ny * q.nz) return;
   const unsigned int r = w / (unsigned int)q.pieces;
