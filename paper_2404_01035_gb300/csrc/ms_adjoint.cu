@@ -690,8 +690,9 @@ struct FusedShape {
   static constexpr int DJ = 0, GCR = NP, DIV = GCR + 2 * NP, M = DIV + NM, MU = M + NM * NM, FX = MU + NM,
                        FY = FX + FS::N, N = FY + FS::N;
 };
-inline dim3 fused_grid(const HostModel& m) {
-  return dim3((unsigned)((m.nx + kFusedTX - 1) / kFusedTX), (unsigned)((m.ny + kFusedTY - 1) / kFusedTY));
+// (one-dimensional: a grid's y extent ends at 65535 blocks)
+inline long long fused_blocks(const HostModel& m) {
+  return (long long)((m.nx + kFusedTX - 1) / kFusedTX) * ((m.ny + kFusedTY - 1) / kFusedTY);
 }
 
 template <int NP, int NM, class Real>
@@ -710,7 +711,8 @@ __global__ void __launch_bounds__(FusedShape<NP, NM>::THREADS, 2)
   __shared__ double red[NW][NPRM];
   const int tid = threadIdx.x, lane = tid & 31;
   const int lx = lane - 1, ly = (tid >> 5) - 1;
-  const int gx = (int)blockIdx.x * kFusedTX + lx, gy = (int)blockIdx.y * kFusedTY + ly;
+  const unsigned int tiles_x = (unsigned int)(g.nx + kFusedTX - 1) / kFusedTX, by = blockIdx.x / tiles_x;
+  const int gx = (int)(blockIdx.x - by * tiles_x) * kFusedTX + lx, gy = (int)by * kFusedTY + ly;
   const long long cells = (long long)g.nx * g.ny;
   // the grid cell (vx, vy: there is one) and the padded position to read at
   auto wrap = [](int i, int n, int bc, int& w) {
@@ -903,7 +905,7 @@ __global__ void __launch_bounds__(FusedShape<NP, NM>::THREADS, 2)
   if (tid < NPRM) {
     double v = 0.0;
     for (int w = 0; w < NW; ++w) v += red[w][tid];
-    partials[((long long)blockIdx.y * gridDim.x + blockIdx.x) * NPRM + tid] += v;   // summed over the reverse steps
+    partials[(long long)blockIdx.x * NPRM + tid] += v;   // summed over the reverse steps
   }
 }
 
@@ -975,7 +977,7 @@ cudaError_t launch_adjoint(const void* state, const void* lam_in, void* lam_out,
 
 // Parameter partials of a reverse step: one set per block of its cell pass.
 inline long long adjoint_blocks(const AdjKernel& k, const HostModel& m) {
-  if (k.fused) return (long long)fused_grid(m).x * fused_grid(m).y;
+  if (k.fused) return fused_blocks(m);
   return ((long long)m.nx * m.ny * m.nz + 127) / 128;
 }
 
@@ -987,7 +989,7 @@ cudaError_t launch_adjoint_fused(const void* state, const void* lam_in, void* la
   AdjExtra<Real, NP, NM> ex;
   for (int a = 0; a < NP; ++a)
     for (int k = 0; k < NM * NM; ++k) ex.D[a][k] = (Real)m.D[a][k];
-  k_adj_fused<NP, NM, Real><<<fused_grid(m), FusedShape<NP, NM>::THREADS, 0, st>>>(
+  k_adj_fused<NP, NM, Real><<<(unsigned)fused_blocks(m), FusedShape<NP, NM>::THREADS, 0, st>>>(
       reinterpret_cast<const Real*>(state), reinterpret_cast<const Real*>(lam_in), reinterpret_cast<Real*>(lam_out), g,
       ex, partials);
   return cudaGetLastError();
