@@ -348,6 +348,13 @@ ElasticBasis elastic_basis(const HostModel& m) {
       for (int j = 0; j < m.dim; ++j) rem[a][i][j] = m.eig[a][std::max(i, j)][std::min(i, j)];   // symmetric
     top = std::max(top, norm2(rem[a]));
   }
+  for (int a = 0; a < m.N; ++a)
+    if (!std::isfinite(norm2(rem[a]))) {   // no comparison below holds: passed on, the state becomes non-finite
+      b.rank = 1;
+      b.B[0][0][0] = 1.0;
+      for (int p = 0; p < m.N; ++p) b.c[p][0] = norm2(rem[a]);
+      return b;
+    }
   while (b.rank < kElRank) {
     int pick = 0;
     for (int a = 1; a < m.N; ++a)
