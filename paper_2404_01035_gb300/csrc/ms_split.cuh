@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(StreamShape<NP, NM, TY>::NTHREADS, StreamShape
   }
   const int streaming = __syncthreads_count(lane == 0 && any != 0u);   // warps
   if (tid == 0) {
-    for (int i = 0; i < NST; ++i) mbar_init(&empty[i], streaming);
+    for (int i = 0; i < NST; ++i) mbar_init(&empty[i], streaming > 0 ? streaming : 1);   // (a count is at least 1)
     mbar_fence_init();
   }
   __syncthreads();   // the last CTA-wide barrier: roles split below
