@@ -1170,7 +1170,7 @@ ms_status ms_grad(ms_ctx* c, const void* dphi_T, const void* dmu_T, double* dpar
     if (e != cudaSuccess) return cuda_fail(c, e, "segment restore");
     const bool multi = multi_steps(c);
     if (multi && len > 1) {   // as the forward steps went
-      ms_status ms = launch_multi_steps(c, len - 1, slots, c->state_bytes, m.t0 + (double)s0 * m.dt);
+      ms_status ms = launch_multi_steps(c, len - 1, slots, c->state_bytes, s0, m.t0 + (double)s0 * m.dt);
       if (ms != MS_OK) return ms;
     }
     if (!multi && len > 1) {

@@ -96,7 +96,9 @@ struct MultiRun {
   size_t slot_bytes;
   int nsteps;
   double t;                    // time of state 0
-  double off, G, V, dt;        // T - T_ref = off - G V t at the origin of the last axis
+  double t0, dt;               // and of state k > 0: t0 + (step0 + k) dt
+  long long step0;
+  double off, G, z0, V;        // T - T_ref = off - G (z0 + V t) at the origin of the last axis
   unsigned int* counters;      // [0] barrier arrivals, [1] exit tickets; zero between launches
 };
 

@@ -145,7 +145,9 @@ __global__ void __launch_bounds__(MultiShape<NP, NM, Real>::THREADS)
     Real* out = reinterpret_cast<Real*>(r.slots ? r.slots + (size_t)(k + 1) * r.slot_bytes : (char*)r.buf[(k + 1) & 1]);
     MultiAcc<NP, NM, Real> acc;
     acc.g = &g;
-    acc.tz0 = (Real)(r.off - r.G * (r.V * (r.t + (double)k * r.dt)));
+    // (rounded as launch_one_step's time and temp_offset: the steps of a call may be split over calls)
+    const double t = k == 0 ? r.t : __dadd_rn(r.t0, __dmul_rn((double)(r.step0 + k), r.dt));
+    acc.tz0 = (Real)__dsub_rn(r.off, __dmul_rn(r.G, __dadd_rn(r.z0, __dmul_rn(r.V, t))));
     for (int u = wid * gridDim.x + blockIdx.x; u < units; u += total) {
       const int y = u / g.segs, sg = u - y * g.segs;
       const int flag = stage_unit<NP, NM, Real>(g, in, box, lane, sg, y);

@@ -98,8 +98,8 @@ ms_status ensure_at_list(ms_ctx* c);   // the anti-trapping work list, when the 
 ms_status refresh_codes(ms_ctx* c);   // segment codes of the current state
 bool multi_steps(const ms_ctx* c);    // ms_step advances this context by the persistent multi-step kernel
 // n steps by that kernel: between the context's two buffers, or (slots not
-// NULL) from state 0 at slots, time t, to states 1 .. n at slots + k slot_bytes.
-ms_status launch_multi_steps(ms_ctx* c, int n, char* slots, size_t slot_bytes, double t);
+// NULL) from state 0 at slots, step `step` and time t, to states 1 .. n at slots + k slot_bytes.
+ms_status launch_multi_steps(ms_ctx* c, int n, char* slots, size_t slot_bytes, int64_t step, double t);
 // The current state was replaced: its codes now, or when they are next read.
 ms_status state_replaced(ms_ctx* c);
 // Parse a fault-injection spec "step:K,code:X" (K >= 0, X a non-zero

@@ -564,7 +564,7 @@ bool multi_steps(const ms_ctx* c) {
          (long long)c->m.nx * c->m.ny <= kMultiMaxCells[c->m.dtype == MS_F64 ? 1 : 0];
 }
 
-ms_status launch_multi_steps(ms_ctx* c, int n, char* slots, size_t slot_bytes, double t) {
+ms_status launch_multi_steps(ms_ctx* c, int n, char* slots, size_t slot_bytes, int64_t step, double t) {
   MultiRun r = {};
   r.buf[0] = c->buf[c->cur];
   r.buf[1] = c->buf[1 - c->cur];
@@ -572,10 +572,13 @@ ms_status launch_multi_steps(ms_ctx* c, int n, char* slots, size_t slot_bytes, d
   r.slot_bytes = slot_bytes;
   r.nsteps = n;
   r.t = t;
-  r.off = c->m.T0 - c->m.T_ref - c->m.G * c->m.z0;
-  r.G = c->m.G;
-  r.V = c->m.V;
+  r.t0 = c->m.t0;
   r.dt = c->m.dt;
+  r.step0 = step;
+  r.off = c->m.T0 - c->m.T_ref;
+  r.G = c->m.G;
+  r.z0 = c->m.z0;
+  r.V = c->m.V;
   r.counters = c->counters;
   cudaError_t e = c->kern->multi(c->args.data(), r, c->lg.sms, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "multi-step launch");
@@ -893,7 +896,7 @@ ms_status ms_step(ms_ctx* c, int64_t n) {
       if (c->adj.every > 0) k = std::min<int64_t>(k, c->adj.every - (c->step - c->adj.first_step) % c->adj.every);
       if (c->diag_every > 0) k = std::min<int64_t>(k, c->diag_every - c->step % c->diag_every);
       if (c->fault_step > c->step) k = std::min<int64_t>(k, c->fault_step - c->step);
-      s = launch_multi_steps(c, (int)k, nullptr, 0, c->t);
+      s = launch_multi_steps(c, (int)k, nullptr, 0, c->step, c->t);
     } else {
       s = launch_one_step(c);
     }
