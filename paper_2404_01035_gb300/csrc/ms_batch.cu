@@ -348,10 +348,16 @@ cudaError_t batch_set_tiles(ms_batch* b, int ty) {
   }
   cudaError_t e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return e;
+  BatchItem* dev_items = static_cast<BatchItem*>(dev_alloc(b->hook, sizeof(BatchItem) * items.size()));
+  if (!dev_items) return cudaErrorMemoryAllocation;   // (the batch keeps the list it has)
   dev_free(b->hook, b->items);
-  b->items = static_cast<BatchItem*>(dev_alloc(b->hook, sizeof(BatchItem) * items.size()));
-  if (!b->items) return cudaErrorMemoryAllocation;
+  b->items = dev_items;
   b->nitems = (int)items.size();
+  if (b->graph) {   // (it reads the old list)
+    cudaGraphExecDestroy(b->graph);
+    b->graph = nullptr;
+  }
+  b->graph_n = -1;
   e = cudaMemcpyAsync(b->items, items.data(), sizeof(BatchItem) * items.size(), cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   int per_sm = 0, dev = 0, sms = 0;
@@ -363,11 +369,6 @@ cudaError_t batch_set_tiles(ms_batch* b, int ty) {
   b->ty = ty;
   b->grid = std::max(1, per_sm) * sms;
   if (b->units) b->grid = std::min(b->grid, std::max(sms, (b->nitems + BatchShape<kBTY>::WARPS - 1) / BatchShape<kBTY>::WARPS));
-  if (b->graph) {
-    cudaGraphExecDestroy(b->graph);
-    b->graph = nullptr;
-  }
-  b->graph_n = -1;
   return cudaSuccess;
 }
 
