@@ -69,7 +69,10 @@ ms_status cuda_fail(ms_ctx* c, cudaError_t e, const char* what) {
 void* dev_alloc(const AllocHook& h, size_t bytes) {
   if (h.alloc) return h.alloc(bytes, h.user);
   void* p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
+  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    cudaGetLastError();   // reported by the caller, not by the next launch
+    return nullptr;
+  }
   return p;
 }
 void dev_free(const AllocHook& h, void* p) {
