@@ -91,7 +91,8 @@ ms_status cuda_fail(ms_ctx* c, cudaError_t e, const char* what);
 ms_status launch_one_step(ms_ctx* c);
 // Device memory for a context that may hold a split step's scratch (more than
 // the state in FP64): where there is no room, the scratch is given back, the
-// context goes on with the fused step, and the allocation is tried again.
+// context goes on with the fused step (if it is not in use already), and the
+// allocation is tried again.
 void* alloc_with_room(ms_ctx* c, size_t bytes);
 ms_status apply_launch(ms_ctx* c, const StepKernel* k, int zchunk);
 ms_status ensure_at_list(ms_ctx* c);   // the anti-trapping work list, when the current is on

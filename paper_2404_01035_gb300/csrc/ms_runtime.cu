@@ -549,17 +549,19 @@ ms_status apply_launch(ms_ctx* c, const StepKernel* k, int zchunk) {
 
 void* alloc_with_room(ms_ctx* c, size_t bytes) {
   void* p = dev_alloc(c->hook, bytes);
-  if (p || !c->kern || !c->kern->split) return p;
-  for (auto* v : step_variants(c->m.dim, c->m.N, c->m.NM, c->m.dtype)) {
-    if (v->split) continue;
-    if (apply_launch(c, v, 0) != MS_OK || cudaStreamSynchronize(c->stream) != cudaSuccess) return nullptr;
-    dev_free(c->hook, c->lg.cells);
-    dev_free(c->hook, c->iface);
-    c->lg.cells = nullptr;
-    c->iface = c->lg.iface = c->lg.iface2 = nullptr;
-    return dev_alloc(c->hook, bytes);
+  if (p || (!c->lg.cells && !c->iface)) return p;
+  if (c->kern->split) {
+    const StepKernel* fused = nullptr;
+    for (auto* v : step_variants(c->m.dim, c->m.N, c->m.NM, c->m.dtype))
+      if (!v->split && !fused) fused = v;
+    if (!fused || apply_launch(c, fused, 0) != MS_OK) return nullptr;
   }
-  return nullptr;
+  if (cudaStreamSynchronize(c->stream) != cudaSuccess) return nullptr;
+  dev_free(c->hook, c->lg.cells);
+  dev_free(c->hook, c->iface);
+  c->lg.cells = nullptr;
+  c->iface = c->lg.iface = c->lg.iface2 = nullptr;
+  return dev_alloc(c->hook, bytes);
 }
 
 bool multi_steps(const ms_ctx* c) {
