@@ -42,7 +42,10 @@ namespace msgb {
 namespace {
 
 struct FftApi {
-  decltype(&cufftPlanMany) plan_many = nullptr;
+  decltype(&cufftCreate) create = nullptr;
+  decltype(&cufftSetAutoAllocation) auto_allocation = nullptr;
+  decltype(&cufftMakePlanMany) make_plan_many = nullptr;
+  decltype(&cufftSetWorkArea) set_work_area = nullptr;
   decltype(&cufftSetStream) set_stream = nullptr;
   decltype(&cufftExecR2C) r2c = nullptr;
   decltype(&cufftExecC2R) c2r = nullptr;
@@ -61,14 +64,18 @@ const FftApi& fft_api() {
     for (const char* n : names)
       if ((h = dlopen(n, RTLD_NOW | RTLD_LOCAL)) != nullptr) break;
     if (!h) return;
-    api.plan_many = reinterpret_cast<decltype(api.plan_many)>(dlsym(h, "cufftPlanMany"));
+    api.create = reinterpret_cast<decltype(api.create)>(dlsym(h, "cufftCreate"));
+    api.auto_allocation = reinterpret_cast<decltype(api.auto_allocation)>(dlsym(h, "cufftSetAutoAllocation"));
+    api.make_plan_many = reinterpret_cast<decltype(api.make_plan_many)>(dlsym(h, "cufftMakePlanMany"));
+    api.set_work_area = reinterpret_cast<decltype(api.set_work_area)>(dlsym(h, "cufftSetWorkArea"));
     api.set_stream = reinterpret_cast<decltype(api.set_stream)>(dlsym(h, "cufftSetStream"));
     api.r2c = reinterpret_cast<decltype(api.r2c)>(dlsym(h, "cufftExecR2C"));
     api.c2r = reinterpret_cast<decltype(api.c2r)>(dlsym(h, "cufftExecC2R"));
     api.d2z = reinterpret_cast<decltype(api.d2z)>(dlsym(h, "cufftExecD2Z"));
     api.z2d = reinterpret_cast<decltype(api.z2d)>(dlsym(h, "cufftExecZ2D"));
     api.destroy = reinterpret_cast<decltype(api.destroy)>(dlsym(h, "cufftDestroy"));
-    api.ok = api.plan_many && api.set_stream && api.r2c && api.c2r && api.d2z && api.z2d && api.destroy;
+    api.ok = api.create && api.auto_allocation && api.make_plan_many && api.set_work_area && api.set_stream && api.r2c &&
+             api.c2r && api.d2z && api.z2d && api.destroy;
   });
   return api;
 }
@@ -386,6 +393,7 @@ void release_state(ms_ctx* c, ElasticState& s) {
   }
   dev_free(c->hook, s.E);
   dev_free(c->hook, s.spec);
+  dev_free(c->hook, s.work);
   s = ElasticState{};
 }
 // The context's buffers and plans of another rank, once the stream is done with them.
@@ -440,22 +448,34 @@ ms_status elastic_setup(ms_ctx* c) {
   int* inb = m.dim == 3 ? inr : inr + 1;
   int* onb = m.dim == 3 ? onr : onr + 1;
   const bool dbl = m.dtype == MS_F64;
+  // the plans' work area (one: they run one after the other) comes from the
+  // context's allocator like the rest, and can have a split step's scratch for room
   cufftHandle p1 = 0, p2 = 0;
-  const bool ok1 = f.plan_many(&p1, rank, n, inb, 1, idist, onb, 1, odist, dbl ? CUFFT_D2Z : CUFFT_R2C, s.rank) ==
-                   CUFFT_SUCCESS;
-  if (ok1) {
-    s.plan_r2c = p1;
-    s.has_r2c = true;
-  }
-  const bool ok2 = ok1 && f.plan_many(&p2, rank, n, onb, 1, odist, inb, 1, idist, dbl ? CUFFT_Z2D : CUFFT_C2R,
-                                      s.rank) == CUFFT_SUCCESS;
-  if (ok2) {
-    s.plan_c2r = p2;
-    s.has_c2r = true;
-  }
-  if (!ok1 || !ok2) {
+  size_t w1 = 0, w2 = 0;
+  bool ok = f.create(&p1) == CUFFT_SUCCESS;
+  s.plan_r2c = p1;
+  s.has_r2c = ok;
+  ok = ok && f.auto_allocation(p1, 0) == CUFFT_SUCCESS &&
+       f.make_plan_many(p1, rank, n, inb, 1, idist, onb, 1, odist, dbl ? CUFFT_D2Z : CUFFT_R2C, s.rank, &w1) ==
+           CUFFT_SUCCESS &&
+       f.create(&p2) == CUFFT_SUCCESS;
+  s.plan_c2r = p2;
+  s.has_c2r = ok;
+  ok = ok && f.auto_allocation(p2, 0) == CUFFT_SUCCESS &&
+       f.make_plan_many(p2, rank, n, onb, 1, odist, inb, 1, idist, dbl ? CUFFT_Z2D : CUFFT_C2R, s.rank, &w2) ==
+           CUFFT_SUCCESS;
+  if (!ok) {
     release_state(c, s);
     return fail(c, MS_ERR_CUDA, "cuFFT plan creation failed");
+  }
+  const size_t work = std::max(w1, w2);
+  if (work > 0 && !(s.work = alloc_with_room(c, work))) {
+    release_state(c, s);
+    return fail(c, MS_ERR_OOM, "cuFFT work area");
+  }
+  if (work > 0 && (f.set_work_area(p1, s.work) != CUFFT_SUCCESS || f.set_work_area(p2, s.work) != CUFFT_SUCCESS)) {
+    release_state(c, s);
+    return fail(c, MS_ERR_CUDA, "cuFFT work area");
   }
   if (f.set_stream(p1, c->stream) != CUFFT_SUCCESS || f.set_stream(p2, c->stream) != CUFFT_SUCCESS) {
     release_state(c, s);

@@ -40,6 +40,7 @@ struct AdjointStore {
 struct ElasticState {
   void* E = nullptr;      // rank fields, dense: eigenstrain amplitudes, then the potentials p_s
   void* spec = nullptr;   // their half spectra
+  void* work = nullptr;   // work area of the plans
   int plan_r2c = 0, plan_c2r = 0;
   int rank = 0;           // independent eigenstrains
   bool has_r2c = false, has_c2r = false;   // the plan handles hold created plans
