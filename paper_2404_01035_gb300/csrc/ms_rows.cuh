@@ -43,7 +43,9 @@ template <int NP, int NM, bool ANISO, bool GG>
 struct RowsShape {
   static constexpr int WARPS = 4;
   static constexpr int THREADS = 32 * WARPS;
-  static constexpr int MIN_BLOCKS = ANISO ? 4 : GG ? 8 : 6;   // 16 / 32 / 24 warps per SM
+  // (isotropic rows with the driving force: 54 us a step of 7 grains in 128^3 with 24 warps
+  // per SM, which spill, 50 with 16)
+  static constexpr int MIN_BLOCKS = GG && !ANISO ? 8 : 4;   // 32 / 16 warps per SM
 };
 
 // Threshold of the simplex projection (phi = max(v - theta, 0)): sorted values,
