@@ -285,7 +285,10 @@ ms_status ms_shift(ms_ctx* ctx, int planes, const double* mu_fill);
 ms_status ms_front(ms_ctx* ctx, int* last_plane);
 
 /* Launch shape: tile (index into ms_tile_shapes) and z-chunk (planes marched
- * per CTA, 3-D only; 0 = automatic; values above 64 are clamped to 64). */
+ * per CTA, 3-D only; 0 = automatic; values above 64 are clamped to 64).  A
+ * 2-D grid of few cells, which takes many steps per launch until then, steps
+ * by one launch of the chosen variant from here on (until ms_tune finds the
+ * multi-step launch the faster again). */
 ms_status ms_set_launch(ms_ctx* ctx, int tile, int zchunk);
 /* Number of tile shapes compiled for this context and their (tx, ty). */
 int ms_tile_count(const ms_ctx* ctx);
@@ -304,7 +307,8 @@ int ms_tile_split(const ms_ctx* ctx, int tile);
 /* Current launch: tile index and z-chunk (either pointer may be NULL). */
 ms_status ms_get_launch(const ms_ctx* ctx, int* tile, int* zchunk);
 
-/* Autotuner: times every compiled tile shape and a set of z-chunk sizes on
+/* Autotuner: times every compiled tile shape and a set of z-chunk sizes, and the
+ * multi-step launch of 2-D grids of few cells, on
  * the current state (the state is saved and restored), keeps the fastest and,
  * when cache_path is not NULL, records it in that JSON file keyed by device,
  * dim, N, K, dtype and grid, reusing a cached entry when present.
@@ -380,13 +384,14 @@ int64_t ms_batch_cells(const ms_batch* b);   /* total cells over all simulations
 /* Strip height of the batched work list: the persistent kernel is compiled for
  * strips of 128 x 4, 128 x 8 (the default) and 128 x 16 cells; a change rebuilds
  * the work list (synchronous) and recaptures the graph at the next
- * ms_batch_step.  MS_ERR_ARG for another height. */
+ * ms_batch_step.  A batch of few cells, which steps by row segments until then,
+ * steps by strips once a height is set.  MS_ERR_ARG for another height. */
 ms_status ms_batch_set_tile(ms_batch* b, int tile_height);
 int ms_batch_tile(const ms_batch* b);        /* current tile height, 0 for NULL */
 /* Autotuner of the batched form: times steps_per_trial steps (after one
- * warm-up launch of the same length) with every compiled tile height on the
- * current states, restores the states (a device copy of all of them is held
- * during the call) and keeps the fastest height; best_ms_per_step (may be
+ * warm-up launch of the same length) with every compiled strip height, and for
+ * batches of few cells by row segments, on the current states, restores the states (a device copy of all of them is held
+ * during the call) and keeps the fastest; best_ms_per_step (may be
  * NULL) receives its time per step.  Synchronous. */
 ms_status ms_batch_tune(ms_batch* b, int steps_per_trial, double* best_ms_per_step);
 

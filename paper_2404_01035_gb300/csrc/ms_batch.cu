@@ -248,6 +248,8 @@ using namespace msgb;
 
 struct ms_batch {
   bool units = false;                   // steps by k_batch_units
+  bool units_fit = false;               // few enough cells for it
+  bool codes_ok = true;                 // the segment codes describe the states (k_batch_units keeps none)
   int nsims = 0, N = 0, NM = 0, dtype = 0;
   std::vector<HostModel> models;
   std::vector<size_t> off;              // byte offset of each simulation's two state buffers
@@ -288,9 +290,9 @@ constexpr int kNBTY = 3;
 // 4 x 400^2 17.8 / 13.5, 64 x 128^2 31.0 / 20.8).
 constexpr long long kBatchUnitCells = 400000;
 
-void* batch_kernel_for(const ms_batch* b, int ty) {
-  return b->units  ? reinterpret_cast<void*>(k_batch_units<2, 1>)
-         : ty == 4    ? reinterpret_cast<void*>(k_batch<2, 1, 4>)
+void* batch_kernel_for(bool units, int ty) {
+  return units      ? reinterpret_cast<void*>(k_batch_units<2, 1>)
+         : ty == 4  ? reinterpret_cast<void*>(k_batch<2, 1, 4>)
          : ty == 16 ? reinterpret_cast<void*>(k_batch<2, 1, 16>)
                     : reinterpret_cast<void*>(k_batch<2, 1, 8>);
 }
@@ -337,14 +339,15 @@ cudaError_t launch_batch(ms_batch* b, int64_t n) {
   return cudaLaunchKernelEx(&cfg, kern, sims, items, b->nitems, b->rows, (int)n, b->parity, b->barrier, b->status);
 }
 
-// Work list and persistent grid for strips of ty rows (one of kBTYs): items are
-// (simulation, strip) pairs in simulation order.  Drops the captured graph.
-cudaError_t batch_set_tiles(ms_batch* b, int ty) {
+// Work list and persistent grid for strips of ty rows (one of kBTYs), or for
+// units: items are (simulation, strip or segment) pairs in simulation order.  Drops
+// the captured graph.
+cudaError_t batch_set_tiles(ms_batch* b, int ty, bool units) {
   std::vector<BatchItem> items;
   for (int i = 0; i < b->nsims; ++i) {
     const HostModel& m = b->models[i];
-    for (int y0 = 0; y0 < m.ny; y0 += b->units ? 1 : ty)
-      for (int sx = 0; (b->units ? 32 : 128) * sx < m.nx; ++sx) items.push_back(BatchItem{i, sx, y0, 0});
+    for (int y0 = 0; y0 < m.ny; y0 += units ? 1 : ty)
+      for (int sx = 0; (units ? 32 : 128) * sx < m.nx; ++sx) items.push_back(BatchItem{i, sx, y0, 0});
   }
   cudaError_t e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return e;
@@ -360,16 +363,29 @@ cudaError_t batch_set_tiles(ms_batch* b, int ty) {
   b->graph_n = -1;
   e = cudaMemcpyAsync(b->items, items.data(), sizeof(BatchItem) * items.size(), cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+  b->ty = ty;
+  b->units = units;
   int per_sm = 0, dev = 0, sms = 0;
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel_for(b, ty), BatchShape<kBTY>::THREADS, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel_for(units, ty), BatchShape<kBTY>::THREADS, 0);
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  b->ty = ty;
   b->grid = std::max(1, per_sm) * sms;
   if (b->units) b->grid = std::min(b->grid, std::max(sms, (b->nitems + BatchShape<kBTY>::WARPS - 1) / BatchShape<kBTY>::WARPS));
   return cudaSuccess;
+}
+
+// Codes of the current states, none of which lets a step keep phi.
+cudaError_t batch_refresh_codes(ms_batch* b) {
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < b->nsims && e == cudaSuccess; ++i) {
+    const size_t half = (b->sbytes[i] + 255) / 256 * 256;
+    e = step_variants(2, 2, 1, 0).front()->codes(static_cast<char*>(b->state) + b->off[i] + b->parity * half, b->models[i],
+                                                 codes_of(b, i, b->parity), b->stream);
+  }
+  b->codes_ok = e == cudaSuccess;
+  return e;
 }
 
 }  // namespace
@@ -430,7 +446,7 @@ ms_status ms_batch_create(int nsims, const ms_grid* grids, int n_phases, int n_c
     tot += 2 * ((sb + 255) / 256 * 256);
     nrows += (size_t)segments(m) * m.ny;
   }
-  b->units = ms_batch_cells(b) <= kBatchUnitCells;
+  b->units_fit = ms_batch_cells(b) <= kBatchUnitCells;
   for (int i = 0; i < nsims; ++i) {
     b->coff.push_back(tot);
     tot += (2 * code_bytes(b->models[i]) + 15) / 16 * 16;
@@ -470,7 +486,7 @@ ms_status ms_batch_create(int nsims, const ms_grid* grids, int n_phases, int n_c
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->sims, hs.data(), sizeof(hs[0]) * nsims, cudaMemcpyHostToDevice, b->stream);
   // work list and persistent grid (every CTA resident at once)
-  if (e == cudaSuccess) e = batch_set_tiles(b, kBTY);
+  if (e == cudaSuccess) e = batch_set_tiles(b, kBTY, b->units_fit);
   if (e != cudaSuccess) {
     std::string m = std::string("batch set-up: ") + cudaGetErrorString(e);
     batch_free(b);
@@ -544,7 +560,8 @@ ms_status ms_batch_step(ms_batch* b, int64_t n) {
   if (n > ((int64_t)1 << 20)) return bfail(b, MS_ERR_BOUNDS, "at most 1048576 steps per ms_batch_step call");
   // the launch (barrier reset + cooperative kernel) is captured once per
   // (n, parity) and replayed
-  cudaError_t e = cudaSuccess;
+  cudaError_t e = b->units || b->codes_ok ? cudaSuccess : batch_refresh_codes(b);
+  if (e != cudaSuccess) return bfail(b, MS_ERR_CUDA, std::string("batch codes: ") + cudaGetErrorString(e));
   if (!b->graph || b->graph_n != n * 2 + b->parity) {
     if (b->graph) {
       cudaGraphExecDestroy(b->graph);
@@ -576,6 +593,7 @@ ms_status ms_batch_step(ms_batch* b, int64_t n) {
   if (e != cudaSuccess) return bfail(b, MS_ERR_CUDA, std::string("batch launch: ") + cudaGetErrorString(e));
   b->parity = (int)((b->parity + n) & 1);
   b->steps_done += n;
+  b->codes_ok = !b->units;
   return MS_OK;
 }
 
@@ -594,8 +612,8 @@ ms_status ms_batch_set_tile(ms_batch* b, int ty) {
   bool ok = false;
   for (int k = 0; k < kNBTY; ++k) ok = ok || kBTYs[k] == ty;
   if (!ok) return bfail(b, MS_ERR_ARG, "tile height must be one of 4, 8, 16");
-  if (ty == b->ty) return MS_OK;
-  cudaError_t e = batch_set_tiles(b, ty);
+  if (ty == b->ty && !b->units) return MS_OK;
+  cudaError_t e = batch_set_tiles(b, ty, false);   // strips, also where units were the default
   if (e != cudaSuccess) return bfail(b, MS_ERR_CUDA, std::string("batch tiles: ") + cudaGetErrorString(e));
   return MS_OK;
 }
@@ -610,14 +628,17 @@ ms_status ms_batch_tune(ms_batch* b, int steps_per_trial, double* best_ms_per_st
   if (!save) return bfail(b, MS_ERR_OOM, "batch tuner: state copy allocation failed");
   const int parity0 = b->parity;
   const int64_t done0 = b->steps_done;
+  const bool codes0 = b->codes_ok;
   cudaError_t e = cudaMemcpyAsync(save, b->state, tot, cudaMemcpyDeviceToDevice, b->stream);
   cudaEvent_t t0 = nullptr, t1 = nullptr;
   if (e == cudaSuccess) e = cudaEventCreate(&t0);
   if (e == cudaSuccess) e = cudaEventCreate(&t1);
   int best = b->ty;
+  bool best_units = b->units;
   float best_ms = 0.0f;
-  for (int k = 0; k < kNBTY && e == cudaSuccess; ++k) {
-    e = batch_set_tiles(b, kBTYs[k]);
+  for (int k = 0; k < kNBTY + (b->units_fit ? 1 : 0) && e == cudaSuccess; ++k) {   // the heights, then the units
+    const bool units = k == kNBTY;
+    e = batch_set_tiles(b, units ? kBTY : kBTYs[k], units);
     if (e != cudaSuccess) break;
     // a warm-up launch captures the graph for this step count
     if (ms_batch_step(b, steps_per_trial) != MS_OK) {
@@ -632,18 +653,20 @@ ms_status ms_batch_tune(ms_batch* b, int steps_per_trial, double* best_ms_per_st
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, t0, t1);
     if (e == cudaSuccess && (k == 0 || ms < best_ms)) {
       best_ms = ms;
-      best = kBTYs[k];
+      best = b->ty;
+      best_units = units;
     }
     // back to the saved state
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->state, save, tot, cudaMemcpyDeviceToDevice, b->stream);
     b->parity = parity0;
     b->steps_done = done0;
+    b->codes_ok = codes0;   // (the copy holds the codes as well)
   }
   if (t0) cudaEventDestroy(t0);
   if (t1) cudaEventDestroy(t1);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   dev_free(b->hook, save);
-  if (e == cudaSuccess) e = batch_set_tiles(b, best);
+  if (e == cudaSuccess) e = batch_set_tiles(b, best, best_units);
   if (e != cudaSuccess) return bfail(b, MS_ERR_CUDA, std::string("batch tuner: ") + cudaGetErrorString(e));
   if (best_ms_per_step) *best_ms_per_step = best_ms / steps_per_trial;
   return ms_batch_sync(b);

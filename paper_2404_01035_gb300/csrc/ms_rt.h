@@ -60,6 +60,7 @@ struct ms_ctx {
   void* buf[2] = {nullptr, nullptr};
   uint8_t* codes[2] = {nullptr, nullptr};   // segment codes of buf[0] / buf[1]
   bool codes_stale = false;                 // the codes do not describe the current state (refresh_codes)
+  bool single_steps = false;                // a variant was chosen (ms_set_launch, ms_tune): one launch of it per step
   unsigned int* iface = nullptr;            // work list of the split step (lazily allocated)
   unsigned int* at_list = nullptr;          // anti-trapping work list (allocated while it is on)
   size_t state_bytes = 0;
@@ -98,7 +99,8 @@ void* alloc_with_room(ms_ctx* c, size_t bytes);
 ms_status apply_launch(ms_ctx* c, const StepKernel* k, int zchunk);
 ms_status ensure_at_list(ms_ctx* c);   // the anti-trapping work list, when the current is on
 ms_status refresh_codes(ms_ctx* c);   // segment codes of the current state
-bool multi_steps(const ms_ctx* c);    // ms_step advances this context by the persistent multi-step kernel
+bool multi_fits(const ms_ctx* c);     // the persistent multi-step kernel takes this context's grid and model
+bool multi_steps(const ms_ctx* c);    // and ms_step advances it so
 // n steps by that kernel: between the context's two buffers, or (slots not
 // NULL) from state 0 at slots, step `step` and time t, to states 1 .. n at slots + k slot_bytes.
 ms_status launch_multi_steps(ms_ctx* c, int n, char* slots, size_t slot_bytes, int64_t step, double t);

@@ -564,10 +564,12 @@ void* alloc_with_room(ms_ctx* c, size_t bytes) {
   return dev_alloc(c->hook, bytes);
 }
 
-bool multi_steps(const ms_ctx* c) {
+bool multi_fits(const ms_ctx* c) {
   return c->kern->multi && !c->m.at && !c->m.el && c->m.noise_amp == 0.0 &&
          (long long)c->m.nx * c->m.ny <= kMultiMaxCells[c->m.dtype == MS_F64 ? 1 : 0];
 }
+
+bool multi_steps(const ms_ctx* c) { return !c->single_steps && multi_fits(c); }
 
 ms_status launch_multi_steps(ms_ctx* c, int n, char* slots, size_t slot_bytes, int64_t step, double t) {
   MultiRun r = {};
@@ -1048,7 +1050,9 @@ ms_status ms_set_launch(ms_ctx* c, int tile, int zchunk) {
   if (!c) return fail(nullptr, MS_ERR_ARG, "ctx is NULL");
   auto v = step_variants(c->m.dim, c->m.N, c->m.NM, c->m.dtype);
   if (tile < 0 || tile >= (int)v.size() || zchunk < 0) return fail(c, MS_ERR_ARG, "bad tile or zchunk");
-  return apply_launch(c, v[tile], zchunk);
+  const ms_status s = apply_launch(c, v[tile], zchunk);
+  if (s == MS_OK) c->single_steps = true;
+  return s;
 }
 
 }  // extern "C"

@@ -34,6 +34,7 @@ std::string cache_key(const ms_ctx* c) {
 
 // Entries are lines of the form
 //   "key": {"tx": 32, "ty": 8, "split": 1, "zchunk": 16, "ms": 0.1},
+// with , "multi": 1 (or 0) where the multi-step kernel was a candidate.
 std::map<std::string, std::string> read_cache(const char* path) {
   std::map<std::string, std::string> m;
   std::ifstream in(path);
@@ -76,8 +77,9 @@ extern "C" ms_status ms_tune(ms_ctx* c, const char* cache_path, int steps, doubl
   if (cache_path) {
     cache = read_cache(cache_path);
     auto it = cache.find(key);
-    int tx, ty, zc, split = 0;
-    if (it != cache.end() && parse_int(it->second, "tx", &tx) && parse_int(it->second, "ty", &ty) &&
+    int tx, ty, zc, split = 0, multi = 0;
+    // (where the multi-step kernel is a candidate, entries that do not say whether it won are no answer)
+    if (it != cache.end() && (!multi_fits(c) || parse_int(it->second, "multi", &multi)) && parse_int(it->second, "tx", &tx) && parse_int(it->second, "ty", &ty) &&
         parse_int(it->second, "zchunk", &zc)) {
       parse_int(it->second, "split", &split);
       for (auto* v : variants)
@@ -89,6 +91,7 @@ extern "C" ms_status ms_tune(ms_ctx* c, const char* cache_path, int steps, doubl
             *best_ms = ms;
           }
           const ms_status as = apply_launch(c, v, zc);
+          if (as == MS_OK) c->single_steps = multi == 0;
           if (as == MS_OK || !v->split) return as;
           break;   // no scratch for the split step that won elsewhere: time the candidates
         }
@@ -116,26 +119,36 @@ extern "C" ms_status ms_tune(ms_ctx* c, const char* cache_path, int steps, doubl
   int best_zc = 1;
   double best_t = 1e300;
   ms_status st = MS_OK;
+  // ms a step of the current launch, or of the multi-step kernel, from the saved state
+  auto trial = [&](bool multi) {
+    auto run = [&](int n) {
+      for (int k; n > 0 && st == MS_OK; n -= k) {
+        k = multi ? std::min(n, kMultiMaxSteps) : 1;
+        st = multi ? launch_multi_steps(c, k, nullptr, 0, c->step, c->t) : launch_one_step(c);
+      }
+    };
+    c->cur = cur0;
+    e = cudaMemcpyAsync(c->buf[c->cur], saved, c->state_bytes, cudaMemcpyDeviceToDevice, c->stream);
+    if ((st = refresh_codes(c)) != MS_OK) return 0.0;
+    c->step = step0;
+    c->t = t0;
+    run(2);
+    cudaEventRecord(ev0, c->stream);
+    run(steps);
+    cudaEventRecord(ev1, c->stream);
+    if (st != MS_OK || (e = cudaEventSynchronize(ev1)) != cudaSuccess) return 0.0;
+    float ms = 0;
+    cudaEventElapsedTime(&ms, ev0, ev1);
+    return (double)ms / steps;
+  };
   for (auto* v : variants) {
     for (int zc : zcs) {
       if ((st = apply_launch(c, v, zc)) != MS_OK) {
         if (v->split) st = MS_OK;   // no scratch for it here: not a candidate
         break;
       }
-      c->cur = cur0;
-      e = cudaMemcpyAsync(c->buf[c->cur], saved, c->state_bytes, cudaMemcpyDeviceToDevice, c->stream);
-      if ((st = refresh_codes(c)) != MS_OK) break;
-      c->step = step0;
-      c->t = t0;
-      for (int i = 0; i < 2 && st == MS_OK; ++i) st = launch_one_step(c);
-      cudaEventRecord(ev0, c->stream);
-      for (int i = 0; i < steps && st == MS_OK; ++i) st = launch_one_step(c);
-      cudaEventRecord(ev1, c->stream);
-      if (st != MS_OK) break;
-      if ((e = cudaEventSynchronize(ev1)) != cudaSuccess) break;
-      float ms = 0;
-      cudaEventElapsedTime(&ms, ev0, ev1);
-      const double per = ms / steps;
+      const double per = trial(false);
+      if (st != MS_OK || e != cudaSuccess) break;
       if (per < best_t) {
         best_t = per;
         best = v;
@@ -143,6 +156,15 @@ extern "C" ms_status ms_tune(ms_ctx* c, const char* cache_path, int steps, doubl
       }
     }
     if (st != MS_OK || e != cudaSuccess) break;
+  }
+  // what a step of a small 2-D grid takes unless a variant is faster (one kernel, whatever the variant)
+  bool multi = false;
+  if (st == MS_OK && e == cudaSuccess && multi_fits(c)) {
+    const double per = trial(true);
+    if (st == MS_OK && e == cudaSuccess && per < best_t) {
+      best_t = per;
+      multi = true;
+    }
   }
   c->cur = cur0;
   cudaMemcpyAsync(c->buf[c->cur], saved, c->state_bytes, cudaMemcpyDeviceToDevice, c->stream);
@@ -158,12 +180,14 @@ extern "C" ms_status ms_tune(ms_ctx* c, const char* cache_path, int steps, doubl
   if (!best) return fail(c, MS_ERR_STATE, "no tile variant ran");
   st = apply_launch(c, best, best_zc);
   if (st != MS_OK) return st;
+  c->single_steps = !multi;
   if (best_ms) *best_ms = best_t;
   if (cache_path) {
     char buf[160];
-    std::snprintf(buf, sizeof buf, "{\"tx\": %d, \"ty\": %d, \"split\": %d, \"zchunk\": %d, \"ms\": %.9g}",
-                  best->tx, best->ty, best->split, c->lg.zchunk, best_t);
+    std::snprintf(buf, sizeof buf, "{\"tx\": %d, \"ty\": %d, \"split\": %d, \"zchunk\": %d, \"ms\": %.9g", best->tx,
+                  best->ty, best->split, c->lg.zchunk, best_t);
     cache[key] = buf;
+    cache[key] += multi_fits(c) ? (multi ? ", \"multi\": 1}" : ", \"multi\": 0}") : "}";
     write_cache(cache_path, cache);
   }
   return MS_OK;
