@@ -506,7 +506,7 @@ ms_status ms_batch_set_fields(ms_batch* b, int sim, const void* phi, const void*
   const size_t half = (b->sbytes[sim] + 255) / 256 * 256;
   char* buf = static_cast<char*>(b->state) + b->off[sim] + b->parity * half;
   cudaError_t e = cudaSuccess;
-  if (on_device || b->stage) {
+  if (on_device ? field_kernel_reaches(phi) && field_kernel_reaches(mu) : b->stage != nullptr) {
     // (host fields: dense copies; strided ones run at a tenth of their rate)
     const void *p = phi, *q = mu;
     if (!on_device) {
@@ -535,9 +535,9 @@ ms_status ms_batch_get_fields(ms_batch* b, int sim, void* phi, void* mu, int on_
   const size_t half = (b->sbytes[sim] + 255) / 256 * 256;
   char* buf = static_cast<char*>(b->state) + b->off[sim] + b->parity * half;
   cudaError_t e = cudaSuccess;
-  if (on_device) {
+  if (on_device && field_kernel_reaches(phi) && field_kernel_reaches(mu)) {
     e = unload_fields(m, buf, phi, mu, b->stream);
-  } else if (b->stage) {   // as the way in
+  } else if (!on_device && b->stage) {   // as the way in
     char* s = static_cast<char*>(b->stage);
     const size_t np = sizeof(float) * m.N * m.nx * m.ny, nm = sizeof(float) * m.NM * m.nx * m.ny;
     e = unload_fields(m, buf, phi ? s : nullptr, mu ? s + np : nullptr, b->stream);

@@ -11,6 +11,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "ms_pointer.h"
 #include "ms_rt.h"
 
 namespace msgb {
@@ -200,11 +201,24 @@ cudaError_t unload(const HostModel& m, const void* padded, void* phi, void* mu, 
   return cudaGetLastError();
 }
 
+static_assert((int)cudaMemoryTypeDevice == kMemDevice && (int)cudaMemoryTypeManaged == kMemManaged, "ms_pointer.h");
+
 }  // namespace
 
 // Row pieces are counted with 32 bits.
 bool field_kernels_fit(const HostModel& m) {
   return (long long)((m.nx + 31) / 32) * m.ny * m.nz < 0x7FFFFFF0ll;
+}
+
+bool field_kernel_reaches(const void* p) {
+  if (!p) return true;
+  cudaPointerAttributes a;
+  int here = 0;
+  if (cudaGetDevice(&here) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return kernel_reaches((int)a.type, a.device, here);
 }
 
 cudaError_t load_fields(const HostModel& m, void* padded, const void* phi, const void* mu, uint8_t* codes,

@@ -126,6 +126,7 @@ cudaError_t fill_ghosts(const HostModel& m, void* buf, int nf, cudaStream_t st);
 // Dense device-resident fields to a padded state with its ghosts and segment
 // codes (codes may be NULL), and back (phi or mu may be NULL); ms_fields.cu.
 bool field_kernels_fit(const HostModel& m);
+bool field_kernel_reaches(const void* p);   // the pointer (NULL: nothing to reach) is one for those kernels
 cudaError_t load_fields(const HostModel& m, void* padded, const void* phi, const void* mu, uint8_t* codes,
                         cudaStream_t st);
 cudaError_t unload_fields(const HostModel& m, const void* padded, void* phi, void* mu, cudaStream_t st);

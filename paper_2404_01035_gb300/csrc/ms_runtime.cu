@@ -839,7 +839,7 @@ ms_status ms_update_params(ms_ctx* c, const ms_params* p) {
 
 ms_status ms_set_fields(ms_ctx* c, const void* phi, const void* mu, int on_device) {
   if (!c || !phi || !mu) return fail(c, MS_ERR_ARG, "ctx, phi and mu are required");
-  if (on_device && field_kernels_fit(c->m)) {
+  if (on_device && field_kernels_fit(c->m) && field_kernel_reaches(phi) && field_kernel_reaches(mu)) {
     // (the multi-step kernel keeps no codes: they wait for a reader)
     c->codes_stale = multi_steps(c);
     MS_CUDA(c, load_fields(c->m, c->buf[c->cur], phi, mu, c->codes_stale ? nullptr : c->codes[c->cur], c->stream));
@@ -860,7 +860,7 @@ ms_status ms_set_fields(ms_ctx* c, const void* phi, const void* mu, int on_devic
 
 ms_status ms_get_fields(ms_ctx* c, void* phi, void* mu, int on_device) {
   if (!c) return fail(nullptr, MS_ERR_ARG, "ctx is NULL");
-  if (on_device && field_kernels_fit(c->m)) {
+  if (on_device && field_kernels_fit(c->m) && field_kernel_reaches(phi) && field_kernel_reaches(mu)) {
     MS_CUDA(c, unload_fields(c->m, c->buf[c->cur], phi, mu, c->stream));
   } else {
     if (phi) MS_CUDA(c, copy_fields(c->m, c->buf[c->cur], 0, c->m.N, nullptr, phi, on_device, c->stream));
