@@ -480,6 +480,25 @@ int default_zchunk(const HostModel& m, const StepKernel& k) {
   return std::min(zc, m.nz);
 }
 
+// In FP32 the split step of many phases sums the pairs in another order than the
+// fused one, which the anti-trapping current makes large differences of (see
+// at_axis): with the current on such models start fused.
+static bool fixed_order(const HostModel& m) { return m.at && m.dtype == MS_F32 && m.N > 3; }
+
+// The split step a context starts with, or NULL.  Where one is compiled (3-D) it is
+// faster than the fused kernels at every size measured on a GB300 (us a step, fused /
+// split, FP32: eutectic 24^3 87 / 17, 150x133x97 158 / 80, 256^3 769 / 196; 8-phase
+// multigrain 24^3 329 / 19, 128^3 1733 / 231, 384^3 3646 / 389).  A grid too
+// large for its work lists, or without memory for them, gets the fused kernel.
+static const StepKernel* default_split(const HostModel& m) {
+  const StepKernel* split = nullptr;
+  if (!fixed_order(m) && (m.dim == 3 ? (m.dtype == MS_F64 ? cells_fit(m) : list_entry_fits(m))
+                                     : m.dtype == MS_F32 && list_entry_fits(m) && (long long)m.nx * m.ny >= kPlaneMinCells))
+    for (auto* v : step_variants(m.dim, m.N, m.NM, m.dtype))
+      if (v->split) split = v;
+  return split;
+}
+
 ms_status ensure_at_list(ms_ctx* c) {
   if (!c->m.at || c->at_list) return MS_OK;
   // count, ticket and one entry per row segment
@@ -752,19 +771,7 @@ ms_status ms_create(const ms_grid* grid, int n_phases, int n_components, const m
     ms_destroy(c);
     return r;
   }
-  // the split step where one is compiled (3-D): faster than the fused
-  // kernels at every size measured on a GB300 (us a step, fused / split, FP32:
-  // eutectic 24^3 87 / 17, 150x133x97 158 / 80, 256^3 769 / 196; 8-phase
-  // multigrain 24^3 329 / 19, 128^3 1733 / 231, 384^3 3646 / 389).  A grid too
-  // large for its work lists, or without memory for them, gets the fused kernel,
-  // and so do many phases with the anti-trapping current in FP32, whose split step
-  // sums the pairs in another order (see at_axis for what that does to the current).
-  const StepKernel* split = nullptr;
-  const bool fixed_order = c->m.at && c->m.dtype == MS_F32 && c->m.N > 3;
-  if (!fixed_order && (c->m.dim == 3 ? (c->m.dtype == MS_F64 ? cells_fit(c->m) : list_entry_fits(c->m))
-                    : c->m.dtype == MS_F32 && list_entry_fits(c->m) && (long long)c->m.nx * c->m.ny >= kPlaneMinCells))
-    for (auto* v : step_variants(c->m.dim, c->m.N, c->m.NM, c->m.dtype))
-      if (v->split) split = v;
+  const StepKernel* split = default_split(c->m);
   s = MS_ERR_UNSUPPORTED;
   if (split) s = apply_launch(c, split, 0);
   if (s != MS_OK) s = apply_launch(c, k, 0);
@@ -831,6 +838,13 @@ ms_status ms_update_params(ms_ctx* c, const ms_params* p) {
     return fail(c, es, msg);
   }
   c->kern->fill(c->args.data(), c->m, c->lg.zchunk, c->status);
+  if (fixed_order(before) != fixed_order(c->m) && !c->single_steps) {   // (nothing was chosen)
+    const StepKernel* k = default_split(c->m);
+    if (!k || apply_launch(c, k, 0) != MS_OK) {
+      k = find_step(c->m.dim, c->m.N, c->m.NM, c->m.dtype, 32, 8);
+      if (k && (es = apply_launch(c, k, 0)) != MS_OK) return es;
+    }
+  }
   // recorded adjoint snapshots belong to the old parameters: the recording
   // restarts at the current step
   if (c->adj.every > 0 && c->step > c->adj.first_step) ms_reset_extra(c);

@@ -87,3 +87,24 @@ def test_many_phases_with_the_current_start_fused():
         sim = Simulation(p.copy(anti_trapping=current), dtype="f32")
         assert sim.tiles()[sim.launch()[0]][2] == split
         sim.close()
+
+
+def test_turning_the_current_on_and_off_with_many_phases():
+    from paper_2404_01035_gb300 import Simulation
+    p = W.small_multiphase(n=12, dim=3, N=8, NM=1, seed=3)
+    out = []
+    for how in ("created", "updated", "chosen"):
+        sim = Simulation(p.copy(anti_trapping=int(how == "created")), dtype="f32")
+        split = [t[2] for t in sim.tiles()]
+        if how == "chosen":
+            sim.set_launch(split.index(1))
+        if how != "created":
+            sim.update_params(anti_trapping=1)
+        assert split[sim.launch()[0]] == (how == "chosen")
+        sim.set_fields(p.phi0, p.mu0)
+        sim.step(10)
+        out.append(sim.get_fields())
+        sim.update_params(anti_trapping=0)
+        assert split[sim.launch()[0]] == 1
+        sim.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
