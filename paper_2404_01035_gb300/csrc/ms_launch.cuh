@@ -160,19 +160,24 @@ void set_launch_args(StepArgs<Real, NP, NM>& g, const HostModel& m, double t, vo
   g.elw = reinterpret_cast<const Real*>(lg.elw);
 }
 
-// A model that uses none of the optional paths of the cell update (rotated
-// pairs, gamma_abc, phi noise, elasticity, grain growth) and in which only
-// the liquid diffuses (the one-sided model: D = 0 in every other phase).  Nor the
-// anti-trapping current: it makes large differences out of the last bits of phi
-// (at_axis), so its models take one form of the update whatever the launch.
-inline bool plain_model(const HostModel& m) {
+// A model that uses none of the optional terms of the cell update (rotated
+// pairs, gamma_abc, phi noise, elasticity, grain growth).
+inline bool bare_model(const HostModel& m) {
   for (int a = 0; a < m.N; ++a)
     for (int b = 0; b < m.N; ++b)
       if (a != b && m.rotated[a][b]) return false;
+  return !m.has_g3 && m.noise_amp == 0.0 && !m.el && !m.gg;
+}
+
+// And in which only the liquid diffuses (the one-sided model: D = 0 in every other
+// phase).  Nor the anti-trapping current: it makes large differences out of the last
+// bits of phi (at_axis), so its models take one form of the mobility whatever the
+// launch.
+inline bool plain_model(const HostModel& m) {
   for (int a = 0; a + 1 < m.N; ++a)
     for (int k = 0; k < m.NM * m.NM; ++k)
       if (m.DX[a][k] != 0.0) return false;
-  return !m.has_g3 && m.noise_amp == 0.0 && !m.el && !m.gg && !m.at;
+  return bare_model(m) && !m.at;
 }
 
 // One boundary energy for every pair and no triple term: the sums over pairs
@@ -263,42 +268,52 @@ cudaError_t launch_split(const CUtensorMap* tm, const CUtensorMap* tmi, const vo
   // the interface kernel fills the anti-trapping list only when the
   // correction runs after this step (launch_at with LISTED)
   if (!m.at) g.at_list = nullptr;
-  // the interface kernels in two builds: every optional path of the cell
-  // update, and none of them (when the model uses none: the common case)
+  // the interface kernels in builds: every optional path of the cell update (0),
+  // none of them (1: when the model uses none, the common case) and, of few phases,
+  // the one that models with the current keep besides it (2: 118 us a step of the
+  // eutectic 150x133x97 on a GB300, 134 with every path)
+  constexpr int kAtFeat = two ? kFeatAll : kFeatSolidD;
   const bool plain = plain_model(m);
+  const int v = plain ? 1 : m.at && bare_model(m) ? 2 : 0;
   const bool ragged = m.nx % 4 != 0;
   auto ks = ragged ? k_gp_stream<NP, NM, TY, true> : k_gp_stream<NP, NM, TY, false>;
-  auto ki = plain ? k_gp_iface<3, NP, NM, float, 0, 0> : k_gp_iface<3, NP, NM, float, 0, kFeatAll>;
+  auto build = [](int v) {
+    return v == 1   ? k_gp_iface<3, NP, NM, float, 0, 0>
+           : v == 2 ? k_gp_iface<3, NP, NM, float, 0, kAtFeat>
+                    : k_gp_iface<3, NP, NM, float, 0, kFeatAll>;
+  };
+  auto ki = build(v);
   auto kf = plain ? k_gp_iface<3, NP, NM, float, two ? 1 : 0, 0>   // only launched when two
                   : k_gp_iface<3, NP, NM, float, two ? 1 : 0, kFeatAll>;
   static bool configured = false;   // attributes are per function, set once
-  static int iface_per_sm[2] = {0, 0}, full_per_sm[2] = {0, 0};   // resident CTAs per SM (all, plain)
+  static int iface_per_sm[3] = {0, 0, 0}, full_per_sm[2] = {0, 0};   // resident CTAs per SM
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(k_gp_stream<NP, NM, TY, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          Ss::SMEM_BYTES);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k_gp_stream<NP, NM, TY, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Ss::SMEM_BYTES);
-    for (int v = 0; v < 2 && e == cudaSuccess; ++v) {
-      auto vi = v ? k_gp_iface<3, NP, NM, float, 0, 0> : k_gp_iface<3, NP, NM, float, 0, kFeatAll>;
-      auto vf = v ? k_gp_iface<3, NP, NM, float, two ? 1 : 0, 0> : k_gp_iface<3, NP, NM, float, two ? 1 : 0, kFeatAll>;
+    for (int v = 0; v < 3 && e == cudaSuccess; ++v) {
+      auto vi = build(v);
       e = cudaFuncSetAttribute(vi, cudaFuncAttributeMaxDynamicSharedMemorySize, Si::SMEM_BYTES);
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(vi, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
       if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&iface_per_sm[v], vi, Si::THREADS, Si::SMEM_BYTES);
+      iface_per_sm[v] = iface_per_sm[v] < 1 ? 1 : iface_per_sm[v];
+    }
+    for (int v = 0; v < 2 && e == cudaSuccess; ++v) {
+      auto vf = v ? k_gp_iface<3, NP, NM, float, two ? 1 : 0, 0> : k_gp_iface<3, NP, NM, float, two ? 1 : 0, kFeatAll>;
       if (two && e == cudaSuccess)
         e = cudaFuncSetAttribute(vf, cudaFuncAttributeMaxDynamicSharedMemorySize, Si::SMEM_BYTES);
       if (two && e == cudaSuccess)
         e = cudaFuncSetAttribute(vf, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
       if (two && e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&full_per_sm[v], vf, Si::THREADS, Si::SMEM_BYTES);
-      iface_per_sm[v] = iface_per_sm[v] < 1 ? 1 : iface_per_sm[v];
       full_per_sm[v] = full_per_sm[v] < 1 ? 1 : full_per_sm[v];
     }
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  const int v = plain ? 1 : 0;
   ks<<<dim3(lg.tiles, lg.zchunks), Ss::NTHREADS, Ss::SMEM_BYTES, st>>>(*tm, g);
   if constexpr (two)
     if (uniform_gamma(m) && !m.at) {   // (with the current, as plain_model: pairs, in the order of the fused kernel)
@@ -308,7 +323,7 @@ cudaError_t launch_split(const CUtensorMap* tm, const CUtensorMap* tmi, const vo
                   : launch_rows<NP, NM, false, false>(g, in, lg.iface_blocks, st);
     }
   ki<<<lg.iface_blocks * iface_per_sm[v], Si::THREADS, Si::SMEM_BYTES, st>>>(*tmi, g);
-  if constexpr (two) kf<<<lg.iface_blocks * full_per_sm[v], Si::THREADS, Si::SMEM_BYTES, st>>>(*tmi, g);
+  if constexpr (two) kf<<<lg.iface_blocks * full_per_sm[plain ? 1 : 0], Si::THREADS, Si::SMEM_BYTES, st>>>(*tmi, g);
   return cudaGetLastError();
 }
 
