@@ -299,9 +299,13 @@ ms_status ms_tile_shape(const ms_ctx* ctx, int tile, int* tx, int* ty);
  * with the full Sec. 2.1 cell update; results agree with the fused variants to
  * FP rounding.  The split variant allocates its scratch once, through the
  * context's allocator, when first selected: in FP32 work lists of 8 bytes per
- * 32-cell row segment, in FP64 per cell a list entry, two bytes, 3 N fluxes and
- * (K-1)^2 mobilities.  A context starts with the split step in 3-D and for
- * binary 2-D FP32 grids from 1.2 million cells, where its scratch can be had.
+ * 32-cell row segment, in FP64 per cell a list entry and two bytes, and 3 N fluxes
+ * and (K-1)^2 mobilities per cell up to 2^22 cells, beyond for an eighth of them (2^22
+ * at least) and four bytes more per cell: 22 bytes a cell for N = 3, K = 3, 34 for N =
+ * 8, K = 2 on large grids, beside 80 and 144 of state.  A context starts with the split
+ * step in 3-D and for binary 2-D FP32 grids from 1.2 million cells, where its scratch
+ * can be had, so creating it costs that memory; it is given back when an allocation of
+ * the context itself finds no room.
  * 0 for a fused variant, -1 for a bad index. */
 int ms_tile_split(const ms_ctx* ctx, int tile);
 /* Current launch: tile index and z-chunk (either pointer may be NULL). */

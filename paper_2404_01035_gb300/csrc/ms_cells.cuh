@@ -30,16 +30,20 @@ struct CellsScratch {
   unsigned int* list;      // [0] count, [1] exit ticket, [2..] listed cells (linear index)
   uint8_t* mask;           // phases in the block of listed cell k
   uint8_t* kind;           // per cell: pure phase + 1 where bulk, 0 where listed
-  Real* J;                 // [3 NP][cells] upper-face fluxes of listed cells, [D NP + a]
-  Real* M;                 // [NM NM][cells] mobilities of listed cells
-  long long cells;
+  unsigned int* pos;       // per cell: its place in the list where listed; NULL: fluxes are stored by cell
+  Real* J;                 // [3 NP][slots] upper-face fluxes of listed cells, [D NP + a], by cell or place
+  Real* M;                 // [NM NM][slots] mobilities of listed cells
+  long long slots;         // (see cell_slots)
+  // where the fluxes of listed cell i, the k-th, are, or (place past the end) none are stored
+  __device__ __forceinline__ unsigned int slot(unsigned int i, unsigned int k) const { return pos ? k : i; }
+  __device__ __forceinline__ unsigned int slot_of(long long i) const { return pos ? pos[i] : (unsigned int)i; }
 };
 
 // (cells_scratch_bytes in ms_runtime.cu adds up the same parts)
 template <class Real>
 CellsScratch<Real> cells_layout(void* base, const HostModel& m) {
   CellsScratch<Real> c;
-  const size_t cells = (size_t)m.nx * m.ny * m.nz;
+  const size_t cells = (size_t)m.nx * m.ny * m.nz, slots = cell_slots(cells);
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
   char* p = static_cast<char*>(base);
   c.list = reinterpret_cast<unsigned int*>(p);
@@ -48,10 +52,12 @@ CellsScratch<Real> cells_layout(void* base, const HostModel& m) {
   p += up(cells);
   c.kind = reinterpret_cast<uint8_t*>(p);
   p += up(cells);
+  c.pos = slots < cells ? reinterpret_cast<unsigned int*>(p) : nullptr;
+  if (c.pos) p += up(cells * 4);
   c.J = reinterpret_cast<Real*>(p);
-  p += up(3 * m.N * cells * sizeof(Real));
+  p += up(3 * m.N * slots * sizeof(Real));
   c.M = reinterpret_cast<Real*>(p);
-  c.cells = (long long)cells;
+  c.slots = (long long)slots;
   return c;
 }
 
@@ -146,6 +152,7 @@ __global__ void __launch_bounds__(256) k_c_scan(const __grid_constant__ StepArgs
   if (want) {
     c.list[2 + k] = cell;
     c.mask[k] = (uint8_t)present;
+    if (c.pos) c.pos[cell] = k;
   }
 }
 
@@ -177,7 +184,8 @@ __global__ void __launch_bounds__(64) k_c_faces(const __grid_constant__ StepArgs
   const long long plane = (long long)g.nyp * g.pitch;
   const auto dp = plain_prm<Real, NP, NM>(g);
   for (unsigned int k = blockIdx.x * 64u + threadIdx.x; k < count; k += gridDim.x * 64u) {
-    const unsigned int i = c.list[2 + k], r = i / (unsigned int)g.nx;
+    const unsigned int i = c.list[2 + k], r = i / (unsigned int)g.nx, at = c.slot(i, k);
+    if (at >= c.slots) break;   // (later cells have none either)
     const int x = (int)(i - r * g.nx), y = (int)(r % (unsigned int)g.ny), z = (int)(r / (unsigned int)g.ny);
     PadAcc<NP, NM, Real> A{in + (long long)(z + g.zoff) * plane + (long long)(y + 1) * g.pitch + x + g.xoff,
                            g.fstride, plane, g.pitch, c.mask[k], &g};
@@ -185,46 +193,55 @@ __global__ void __launch_bounds__(64) k_c_faces(const __grid_constant__ StepArgs
     Real J[NP];
     face_flux<3, 0, NP, NM, Real, Real>(A, g, dp, A.m, 1, tan, J);
 #pragma unroll
-    for (int a = 0; a < NP; ++a) c.J[a * c.cells + i] = J[a];
+    for (int a = 0; a < NP; ++a) c.J[a * c.slots + at] = J[a];
     face_flux<3, 1, NP, NM, Real, Real>(A, g, dp, A.m, 1, tan, J);
 #pragma unroll
-    for (int a = 0; a < NP; ++a) c.J[(NP + a) * c.cells + i] = J[a];
+    for (int a = 0; a < NP; ++a) c.J[(NP + a) * c.slots + at] = J[a];
     face_flux<3, 2, NP, NM, Real, Real>(A, g, dp, A.m, 1, tan, J);
 #pragma unroll
-    for (int a = 0; a < NP; ++a) c.J[(2 * NP + a) * c.cells + i] = J[a];
+    for (int a = 0; a < NP; ++a) c.J[(2 * NP + a) * c.slots + at] = J[a];
     if (!g.gg) {
       Real ph[NP], M[NM * NM];
 #pragma unroll
       for (int a = 0; a < NP; ++a) ph[a] = A.phi(a, 0, 0, 0);
       cell_mobility<NP, NM>(ph, g.DX, M);
 #pragma unroll
-      for (int q = 0; q < NM * NM; ++q) c.M[q * c.cells + i] = M[q];
+      for (int q = 0; q < NM * NM; ++q) c.M[q * c.slots + at] = M[q];
     }
   }
 }
 
 // One axis of a listed cell: adds (J_upper - J_lower) / dx to divJ and the mu
-// flux through both faces to div.  `pos`, n, bc: the cell's index along the
-// axis, its extent and boundary code; `step`: linear cells to its neighbour.
+// flux through both faces to div.  `at`: where the cell's own fluxes are; `pos`, n,
+// bc: its index along the axis, its extent and boundary code; `step`: linear cells to
+// its neighbour.  What no cell stores (no cell below a boundary face, no place left)
+// is evaluated here.
 template <int D, int NP, int NM, class Real, class DP>
 __device__ __forceinline__ void axis_terms(const StepArgs<Real, NP, NM>& g, const CellsScratch<Real>& c,
-                                           const PadAcc<NP, NM, Real>& A, const DP& dp, unsigned int i, int pos, int n,
+                                           const PadAcc<NP, NM, Real>& A, const DP& dp, unsigned int i, unsigned int at, int pos, int n,
                                            int bc, long long step, bool tan, const Real* Mc, const Real* mc, Real* divJ,
                                            Real* div) {
   // linear index of the lower / upper neighbour where it is a cell of the grid
   const bool lo_in = pos > 0 || bc == 3, hi_in = pos < n - 1 || bc == 3;
   const long long lo = (long long)i + (pos > 0 ? -step : (long long)(n - 1) * step);
   const long long hi = (long long)i + (pos < n - 1 ? step : -(long long)(n - 1) * step);
-  Real Jl[NP];
-  if (!lo_in) {
-    face_flux<3, D, NP, NM, Real, Real>(A, g, dp, A.m, 0, tan, Jl);   // a face of the boundary: no cell below it
-  } else {
-    const bool stored = c.kind[lo] == 0;
+  // flux of the lower (0) / upper (1) face: from its place, zero (listed = false:
+  // the face lies in a pure block), or evaluated
+  auto flux = [&](int side, bool listed, unsigned int place, bool eval, Real* J) {
+    if (eval) {
+      face_flux<3, D, NP, NM, Real, Real>(A, g, dp, A.m, side, tan, J);
+    } else {
 #pragma unroll
-    for (int a = 0; a < NP; ++a) Jl[a] = stored ? c.J[(D * NP + a) * c.cells + lo] : Real(0);
-  }
+      for (int a = 0; a < NP; ++a) J[a] = listed ? c.J[(D * NP + a) * c.slots + place] : Real(0);
+    }
+  };
+  const bool below = lo_in && c.kind[lo] == 0;
+  const unsigned int pl = below ? c.slot_of(lo) : 0u;
+  Real Jl[NP], Ju[NP];
+  flux(0, below, pl, !lo_in || pl >= c.slots, Jl);
+  flux(1, true, at, at >= c.slots, Ju);
 #pragma unroll
-  for (int a = 0; a < NP; ++a) divJ[a] += (c.J[(D * NP + a) * c.cells + i] - Jl[a]) * g.inv_dx;
+  for (int a = 0; a < NP; ++a) divJ[a] += (Ju[a] - Jl[a]) * g.inv_dx;
   if (g.gg) return;
 #pragma unroll
   for (int sd = 0; sd < 2; ++sd) {
@@ -232,15 +249,16 @@ __device__ __forceinline__ void axis_terms(const StepArgs<Real, NP, NM>& g, cons
     const long long nb = sd ? hi : lo;
     const int d = sd ? 1 : -1;
     Real Mn[NM * NM];
-    if (!inside) {
+    const int kd = inside ? c.kind[nb] : 0;
+    const unsigned int pn = inside && kd == 0 ? c.slot_of(nb) : 0u;
+    if (!inside || pn >= c.slots) {
       Real ph[NP];
 #pragma unroll
       for (int a = 0; a < NP; ++a) ph[a] = A.phi(a, D == 0 ? d : 0, D == 1 ? d : 0, D == 2 ? d : 0);
       cell_mobility<NP, NM>(ph, g.DX, Mn);
     } else {
-      const int kd = c.kind[nb];
 #pragma unroll
-      for (int q = 0; q < NM * NM; ++q) Mn[q] = kd == 0 ? c.M[q * c.cells + nb] : g.DX[kd - 1][q];
+      for (int q = 0; q < NM * NM; ++q) Mn[q] = kd == 0 ? c.M[q * c.slots + pn] : g.DX[kd - 1][q];
     }
 #pragma unroll
     for (int r = 0; r < NM; ++r)
@@ -260,7 +278,7 @@ __global__ void __launch_bounds__(64) k_c_update(const __grid_constant__ StepArg
   const long long plane = (long long)g.nyp * g.pitch;
   const auto dp = plain_prm<Real, NP, NM>(g);
   for (unsigned int k = blockIdx.x * 64u + threadIdx.x; k < count; k += gridDim.x * 64u) {
-    const unsigned int i = c.list[2 + k], r = i / (unsigned int)g.nx;
+    const unsigned int i = c.list[2 + k], r = i / (unsigned int)g.nx, at = c.slot(i, k);
     const int x = (int)(i - r * g.nx), y = (int)(r % (unsigned int)g.ny), z = (int)(r / (unsigned int)g.ny);
     PadAcc<NP, NM, Real> A{in + (long long)(z + g.zoff) * plane + (long long)(y + 1) * g.pitch + x + g.xoff,
                            g.fstride, plane, g.pitch, c.mask[k], &g};
@@ -278,10 +296,11 @@ __global__ void __launch_bounds__(64) k_c_update(const __grid_constant__ StepArg
       div[q] = Real(0);
     }
 #pragma unroll
-    for (int q = 0; q < NM * NM; ++q) Mc[q] = g.gg ? Real(0) : c.M[q * c.cells + i];
-    axis_terms<0>(g, c, A, dp, i, x, g.nx, g.bc[0], 1ll, tan, Mc, mc, divJ, div);
-    axis_terms<1>(g, c, A, dp, i, y, g.ny, g.bc[1], (long long)g.nx, tan, Mc, mc, divJ, div);
-    axis_terms<2>(g, c, A, dp, i, z, g.nz, g.bc[2], (long long)g.nx * g.ny, tan, Mc, mc, divJ, div);
+    for (int q = 0; q < NM * NM; ++q) Mc[q] = g.gg || at >= c.slots ? Real(0) : c.M[q * c.slots + at];
+    if (!g.gg && at >= c.slots) cell_mobility<NP, NM>(ph, g.DX, Mc);
+    axis_terms<0>(g, c, A, dp, i, at, x, g.nx, g.bc[0], 1ll, tan, Mc, mc, divJ, div);
+    axis_terms<1>(g, c, A, dp, i, at, y, g.ny, g.bc[1], (long long)g.nx, tan, Mc, mc, divJ, div);
+    axis_terms<2>(g, c, A, dp, i, at, z, g.nz, g.bc[2], (long long)g.nx * g.ny, tan, Mc, mc, divJ, div);
     Real gcr[NP][3];
 #pragma unroll
     for (int a = 0; a < NP; ++a) {

@@ -169,6 +169,14 @@ struct DiagKernel {
 };
 
 size_t cells_scratch_bytes(const HostModel& m);   // of the cell-list step
+// Listed cells whose fluxes and mobilities the cell-list step stores (8 (3 N +
+// (K-1)^2) bytes each): all there can be on grids of up to 2^22 cells, an eighth of
+// the cells beyond, where the rest, if that many are ever listed, evaluate the faces
+// of a neighbour without a place themselves.  By cell instead, the scratch of a
+// 3-D FP64 context was more than its state (110 bytes a cell beside 80 for N = 3, 206
+// beside 144 for N = 8), now 22 and 34.
+constexpr size_t kCellSlots = size_t(1) << 22;
+inline size_t cell_slots(size_t cells) { return cells <= kCellSlots ? cells : cells / 8 > kCellSlots ? cells / 8 : kCellSlots; }
 // The cell-list step indexes cells with 32 bits.
 inline bool cells_fit(const HostModel& m) { return (long long)m.nx * m.ny * m.nz < 0xFFFFFFF0ll; }
 

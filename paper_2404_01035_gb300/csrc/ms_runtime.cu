@@ -516,7 +516,9 @@ ms_status ensure_at_list(ms_ctx* c) {
 size_t cells_scratch_bytes(const HostModel& m) {
   const size_t cells = (size_t)m.nx * m.ny * m.nz, s = m.dtype == MS_F64 ? 8 : 4;
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
-  return up((cells + 2) * 4) + 2 * up(cells) + up(3 * m.N * cells * s) + up((size_t)m.NM * m.NM * cells * s);
+  const size_t slots = cell_slots(cells);
+  return up((cells + 2) * 4) + 2 * up(cells) + (slots < cells ? up(cells * 4) : 0) + up(3 * m.N * slots * s) +
+         up((size_t)m.NM * m.NM * slots * s);
 }
 
 ms_status apply_launch(ms_ctx* c, const StepKernel* k, int zchunk) {
