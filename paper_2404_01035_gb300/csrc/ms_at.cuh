@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(AtShape<Real>::THREADS, AtShape<Real>::MIN_BLO
       Real pn[NP], h[NP];
 #pragma unroll
       for (int a = 0; a < NP; ++a) pn[a] = A.phin(a, 0, 0, 0);
-      interp_h<NP>(pn, h);
+      interp_h<NP, true>(pn, h);
       Real chi[NM * NM], rhs[NM], dmu[NM], mn[NM];
 #pragma unroll
       for (int q = 0; q < NM * NM; ++q) {

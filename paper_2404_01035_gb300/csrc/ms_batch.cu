@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(BatchShape<R>::THREADS, BatchShape<R>::MIN_BLO
 #pragma unroll
         for (int p = 0; p < StepArgs<float, NP, NM>::P; ++p) dp.delta[p] = g.delta[p];
         float pn[NP], mn[NM];
-        gp_cell<2, NP, NM, float, float>(acc, g, dp, y + g.zorg, 0ull, pn, mn);
+        gp_cell<2, NP, NM, float, float, MultiAcc<NP, NM, float>, kFeatNoAt>(acc, g, dp, y + g.zorg, 0ull, pn, mn);
         uint32_t nzm = 0, one = 0;
 #pragma unroll
         for (int q = 0; q < NP; ++q) {

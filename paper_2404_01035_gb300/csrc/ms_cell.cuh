@@ -48,7 +48,9 @@ constexpr int kFeatNoise = 4;    // phi noise
 constexpr int kFeatElastic = 8;  // elastic potentials added to psi
 constexpr int kFeatGG = 16;      // grain growth (no chemical driving force, mu held)
 constexpr int kFeatSolidD = 32;  // phases other than the liquid diffuse (else M = h_l D^l chi^l)
-constexpr int kFeatAll = 63;
+constexpr int kFeatAt = 64;      // models with the anti-trapping current run it (see WrittenOut)
+constexpr int kFeatAll = 127;
+constexpr int kFeatNoAt = kFeatAll & ~kFeatAt;
 
 // g = dA/dq of the unrotated anisotropic pair, evaluated in real arithmetic
 // through the factorisation g_i = 2 gamma a_c q_i (a_c + 16 delta (q_i^2 /
@@ -293,57 +295,82 @@ __device__ __forceinline__ void face_flux_pair(const Acc& A, const StepArgs<floa
 
 // Cell mobilities M = sum_a h_a D^a chi^a of the two neighbours along axis d
 // at once (low half: the -d neighbour, high half: the +d one), paired FP32.
-template <int DIM, int NP, int NM, class Acc>
+template <int DIM, int NP, int NM, bool AT, class Acc>
 __device__ __forceinline__ void mobility_pair(const Acc& A, const StepArgs<float, NP, NM>& g, int d, F2* M) {
   const Off<DIM> m = unit<DIM>(d, -1), p = unit<DIM>(d, 1);
   F2 f[NP];
 #pragma unroll
   for (int a = 0; a < NP; ++a) f[a] = f2(A.phi(a, m.x, m.y, m.z), A.phi(a, p.x, p.y, p.z));
-  F2 e1 = f[0], e2 = f2s(0.0f), run = f[0];
+  F2 h[NP];
+  if constexpr (WrittenOut<float, AT>::value && NP <= 3) {
 #pragma unroll
-  for (int a = 1; a < NP; ++a) {
-    e1 = e1 + f[a];
-    e2 = fma2(f[a], run, e2);
-    run = run + f[a];
+    for (int a = 0; a < NP; ++a) {   // p^2 (3 - 2 p) + 2 p (product of the others)
+      h[a] = f[a] * f[a] * fma2(f2s(-2.0f), f[a], f2s(3.0f));
+      if constexpr (NP == 3) h[a] = fma2(f2s(2.0f) * f[a], f[(a + 1) % 3] * f[(a + 2) % 3], h[a]);
+    }
+  } else {
+    F2 e1 = f[0], e2 = f2s(0.0f), run = f[0];
+#pragma unroll
+    for (int a = 1; a < NP; ++a) {
+      e1 = e1 + f[a];
+      e2 = fma2(f[a], run, e2);
+      run = run + f[a];
+    }
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+      const F2 rest = e2 - f[a] * (e1 - f[a]);
+      const F2 p2 = f[a] * f[a];
+      h[a] = f2s(3.0f) * p2 - f2s(2.0f) * p2 * f[a] + f2s(2.0f) * f[a] * rest;
+    }
   }
 #pragma unroll
-  for (int a = 0; a < NP; ++a) {
-    const F2 rest = e2 - f[a] * (e1 - f[a]);
-    const F2 p2 = f[a] * f[a];
-    const F2 h = f2s(3.0f) * p2 - f2s(2.0f) * p2 * f[a] + f2s(2.0f) * f[a] * rest;
+  for (int a = 0; a < NP; ++a)
 #pragma unroll
-    for (int k = 0; k < NM * NM; ++k) M[k] = a == 0 ? h * f2s(g.DX[0][k]) : fma2(h, f2s(g.DX[a][k]), M[k]);
-  }
+    for (int k = 0; k < NM * NM; ++k) M[k] = a == 0 ? h[0] * f2s(g.DX[0][k]) : fma2(h[a], f2s(g.DX[a][k]), M[k]);
 }
 
 // As mobility_pair when only the liquid (phase NP-1) diffuses: M = h_l D^l
 // chi^l, h_l = phi_l^2 (3 - 2 phi_l) + 2 phi_l sum_{b<c<l} phi_b phi_c.
-template <int DIM, int NP, int NM, class Acc>
+template <int DIM, int NP, int NM, bool AT, class Acc>
 __device__ __forceinline__ void mobility_pair_liquid(const Acc& A, const StepArgs<float, NP, NM>& g, int d, F2* M) {
   const Off<DIM> m = unit<DIM>(d, -1), p = unit<DIM>(d, 1);
   constexpr int L = NP - 1;
   F2 f[NP];
 #pragma unroll
   for (int a = 0; a < NP; ++a) f[a] = f2(A.phi(a, m.x, m.y, m.z), A.phi(a, p.x, p.y, p.z));
-  F2 rest = f2s(0.0f), run = f[0];
+  F2 h;
+  if constexpr (WrittenOut<float, AT>::value) {
+    h = f[L] * f[L] * fma2(f2s(-2.0f), f[L], f2s(3.0f));
+    if constexpr (NP > 2) {
+      F2 rest = f[0] * f[1], run = f[0] + f[1];
 #pragma unroll
-  for (int b = 1; b < L; ++b) {
-    rest = fma2(f[b], run, rest);
-    run = run + f[b];
+      for (int b = 2; b < L; ++b) {
+        rest = fma2(f[b], run, rest);
+        run = run + f[b];
+      }
+      h = fma2(f2s(2.0f) * f[L], rest, h);
+    }
+  } else {
+    F2 rest = f2s(0.0f), run = f[0];
+#pragma unroll
+    for (int b = 1; b < L; ++b) {
+      rest = fma2(f[b], run, rest);
+      run = run + f[b];
+    }
+    const F2 p2 = f[L] * f[L];
+    h = f2s(3.0f) * p2 - f2s(2.0f) * p2 * f[L] + f2s(2.0f) * f[L] * rest;
   }
-  const F2 p2 = f[L] * f[L];
-  const F2 h = f2s(3.0f) * p2 - f2s(2.0f) * p2 * f[L] + f2s(2.0f) * f[L] * rest;
 #pragma unroll
   for (int k = 0; k < NM * NM; ++k) M[k] = h * f2s(g.DX[L][k]);
 }
 
 // The cell's own mobility when only the liquid diffuses (scalar).
-template <int NP, int NM, class Real>
+template <int NP, int NM, class Real, bool AT>
 __device__ __forceinline__ void mobility_liquid(const Real* ph, const StepArgs<Real, NP, NM>& g, Real* M) {
   constexpr int L = NP - 1;
   const Real p2 = ph[L] * ph[L];
   Real h;
-  if constexpr (WrittenOut<Real>::value) {
+  if constexpr (WrittenOut<Real, AT>::value) {
     h = Real(3) * p2 - Real(2) * p2 * ph[L];
     if constexpr (NP > 2) {
       Real rest = ph[0] * ph[1], run = ph[0] + ph[1];
@@ -543,8 +570,9 @@ __device__ __forceinline__ void phase_update(const StepArgs<Real, NP, NM>& g, co
   // dh_a/dphi_a = 6 phi_a (1 - phi_a) + 2 rest_a; dh_b/dphi_a = 2 phi_b sum_{c
   // != a, b} phi_c, which two phases do not have and three share as 2 phi_b phi_c
   // (written out so where WrittenOut says)
+  constexpr bool kWritten = WrittenOut<S, (FEAT & kFeatAt) != 0>::value;
   S rest[NP], e1 = ph[0], e2 = S(Real(0));
-  if constexpr (WrittenOut<S>::value) {
+  if constexpr (kWritten) {
     other_products<NP>(ph, rest);
     if constexpr (NP > 3) {
 #pragma unroll
@@ -564,13 +592,13 @@ __device__ __forceinline__ void phase_update(const StepArgs<Real, NP, NM>& g, co
 #pragma unroll
   for (int a = 0; a < NP; ++a) {
     S P;
-    if constexpr (WrittenOut<S>::value && NP <= 3) {
+    if constexpr (kWritten && NP <= 3) {
       S dh = Real(6) * ph[a] - Real(6) * (ph[a] * ph[a]);
       if constexpr (NP > 2) dh = dh + Real(2) * rest[a];
       P = psi[a] * dh;
       if constexpr (NP == 3) P += (psi[(a + 1) % 3] + psi[(a + 2) % 3]) * (Real(2) * rest[a]);
     } else {
-      const S r2 = WrittenOut<S>::value ? rest[a] : e2 - ph[a] * (e1 - ph[a]);
+      const S r2 = kWritten ? rest[a] : e2 - ph[a] * (e1 - ph[a]);
       P = psi[a] * (Real(6) * ph[a] - Real(6) * (ph[a] * ph[a]) + Real(2) * r2);
 #pragma unroll
       for (int b = 0; b < NP; ++b) {
@@ -592,17 +620,17 @@ __device__ __forceinline__ void phase_update(const StepArgs<Real, NP, NM>& g, co
 // the mu step of Eq. (Mu_explicit_temperature) with chi(h(phi^{n+1})),
 // c^a(mu^n) and dh/dt, dT/dt as one-step differences.  bulk: phi^{n+1} =
 // phi^n (no dh term).
-template <int NP, int NM, class Real, class S>
+template <int NP, int NM, class Real, class S, bool AT = false>
 __device__ __forceinline__ void mu_update(const StepArgs<Real, NP, NM>& g, const S* ph, const S* pn, const S* mc,
                                           const S* div, Real s, bool bulk, S* mn) {
   S h_new[NP];
-  interp_h<NP>(pn, h_new);
+  interp_h<NP, AT>(pn, h_new);
   S rhs[NM];
 #pragma unroll
   for (int i = 0; i < NM; ++i) rhs[i] = g.dt * div[i];
   if (!bulk) {
     S h_old[NP];
-    interp_h<NP>(ph, h_old);
+    interp_h<NP, AT>(ph, h_old);
 #pragma unroll
     for (int a = 0; a < NP; ++a) {
       S dh = h_new[a] - h_old[a];
@@ -647,6 +675,7 @@ template <int DIM, int NP, int NM, class Real, class S, class Acc, int FEAT = kF
 __device__ __forceinline__ void gp_cell(const Acc& A, const StepArgs<Real, NP, NM>& g,
                                         const DiffPrm<S, NP*(NP - 1) / 2>& dp, int kz, unsigned long long gcell,
                                         S* pn, S* mn) {
+  constexpr bool AT = (FEAT & kFeatAt) != 0;
   const bool gg = (FEAT & kFeatGG) && g.gg;
   S ph[NP];
 #pragma unroll
@@ -708,9 +737,9 @@ __device__ __forceinline__ void gp_cell(const Acc& A, const StepArgs<Real, NP, N
     S phc[NP];
 #pragma unroll
     for (int a = 0; a < NP; ++a) phc[a] = A.phi(a, 0, 0, 0);
-    mobility_liquid<NP, NM, Real>(phc, g, Mc);
+    mobility_liquid<NP, NM, Real, AT>(phc, g, Mc);
   } else {
-    A.mobility(0, 0, 0, Mc);
+    A.template mobility<AT>(0, 0, 0, Mc);
   }
   S div[NM];
 #pragma unroll
@@ -725,9 +754,9 @@ __device__ __forceinline__ void gp_cell(const Acc& A, const StepArgs<Real, NP, N
       const Off<DIM> m = unit<DIM>(d, -1), p = unit<DIM>(d, 1);
       F2 Mn[NM * NM];
       if constexpr (FEAT & kFeatSolidD)
-        mobility_pair<DIM, NP, NM>(A, g, d, Mn);
+        mobility_pair<DIM, NP, NM, AT>(A, g, d, Mn);
       else
-        mobility_pair_liquid<DIM, NP, NM>(A, g, d, Mn);
+        mobility_pair_liquid<DIM, NP, NM, AT>(A, g, d, Mn);
 #pragma unroll
       for (int i = 0; i < NM; ++i) {
 #pragma unroll
@@ -751,9 +780,9 @@ __device__ __forceinline__ void gp_cell(const Acc& A, const StepArgs<Real, NP, N
           S phn[NP];
 #pragma unroll
           for (int a = 0; a < NP; ++a) phn[a] = A.phi(a, o.x, o.y, o.z);
-          mobility_liquid<NP, NM, Real>(phn, g, Mn);
+          mobility_liquid<NP, NM, Real, AT>(phn, g, Mn);
         } else {
-          A.mobility(o.x, o.y, o.z, Mn);
+          A.template mobility<AT>(o.x, o.y, o.z, Mn);
         }
 #pragma unroll
         for (int i = 0; i < NM; ++i) {
@@ -766,7 +795,7 @@ __device__ __forceinline__ void gp_cell(const Acc& A, const StepArgs<Real, NP, N
       }
     }
   }
-  mu_update<NP, NM, Real, S>(g, ph, pn, mc, div, s, bulk, mn);
+  mu_update<NP, NM, Real, S, AT>(g, ph, pn, mc, div, s, bulk, mn);
 }
 
 // ------------------------------------------------------------------------

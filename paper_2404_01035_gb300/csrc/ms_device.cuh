@@ -472,15 +472,15 @@ __device__ __forceinline__ void pair_grad(const S* q, Real gam2, const S& del, b
   }
 }
 
-// Scalars whose interpolation and driving force are written out for two and
-// three phases: doubles and dual numbers, whose arithmetic bounds their kernels
+// Where interpolation and driving force are written out for two and three phases
 // (FP64 dendrite 128^2 on a GB300 16.4 -> 13.6 us a step, an FP32 reverse step 15.0
-// -> 13.7).  Plain FP32 keeps one form for every phase count: its kernels do not
-// gain, and the anti-trapping current, which switches on at |grad phi|^2 >= 1e-12,
-// makes differences of 1e-2 in single cells out of another rounding of phi.
-template <class S>
+// -> 13.7, 100 FP32 steps of 256^2 560 -> 510).  Not in the FP32 kernels that models
+// with the anti-trapping current run (AT): the current switches on at |grad phi|^2
+// >= 1e-12 and makes differences of 1e-2 in single cells out of another rounding of
+// phi, so they all keep the one form for every phase count.
+template <class S, bool AT>
 struct WrittenOut {
-  static constexpr bool value = !std::is_same<S, float>::value;
+  static constexpr bool value = !(AT && std::is_same<S, float>::value);
 };
 
 // sum_{b<c; b,c != a} phi_b phi_c for every a: nothing for two phases, the
@@ -508,10 +508,10 @@ __device__ __forceinline__ void other_products(const S* ph, S* rest) {
 }
 
 // Interpolation h_a = phi_a^2 (3 - 2 phi_a) + 2 phi_a sum_{b<c; b,c != a} phi_b phi_c (Eq. hphi).
-template <int NP, class S>
+template <int NP, bool AT = false, class S>
 __device__ __forceinline__ void interp_h(const S* ph, S* h) {
   using R = decltype(val(ph[0]));
-  if constexpr (WrittenOut<S>::value) {
+  if constexpr (WrittenOut<S, AT>::value) {
     S rest[NP];
     other_products<NP>(ph, rest);
 #pragma unroll
@@ -539,10 +539,10 @@ __device__ __forceinline__ void interp_h(const S* ph, S* h) {
 }
 
 // Cell mobility M = sum_a h_a(phi) D^a chi^a (Eq. Mass_conservation).
-template <int NP, int NM, class S, class DXT>
+template <int NP, int NM, bool AT = false, class S, class DXT>
 __device__ __forceinline__ void cell_mobility(const S* ph, const DXT& DX, S* M) {
   S h[NP];
-  interp_h<NP>(ph, h);
+  interp_h<NP, AT>(ph, h);
 #pragma unroll
   for (int k = 0; k < NM * NM; ++k) {
     M[k] = h[0] * DX[0][k];

@@ -268,31 +268,33 @@ cudaError_t launch_split(const CUtensorMap* tm, const CUtensorMap* tmi, const vo
   // the interface kernel fills the anti-trapping list only when the
   // correction runs after this step (launch_at with LISTED)
   if (!m.at) g.at_list = nullptr;
-  // the interface kernels in builds: every optional path of the cell update (0),
-  // none of them (1: when the model uses none, the common case) and, of few phases,
-  // the one that models with the current keep besides it (2: 118 us a step of the
-  // eutectic 150x133x97 on a GB300, 134 with every path)
-  constexpr int kAtFeat = two ? kFeatAll : kFeatSolidD;
+  // the interface kernels in builds: every optional path of the cell update (0) or
+  // none of them (1: when the model uses none, the common case), and the same for
+  // models with the current, which always keep the general mobility (2: every path,
+  // 3: that alone; 118 us a step of the eutectic 150x133x97 on a GB300, 134 with
+  // every path).  Many phases have one form: 0 for 2 and 3.
+  constexpr int kNoAt = two ? kFeatAll : kFeatNoAt, kAtBare = two ? kFeatAll : kFeatSolidD | kFeatAt;
   const bool plain = plain_model(m);
-  const int v = plain ? 1 : m.at && bare_model(m) ? 2 : 0;
+  const int v = plain ? 1 : !m.at ? 0 : bare_model(m) ? 3 : 2;
   const bool ragged = m.nx % 4 != 0;
   auto ks = ragged ? k_gp_stream<NP, NM, TY, true> : k_gp_stream<NP, NM, TY, false>;
   auto build = [](int v) {
     return v == 1   ? k_gp_iface<3, NP, NM, float, 0, 0>
-           : v == 2 ? k_gp_iface<3, NP, NM, float, 0, kAtFeat>
-                    : k_gp_iface<3, NP, NM, float, 0, kFeatAll>;
+           : v == 3 ? k_gp_iface<3, NP, NM, float, 0, kAtBare>
+           : v == 2 ? k_gp_iface<3, NP, NM, float, 0, kFeatAll>
+                    : k_gp_iface<3, NP, NM, float, 0, kNoAt>;
   };
   auto ki = build(v);
   auto kf = plain ? k_gp_iface<3, NP, NM, float, two ? 1 : 0, 0>   // only launched when two
                   : k_gp_iface<3, NP, NM, float, two ? 1 : 0, kFeatAll>;
   static bool configured = false;   // attributes are per function, set once
-  static int iface_per_sm[3] = {0, 0, 0}, full_per_sm[2] = {0, 0};   // resident CTAs per SM
+  static int iface_per_sm[4] = {0, 0, 0, 0}, full_per_sm[2] = {0, 0};   // resident CTAs per SM
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(k_gp_stream<NP, NM, TY, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          Ss::SMEM_BYTES);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k_gp_stream<NP, NM, TY, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Ss::SMEM_BYTES);
-    for (int v = 0; v < 3 && e == cudaSuccess; ++v) {
+    for (int v = 0; v < 4 && e == cudaSuccess; ++v) {
       auto vi = build(v);
       e = cudaFuncSetAttribute(vi, cudaFuncAttributeMaxDynamicSharedMemorySize, Si::SMEM_BYTES);
       if (e == cudaSuccess)

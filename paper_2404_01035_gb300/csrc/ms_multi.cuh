@@ -36,11 +36,12 @@ struct MultiAcc {
   __device__ __forceinline__ Real phi(int a, int dx, int dy, int) const { return s[a * (3 * Sh::BX) + dy * Sh::BX + dx]; }
   __device__ __forceinline__ Real mu(int i, int dx, int dy, int) const { return phi(NP + i, dx, dy, 0); }
   __device__ __forceinline__ uint32_t mask() const { return stencil_mask<2, NP>(*this); }
+  template <bool AT>
   __device__ __forceinline__ void mobility(int dx, int dy, int dz, Real* M) const {
     Real ph[NP];
 #pragma unroll
     for (int a = 0; a < NP; ++a) ph[a] = phi(a, dx, dy, dz);
-    cell_mobility<NP, NM>(ph, g->DX, M);
+    cell_mobility<NP, NM, AT>(ph, g->DX, M);
   }
 };
 template <int NP, int NM, class Real>
@@ -104,7 +105,7 @@ __device__ __forceinline__ void update_unit(const StepArgs<Real, NP, NM>& g, Mul
     if (flag != 0)
       bulk_cell<2, NP, NM, Real>(acc, g, flag - 1, pn, mn);
     else
-      gp_cell<2, NP, NM, Real, Real>(acc, g, dp, y + g.zorg, 0ull, pn, mn);
+      gp_cell<2, NP, NM, Real, Real, MultiAcc<NP, NM, Real>, kFeatNoAt>(acc, g, dp, y + g.zorg, 0ull, pn, mn);
     store_cell_to<2>(g, out, x, y, 0, pn, mn);
   }
 }

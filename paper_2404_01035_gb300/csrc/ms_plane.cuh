@@ -51,11 +51,12 @@ struct PlaneAcc {
   __device__ __forceinline__ float phi(int a, int dx, int dy, int) const { return __ldg(s + a * fs + dy * pitch + dx); }
   __device__ __forceinline__ float mu(int i, int dx, int dy, int) const { return phi(NP + i, dx, dy, 0); }
   __device__ __forceinline__ uint32_t mask() const { return stencil_mask<2, NP>(*this); }
+  template <bool AT>
   __device__ __forceinline__ void mobility(int dx, int dy, int dz, float* M) const {
     float ph[NP];
 #pragma unroll
     for (int a = 0; a < NP; ++a) ph[a] = phi(a, dx, dy, dz);
-    cell_mobility<NP, NM>(ph, g->DX, M);
+    cell_mobility<NP, NM, AT>(ph, g->DX, M);
   }
 };
 

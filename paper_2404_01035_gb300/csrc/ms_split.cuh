@@ -413,11 +413,12 @@ struct BoxAcc {
   __device__ __forceinline__ Real phi(int a, int dx, int dy, int dz) const { return ld(a, dx, dy, dz); }
   __device__ __forceinline__ Real mu(int i, int dx, int dy, int dz) const { return ld(NP + i, dx, dy, dz); }
   __device__ __forceinline__ uint32_t mask() const { return wmask; }
+  template <bool AT>
   __device__ __forceinline__ void mobility(int dx, int dy, int dz, Real* M) const {
     Real ph[NP];
 #pragma unroll
     for (int a = 0; a < NP; ++a) ph[a] = phi(a, dx, dy, dz);
-    cell_mobility<NP, NM>(ph, g->DX, M);
+    cell_mobility<NP, NM, AT>(ph, g->DX, M);
   }
 };
 

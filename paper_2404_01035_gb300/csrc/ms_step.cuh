@@ -135,11 +135,12 @@ struct SmemAcc {
   }
   __device__ __forceinline__ uint32_t mask() const { return stencil_mask<DIM, NP>(*this); }
   // cell mobility M = sum_a h_a D^a chi^a of a neighbour, from its phi
+  template <bool AT>
   __device__ __forceinline__ void mobility(int dx, int dy, int dz, Real* M) const {
     Real ph[NP];
 #pragma unroll
     for (int a = 0; a < NP; ++a) ph[a] = phi(a, dx, dy, dz);
-    cell_mobility<NP, NM>(ph, g->DX, M);
+    cell_mobility<NP, NM, AT>(ph, g->DX, M);
   }
 };
 
