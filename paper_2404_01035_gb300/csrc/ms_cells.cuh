@@ -215,8 +215,8 @@ __global__ void __launch_bounds__(64) k_c_faces(const __grid_constant__ StepArgs
 // flux through both faces to div.  `at`: where the cell's own fluxes are; `pos`, n,
 // bc: its index along the axis, its extent and boundary code; `step`: linear cells to
 // its neighbour.  What no cell stores (no cell below a boundary face, no place left)
-// is evaluated here.
-template <int D, int NP, int NM, class Real, class DP>
+// is evaluated here.  PLACES: there may be places for some cells only.
+template <int D, bool PLACES, int NP, int NM, class Real, class DP>
 __device__ __forceinline__ void axis_terms(const StepArgs<Real, NP, NM>& g, const CellsScratch<Real>& c,
                                            const PadAcc<NP, NM, Real>& A, const DP& dp, unsigned int i, unsigned int at, int pos, int n,
                                            int bc, long long step, bool tan, const Real* Mc, const Real* mc, Real* divJ,
@@ -236,10 +236,10 @@ __device__ __forceinline__ void axis_terms(const StepArgs<Real, NP, NM>& g, cons
     }
   };
   const bool below = lo_in && c.kind[lo] == 0;
-  const unsigned int pl = below ? c.slot_of(lo) : 0u;
+  const unsigned int pl = !below ? 0u : PLACES ? c.slot_of(lo) : (unsigned int)lo;
   Real Jl[NP], Ju[NP];
-  flux(0, below, pl, !lo_in || pl >= c.slots, Jl);
-  flux(1, true, at, at >= c.slots, Ju);
+  flux(0, below, pl, !lo_in || (PLACES && pl >= c.slots), Jl);
+  flux(1, true, at, PLACES && at >= c.slots, Ju);
 #pragma unroll
   for (int a = 0; a < NP; ++a) divJ[a] += (Ju[a] - Jl[a]) * g.inv_dx;
   if (g.gg) return;
@@ -250,8 +250,8 @@ __device__ __forceinline__ void axis_terms(const StepArgs<Real, NP, NM>& g, cons
     const int d = sd ? 1 : -1;
     Real Mn[NM * NM];
     const int kd = inside ? c.kind[nb] : 0;
-    const unsigned int pn = inside && kd == 0 ? c.slot_of(nb) : 0u;
-    if (!inside || pn >= c.slots) {
+    const unsigned int pn = !inside || kd != 0 ? 0u : PLACES ? c.slot_of(nb) : (unsigned int)nb;
+    if (!inside || (PLACES && pn >= c.slots)) {
       Real ph[NP];
 #pragma unroll
       for (int a = 0; a < NP; ++a) ph[a] = A.phi(a, D == 0 ? d : 0, D == 1 ? d : 0, D == 2 ? d : 0);
@@ -270,7 +270,7 @@ __device__ __forceinline__ void axis_terms(const StepArgs<Real, NP, NM>& g, cons
   }
 }
 
-template <int NP, int NM, class Real>
+template <int NP, int NM, class Real, bool PLACES>
 __global__ void __launch_bounds__(64) k_c_update(const __grid_constant__ StepArgs<Real, NP, NM> g,
                                                  const Real* __restrict__ in,
                                                  const __grid_constant__ CellsScratch<Real> c) {
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(64) k_c_update(const __grid_constant__ StepArg
   const long long plane = (long long)g.nyp * g.pitch;
   const auto dp = plain_prm<Real, NP, NM>(g);
   for (unsigned int k = blockIdx.x * 64u + threadIdx.x; k < count; k += gridDim.x * 64u) {
-    const unsigned int i = c.list[2 + k], r = i / (unsigned int)g.nx, at = c.slot(i, k);
+    const unsigned int i = c.list[2 + k], r = i / (unsigned int)g.nx, at = PLACES ? c.slot(i, k) : i;
     const int x = (int)(i - r * g.nx), y = (int)(r % (unsigned int)g.ny), z = (int)(r / (unsigned int)g.ny);
     PadAcc<NP, NM, Real> A{in + (long long)(z + g.zoff) * plane + (long long)(y + 1) * g.pitch + x + g.xoff,
                            g.fstride, plane, g.pitch, c.mask[k], &g};
@@ -296,11 +296,11 @@ __global__ void __launch_bounds__(64) k_c_update(const __grid_constant__ StepArg
       div[q] = Real(0);
     }
 #pragma unroll
-    for (int q = 0; q < NM * NM; ++q) Mc[q] = g.gg || at >= c.slots ? Real(0) : c.M[q * c.slots + at];
-    if (!g.gg && at >= c.slots) cell_mobility<NP, NM>(ph, g.DX, Mc);
-    axis_terms<0>(g, c, A, dp, i, at, x, g.nx, g.bc[0], 1ll, tan, Mc, mc, divJ, div);
-    axis_terms<1>(g, c, A, dp, i, at, y, g.ny, g.bc[1], (long long)g.nx, tan, Mc, mc, divJ, div);
-    axis_terms<2>(g, c, A, dp, i, at, z, g.nz, g.bc[2], (long long)g.nx * g.ny, tan, Mc, mc, divJ, div);
+    for (int q = 0; q < NM * NM; ++q) Mc[q] = g.gg || (PLACES && at >= c.slots) ? Real(0) : c.M[q * c.slots + at];
+    if (PLACES && !g.gg && at >= c.slots) cell_mobility<NP, NM>(ph, g.DX, Mc);
+    axis_terms<0, PLACES>(g, c, A, dp, i, at, x, g.nx, g.bc[0], 1ll, tan, Mc, mc, divJ, div);
+    axis_terms<1, PLACES>(g, c, A, dp, i, at, y, g.ny, g.bc[1], (long long)g.nx, tan, Mc, mc, divJ, div);
+    axis_terms<2, PLACES>(g, c, A, dp, i, at, z, g.nz, g.bc[2], (long long)g.nx * g.ny, tan, Mc, mc, divJ, div);
     Real gcr[NP][3];
 #pragma unroll
     for (int a = 0; a < NP; ++a) {

@@ -367,20 +367,25 @@ cudaError_t launch_cells(const CUtensorMap*, const CUtensorMap*, const void* in,
   const CellsScratch<Real> c = cells_layout<Real>(lg.cells, m);
   const Real* p = reinterpret_cast<const Real*>(in);
   auto kf = k_c_faces<NP, NM, Real>;
-  auto ku = k_c_update<NP, NM, Real>;
-  static int faces_per_sm = 0, update_per_sm = 0;   // resident CTAs per SM
-  if (update_per_sm == 0) {
+  // few phases: a build for grids with a place for every cell (206 registers, 244
+  // with the other form: 1.5% of a step of the eutectic 67x50x61)
+  constexpr bool kOne = NP > kSparseK;
+  const int v = kOne || c.pos ? 1 : 0;
+  auto ku = v ? k_c_update<NP, NM, Real, true> : k_c_update<NP, NM, Real, kOne>;
+  static int faces_per_sm = 0, update_per_sm[2] = {0, 0};   // resident CTAs per SM
+  if (update_per_sm[1] == 0) {
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&faces_per_sm, kf, 64, 0);
-    int u = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&u, ku, 64, 0);
+    int u[2] = {0, 0};
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&u[0], k_c_update<NP, NM, Real, kOne>, 64, 0);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&u[1], k_c_update<NP, NM, Real, true>, 64, 0);
     if (e != cudaSuccess) return e;
     faces_per_sm = faces_per_sm < 1 ? 1 : faces_per_sm;
-    update_per_sm = u < 1 ? 1 : u;
+    for (int k = 0; k < 2; ++k) update_per_sm[k] = u[k] < 1 ? 1 : u[k];
   }
   const long long nseg = (long long)segments(m) * m.ny * m.nz;
   k_c_scan<NP, NM, Real><<<(unsigned)((nseg + 7) / 8), 256, 0, st>>>(g, p, c);
   kf<<<lg.sms * faces_per_sm, 64, 0, st>>>(g, p, c);
-  ku<<<lg.sms * update_per_sm, 64, 0, st>>>(g, p, c);
+  ku<<<lg.sms * update_per_sm[v], 64, 0, st>>>(g, p, c);
   return cudaGetLastError();
 }
 
