@@ -110,9 +110,11 @@ __device__ __forceinline__ void update_unit(const StepArgs<Real, NP, NM>& g, Mul
   }
 }
 
-// Arrive and wait until `target` arrivals are in; false after the time limit.
-__device__ __forceinline__ bool multi_barrier(unsigned int* counter, unsigned int target) {
+__device__ __forceinline__ void multi_arrive(unsigned int* counter) {
   asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
+}
+// Waits until `target` arrivals are in; false after the time limit.
+__device__ __forceinline__ bool multi_wait(unsigned int* counter, unsigned int target) {
   unsigned int v;
   unsigned long long t0 = 0;
   for (;;) {
@@ -127,12 +129,18 @@ __device__ __forceinline__ bool multi_barrier(unsigned int* counter, unsigned in
   }
 }
 
+__device__ __forceinline__ bool multi_barrier(unsigned int* counter, unsigned int target) {
+  multi_arrive(counter);
+  return multi_wait(counter, target);
+}
+
 template <int NP, int NM, class Real>
 __global__ void __launch_bounds__(MultiShape<NP, NM, Real>::THREADS)
     k_gp_multi(const __grid_constant__ StepArgs<Real, NP, NM> g, const __grid_constant__ MultiRun r) {
   using Sh = MultiShape<NP, NM, Real>;
   __shared__ Real s_box[Sh::WARPS][Sh::BOX];
   __shared__ int s_ok;
+  __shared__ Real s_tz0;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   Real* const box = s_box[wid];
   const int units = g.segs * g.ny, total = gridDim.x * Sh::WARPS;
@@ -141,14 +149,15 @@ __global__ void __launch_bounds__(MultiShape<NP, NM, Real>::THREADS)
 #pragma unroll
   for (int p = 0; p < StepArgs<Real, NP, NM>::P; ++p) dp.delta[p] = g.delta[p];
   bool ok = true;
+  // T - T_ref at the origin of the last axis (rounded as temp_offset)
+  auto origin = [&](double t) { return (Real)__dsub_rn(r.off, __dmul_rn(r.G, __dadd_rn(r.z0, __dmul_rn(r.V, t)))); };
+  Real tz0 = origin(r.t);
   for (int k = 0; k < r.nsteps; ++k) {
     const Real* in = reinterpret_cast<const Real*>(r.slots ? r.slots + (size_t)k * r.slot_bytes : (char*)r.buf[k & 1]);
     Real* out = reinterpret_cast<Real*>(r.slots ? r.slots + (size_t)(k + 1) * r.slot_bytes : (char*)r.buf[(k + 1) & 1]);
     MultiAcc<NP, NM, Real> acc;
     acc.g = &g;
-    // (rounded as launch_one_step's time and temp_offset: the steps of a call may be split over calls)
-    const double t = k == 0 ? r.t : __dadd_rn(r.t0, __dmul_rn((double)(r.step0 + k), r.dt));
-    acc.tz0 = (Real)__dsub_rn(r.off, __dmul_rn(r.G, __dadd_rn(r.z0, __dmul_rn(r.V, t))));
+    acc.tz0 = tz0;
     for (int u = wid * gridDim.x + blockIdx.x; u < units; u += total) {
       const int y = u / g.segs, sg = u - y * g.segs;
       const int flag = stage_unit<NP, NM, Real>(g, in, box, lane, sg, y);
@@ -157,9 +166,17 @@ __global__ void __launch_bounds__(MultiShape<NP, NM, Real>::THREADS)
     }
     if (k + 1 == r.nsteps) break;
     __syncthreads();
-    if (threadIdx.x == 0) s_ok = multi_barrier(&r.counters[0], (unsigned int)(k + 1) * gridDim.x) ? 1 : 0;
+    if (threadIdx.x == 0) {
+      multi_arrive(&r.counters[0]);
+      // the time of step k + 1, rounded as launch_one_step's (the steps of a call may be
+      // split over calls); by one thread while it waits: every FP64 instruction of a
+      // warp holds the pipe for 16 cycles (all warps: 5.4 us a step at 256^2, 5.0 so)
+      s_tz0 = origin(__dadd_rn(r.t0, __dmul_rn((double)(r.step0 + k + 1), r.dt)));
+      s_ok = multi_wait(&r.counters[0], (unsigned int)(k + 1) * gridDim.x) ? 1 : 0;
+    }
     __syncthreads();
     ok = s_ok != 0;
+    tz0 = s_tz0;
     if (!ok) {
       if (threadIdx.x == 0) atomicOr(g.status, kStatusTimeout);
       break;
