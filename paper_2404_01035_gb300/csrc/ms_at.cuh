@@ -57,7 +57,7 @@ template <class Real>
 struct AtShape {
   static constexpr int THREADS = 128;
   static constexpr int WARPS = THREADS / 32;
-  static constexpr int MIN_BLOCKS = sizeof(Real) == 4 ? 6 : 2;   // FP32: 80 registers, 24 warps per SM
+  static constexpr int MIN_BLOCKS = sizeof(Real) == 4 ? 6 : 2;   // FP32: 24 warps per SM
 };
 
 // dt times the normal component along axis d of j_at_i (the rates are taken
@@ -244,7 +244,9 @@ __global__ void __launch_bounds__(256) k_at_list(const __grid_constant__ StepArg
 // (whole rows; L1 holds what the offsets share).  The last CTA to finish clears
 // the list (ticket), so the launches replay from a graph.  FP32 evaluates the
 // two faces of an axis together.  What bounds it: the latency of its loads, so 24
-// warps per SM: eutectic 150x133x97 on a GB300 takes 40 us a step, 53 with 16
+// warps per SM, also where the builds for that many spill a little (us a step of all
+// kernels, 24 / 20 / 16 warps: three phases 133 / 135 / 142, two 67 / 69 / 71, eight
+// 1616 / 1662 / 1681): eutectic 150x133x97 on a GB300 takes 42 us a step, 53 with 16
 // warps, 63 with the block staged element by element in shared memory, every face
 // on its own and the rows without a current corrected too.
 template <int DIM, int NP, int NM, class Real>

@@ -13,7 +13,7 @@
 // the rows are other SMs' stores of the previous phase.
 //
 // What bounds it: the two barriers and the latency of each phase.  32 simulations
-// of 64^2 .. 512^2 (3.2 M cells) on a GB300: 19.6 us a step; 60 us with every tile
+// of 64^2 .. 512^2 (3.2 M cells) on a GB300: 20.4 us a step; 60 us with every tile
 // staged through a TMA ring, a cell per thread, and phi tested cell by cell.
 #include <cuda.h>
 #include <cuda_runtime.h>

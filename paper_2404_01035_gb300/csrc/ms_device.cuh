@@ -470,7 +470,7 @@ __device__ __forceinline__ void pair_grad(const S* q, Real gam2, const S& del, b
 
 // Where interpolation and driving force are written out for two and three phases
 // (FP64 dendrite 128^2 on a GB300 16.4 -> 13.6 us a step, an FP32 reverse step 15.0
-// -> 13.7, 100 FP32 steps of 256^2 560 -> 510).  Not in the FP32 kernels that models
+// -> 13.7, binary FP32 150x133x97 42.6 -> 40.7).  Not in the FP32 kernels that models
 // with the anti-trapping current run (AT): the current switches on at |grad phi|^2
 // >= 1e-12 and makes differences of 1e-2 in single cells out of another rounding of
 // phi, so they all keep the one form for every phase count.

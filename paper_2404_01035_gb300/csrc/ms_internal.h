@@ -132,14 +132,14 @@ struct StepKernel {
 
 // Cells up to which a 2-D grid is stepped by the persistent multi-step kernel
 // (FP32, FP64): us a step on a GB300, one launch a step / multi-step: FP32
-// binary 128^2 6.2 / 3.9, 256^2 6.2 / 5.0, 384^2 6.2 / 8.8, ternary 200^2
-// 10.3 / 9.4, 400^2 18.7 / 23.7; FP64 binary 128^2 30.9 / 16.4, 512^2 62 / 41,
-// 900^2 99 / 116, ternary 512^2 424 / 408.
+// binary 128^2 6.2 / 3.7, 256^2 6.2 / 4.5, 384^2 6.2 / 7.7, ternary 200^2
+// 10.3 / 9.0, 400^2 18.3 / 20.3; FP64 binary 128^2 24.6 / 11.6, 512^2 50 / 20,
+// 900^2 77 / 51, ternary 512^2 344 / 307.  (The FP64 line stands below the crossover.)
 constexpr long long kMultiMaxCells[2] = {80000, 300000};
 // Cells from which a binary 2-D FP32 context starts with the split step: its two
-// launches cost 14 us however small the grid (us a step on a GB300, fused / split,
-// a dendrite: 290^2 6.2 / 14.4, 700^2 10.3 / 15.4, 1000^2 16.4 / 16.4, 1537x1411
-// 28.9 / 18.6, 2048^2 51.4 / 28.3).
+// launches cost 13 us however small the grid (us a step on a GB300, fused / split,
+// a dendrite: 290^2 6.2 / 13.4, 700^2 10.9 / 16.3, 1000^2 16.4 / 16.4, 1537x1411
+// 29.4 / 18.6, 2048^2 52.7 / 28.2).
 constexpr long long kPlaneMinCells = 1200000;
 // Steps of one multi-step launch at most (the barrier counts steps x CTAs in 32 bits).
 constexpr int kMultiMaxSteps = 1 << 16;

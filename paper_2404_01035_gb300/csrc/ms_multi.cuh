@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(MultiShape<NP, NM, Real>::THREADS)
       multi_arrive(&r.counters[0]);
       // the time of step k + 1, rounded as launch_one_step's (the steps of a call may be
       // split over calls); by one thread while it waits: every FP64 instruction of a
-      // warp holds the pipe for 16 cycles (all warps: 5.4 us a step at 256^2, 5.0 so)
+      // warp holds the pipe for 16 cycles (by all warps: 5.4 us a step at 256^2, 4.5 so)
       s_tz0 = origin(__dadd_rn(r.t0, __dmul_rn((double)(r.step0 + k + 1), r.dt)));
       s_ok = multi_wait(&r.counters[0], (unsigned int)(k + 1) * gridDim.x) ? 1 : 0;
     }

@@ -3,8 +3,8 @@
 // pure phase, which reads and writes mu alone (phi only where the output buffer
 // does not hold it, as in the 3-D split step), and an interface kernel, a warp
 // per remaining segment.  What bounds them is latency, of the loads and of the
-// dependent arithmetic of a row.  Binary, 1537 x 1411 on a GB300: 6.8 + 9.0 us, 28.4
-// us in the fused kernel.  One kernel that keeps each CTA's list in shared memory
+// dependent arithmetic of a row.  Binary, 1537 x 1411 on a GB300: 6.8 + 9.1 us (18.6 a
+// step with the gaps), 29.4 us in the fused kernel.  One kernel that keeps each CTA's list in shared memory
 // takes 33: few CTAs hold all of an interface.  With three phases and interfaces
 // over half of the grid the fused kernel is faster (1400^2 150 us, this form 220).
 #pragma once

@@ -29,9 +29,9 @@
 // anisotropic pairs the instruction cache (so one code path for rotated and
 // unrotated pairs, and builds of their own for grain growth).  Measured on a
 // GB300, interface rows of one step, by pairs / with the sums taken face by
-// face / here: 8 grains filling 192^3 (isotropic) 5846 / 340 / 233 us; 7 rotated
-// grains in 128^3 with an eigenstrain - / 141 / 109 us; in 512^3 (few interface
-// rows) 698 / 186 / 142 us.  Models with unequal gamma, the triple term or the
+// face / here: 8 grains filling 192^3 (isotropic) 5846 / 340 / 222 us; 7 rotated
+// grains in 128^3 with an eigenstrain - / 141 / 111 us; in 512^3 (few interface
+// rows) 698 / 186 / 144 us.  Models with unequal gamma, the triple term or the
 // anti-trapping current keep the pair form (k_gp_iface).
 #pragma once
 
