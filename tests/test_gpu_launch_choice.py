@@ -27,6 +27,7 @@ def _profiler_is_up():
     for _ in range(10):
         if "kernel" in _kernels(lambda: torch.ones(1000, device="cuda").add_(1.0)):
             return
+    pytest.skip("the profiler names no kernels here")
 
 
 def _problem(N, nx, ny):
